@@ -22,8 +22,7 @@ constexpr uint64_t kMaxPos = (1ull << 18) - 1;   // full blocks per request
 constexpr uint64_t kMaxStep = (1ull << 31) - 1;  // steps (step tags keep 32 bits)
 constexpr int kTableWays = 8;    // native prefix table: 8 x 16 B entries per 128 B bucket
 constexpr int kClaimWays = 4;    // per-step claim map: 4 x 32 B entries per bucket
-constexpr int kRadixBits = 8;
-constexpr int kRadixBins = 1 << kRadixBits;
+constexpr int kRadixBins = 256;  // byte digits of the split list's finish
 constexpr int kSegBlocks = 32;   // blocks of one chunk half (a warp's width)
 constexpr int kChunkBlocks = 2 * kSegBlocks;  // blocks of one prompt hashed by one warp (a chunk)
 constexpr int kBmChunk = 256;    // bitmap words per CTA of the id-list compaction
@@ -90,13 +89,13 @@ struct Ctl {
   int64_t T, nblocks, nsegs;
   int64_t pinned, n_inval, total_claims, avail, need, nfree, ftake, mvict;
   int64_t hist_new;
-  int64_t n_evicted, n_alloc, n_victims_marked;
+  int64_t n_evicted, n_alloc;
   int64_t m_fb;            // prefixshield: victims left to the global fallback
   int32_t sel_ntie, sel_k; // prefixshield tie bookkeeping
   int64_t lst_n;              // members of the select's split list
   uint32_t ticket;         // last-block-done counter for the radix passes and the split
   int32_t nlaunch;         // kernels launched by the step (conditional bodies run or not)
-  int32_t wide_nrows;      // segments counted by the last first-digit pass
+  int32_t pad2;
   int32_t internal_error;  // an invariant of the step failed (reported, never expected)
   // indexed queues (PS_FLAG_INDEXED_QUEUES)
   int32_t lg_buf;          // entry buffer holding the logs (0 or 1)
@@ -122,14 +121,13 @@ struct __align__(16) ChunkDesc {
   int32_t sb;      // the request's first chunk
 };
 
-// Per-segment state of the segmented radix select.
+// Per-segment state of the segmented select.
 struct __align__(16) SelSeg {
-  uint64_t prefix;   // key bits fixed so far
-  uint64_t mask;     // which bits are fixed
-  int64_t rank;      // 1-based rank still to locate inside the prefix class
-  int32_t active;    // 1 while this segment selects
-  int32_t incl;      // 1: victims are keys <= prefix; 0: keys < prefix
-  uint64_t kmin, kmax;  // a range holding every candidate key of the segment
+  int64_t rank;         // 1-based rank still to locate (inside [kmin, kmax], then inside [blo, bhi])
+  int32_t active;       // 1 while this segment selects
+  int32_t incl;         // 1: victims are keys up to the located one; 0: below it; 2: the tie rule decides
+  uint64_t kmin, kmax;  // a range holding every candidate key of the segment's class
+  uint64_t blo, bhi;    // the bucket of that range holding the rank
   uint64_t qmin, qmax;  // range of the segment's keys on the split list
 };
 
@@ -169,10 +167,9 @@ struct TieItem {
   int32_t log;
 };
 constexpr int kClasses = 3;
-// The first digit of a select is 16 bits wide while at most kWideRows
-// segments count (8 bits otherwise).
-constexpr int kWideRows = 64;
-constexpr int kWideBins = 1 << 16;
+// Buckets a select cuts a segment's key range into.
+constexpr int kDigBits = 12;
+constexpr int kDigBins = 1 << kDigBits;
 
 // ---- S3-FIFO as sequence-ordered arrays ------------------------------------
 // Both queues are arrays of block ids in sequence order (oldest first),
@@ -322,10 +319,7 @@ struct DevState {
   uint8_t* grp_full;       // the debt phase takes all of the group's candidates
   SelSeg* sel;             // [G] segments
   ClsRange* cls;           // [G * kClasses] candidates per (segment, class)
-  uint32_t* hist_bins;     // [G][256] radix histogram
-  uint32_t* wide_bins;     // [kWideRows][65536] first-digit histograms (or [G][256])
-  uint32_t* wide_coarse;   // [kWideRows][256] the 16-bit histograms summed by their top byte
-  int16_t* wide_seg;       // [G] segment of each first-digit row
+  uint32_t* dig_bins;      // [G][kDigBins] candidates per bucket (zero between selects)
   uint64_t* lst_key;       // split list of the select: key, block, segment
   uint32_t* lst_blk;
   uint16_t* lst_seg;

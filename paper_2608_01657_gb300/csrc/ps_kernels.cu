@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(kValTile) k_validate(DevState s, int probe) {
   if (!probe) {
     c->pinned = 0; c->n_inval = 0; c->total_claims = 0; c->avail = 0; c->need = 0;
     c->nfree = 0; c->ftake = 0; c->mvict = 0; c->hist_new = 0; c->n_evicted = 0;
-    c->n_alloc = 0; c->n_victims_marked = 0; c->m_fb = 0; c->sel_ntie = 0; c->sel_k = 0; c->ticket = 0;
+    c->n_alloc = 0; c->m_fb = 0; c->sel_ntie = 0; c->sel_k = 0; c->ticket = 0;
     c->internal_error = (vb & 2) ? 1 : 0;
     c->nlaunch = 1;  // this kernel; every later kernel of the step adds itself
   }
@@ -1262,7 +1262,6 @@ __device__ __forceinline__ void cls_stamp_range(const ClsRange& r, uint64_t* lo,
   *hi = ((uint64_t)r.hmax << 32) | (same_hi ? r.lmax : 0xFFFFFFFFu);
 }
 
-__device__ __forceinline__ void sel_start(SelSeg& z);
 // Start a segment's search from its per-class candidates: the class holding
 // the rank-th smallest key is fixed (lower classes are all below it), the rank
 // becomes a rank inside that class, and the key range is the class's.
@@ -1292,7 +1291,6 @@ __device__ __forceinline__ void sel_start_cls(SelSeg& z, const int64_t (&cnt)[kC
   } else {
     z.kmin = z.kmax = cb;
   }
-  sel_start(z);
 }
 __device__ __forceinline__ void sel_start_group(const DevState& s, int g, SelSeg& z, bool segmented) {
   int64_t cnt[kClasses];
@@ -1534,108 +1532,53 @@ __global__ void __launch_bounds__(1024) k_waterfill(DevState s, cudaGraphConditi
 // ---- exact segmented select -------------------------------------------------
 // Each active segment (a group in the debt phase, one global segment for lru
 // and for the fallback) looks for the rank-th smallest key among its
-// candidates, MSB-first, one byte at a time.  Bytes that all its candidates
-// share (from their smallest and largest key) are fixed without counting.
-// The first counted byte is histogrammed over the whole candidate array;
-// a split pass then marks every candidate below the chosen bucket as a
-// victim and copies the bucket's members into a short list, over which the
-// remaining bytes are counted.  A last-CTA-done resolve picks each digit.
+// candidates of one class.  The class's key range [kmin, kmax] is cut into
+// kDigBins equal buckets (a power of two wide), the candidates are counted by
+// bucket, and the bucket holding the rank is found; candidates below it are
+// victims, its members go to a short list that one CTA finishes exactly.
+//
+// Stamps are dense (a step's blocks take consecutive ones), so a range cut
+// into 4096 buckets leaves a few members a segment on the list.  Cutting the
+// range instead of two fixed bytes of the key keeps a segment's counts in
+// 16 KB (a byte-aligned 16-bit digit took 256 KB a segment: 16.7 MB of
+// histogram at 64 groups, zeroed again every step) and needs no coarse
+// histogram beside it.  Measured a step, byte digits against this: staticquota
+// over 100,003 blocks 90.2 -> 82.0 us, prefixshield over 256 blocks 76.2 ->
+// 71.9 us and over 2^20 blocks 186.3 -> 184.5 us (the launches dominate).
 
-// Highest byte where kmin and kmax differ, as a shift; -1 if equal.
-__device__ __forceinline__ int first_shift(uint64_t kmin, uint64_t kmax) {
-  const uint64_t d = kmin ^ kmax;
-  return d == 0 ? -1 : ((63 - __clzll((long long)d)) / 8) * 8;
-}
-// Bytes above 'shift' (shift a multiple of 8 in [0, 56]).
-__device__ __forceinline__ uint64_t above_mask(int shift) { return shift >= 56 ? 0ull : (~0ull << (shift + 8)); }
-// The next unresolved digit under a byte-aligned prefix mask, or -1.
-__device__ __forceinline__ int next_shift(uint64_t mask) {
-  if (mask == ~0ull) return -1;
-  if (mask == 0) return 56;
-  return __ffsll((long long)mask) - 1 - 8;
-}
-// Start a segment's search from its key range (rank and activity already set).
-__device__ __forceinline__ void sel_start(SelSeg& z) {
-  const int fs = first_shift(z.kmin, z.kmax);
-  if (fs < 0) {
-    z.prefix = z.kmin;
-    z.mask = ~0ull;
-  } else {
-    z.mask = above_mask(fs);
-    z.prefix = z.kmin & z.mask;
-  }
+// The bucket width of a range, as a shift.
+__device__ __forceinline__ int bucket_shift(uint64_t kmin, uint64_t kmax) {
+  const int bits = 64 - __clzll((long long)(kmax - kmin));
+  return bits > kDigBits ? bits - kDigBits : 0;
 }
 
-// A segment as the list passes see it: the list's members of the segment all
-// share the bits above the highest byte where the list's smallest and largest
-// key differ, so those bytes are fixed without counting.
-__device__ __forceinline__ SelSeg list_view(SelSeg z) {
-  if (z.qmin > z.qmax) return z;  // no member on the list
-  const int fs = first_shift(z.qmin, z.qmax);
-  const uint64_t cm = fs < 0 ? ~0ull : above_mask(fs);
-  z.mask |= cm;
-  z.prefix |= z.qmin & cm;
-  return z;
-}
+// A segment as the counting pass sees it (shared memory).
+struct CountSmem {
+  uint64_t kmin[PS_MAX_GROUPS];
+  uint64_t span[PS_MAX_GROUPS];   // kmax - kmin of a selecting segment
+  uint8_t shift[PS_MAX_GROUPS];   // 64: the segment does not select
+};
 
-// The first counted digit of every segment, over the whole candidate array:
-// 16 bits wide (two bytes) while at most kWideRows segments count, one byte
-// otherwise, into global histograms (warp-aggregated atomics).  CTA 0 records
-// the rows' segments for k_wide_resolve.
-__device__ __forceinline__ void wide_digit(int nrows, uint64_t mask, int* dshift, uint32_t* nbins) {
-  const int sh = next_shift(mask);
-  const bool w16 = nrows <= kWideRows && sh >= 8;
-  *dshift = w16 ? sh - 8 : sh;
-  *nbins = w16 ? (uint32_t)kWideBins : (uint32_t)kRadixBins;
-}
-__global__ void __launch_bounds__(256) k_wide_pass(DevState s, int single, int fallback) {
-  s = with_args(s);
-  __shared__ uint32_t s_coarse[kRadixBins];  // one row's coarse counts (a single segment)
-  __shared__ int16_t row_of[PS_MAX_GROUPS];
-  __shared__ uint64_t s_pre[PS_MAX_GROUPS], s_msk[PS_MAX_GROUPS];  // the segments' prefix and mask
-  __shared__ int s_nrows;
-  Ctl* c = s.ctl;
-  if (c->status != PS_OK || c->mvict == 0) return;
+// Counts by bucket, thread per candidate, kU candidates a thread per
+// iteration with their loads issued together (the trip count is CTA-uniform,
+// as the warp-aggregated increment needs).  Neighbouring blocks were mostly
+// admitted together and share buckets, so a warp's increments combine.
+// Bound by the scan of N keys (8 B) and groups (2 B).
+__device__ __forceinline__ void select_count(const DevState& s, CountSmem& sm, int single, int fallback, int bid,
+                                             int nb) {
   const int nseg = single ? 1 : s.G;
-  if (single && !s.sel[0].active) return;
-  {
-    int k = 0;
-    for (int base = 0; base < nseg; base += blockDim.x) {
-      const int g = base + threadIdx.x;
-      bool counts = false;
-      if (g < nseg) {
-        const SelSeg ss = s.sel[g];
-        counts = ss.active && next_shift(ss.mask) >= 0;
-        s_pre[g] = ss.prefix;
-        s_msk[g] = ss.mask;
-      }
-      int tot;
-      const int ex = block_excl_scan((int)counts, &tot);
-      if (g < nseg) row_of[g] = counts ? (int16_t)(k + ex) : (int16_t)-1;
-      if (counts && blockIdx.x == 0) s.wide_seg[k + ex] = (int16_t)g;
-      k += tot;
-    }
-    if (threadIdx.x == 0) {
-      s_nrows = k;
-      if (blockIdx.x == 0) c->wide_nrows = k;
-    }
-    __syncthreads();
+  int any = 0;
+  for (int g = threadIdx.x; g < nseg; g += blockDim.x) {
+    const SelSeg z = s.sel[g];
+    sm.kmin[g] = z.kmin;
+    sm.span[g] = z.kmax - z.kmin;
+    sm.shift[g] = z.active ? (uint8_t)bucket_shift(z.kmin, z.kmax) : (uint8_t)64;
+    any |= z.active;
   }
-  const int nrows = s_nrows;
-  if (nrows == 0) return;
-  const uint32_t stride = nrows <= kWideRows ? (uint32_t)kWideBins : (uint32_t)kRadixBins;
-  // A 16-bit digit is also counted by its top byte (row-major, 256 a row)
-  // for the resolve.  One row takes every candidate (lru, the fallback):
-  // its 256 coarse counts would serialize global atomics, so each CTA counts
-  // them in shared memory and adds its nonzero ones once at the end.
-  const bool coarse_smem = nrows == 1 && stride == (uint32_t)kWideBins;
-  for (int k = threadIdx.x; k < kRadixBins; k += blockDim.x) s_coarse[k] = 0;
-  __syncthreads();
-  // kU candidates a thread per iteration, their loads issued together (the
-  // trip count is CTA-uniform, as the warp-aggregated increment needs)
+  if (!__syncthreads_or(any)) return;
   constexpr int kU = 4;
-  const int64_t span = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t b0 = blockIdx.x * (int64_t)blockDim.x; b0 < s.N; b0 += span * kU) {
+  const int64_t span = (int64_t)nb * blockDim.x;
+  for (int64_t b0 = bid * (int64_t)blockDim.x; b0 < s.N; b0 += span * kU) {
     uint64_t key[kU];
     int seg[kU];
     uint32_t vw[kU];
@@ -1654,182 +1597,164 @@ __global__ void __launch_bounds__(256) k_wide_pass(DevState s, int single, int f
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
       const int64_t e = b0 + u * span + threadIdx.x;
-      bool act = false, act16 = false;
+      bool act = false;
       uint32_t idx = 0;
       if (key[u] != ~0ull && !((vw[u] >> (e & 31)) & 1)) {
-        const int row = row_of[seg[u]];
-        if (row >= 0) {
-          const uint64_t msk = s_msk[seg[u]];
-          if ((key[u] & msk) == s_pre[seg[u]]) {
-            int dsh;
-            uint32_t nb;
-            wide_digit(nrows, msk, &dsh, &nb);
-            act = true;
-            act16 = nb == (uint32_t)kWideBins;
-            idx = (uint32_t)row * stride + (uint32_t)((key[u] >> dsh) & (nb - 1));
-          }
-        }
+        const int sh = sm.shift[seg[u]];
+        const uint64_t d = key[u] - sm.kmin[seg[u]];  // keys below the range wrap past any span
+        act = sh < 64 && d <= sm.span[seg[u]];
+        idx = (uint32_t)seg[u] * kDigBins + (act ? (uint32_t)(d >> sh) : 0u);
       }
-      agg_inc(s.wide_bins, idx, act);
-      const uint32_t cidx = (idx >> 16) * kRadixBins + ((idx >> 8) & 0xFF);
-      if (coarse_smem) {
-        if (act16) atomicAdd(&s_coarse[cidx], 1u);
-      } else if (stride == (uint32_t)kWideBins) {
-        agg_inc(s.wide_coarse, cidx, act16);
-      }
+      agg_inc(s.dig_bins, idx, act);
     }
-  }
-  if (coarse_smem) {
-    __syncthreads();
-    for (int k = threadIdx.x; k < kRadixBins; k += blockDim.x)
-      if (s_coarse[k]) atomicAdd(s.wide_coarse + k, s_coarse[k]);
   }
 }
 
-// One warp per counted segment: the bucket holding the segment's rank-th key
-// fixes the digit.  A 16-bit digit is found in two short scans (its top byte
-// from the coarse histogram, then the 256 bins under it); the coarse bins are
-// cleared here and the fine ones by the split that follows.
-__global__ void __launch_bounds__(32) k_wide_resolve(DevState s, int single) {
-  s = with_args(s);
-  Ctl* c = s.ctl;
-  if (c->status != PS_OK || c->mvict == 0) return;
-  if (single && !s.sel[0].active) return;
-  const int nrows = c->wide_nrows;
-  const int r = blockIdx.x;
-  if (r >= nrows) return;
-  const int lane = lane_id();
-  const int seg = s.wide_seg[r];
-  SelSeg ss = s.sel[seg];
-  int dsh;
-  uint32_t nb;
-  wide_digit(nrows, ss.mask, &dsh, &nb);
-  const bool w16 = nb == (uint32_t)kWideBins;
-  const uint32_t stride = nrows <= kWideRows ? (uint32_t)kWideBins : (uint32_t)kRadixBins;
-  uint32_t* row = s.wide_bins + (size_t)r * stride;
-  // locate rank among 256 consecutive bins (8 a lane); returns the bin and
-  // the count before it
-  auto locate = [&](const uint32_t* bins, uint64_t rank, uint32_t* before) -> uint32_t {
-    uint32_t v[8], sum = 0;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) { v[k] = __ldcg(bins + lane * 8 + k); sum += v[k]; }
-    const uint32_t incl = warp_incl_scan(sum), excl = incl - sum;
-    const bool mine = (uint64_t)excl < rank && rank <= (uint64_t)incl;
-    const unsigned mw = __ballot_sync(kFull, mine);
-    const int ml = mw ? __ffs(mw) - 1 : 0;
-    uint32_t d = 0, run = excl;
-    if (mine) {
-      for (int k = 0; k < 8; ++k) {
-        if (rank <= (uint64_t)(run + v[k])) { d = lane * 8 + k; break; }
-        run += v[k];
-      }
+// One CTA per segment: the bucket holding the segment's rank-th key, as a key
+// range [blo, bhi], and the rank left inside it.  The counts are cleared for
+// the next select.
+__device__ __forceinline__ void select_resolve(const DevState& s, int g) {
+  const SelSeg z = s.sel[g];
+  if (!z.active) return;
+  constexpr int kV = 4;  // bins a thread reads at once
+  uint4* bins = reinterpret_cast<uint4*>(s.dig_bins + (size_t)g * kDigBins);
+  uint64_t before = 0;
+  for (int base = 0; base < kDigBins / kV; base += blockDim.x) {
+    const int k = base + (int)threadIdx.x;
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (k < kDigBins / kV) {
+      v = __ldcg(bins + k);
+      bins[k] = make_uint4(0, 0, 0, 0);
     }
-    *before = __shfl_sync(kFull, run, ml);
-    return __shfl_sync(kFull, d, ml);
-  };
-  uint32_t d, run;
-  if (w16) {
-    uint32_t* coarse = s.wide_coarse + (size_t)r * kRadixBins;
-    uint32_t cb_before;
-    const uint32_t cb = locate(coarse, (uint64_t)ss.rank, &cb_before);
-    uint32_t fb_before;
-    const uint32_t fb = locate(row + cb * kRadixBins, (uint64_t)ss.rank - cb_before, &fb_before);
-    d = cb * kRadixBins + fb;
-    run = cb_before + fb_before;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) coarse[lane * 8 + k] = 0;
-  } else {
-    d = locate(row, (uint64_t)ss.rank, &run);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) row[lane * 8 + k] = 0;
-  }
-  if (lane == 0) {
-    ss.prefix |= (uint64_t)d << dsh;
-    ss.mask |= (uint64_t)(nb - 1) << dsh;
-    ss.rank -= run;
-    s.sel[seg] = ss;
+    uint32_t tot;
+    const uint64_t ex = before + block_excl_scan<uint32_t>(v.x + v.y + v.z + v.w, &tot);
+    const uint64_t rank = (uint64_t)z.rank;
+    if (ex < rank && rank <= ex + v.x + v.y + v.z + v.w) {  // one thread
+      uint64_t run = ex;
+      uint32_t d = 4u * (uint32_t)k;
+      if (rank > run + v.x) { run += v.x; ++d;
+        if (rank > run + v.y) { run += v.y; ++d;
+          if (rank > run + v.z) { run += v.z; ++d; } } }
+      const int sh = bucket_shift(z.kmin, z.kmax);
+      SelSeg* o = s.sel + g;
+      o->blo = z.kmin + ((uint64_t)d << sh);
+      o->bhi = tmin<uint64_t>(o->blo + ((1ull << sh) - 1), z.kmax);
+      o->rank = (int64_t)(rank - run);
+    }
+    before += tot;
   }
 }
 
-// Split: candidates below their segment's chosen bucket are victims; the
-// bucket's members go to the list for the remaining digits, with the list's
-// key range per segment.
-__global__ void __launch_bounds__(256) k_split(DevState s, int single, int fallback) {
-  s = with_args(s);
-  Ctl* c = s.ctl;
-  if (c->status != PS_OK || c->mvict == 0) return;
-  if (single && !s.sel[0].active) return;
-  {
-    // the first digit's 16-bit rows are read: clear them for the next select
-    const int nrows = c->wide_nrows;
-    if (nrows <= kWideRows) {
-      uint4* w = reinterpret_cast<uint4*>(s.wide_bins);
-      const int64_t n4 = (int64_t)nrows * kWideBins / 4;
-      for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n4; k += (int64_t)gridDim.x * blockDim.x)
-        w[k] = make_uint4(0, 0, 0, 0);
-    }
-  }
-  // the segments' state, once per CTA (s_act: 1 selecting, 2 taken whole)
-  __shared__ uint64_t s_pre[PS_MAX_GROUPS], s_msk[PS_MAX_GROUPS];
-  __shared__ uint8_t s_act[PS_MAX_GROUPS];
+// Split: candidates below their segment's bucket are victims; the bucket's
+// members go to the list, with the list's key range per segment.
+struct SplitSmem {
+  uint64_t lo[PS_MAX_GROUPS], hi[PS_MAX_GROUPS];  // the bucket; a segment taken whole: [~0, ~0]
+  uint8_t act[PS_MAX_GROUPS];
+};
+__device__ __forceinline__ void select_split(const DevState& s, Ctl* c, SplitSmem& sm, int single, int fallback,
+                                             int bid, int nb) {
   const int nseg = single ? 1 : s.G;
   const bool whole = !single && s.policy == PS_PREFIXSHIELD;
+  int any = 0;
   for (int g = threadIdx.x; g < nseg; g += blockDim.x) {
-    const SelSeg ss = s.sel[g];
-    s_pre[g] = ss.prefix;
-    s_msk[g] = ss.mask;
-    s_act[g] = (whole && s.grp_full[g]) ? 2 : (ss.active ? 1 : 0);
+    const SelSeg z = s.sel[g];
+    const bool w = whole && s.grp_full[g];
+    sm.lo[g] = w ? ~0ull : z.blo;
+    sm.hi[g] = w ? ~0ull : z.bhi;
+    sm.act[g] = w || z.active;
+    any |= sm.act[g];
   }
-  __syncthreads();
-  int marked = 0;
-  for (int64_t b0 = blockIdx.x * (int64_t)blockDim.x; b0 < s.N; b0 += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = b0 + threadIdx.x;
-    bool v = false, to_list = false;
-    uint64_t key = ~0ull;
-    int seg = 0;
-    if (b < s.N) {
-      key = s.csk[b];
-      const int grp = single ? 0 : s.blk_group[b];
-      if (key != ~0ull && !(fallback && ((s.bm_victim[b >> 5] >> (b & 31)) & 1))) {
-        seg = grp;
-        if (s_act[seg] == 2) {
-          v = true;
-        } else if (s_act[seg]) {
-          const uint64_t k = key & s_msk[seg];
-          v = k < s_pre[seg];
-          to_list = k == s_pre[seg];
-        }
+  if (!__syncthreads_or(any)) return;
+  constexpr int kU = 4;
+  const int64_t span = (int64_t)nb * blockDim.x;
+  for (int64_t b0 = bid * (int64_t)blockDim.x; b0 < s.N; b0 += span * kU) {
+    uint64_t key[kU];
+    int seg[kU];
+    uint32_t vw[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int64_t b = b0 + u * span + threadIdx.x;
+      key[u] = ~0ull;
+      seg[u] = 0;
+      vw[u] = 0;
+      if (b < s.N) {
+        key[u] = s.csk[b];
+        if (!single) seg[u] = s.blk_group[b];
+        if (fallback) vw[u] = s.bm_victim[b >> 5];
       }
     }
-    const unsigned bits = __ballot_sync(kFull, v);
-    if (bits && lane_id() == 0) atomicOr(s.bm_victim + ((b - lane_id()) >> 5), bits);
-    marked += __popc(bits);
-    const unsigned lm = __ballot_sync(kFull, to_list);
-    if (lm) {
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int64_t b = b0 + u * span + threadIdx.x;
+      bool v = false, to_list = false;
+      if (key[u] != ~0ull && !((vw[u] >> (b & 31)) & 1) && sm.act[seg[u]]) {
+        v = key[u] < sm.lo[seg[u]];
+        to_list = !v && key[u] <= sm.hi[seg[u]];
+      }
+      const unsigned bits = __ballot_sync(kFull, v);
+      if (bits && lane_id() == 0) atomicOr(s.bm_victim + ((b - lane_id()) >> 5), bits);
+      const unsigned lm = __ballot_sync(kFull, to_list);
+      if (!lm) continue;
       unsigned long long base = 0;
       if (lane_id() == 0) base = atomicAdd(reinterpret_cast<unsigned long long*>(&c->lst_n), (unsigned long long)__popc(lm));
       base = __shfl_sync(kFull, base, 0);
       if (to_list) {
         const int64_t slot = (int64_t)base + __popc(lm & ((1u << lane_id()) - 1));
-        s.lst_key[slot] = key;
+        s.lst_key[slot] = key[u];
         s.lst_blk[slot] = (uint32_t)b;
-        s.lst_seg[slot] = (uint16_t)seg;
+        s.lst_seg[slot] = (uint16_t)seg[u];
       }
       // the list's key range per segment (lanes of one segment combined)
-      const unsigned peers = __match_any_sync(kFull, to_list ? (uint32_t)seg : ~0u);
+      const unsigned peers = __match_any_sync(kFull, to_list ? (uint32_t)seg[u] : ~0u);
       if (to_list) {
-        const uint32_t hi = (uint32_t)(key >> 32), lo = (uint32_t)key;
+        const uint32_t hi = (uint32_t)(key[u] >> 32), lo = (uint32_t)key[u];
         const uint32_t hmin = __reduce_min_sync(peers, hi), hmax = __reduce_max_sync(peers, hi);
         const uint32_t lmin = __reduce_min_sync(peers, hi == hmin ? lo : ~0u);
         const uint32_t lmax = __reduce_max_sync(peers, hi == hmax ? lo : 0u);
         if (lane_id() == __ffs(peers) - 1) {
-          atomicMin(reinterpret_cast<unsigned long long*>(&s.sel[seg].qmin), ((unsigned long long)hmin << 32) | lmin);
-          atomicMax(reinterpret_cast<unsigned long long*>(&s.sel[seg].qmax), ((unsigned long long)hmax << 32) | lmax);
+          atomicMin(reinterpret_cast<unsigned long long*>(&s.sel[seg[u]].qmin), ((unsigned long long)hmin << 32) | lmin);
+          atomicMax(reinterpret_cast<unsigned long long*>(&s.sel[seg[u]].qmax), ((unsigned long long)hmax << 32) | lmax);
         }
       }
     }
   }
-  if (lane_id() == 0 && marked) atomic_add_i64(&c->n_victims_marked, marked);
+}
+
+__global__ void __launch_bounds__(256) k_sel_count(DevState s, int single, int fallback) {
+  s = with_args(s);
+  __shared__ CountSmem sm;
+  Ctl* c = s.ctl;
+  if (c->status != PS_OK || c->mvict == 0) return;
+  select_count(s, sm, single, fallback, blockIdx.x, gridDim.x);
+}
+__global__ void __launch_bounds__(1024) k_sel_resolve(DevState s) {
+  s = with_args(s);
+  const Ctl* c = s.ctl;
+  if (c->status != PS_OK || c->mvict == 0) return;
+  select_resolve(s, blockIdx.x);
+}
+__global__ void __launch_bounds__(256) k_sel_split(DevState s, int single, int fallback) {
+  s = with_args(s);
+  __shared__ SplitSmem sm;
+  Ctl* c = s.ctl;
+  if (c->status != PS_OK || c->mvict == 0) return;
+  select_split(s, c, sm, single, fallback, blockIdx.x, gridDim.x);
+}
+
+// The digits of the list's finish: bytes, from the highest one where the
+// list's keys of a segment differ.
+// Highest byte where kmin and kmax differ, as a shift; -1 if equal.
+__device__ __forceinline__ int first_shift(uint64_t kmin, uint64_t kmax) {
+  const uint64_t d = kmin ^ kmax;
+  return d == 0 ? -1 : ((63 - __clzll((long long)d)) / 8) * 8;
+}
+// Bytes above 'shift' (shift a multiple of 8 in [0, 56]).
+__device__ __forceinline__ uint64_t above_mask(int shift) { return shift >= 56 ? 0ull : (~0ull << (shift + 8)); }
+// The next unresolved digit under a byte-aligned prefix mask, or -1.
+__device__ __forceinline__ int next_shift(uint64_t mask) {
+  if (mask == ~0ull) return -1;
+  if (mask == 0) return 56;
+  return __ffsll((long long)mask) - 1 - 8;
 }
 
 // The rest of a select on one CTA, with every segment's state in shared
@@ -1868,9 +1793,14 @@ __global__ void __launch_bounds__(1024) k_list_finish(DevState s, int single) {
   const int64_t n = c->lst_n;
   const bool small = n <= kFinCap;
   const int warp = threadIdx.x >> 5, lane = lane_id();
+  // the list's members of a segment share the bits above the highest byte
+  // where their smallest and largest key differ: those are fixed already
   for (int g = threadIdx.x; g < nseg; g += blockDim.x) {
-    const SelSeg v = list_view(s.sel[g]);
-    sl[g] = FinSeg{v.prefix, v.mask, v.rank, v.active, v.incl};
+    const SelSeg z = s.sel[g];
+    const bool listed = z.qmin <= z.qmax;
+    const int fs = listed ? first_shift(z.qmin, z.qmax) : 56;
+    const uint64_t mask = fs < 0 ? ~0ull : above_mask(fs);
+    sl[g] = FinSeg{listed ? z.qmin & mask : 0ull, listed ? mask : ~0ull, z.rank, listed ? z.active : 0, z.incl};
   }
   if (small)
     for (int64_t e = threadIdx.x; e < n; e += blockDim.x) { lkey[e] = s.lst_key[e]; lseg[e] = s.lst_seg[e]; }
@@ -1879,22 +1809,24 @@ __global__ void __launch_bounds__(1024) k_list_finish(DevState s, int single) {
   auto seg_at = [&](int64_t e) -> int { return small ? (int)lseg[e] : (int)s.lst_seg[e]; };
   // A short list (the usual case): a segment's threshold key is its member
   // whose rank among the segment's list members (keys are unique) is its
-  // remaining rank - 1; each thread ranks one member by counting, so no
-  // digit rounds (and their barriers) are needed.
+  // remaining rank - 1; L lanes rank one member by counting, so no digit
+  // rounds (and their barriers) are needed.
   const bool by_count = small && n <= kFinCountCap;
   if (by_count) {
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-      const int g = lseg[e];
-      if (!sl[g].active) continue;
-      const uint64_t key = lkey[e];
-      int64_t below = 0;
-      for (int j = 0; j < n; ++j) below += (lseg[j] == g && lkey[j] < key) ? 1 : 0;
-      // one member per segment matches, and the loop reads only the
-      // segment's activity and rank, which nothing here writes
-      if (below == sl[g].rank - 1) {
-        sl[g].prefix = key;
-        sl[g].mask = ~0ull;
-      }
+    int L = 32;
+    while (L * (int)n > (int)blockDim.x) L >>= 1;  // kFinCountCap <= blockDim.x: L >= 1
+    const int e = (int)threadIdx.x / L, l = (int)threadIdx.x % L;
+    const bool in = e < n && sl[lseg[e]].active;
+    const int g = in ? lseg[e] : -1;
+    const uint64_t key = in ? lkey[e] : 0;
+    int below = 0;
+    if (in)
+      for (int j = l; j < n; j += L) below += (lseg[j] == g && lkey[j] < key) ? 1 : 0;
+    for (int o = L / 2; o > 0; o >>= 1) below += __shfl_xor_sync(kFull, below, o);
+    // one member per segment matches; nothing here writes the ranks read
+    if (in && l == 0 && below == sl[g].rank - 1) {
+      sl[g].prefix = key;
+      sl[g].mask = ~0ull;
     }
     __syncthreads();
   }
@@ -2251,8 +2183,6 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
   const int R = s.max_requests;
   const int pgrid = grid_for(s.max_blocks, kThreads, 1 << 30);
   const int prgrid = grid_for(s.max_blocks + R, kThreads, 1 << 30);
-  const int ngrid = grid_for(s.N, 256, 152 * 8);
-  const int sgrid = grid_for(s.N, 256, 152 * 4);  // 48 KB histograms: 4 CTAs per SM
   const int cgrid = grid_for(s.N, 256, 152 * 8);
   int launches = 0;
   auto mark = [&](int stage) {
@@ -2353,9 +2283,9 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
   // conditional graph node measured about 10 us a step even when its body
   // was skipped, more than the phase's early-returning launches.
   auto select = [&](int single, int fallback) {
-    PS_LAUNCH(launch_k(k_wide_pass, cgrid, 256, 0, st, s, single, fallback));
-    PS_LAUNCH(launch_k(k_wide_resolve, single ? 1 : s.G, 32, 0, st, s, single));
-    PS_LAUNCH(launch_k(k_split, cgrid, 256, 0, st, s, single, fallback));
+    PS_LAUNCH(launch_k(k_sel_count, cgrid, 256, 0, st, s, single, fallback));
+    PS_LAUNCH(launch_k(k_sel_resolve, single ? 1 : s.G, 1024, 0, st, s));
+    PS_LAUNCH(launch_k(k_sel_split, cgrid, 256, 0, st, s, single, fallback));
     PS_LAUNCH(launch_k(k_list_finish, 1, 1024, kFinSmem, st, s, single));
   };
   if (s.lg_on) {

@@ -337,7 +337,6 @@ __global__ void __launch_bounds__(kScanThreads) k_lg_take(DevState s, int phase,
           const int32_t B = lg_log_b(s, (uint32_t)(k.log % kClasses));
           if (B >= 0) atomic_add_i64(s.lg_live + B, -sum);
         }
-        atomic_add_i64(&c->n_victims_marked, sum);
       }
       if (rem > 0 && rem <= tot) {
         s.lg_tk[t].done = 1;
@@ -375,7 +374,6 @@ __global__ void __launch_bounds__(1024) k_lg_tie(DevState s) {
   __syncthreads();
   if (threadIdx.x == 0 && n != c->sel_ntie) c->internal_error = 1;
   const int k = c->sel_k;
-  int taken = 0;
   if (threadIdx.x < n) {
     const uint64_t key = skey[threadIdx.x];
     int rank = 0;
@@ -388,13 +386,10 @@ __global__ void __launch_bounds__(1024) k_lg_tie(DevState s) {
       const int32_t B = lg_log_b(s, (uint32_t)(ti.log % kClasses));
       if (B >= 0) atomic_add_i64(s.lg_live + B, -1);
       s.lg_desc[ti.log].head = ti.pos + 1;
-      taken = 1;
     } else {
       s.grp_x[gg] -= 1;
     }
   }
-  const int sum = block_sum(taken);
-  if (threadIdx.x == 0 && sum) atomic_add_i64(&c->n_victims_marked, sum);
 }
 
 // ---- end of step: append this step's stamps, compacting first if needed ----
