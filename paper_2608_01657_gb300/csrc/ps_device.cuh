@@ -99,15 +99,14 @@ __device__ __forceinline__ void atomic_add_i64(int64_t* p, int64_t v) {
 __device__ __forceinline__ int64_t* stat_ptr(const DevState& s, int g, int k) {
   return s.stats + (int64_t)g * PS_NUM_STATS + k;
 }
-// Add v to stat k of group g, combining lanes of the warp with equal g.
+// Add v (the same for every lane) to stat k of group g once per lane with
+// 'active', lanes of equal g combined: their number is known from the match,
+// so nothing is summed lane by lane.
 __device__ __forceinline__ void agg_stat(const DevState& s, uint32_t g, int k, int64_t v, bool active) {
-  const bool on = active && v != 0;
-  const unsigned act = __ballot_sync(kFull, on);
-  if (!on) return;
+  const unsigned act = __ballot_sync(kFull, active);
+  if (!active) return;
   const unsigned peers = __match_any_sync(act, g);
-  int64_t sum = 0;
-  for (unsigned m = peers; m; m &= m - 1) sum += __shfl_sync(peers, v, __ffs(m) - 1);
-  if (lane_id() == __ffs(peers) - 1) atomic_add_i64(stat_ptr(s, (int)g, k), sum);
+  if (lane_id() == __ffs(peers) - 1) atomic_add_i64(stat_ptr(s, (int)g, k), v * __popc(peers));
 }
 // Warp-aggregated increment of bins[idx] for the lanes with 'active'.
 __device__ __forceinline__ void agg_inc(uint32_t* bins, uint32_t idx, bool active) {
@@ -116,15 +115,13 @@ __device__ __forceinline__ void agg_inc(uint32_t* bins, uint32_t idx, bool activ
   const unsigned peers = __match_any_sync(act, idx);
   if (lane_id() == __ffs(peers) - 1) atomicAdd(bins + idx, (uint32_t)__popc(peers));
 }
-// base[i] += v, lanes of the warp with equal i combined first (every lane of
-// the warp must call it).
+// base[i] += v (the same for every lane), lanes of the warp with equal i
+// combined first (every lane of the warp must call it).
 __device__ __forceinline__ void agg_add_i64(int64_t* base, uint32_t i, int64_t v, bool active) {
   const unsigned act = __ballot_sync(kFull, active);
   if (!active) return;
   const unsigned peers = __match_any_sync(act, i);
-  int64_t sum = 0;
-  for (unsigned m = peers; m; m &= m - 1) sum += __shfl_sync(peers, v, __ffs(m) - 1);
-  if (lane_id() == __ffs(peers) - 1) atomicAdd(reinterpret_cast<unsigned long long*>(base + i), (unsigned long long)sum);
+  if (lane_id() == __ffs(peers) - 1) atomic_add_i64(base + i, v * __popc(peers));
 }
 // atomicMin of v into base[i], lanes of the warp with equal i combined first
 // (every lane of the warp must call it).

@@ -1142,7 +1142,7 @@ __global__ void __launch_bounds__(kThreads) k_touch2(DevState s) {
   if (c->status != PS_OK) return;
   const int64_t pos = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   PosRef r;
-  int gated = 0, promoted = 0;
+  bool gated = false, promoted = false;
   uint32_t g = 0;
   if (pos_ref(s, pos, &r) && r.m < s.rq_h[r.i] + s.rq_e[r.i] && s.pos_elig[pos]) {
     const uint32_t i = r.i;
@@ -1158,12 +1158,12 @@ __global__ void __launch_bounds__(kThreads) k_touch2(DevState s) {
     if (!gate) {
       gated = i < promoter;
     } else if (i == promoter) {
-      promoted = 1;
+      promoted = true;
       if (b != kNone) s.blk_klass[b] = kReuse;
     }
   }
-  agg_stat(s, g, PS_STAT_GATED_REUSES, gated, gated != 0);
-  agg_stat(s, g, PS_STAT_PROMOTIONS, promoted, promoted != 0);
+  agg_stat(s, g, PS_STAT_GATED_REUSES, 1, gated);
+  agg_stat(s, g, PS_STAT_PROMOTIONS, 1, promoted);
 }
 
 // ===========================================================================
