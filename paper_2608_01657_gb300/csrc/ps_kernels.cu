@@ -755,11 +755,15 @@ __global__ void __launch_bounds__(kThreads) k_claims(DevState s) {
   bool own = false;
   const bool valid = pos_ref(s, pos, &r);
   if (valid) {
+    // the position's records in one round of loads, then what they point to
     const int h = s.rq_h[r.i];
-    own = r.m >= h && ldcg_u32(&s.claims[s.pos_claim[pos]].minreq) == r.i;
-    if (r.m > h) {
-      const uint32_t b = s.pos_blk[pos];
-      if (b != kNone && ldcg_u32(s.blk_pin + b) != step32 && atomicExch(s.blk_inval + b, step32) != step32) {
+    const uint32_t slot = s.pos_claim[pos], b = s.pos_blk[pos];
+    const bool past = r.m > h && b != kNone;
+    const uint32_t minreq = r.m >= h ? ldcg_u32(&s.claims[slot].minreq) : kNone;
+    const uint32_t pin = past ? ldcg_u32(s.blk_pin + b) : step32;
+    own = minreq == r.i;
+    if (past) {
+      if (pin != step32 && atomicExch(s.blk_inval + b, step32) != step32) {
         ginv = drop_block(s, b);
         if (s.lg_on) kinv = s.blk_klass[b];
         atomicOr(s.bm_inval + (b >> 5), 1u << (b & 31));
@@ -938,10 +942,17 @@ __global__ void __launch_bounds__(kThreads) k_instep(DevState s) {
   PosRef r;
   bool past = false;
   const bool valid = pos_ref(s, pos, &r);
-  if (valid && r.m >= s.rq_h[r.i] && r.m < s.rq_s[r.i]) {
+  int h = 0, sown = 0;
+  uint32_t slot = kNone;
+  if (valid) {  // one round of loads
+    h = s.rq_h[r.i];
+    sown = s.rq_s[r.i];
+    slot = s.pos_claim[pos];
+  }
+  if (valid && r.m >= h && r.m < sown) {
     // the owner's claims are ranked consecutively: its key here is granted
     // iff it is among the owner's first a_j
-    const uint32_t j = s.claims[s.pos_claim[pos]].minreq;
+    const uint32_t j = s.claims[slot].minreq;
     past = r.m - s.rq_s[j] >= s.rq_a[j];
   }
   agg_min_u32(s.rq_fu, valid ? r.i : 0u, valid ? (uint32_t)r.m : 0u, past);
@@ -1103,34 +1114,38 @@ __global__ void __launch_bounds__(kThreads) k_touch(DevState s) {
   const int64_t pos = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   PosRef r;
   if (!pos_ref(s, pos, &r)) return;
+  // every record of the position and its request in one round of loads (an
+  // atomic in between would hold back the loads after it), then the block's
   const uint32_t i = r.i;
   const int m = r.m;
-  const int h = s.rq_h[i];
-  if (m >= h + s.rq_e[i]) return;
+  const int h = s.rq_h[i], re = s.rq_e[i], n = s.rq_n[i], pbase = s.rq_pbase[i], cid = s.rq_cid[i];
   const uint8_t fl = s.rq_flags[i];
-  const bool proven = fl & 1, gate = fl & 2;
-  const int cid = s.rq_cid[i];
   const uint64_t p = s.rq_p[i];
-  const uint64_t step = c->step;
+  const uint32_t b = s.pos_blk[pos], slot = s.pos_claim[pos];
+  const uint64_t step = c->step, base = c->stamp_base;
+  if (m >= h + re) return;
+  const bool proven = fl & 1, gate = fl & 2;
+  const uint64_t stamp = make_stamp(base, pbase, n, m);
   bool elig;
   if (m < h) {
-    const uint32_t b = s.pos_blk[pos];
-    atomicMax(reinterpret_cast<unsigned long long*>(s.blk_stamp + b),
-              (unsigned long long)make_stamp(c->stamp_base, s.rq_pbase[i], s.rq_n[i], m));
-    if (s.lg_on) s.lg_slot[s.rq_pbase[i] + (s.rq_n[i] - 1 - m)] = b;  // the queues' append reads it back
+    const uint8_t bc = s.blk_contract[b], bk = s.blk_klass[b];
+    const uint64_t bp = s.blk_prefix[b];
+    atomicMax(reinterpret_cast<unsigned long long*>(s.blk_stamp + b), (unsigned long long)stamp);
+    if (s.lg_on) s.lg_slot[pbase + (n - 1 - m)] = b;  // the queues' append reads it back
     atomicAdd(s.blk_acc + b, 1u);
     atomicAdd(s.blk_freq + b, 1u);
-    elig = proven && s.blk_contract[b] == cid && s.blk_prefix[b] == p && s.blk_klass[b] != kReuse;
+    elig = proven && bc == cid && bp == p && bk != kReuse;
     if (elig && gate)
       atomicMax(reinterpret_cast<unsigned long long*>(s.blk_promo + b), (unsigned long long)step_tag(step, i));
   } else {
-    ClaimEntry* e = s.claims + s.pos_claim[pos];
+    ClaimEntry* e = s.claims + slot;
     const uint32_t j = e->minreq;
+    const int jc = s.rq_cid[j];
+    const uint64_t jp = s.rq_p[j];
     // later requests give larger stamps: the maximum is the latest touch's
-    atomicMax(reinterpret_cast<unsigned long long*>(&e->stamp),
-              (unsigned long long)make_stamp(c->stamp_base, s.rq_pbase[i], s.rq_n[i], m));
+    atomicMax(reinterpret_cast<unsigned long long*>(&e->stamp), (unsigned long long)stamp);
     atomicAdd(&e->tcnt, 1u);
-    elig = proven && s.rq_cid[j] == cid && s.rq_p[j] == p;  // new blocks are never Reuse yet
+    elig = proven && jc == cid && jp == p;  // new blocks are never Reuse yet
     if (elig && gate) atomicMin(&e->promo, i);
   }
   s.pos_elig[pos] = elig;
@@ -1144,16 +1159,30 @@ __global__ void __launch_bounds__(kThreads) k_touch2(DevState s) {
   PosRef r;
   bool gated = false, promoted = false;
   uint32_t g = 0;
-  if (pos_ref(s, pos, &r) && r.m < s.rq_h[r.i] + s.rq_e[r.i] && s.pos_elig[pos]) {
+  bool elig = false;
+  int h = 0;
+  uint32_t b = kNone, slot = kNone;
+  uint8_t fl = 0;
+  const uint64_t step = c->step;
+  if (pos_ref(s, pos, &r)) {  // one round of loads (an untouched position's eligibility is stale, and not used)
+    const uint8_t el = s.pos_elig[pos];
+    const int re = s.rq_e[r.i];
+    h = s.rq_h[r.i];
+    b = s.pos_blk[pos];
+    slot = s.pos_claim[pos];
+    fl = s.rq_flags[r.i];
+    g = (uint32_t)s.in_group[r.i];
+    elig = r.m < h + re && el;
+  }
+  if (elig) {
     const uint32_t i = r.i;
-    g = (uint32_t)s.in_group[i];
-    const bool gate = s.rq_flags[i] & 2;
-    uint32_t promoter, b = kNone;
-    if (r.m < s.rq_h[i]) {
-      b = s.pos_blk[pos];
-      promoter = tag_req(ldcg_u64(s.blk_promo + b), c->step);
+    const bool gate = fl & 2;
+    uint32_t promoter;
+    if (r.m < h) {
+      promoter = tag_req(ldcg_u64(s.blk_promo + b), step);
     } else {
-      promoter = ldcg_u32(&s.claims[s.pos_claim[pos]].promo);
+      b = kNone;
+      promoter = ldcg_u32(&s.claims[slot].promo);
     }
     if (!gate) {
       gated = i < promoter;
@@ -2030,7 +2059,7 @@ __global__ void __launch_bounds__(kBmChunk) k_bm_write(DevState s) {
 // then clears its claim-map slot (no other thread reads it here), and each
 // request's first position commits its OnRequest / RecordSuccessfulAdmission
 // history update.
-__global__ void __launch_bounds__(kThreads) k_insert(DevState s) {
+__global__ void __launch_bounds__(kThreads, 5) k_insert(DevState s) {
   s = with_args(s);
   Ctl* c = s.ctl;
   if (c->status != PS_OK) return;
@@ -2040,50 +2069,69 @@ __global__ void __launch_bounds__(kThreads) k_insert(DevState s) {
   bool placed = false, evicted = false;
   uint32_t g = 0, gold = 0;
   if (pos_ref(s, pos, &r)) {
+    // Three rounds of loads, each issued as a whole before anything is stored
+    // (a store or an atomic in between would hold back the loads after it):
+    // the position's and its request's records; the id and the claim; the
+    // id's old record.
     const uint32_t i = r.i;
-    const int si = s.rq_s[i], a = s.rq_a[i];
+    const int si = s.rq_s[i], a = s.rq_a[i], cbase = s.rq_cbase[i], n = s.rq_n[i], pbase = s.rq_pbase[i];
+    const int cid = s.rq_cid[i];
+    const uint32_t hs = s.rq_hs[i];
+    const uint64_t p = s.rq_p[i], key = s.pos_key[pos];
+    const uint8_t knew = s.rq_knew[i];
+    const uint32_t pc = s.pos_claim[pos];
+    const int64_t n_alloc = c->n_alloc;
+    const uint64_t base = c->stamp_base;
     g = (uint32_t)s.in_group[i];
-    if (r.m == 0) {  // history commit of request i (it has a full block)
-      const uint32_t hs = s.rq_hs[i];
-      if (hs != kNone) {
-        atomicAdd(&s.hist[hs].refadm, 1u);
-        if (a > 0) atomicOr(&s.hist[hs].refadm, 0x80000000u);
-      }
+    const uint32_t slot = r.m >= si ? pc : kNone;  // an own claim
+    const bool grant = r.m >= si && r.m < si + a;
+    const int64_t rank = (int64_t)cbase + (r.m - si);
+    ClaimEntry e{};
+    uint32_t b = kNone;
+    if (grant) {
+      e = s.claims[slot];
+      if (rank < n_alloc) b = (uint32_t)s.out.admitted_ids[rank];
     }
-    const uint32_t slot = r.m >= si ? s.pos_claim[pos] : kNone;  // an own claim
-    if (r.m >= si && r.m < si + a) {
-      const int64_t rank = (int64_t)s.rq_cbase[i] + (r.m - si);
-      const uint32_t b = rank < c->n_alloc ? (uint32_t)s.out.admitted_ids[rank] : kNone;
+    uint8_t ofl = 0;
+    uint32_t oslot = 0;
+    uint64_t okey = 0;
+    uint16_t ogrp = 0;
+    if (b < (uint64_t)s.N) {
+      // a resident id is a victim, whose old content (table entry, record)
+      // leaves first
+      ofl = s.blk_flags[b];
+      oslot = s.blk_slot[b];
+      okey = s.blk_key[b];
+      ogrp = s.blk_group[b];
+    }
+    if (r.m == 0 && hs != kNone) {  // history commit of request i (it has a full block)
+      atomicAdd(&s.hist[hs].refadm, 1u);
+      if (a > 0) atomicOr(&s.hist[hs].refadm, 0x80000000u);
+    }
+    if (grant) {
       if (b >= (uint64_t)s.N) {
         c->internal_error = 1;  // the allocated set is short: never expected
       } else {
-        const ClaimEntry e = s.claims[slot];
-        const uint64_t key = s.pos_key[pos];
-        // the id's old record, loaded together: a resident id is a victim,
-        // whose old content (table entry, record) leaves first
-        const uint8_t ofl = s.blk_flags[b];
-        const uint32_t oslot = s.blk_slot[b];
-        const uint64_t okey = s.blk_key[b];
-        const uint16_t ogrp = s.blk_group[b];
         if (ofl & 1) {
           table_delete_known(s, oslot, okey, ogrp);
           gold = ogrp;
           evicted = true;
         }
-        s.blk_key[b] = key;
-        s.blk_group[b] = (uint16_t)g;
-        s.blk_contract[b] = (uint8_t)s.rq_cid[i];
-        s.blk_prefix[b] = s.rq_p[i];
-        s.blk_klass[b] = e.promo != kNone ? (uint8_t)kReuse : s.rq_knew[i];
+        const uint32_t nslot = table_insert(s, key, g, b);
         // the latest request that touched it: an in-step toucher's stamp, or
         // the owner's own
-        const uint64_t st = tmax<uint64_t>(e.stamp, make_stamp(c->stamp_base, s.rq_pbase[i], s.rq_n[i], r.m));
+        const uint64_t st = tmax<uint64_t>(e.stamp, make_stamp(base, pbase, n, r.m));
+        s.blk_key[b] = key;
+        s.blk_group[b] = (uint16_t)g;
+        s.blk_contract[b] = (uint8_t)cid;
+        s.blk_prefix[b] = p;
+        s.blk_klass[b] = e.promo != kNone ? (uint8_t)kReuse : knew;
         s.blk_stamp[b] = st;
-        if (s.lg_on) s.lg_slot[st - c->stamp_base] = b;
+        if (s.lg_on) s.lg_slot[st - base] = b;
         s.blk_acc[b] = e.tcnt;
         s.blk_freq[b] = e.tcnt;
         s.blk_flags[b] = 1;
-        s.blk_slot[b] = table_insert(s, key, g, b);
+        s.blk_slot[b] = nslot;
         placed = true;  // its resident bit was set with the allocated set
       }
     }
