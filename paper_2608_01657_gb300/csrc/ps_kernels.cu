@@ -1990,63 +1990,100 @@ __global__ void __launch_bounds__(kBmChunk) k_bm_count(DevState s) {
 // at most 8192 ids of each kind), so one block scan carries all three.
 __device__ __forceinline__ uint64_t pack3(uint64_t a, uint64_t b, uint64_t c) { return a | b << 21 | c << 42; }
 __device__ __forceinline__ int64_t field3(uint64_t v, int k) { return (int64_t)((v >> (21 * k)) & 0x1FFFFF); }
-__global__ void __launch_bounds__(kBmChunk) k_bm_write(DevState s) {
+// The lowest 'want' set bits of f, 0 <= want <= popc(f) (a search for the
+// want-th set bit by halves; __fns is a loop of up to 32 rounds).
+__device__ __forceinline__ uint32_t lowest_bits(uint32_t f, int want) {
+  if (want == 0) return 0;
+  int left = want, p = 0;
+#pragma unroll
+  for (int st = 16; st > 0; st >>= 1) {
+    const int n = __popc((f >> p) & ((1u << st) - 1u));
+    if (left > n) {
+      left -= n;
+      p += st;
+    }
+  }
+  return f & ((2u << p) - 1u);
+}
+// The ids of nw bitmap words from w0 on to the three lists: a warp takes a
+// word, a lane an id, so a list's stores coalesce (a thread a word wrote up to
+// 32 ids one after the other, in as many rounds as the fullest word).
+struct ListSmem {
+  uint32_t word[3][kBmChunk];  // allocated, evicted, invalidated ids of each word
+  int32_t base[3][kBmChunk];   // where they go
+};
+__device__ __forceinline__ void write_ids(const DevState& s, const ListSmem& sm, int64_t w0, int nw) {
+  int32_t* outs[3] = {s.out.admitted_ids, s.out.evicted_ids, s.out.invalidated_ids};
+  const int lane = lane_id();
+  const unsigned lt = (1u << lane) - 1u;
+  for (int w = (int)(threadIdx.x >> 5); w < nw; w += (int)(blockDim.x >> 5)) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const uint32_t bits = sm.word[k][w];
+      const int64_t o = (int64_t)sm.base[k][w] + __popc(bits & lt);
+      if (((bits >> lane) & 1u) && o < s.max_blocks) outs[k][o] = (int32_t)((w0 + w) * 32 + lane);
+    }
+  }
+}
+constexpr int kBmThreads = 512;
+__global__ void __launch_bounds__(kBmThreads, 3) k_bm_write(DevState s) {
   s = with_args(s);
+  __shared__ ListSmem sm;
   Ctl* c = s.ctl;
   if (c->status != PS_OK) return;
-  const int64_t w = (int64_t)blockIdx.x * kBmChunk + threadIdx.x;
+  const int t = (int)threadIdx.x;
+  const int64_t w0 = (int64_t)blockIdx.x * kBmChunk, w = w0 + t;
   const int nchunks = gridDim.x;
-  const bool in = w < s.nwords;
+  const bool in = t < kBmChunk && w < s.nwords;  // the first kBmChunk threads hold a word each
   const int64_t ftake = c->ftake;
-  // earlier chunks' free, evicted and invalidated ids (summed field by field)
+  const uint32_t vic = in ? s.bm_victim[w] : 0u, inv = in ? s.bm_inval[w] : 0u;
+  // earlier chunks' free, evicted and invalidated ids
   int64_t fb = 0, vb = 0, ib = 0;
-  for (int j = threadIdx.x; j < (int)blockIdx.x; j += blockDim.x) {
+  for (int j = t; j < (int)blockIdx.x; j += kBmThreads) {
     fb += s.bm_chunk_cnt[0 * nchunks + j];
     vb += s.bm_chunk_cnt[1 * nchunks + j];
     ib += s.bm_chunk_cnt[2 * nchunks + j];
   }
+  const int64_t here = s.bm_chunk_cnt[blockIdx.x];
   {
-    __shared__ int64_t s_before[3][kBmChunk / 32];
+    __shared__ int64_t s_before[3][kBmThreads / 32];
     fb = warp_sum(fb); vb = warp_sum(vb); ib = warp_sum(ib);
-    if (lane_id() == 0) { s_before[0][threadIdx.x >> 5] = fb; s_before[1][threadIdx.x >> 5] = vb; s_before[2][threadIdx.x >> 5] = ib; }
+    if (lane_id() == 0) { s_before[0][t >> 5] = fb; s_before[1][t >> 5] = vb; s_before[2][t >> 5] = ib; }
     __syncthreads();
-    fb = vb = ib = 0;
-#pragma unroll
-    for (int q = 0; q < kBmChunk / 32; ++q) { fb += s_before[0][q]; vb += s_before[1][q]; ib += s_before[2][q]; }
+    const bool hold = lane_id() < kBmThreads / 32;
+    fb = warp_sum(hold ? s_before[0][lane_id()] : (int64_t)0);
+    vb = warp_sum(hold ? s_before[1][lane_id()] : (int64_t)0);
+    ib = warp_sum(hold ? s_before[2][lane_id()] : (int64_t)0);
   }
-  const int64_t take_here = tmin(ftake, fb + s.bm_chunk_cnt[blockIdx.x]) - tmin(ftake, fb);
+  const int64_t take_here = tmin(ftake, fb + here) - tmin(ftake, fb);
   // this word's taken free ids: the chunk's lowest take_here free ids
   const uint32_t f = (in && take_here > 0) ? free_word(s, w) : 0u;
-  const uint32_t vic = in ? s.bm_victim[w] : 0u, inv = in ? s.bm_inval[w] : 0u;
   uint64_t tot1;
   const uint64_t ex1 = block_excl_scan<uint64_t>(pack3(__popc(f), __popc(vic), __popc(inv)), &tot1);
   const int64_t fl = field3(ex1, 0);
   const int64_t want = tmin<int64_t>(tmax<int64_t>(take_here - fl, 0), __popc(f));
-  // the lowest 'want' set bits of f: everything below the want-th set bit, and it
-  const uint32_t taken = want == 0 ? 0u : (want >= 32 ? f : (f & ((2u << __fns(f, 0, (int)want)) - 1u)));
-  const uint32_t alloc = taken | vic;
-  if (in) s.res_bits[w] |= alloc;  // every allocated id is resident after the step
-  uint64_t tot2;
-  const uint64_t ex2 = block_excl_scan<uint64_t>((uint64_t)__popc(alloc), &tot2);
-  const uint32_t bitsk[3] = {alloc, vic, inv};
-  const int64_t basek[3] = {vb + tmin(ftake, fb) + (int64_t)ex2, vb + field3(ex1, 1), ib + field3(ex1, 2)};
-  int32_t* outs[3] = {s.out.admitted_ids, s.out.evicted_ids, s.out.invalidated_ids};
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    int64_t o = basek[k];
-    for (uint32_t b = bitsk[k]; b; b &= b - 1) {
-      if (o < s.max_blocks) outs[k][o] = (int32_t)(w * 32 + __ffs(b) - 1);
-      ++o;
-    }
-  }
-  if (blockIdx.x == nchunks - 1 && threadIdx.x == 0) {
-    c->n_alloc = vb + tmin(ftake, fb) + (int64_t)tot2;
-    c->n_evicted = vb + field3(tot1, 1);
-  }
+  const uint32_t alloc = lowest_bits(f, (int)want) | vic;
+  // taken ids before the word: the free ones before it, up to take_here
+  const int64_t ex2 = tmin(fl, take_here) + field3(ex1, 1);
   if (in) {
+    s.res_bits[w] |= alloc;  // every allocated id is resident after the step
     s.bm_victim[w] = 0;
     s.bm_inval[w] = 0;
   }
+  if (t < kBmChunk) {
+    sm.word[0][t] = alloc;
+    sm.word[1][t] = vic;
+    sm.word[2][t] = inv;
+    sm.base[0][t] = (int32_t)(vb + tmin(ftake, fb) + ex2);
+    sm.base[1][t] = (int32_t)(vb + field3(ex1, 1));
+    sm.base[2][t] = (int32_t)(ib + field3(ex1, 2));
+  }
+  if (blockIdx.x == nchunks - 1 && t == 0) {
+    c->n_alloc = vb + tmin(ftake, fb) + take_here + field3(tot1, 1);
+    c->n_evicted = vb + field3(tot1, 1);
+  }
+  __syncthreads();
+  write_ids(s, sm, w0, kBmChunk);
 }
 
 // Stage 6: place granted claims (thread per position).  The allocated ids
@@ -2354,7 +2391,7 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
   mark(7);
   const int nchunks = (int)((s.nwords + kBmChunk - 1) / kBmChunk);
   PS_LAUNCH(launch_k(k_bm_count, nchunks, kBmChunk, 0, st, s));
-  PS_LAUNCH(launch_k(k_bm_write, nchunks, kBmChunk, 0, st, s));
+  PS_LAUNCH(launch_k(k_bm_write, nchunks, kBmThreads, 0, st, s));
   mark(8);
   // (evictions happen in k_insert: every victim is allocated again in its step)
   mark(9);
