@@ -233,6 +233,35 @@ __global__ void k_init_ctl(DevState s) {
 // and per-step scalars, and clears the tile words for the next call.
 // 'probe' skips the clock and step checks.  Every write is bounds-checked, so
 // inputs that turn out invalid write nothing outside the scratch arrays.
+// A warp's requests' chunk descriptors, a lane per chunk: its request is found
+// among the warp's by the chunks before it, and the request's values come by
+// shuffles (a loop over the requests took a pass of mostly idle lanes each).
+__device__ __forceinline__ void write_chunks(const DevState& s, int32_t ns, int32_t n, int64_t o0, int32_t sbase,
+                                             int32_t pbase, uint32_t i, uint32_t g) {
+  const int lane = lane_id();
+  const int32_t incl = warp_incl_scan(ns), ex = incl - ns;
+  const int32_t tot = __shfl_sync(kFull, incl, 31);
+  for (int q0 = 0; q0 < tot; q0 += 32) {
+    const int q = q0 + lane;
+    int src = 0;  // the last request with at most q chunks before it
+#pragma unroll
+    for (int st = 16; st > 0; st >>= 1)
+      if (__shfl_sync(kFull, ex, src + st) <= q) src += st;
+    ChunkDesc d;
+    d.o0 = __shfl_sync(kFull, o0, src);
+    d.req = __shfl_sync(kFull, i, src);
+    d.n = __shfl_sync(kFull, n, src);
+    d.pbase = __shfl_sync(kFull, pbase, src);
+    d.k = q - __shfl_sync(kFull, ex, src);
+    d.group = __shfl_sync(kFull, g, src);
+    d.sb = __shfl_sync(kFull, sbase, src);
+    if (q < tot) {
+      s.chunks[d.sb + d.k] = d;
+      s.seg_word[d.sb + d.k] = 0;
+    }
+  }
+}
+
 constexpr uint64_t kTileFlag = 1ull << 63;
 
 __global__ void __launch_bounds__(kValTile) k_validate(DevState s, int probe) {
@@ -251,7 +280,7 @@ __global__ void __launch_bounds__(kValTile) k_validate(DevState s, int probe) {
     o0 = s.in_offsets[i];
     const int64_t o1 = s.in_offsets[i + 1];
     g = s.in_group[i];
-    const int64_t nb = (o1 - o0) / s.bs;
+    const int64_t nb = (o1 - o0) >> (__ffs(s.bs) - 1);  // a power of two
     bad = o1 < o0 || g < 0 || g >= s.G || nb > (int64_t)kMaxPos;
     if (s.in_contract) {
       cid = s.in_contract[i];
@@ -300,29 +329,8 @@ __global__ void __launch_bounds__(kValTile) k_validate(DevState s, int probe) {
       s.rq_p[i] = 0;
     }
   }
-  // each request's chunk descriptors; the warp writes one request's chunks
-  // at a time, so the stores coalesce
-  const bool room = in && pbase + n <= s.max_blocks && sbase + ns <= s.max_segments;
-  for (unsigned todo = __ballot_sync(kFull, room && ns > 0); todo; todo &= todo - 1) {
-    const int src = __ffs(todo) - 1;
-    const int64_t ro0 = __shfl_sync(kFull, o0, src);
-    const int64_t rsb = __shfl_sync(kFull, sbase, src);
-    const int32_t rpb = (int32_t)__shfl_sync(kFull, pbase, src);
-    const int32_t rn = __shfl_sync(kFull, n, src), rns = __shfl_sync(kFull, ns, src);
-    const uint32_t ri = (uint32_t)__shfl_sync(kFull, i, src), rg = (uint32_t)__shfl_sync(kFull, g, src);
-    for (int k = lane_id(); k < rns; k += 32) {
-      ChunkDesc d;
-      d.o0 = ro0;
-      d.req = ri;
-      d.n = rn;
-      d.pbase = rpb;
-      d.k = k;
-      d.group = rg;
-      d.sb = (int32_t)rsb;
-      s.chunks[rsb + k] = d;
-      s.seg_word[rsb + k] = 0;
-    }
-  }
+  write_chunks(s, in && pbase + n <= s.max_blocks && sbase + ns <= s.max_segments ? ns : 0, n, o0, (int32_t)sbase,
+               (int32_t)pbase, (uint32_t)i, (uint32_t)g);
   if (!probe && tile == 0) {  // per-step counts accumulated by later kernels
     if (s.policy == PS_STATICQUOTA)
       for (int gg = threadIdx.x; gg < s.G; gg += blockDim.x) s.grp_pinned[gg] = 0;
