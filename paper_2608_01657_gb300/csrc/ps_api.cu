@@ -457,6 +457,10 @@ int32_t ps_create(ps_handle_t** out, int64_t capacity_blocks, int32_t block_size
     s.beta[c] = c < s.C ? params->beta_fp[c] : 0;
     if (c < s.C && params->rho_fp[c] < s.rho_min) s.rho_min = params->rho_fp[c];
   }
+  for (int c = 0; c < PS_MAX_CONTRACTS; ++c) {
+    s.delta[c] = c < s.C ? (int64_t)(((__int128)1 << s.fp_shift) * s.rho_min / s.rho[c]) : 0;
+    s.delta_rcp[c] = s.delta[c] > 0 ? ~0ull / (uint64_t)s.delta[c] : 0;
+  }
   s.s3_small_pct = params->s3_small_pct; s.s3_freq_cap = params->s3_freq_cap; s.s3_move_min = params->s3_move_min_freq;
   s.s3_small_cap = d.s3_small_cap; s.s3_ghost_cap = d.s3_ghost_cap;
   s.gh_nbuckets_log2 = d.gh_log2; s.ghost_ring_cap = d.ghost_ring_cap;

@@ -237,6 +237,8 @@ struct DevState {
   uint64_t chain_mul, digest_mul;  // Kc, Kd of the key chain (mod 2^61-1)
   int64_t max_segments;
   int64_t rho[PS_MAX_CONTRACTS], beta[PS_MAX_CONTRACTS];
+  int64_t delta[PS_MAX_CONTRACTS];      // Eq. 8 decrement of an indebted contract: floor(2^fp rho_min / rho) >= 1
+  uint64_t delta_rcp[PS_MAX_CONTRACTS]; // floor((2^64 - 1) / delta)
   int64_t rho_min;
   int32_t s3_small_pct, s3_freq_cap, s3_move_min;
   int64_t s3_small_cap, s3_ghost_cap;

@@ -48,12 +48,20 @@ __device__ __forceinline__ uint32_t tag_req(uint64_t tag, uint64_t step) {
   return (tag >> 32) == step ? 0xFFFFFFFFu - (uint32_t)tag : 0xFFFFFFFFu;
 }
 __device__ __forceinline__ int64_t refill(int64_t b, int64_t beta, int64_t rho, int64_t dt) {
-  // Eq. 1, min{beta, b + rho*dt}, without overflow (dt >= ceil(need/rho) saturates).
+  // Eq. 1, min{beta, b + rho*dt}, without overflow and without a division.
+  // rho*dt >= need decides it; a product past 64 bits is past any need.
   const int64_t need = beta - b;
-  if (need <= 0 || dt >= (need + rho - 1) / rho) return beta;
-  return b + rho * dt;
+  const uint64_t add = (uint64_t)rho * (uint64_t)dt;
+  if (need <= 0 || __umul64hi((uint64_t)rho, (uint64_t)dt) != 0 || add >= (uint64_t)need) return beta;
+  return b + (int64_t)add;
 }
+// floor(a * b / c) for a >= 0 and 0 < b <= c.  A 128-bit division is a call of
+// about a microsecond, so the cases without one go first: nothing owed, equal
+// rates (one contract, or the slowest one), a product that fits 64 bits.
 __device__ __forceinline__ int64_t muldiv(int64_t a, int64_t b, int64_t c) {
+  if (a == 0) return 0;
+  if (b == c) return a;
+  if (__umul64hi((uint64_t)a, (uint64_t)b) == 0) return (int64_t)(((uint64_t)a * (uint64_t)b) / (uint64_t)c);
   return (int64_t)(((__int128)a * (__int128)b) / (__int128)c);
 }
 
@@ -858,9 +866,10 @@ __global__ void __launch_bounds__(1024) k_grant(DevState s0) {
   const int64_t carry_c = (int64_t)(carry >> 32);
   const int64_t carry_a = quota ? (int64_t)(uint32_t)carry : tmin(avail, carry_c);
   int64_t qv = 0;  // StaticQuota: the groups' overflows are the victims
-  if (quota)
+  if (quota) {
     for (int g = threadIdx.x; g < s.G; g += blockDim.x) qv += s.grp_x[g];
-  qv = block_sum(qv);
+    qv = block_sum(qv);
+  }
   if (threadIdx.x == 0) {
     const int64_t need = carry_a;
     s.out.admitted_offsets[R] = (int32_t)need;
@@ -879,7 +888,8 @@ __global__ void __launch_bounds__(1024) k_grant(DevState s0) {
   __syncthreads();
   const int64_t unit = (int64_t)1 << s.fp_shift;
   for (int g = threadIdx.x; g < s.G; g += blockDim.x) {
-    int64_t raw = 0, norm = 0, rmax = 0;
+    // the Eq. 8 decrement of the largest indebted rate is the smallest one
+    int64_t raw = 0, norm = 0, delta = 0;
     for (int cc = 0; cc < C; ++cc) {
       const int64_t b0 = refill(s.ledger[g * C + cc], s0.beta[cc], s0.rho[cc], s.now - c->t_prev);
       s.ledger_b0[g * C + cc] = b0;
@@ -888,7 +898,7 @@ __global__ void __launch_bounds__(1024) k_grant(DevState s0) {
       const int64_t def = tmax<int64_t>(0, -b);
       raw += def;                                    // Eq. 3
       norm += muldiv(def, s.rho_min, s0.rho[cc]);    // Eq. 5
-      if (b < 0) rmax = tmax(rmax, s0.rho[cc]);
+      if (b < 0 && (delta == 0 || s0.delta[cc] < delta)) delta = s0.delta[cc];
     }
     int64_t* row = s.stats + (int64_t)g * PS_NUM_STATS;
     row[PS_STAT_DEBT_RAW] = raw;
@@ -896,7 +906,7 @@ __global__ void __launch_bounds__(1024) k_grant(DevState s0) {
     s.out.debt_raw[g] = raw;
     s.out.debt_norm[g] = norm;
     s.grp_P[g] = norm;
-    s.grp_delta[g] = rmax ? muldiv(unit, s.rho_min, rmax) : 0;  // 1/W_g of Eq. 8
+    s.grp_delta[g] = delta;  // 1/W_g of Eq. 8
     SelSeg z{};
     z.kmin = ~0ull;
     z.kmax = 0;
@@ -1420,11 +1430,12 @@ __global__ void __launch_bounds__(1024) k_quota_sel(DevState s) {
 // each) the ones with the smallest candidate keys are taken (resolved after
 // the radix select finds those keys).  What the debt phase cannot cover goes
 // to the global fallback in (class, stamp) order.
-__global__ void __launch_bounds__(1024) k_waterfill(DevState s, cudaGraphConditionalHandle fb_cond, int has_cond) {
-  s = with_args(s);
+__global__ void __launch_bounds__(1024) k_waterfill(DevState s0, cudaGraphConditionalHandle fb_cond, int has_cond) {
+  // contract arrays are read from the parameter block (see k_grant)
+  const DevState s = with_args(s0);
   Ctl* c = s.ctl;
   __shared__ int64_t sP[PS_MAX_GROUPS], sD[PS_MAX_GROUPS], sQ[PS_MAX_GROUPS];
-  __shared__ uint64_t sRcp[PS_MAX_GROUPS];  // floor((2^64 - 1) / d) for the division below
+  __shared__ uint64_t sRcp[PS_MAX_GROUPS];  // floor((2^64 - 1) / d) for the division below (d: some contract's)
   __shared__ int64_t s_pmax;
   const int G = s.G;
   const int64_t eps = s.eps;
@@ -1439,7 +1450,10 @@ __global__ void __launch_bounds__(1024) k_waterfill(DevState s, cudaGraphConditi
     sP[g] = s.grp_P[g];
     sD[g] = s.grp_delta[g];
     sQ[g] = s.grp_qsize[g];
-    sRcp[g] = sD[g] > 1 ? ~0ull / (uint64_t)sD[g] : 0;
+    uint64_t rcp = 0;
+    for (int cc = 0; cc < s.C; ++cc)
+      if (s0.delta[cc] == sD[g]) rcp = s0.delta_rcp[cc];
+    sRcp[g] = rcp;
   }
   if (threadIdx.x == 0) s_pmax = 0;
   __syncthreads();
@@ -1470,6 +1484,7 @@ __global__ void __launch_bounds__(1024) k_waterfill(DevState s, cudaGraphConditi
       const bool full = x > 0 && x == sQ[g];
       s.grp_x[g] = x;
       s.grp_full[g] = full ? 1 : 0;
+      if (x == 0) continue;  // k_grant left the segment inactive
       SelSeg z = s.sel[g];
       z.rank = full ? 0 : x;
       z.active = x > 0 && !full;
@@ -1547,14 +1562,15 @@ __global__ void __launch_bounds__(1024) k_waterfill(DevState s, cudaGraphConditi
     const bool tied = d > 0 && P >= tau && qt * (uint64_t)d == (uint64_t)(P - tau) && (int64_t)qt < q;
     above += xa;
     ntie += tied;
+    s.grp_x[g] = xa + (tied ? 1 : 0);
+    s.grp_full[g] = 0;
+    if (xa == 0 && !tied) continue;  // k_grant left the segment inactive
     SelSeg z = s.sel[g];
     z.rank = xa + (tied ? 1 : 0);
-    z.active = z.rank > 0;
+    z.active = 1;
     z.incl = tied ? 2 : 1;  // 2: the tie item is taken only if the tie rule chooses it
     sel_start_group(s, g, z, seg);
     s.sel[g] = z;
-    s.grp_x[g] = xa + (tied ? 1 : 0);
-    s.grp_full[g] = 0;
   }
   above = block_sum(above);
   ntie = block_sum(ntie);
