@@ -2314,7 +2314,7 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
   // The candidates read pins and residency (final from here on) and the class
   // and stamp of unpinned blocks, which S3-S4 leave alone: under capture
   // they are counted on a side branch that runs beside the rest of S3-S4.
-  // The candidate scan writes per-step scratch only, so it forks before the
+  // The candidate scan writes per-step scratch only, so it forks beside the
   // grants (a step the grant then fails ignores what it wrote); the indexed
   // queues' count applies the step's pins to persistent counts, so it waits
   // for the grant's verdict.
@@ -2331,8 +2331,9 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
     if (s.lg_on) {
       if (launch_queue_cand(s, cs, &launches) != PS_OK) return PS_ERR_CUDA;
     } else if (s.policy != PS_S3FIFO) {
-      // one 512-thread CTA per SM: the main branch keeps room on every SM
-      PS_LAUNCH(k_cand<<<fork ? 152 : grid_for(s.N, 1024 * 4, 152), fork ? 512 : 1024, cand_smem, cs>>>(s));
+      // two 512-thread CTAs an SM, less than all of them: the grants' CTA holds
+      // an SM meanwhile, and CTAs left over would run as a second wave
+      PS_LAUNCH(k_cand<<<fork ? 2 * 152 - 8 : grid_for(s.N, 1024 * 4, 152), fork ? 512 : 1024, cand_smem, cs>>>(s));
     }
     if (fork && cudaEventRecord(cap->join, cs) != cudaSuccess) return PS_ERR_CUDA;
     return PS_OK;
@@ -2356,8 +2357,14 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
     if (cudaEventRecord(cap->fork2, st) != cudaSuccess || cudaStreamWaitEvent(cap->side2, cap->fork2, 0) != cudaSuccess)
       return PS_ERR_CUDA;
     ms = cap->side2;
+    // The candidate scan has the GPU to itself first: the select waits for it,
+    // and beside these kernels it took three times as long (28 us of a 177 us
+    // step at 2^20 blocks); they fill the time of the select's one-CTA kernels
+    // instead.
+    if (early && cudaStreamWaitEvent(ms, cap->join, 0) != cudaSuccess) return PS_ERR_CUDA;
   }
-  PS_LAUNCH(launch_k(k_instep, pgrid, kThreads, 0, ms, s));
+  if (fork2 && early) PS_LAUNCH((k_instep<<<pgrid, kThreads, 0, ms>>>(s)));  // after the join: plain
+  else PS_LAUNCH(launch_k(k_instep, pgrid, kThreads, 0, ms, s));
   mark(4);
   PS_LAUNCH(launch_k(k_meter, s.G, 512, 0, ms, s));
   mark(5);
