@@ -1506,7 +1506,6 @@ __global__ void __launch_bounds__(1024) k_waterfill(DevState s0, cudaGraphCondit
   // more rounds beat several per thread and fewer rounds.
   __shared__ int16_t s_gid[PS_MAX_GROUPS];
   __shared__ int s_ng;
-  __shared__ int s_J[3];
   {
     int k = 0;
     for (int base = 0; base < G; base += blockDim.x) {
@@ -1518,7 +1517,6 @@ __global__ void __launch_bounds__(1024) k_waterfill(DevState s0, cudaGraphCondit
       k += tot;
     }
     if (threadIdx.x == 0) s_ng = k;
-    if (threadIdx.x < 3) s_J[threadIdx.x] = -1;
     __syncthreads();
   }
   const int ng = s_ng;
@@ -1528,7 +1526,7 @@ __global__ void __launch_bounds__(1024) k_waterfill(DevState s0, cudaGraphCondit
     while (L < ng && L < 32) { L <<= 1; --logT; }
     const int T = 1 << logT;
     const int jt = threadIdx.x / L, gl = threadIdx.x % L;
-    for (int r = 0; lo < hi; ++r) {
+    while (lo < hi) {
       const int64_t span = hi - lo;  // >= 1
       const int64_t stride = tmax<int64_t>(1, (span + T - 1) >> logT);
       auto thr = [&](int jj) -> int64_t { return jj == T - 1 ? hi : tmin<int64_t>(hi, lo + 1 + stride * jj); };
@@ -1536,13 +1534,11 @@ __global__ void __launch_bounds__(1024) k_waterfill(DevState s0, cudaGraphCondit
       int64_t cnt = 0;
       for (int k = gl; k < ng; k += L) cnt += items_gt(s_gid[k], t - 1);
       for (int o = L / 2; o > 0; o >>= 1) cnt += __shfl_xor_sync(kFull, cnt, o);
-      // J = the largest threshold still holding m items (counts fall as the
-      // threshold rises); slots rotate over three rounds, so one barrier a
-      // round separates every slot's reset, updates and reads
-      if (threadIdx.x == 0) s_J[(r + 1) % 3] = -1;
-      if (gl == 0 && cnt >= m) atomicMax(&s_J[r % 3], jt);
-      __syncthreads();
-      const int J = s_J[r % 3];
+      // J = the largest threshold still holding m items: counts fall as the
+      // threshold rises, so it is the number of such thresholds less one, and
+      // the round's one barrier counts them (a shared maximum taken by up to
+      // 1024 threads made a round 1.1 us, six of them a search)
+      const int J = __syncthreads_count(gl == 0 && cnt >= m) - 1;
       if (J < 0) {
         hi = lo;
       } else {
