@@ -19,7 +19,8 @@ namespace ps {
 
 constexpr int kFinCap = 8192;  // split lists up to this size are finished by one CTA in shared memory
 constexpr int kFinRows = 32;   // rows k_list_finish counts at once (32 KB)
-constexpr int kFinCountCap = 512;  // split lists up to this size are ranked by counting
+constexpr int kFinCountCap = 512;  // split lists up to this size may be ranked by counting,
+constexpr int kFinShort = 128;     // and up to this size are
 
 // 128-bit compare-and-swap (sm_90+): installs the (p, group) identity of a
 // history entry atomically, so two requests of one (group, prefix) that race
@@ -1806,12 +1807,27 @@ __device__ __forceinline__ int next_shift(uint64_t mask) {
   return __ffsll((long long)mask) - 1 - 8;
 }
 
+// The lowest 'want' set bits of f, 0 <= want <= popc(f) (a search for the
+// want-th set bit by halves; __fns is a loop of up to 32 rounds).
+__device__ __forceinline__ uint32_t lowest_bits(uint32_t f, int want) {
+  if (want == 0) return 0;
+  int left = want, p = 0;
+#pragma unroll
+  for (int st = 16; st > 0; st >>= 1) {
+    const int n = __popc((f >> p) & ((1u << st) - 1u));
+    if (left > n) {
+      left -= n;
+      p += st;
+    }
+  }
+  return f & ((2u << p) - 1u);
+}
 // The rest of a select on one CTA, with every segment's state in shared
-// memory.  A split list of at most kFinCap members is staged in shared memory
-// too; a longer one (rare: a boundary bucket of the first digit holding many
-// candidates) is read from global memory in each round.  The segments'
-// thresholds come from ranking by counting (lists of at most kFinCountCap
-// members) or from the remaining radix digits, one round per digit; then
+// memory.  The segments' thresholds come from bitmaps of their buckets where
+// those are narrow (the usual case: a bucket is a 4096th of the class's
+// stamps), else from ranking the list by counting (at most kFinCountCap
+// members) or from the remaining radix digits, one round per digit, over the
+// list in shared memory (at most kFinCap members) or in global memory; then
 // Eq. 7's tie rule, then the list's victims.  One launch for every list
 // length keeps the step graph free of conditional nodes here.
 struct FinSeg {
@@ -1819,14 +1835,19 @@ struct FinSeg {
   int64_t rank;
   int32_t active, incl;
 };
-constexpr size_t kFinSmem = (size_t)kFinCap * 8 + (size_t)kFinCap * 2 + (size_t)kFinRows * kRadixBins * 4 +
-                            (size_t)PS_MAX_GROUPS * sizeof(FinSeg);
+constexpr size_t kFinList = (size_t)kFinCap * 8 + (size_t)kFinRows * kRadixBins * 4 + (size_t)kFinCap * 2;
+constexpr int kFinWords = (int)(kFinList / 4);  // bitmap words in the list's place
+constexpr int kFinSegWords = 1024;              // of one segment (one warp searches them)
+constexpr size_t kFinSmem = kFinList + (size_t)PS_MAX_GROUPS * (sizeof(FinSeg) + 8 + 4 + 2);
 
 __global__ void __launch_bounds__(1024) k_list_finish(DevState s, int single) {
   s = with_args(s);
   extern __shared__ __align__(16) unsigned char fin_smem[];
   FinSeg* sl = reinterpret_cast<FinSeg*>(fin_smem);
-  uint64_t* lkey = reinterpret_cast<uint64_t*>(sl + PS_MAX_GROUPS);
+  uint64_t* blo = reinterpret_cast<uint64_t*>(sl + PS_MAX_GROUPS);  // the segments' buckets
+  int32_t* woff = reinterpret_cast<int32_t*>(blo + PS_MAX_GROUPS);  // and bitmaps
+  int16_t* wlen = reinterpret_cast<int16_t*>(woff + PS_MAX_GROUPS);
+  uint64_t* lkey = reinterpret_cast<uint64_t*>(wlen + PS_MAX_GROUPS);
   uint32_t* fh = reinterpret_cast<uint32_t*>(lkey + kFinCap);
   uint16_t* lseg = reinterpret_cast<uint16_t*>(fh + kFinRows * kRadixBins);
   __shared__ int16_t row_of[PS_MAX_GROUPS];
@@ -1842,17 +1863,81 @@ __global__ void __launch_bounds__(1024) k_list_finish(DevState s, int single) {
   const int64_t n = c->lst_n;
   const bool small = n <= kFinCap;
   const int warp = threadIdx.x >> 5, lane = lane_id();
-  // the list's members of a segment share the bits above the highest byte
-  // where their smallest and largest key differ: those are fixed already
-  for (int g = threadIdx.x; g < nseg; g += blockDim.x) {
-    const SelSeg z = s.sel[g];
-    const bool listed = z.qmin <= z.qmax;
-    const int fs = listed ? first_shift(z.qmin, z.qmax) : 56;
-    const uint64_t mask = fs < 0 ? ~0ull : above_mask(fs);
-    sl[g] = FinSeg{listed ? z.qmin & mask : 0ull, listed ? mask : ~0ull, z.rank, listed ? z.active : 0, z.incl};
+  // each thread's first member, loaded beside the segments' state
+  uint64_t my_key = 0;
+  uint32_t my_blk = 0;
+  int my_seg = 0;
+  if ((int64_t)threadIdx.x < n) {
+    my_key = s.lst_key[threadIdx.x];
+    my_blk = s.lst_blk[threadIdx.x];
+    my_seg = s.lst_seg[threadIdx.x];
   }
-  if (small)
+  // A segment's list members lie in its bucket [blo, bhi], and stamps are
+  // unique: where the buckets are narrow enough, each segment gets a bitmap of
+  // its bucket, the members set their bits, and the rank-th set bit is the
+  // threshold, whatever the list's length.
+  uint32_t* words = reinterpret_cast<uint32_t*>(lkey);  // lkey, fh and lseg: not in use on this path
+  bool by_bits = n > kFinShort;  // counting a short list needs no bitmaps set up
+  int64_t wtot = 0;
+  for (int g0 = 0; g0 < nseg; g0 += blockDim.x) {
+    const int g = g0 + (int)threadIdx.x;
+    int64_t nw = 0;
+    if (g < nseg) {
+      const SelSeg z = s.sel[g];
+      const bool listed = z.qmin <= z.qmax;
+      // the list's members share the bits above the highest byte where their
+      // smallest and largest key differ: those are fixed already
+      const int fs = listed ? first_shift(z.qmin, z.qmax) : 56;
+      const uint64_t mask = fs < 0 ? ~0ull : above_mask(fs);
+      sl[g] = FinSeg{listed ? z.qmin & mask : 0ull, listed ? mask : ~0ull, z.rank, listed ? z.active : 0, z.incl};
+      blo[g] = z.blo;
+      if (by_bits && sl[g].active) nw = (int64_t)tmin<uint64_t>((z.bhi - z.blo) >> 5, kFinSegWords) + 1;
+    }
+    by_bits = by_bits && !__syncthreads_or(nw > kFinSegWords);
+    if (!by_bits) continue;
+    int64_t tot;
+    const int64_t ex = wtot + block_excl_scan(nw, &tot);
+    if (g < nseg) {
+      woff[g] = (int32_t)tmin<int64_t>(ex, kFinWords);
+      wlen[g] = (int16_t)nw;
+    }
+    wtot += tot;
+  }
+  by_bits = by_bits && wtot <= kFinWords;
+  __syncthreads();
+  if (by_bits) {
+    for (int w = threadIdx.x; w < (int)wtot; w += blockDim.x) words[w] = 0;
+    __syncthreads();
+    for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
+      const bool mine = e == (int64_t)threadIdx.x;
+      const int g = mine ? my_seg : (int)s.lst_seg[e];
+      const uint64_t d = (mine ? my_key : ldcg_u64(s.lst_key + e)) - blo[g];
+      if (sl[g].active) atomicOr(&words[woff[g] + (int)(d >> 5)], 1u << (d & 31));
+    }
+    __syncthreads();
+    for (int g = warp; g < nseg; g += blockDim.x >> 5) {
+      if (!sl[g].active) continue;
+      const int nw = wlen[g];
+      int64_t left = sl[g].rank;
+      for (int w0 = 0; w0 < nw; w0 += 32) {
+        const uint32_t x = w0 + lane < nw ? words[woff[g] + w0 + lane] : 0u;
+        const int p = __popc(x), incl = warp_incl_scan(p);
+        const int tot = __shfl_sync(kFull, incl, 31);
+        if (left > tot) {
+          left -= tot;
+          continue;
+        }
+        if (incl - p < left && left <= incl) {  // one lane
+          const uint32_t low = lowest_bits(x, (int)(left - (incl - p)));
+          sl[g].prefix = blo[g] + (uint64_t)(w0 + lane) * 32 + (uint64_t)(31 - __clz((int)low));
+          sl[g].mask = ~0ull;
+        }
+        break;
+      }
+    }
+  } else if (small) {
     for (int64_t e = threadIdx.x; e < n; e += blockDim.x) { lkey[e] = s.lst_key[e]; lseg[e] = s.lst_seg[e]; }
+  }
   __syncthreads();
   auto key_at = [&](int64_t e) -> uint64_t { return small ? lkey[e] : ldcg_u64(s.lst_key + e); };
   auto seg_at = [&](int64_t e) -> int { return small ? (int)lseg[e] : (int)s.lst_seg[e]; };
@@ -1860,7 +1945,7 @@ __global__ void __launch_bounds__(1024) k_list_finish(DevState s, int single) {
   // whose rank among the segment's list members (keys are unique) is its
   // remaining rank - 1; L lanes rank one member by counting, so no digit
   // rounds (and their barriers) are needed.
-  const bool by_count = small && n <= kFinCountCap;
+  const bool by_count = !by_bits && small && n <= kFinCountCap;
   if (by_count) {
     int L = 32;
     while (L * (int)n > (int)blockDim.x) L >>= 1;  // kFinCountCap <= blockDim.x: L >= 1
@@ -1879,7 +1964,7 @@ __global__ void __launch_bounds__(1024) k_list_finish(DevState s, int single) {
     }
     __syncthreads();
   }
-  for (int iter = 0; !by_count && iter < 8; ++iter) {  // at most 8 digits in a 64-bit key
+  for (int iter = 0; !by_bits && !by_count && iter < 8; ++iter) {  // at most 8 digits in a 64-bit key
     {
       int k = 0;
       for (int base = 0; base < nseg; base += blockDim.x) {
@@ -1951,7 +2036,10 @@ __global__ void __launch_bounds__(1024) k_list_finish(DevState s, int single) {
     for (int g = threadIdx.x; g < nseg; g += blockDim.x) {
       if (!(sl[g].active && sl[g].incl == 2)) continue;
       int rank = 0;
-      for (int h = 0; h < nseg; ++h) rank += sl[h].active && sl[h].incl == 2 && sl[h].prefix < sl[g].prefix;
+      const uint64_t own = sl[g].prefix;
+#pragma unroll 4
+      for (int h = 0; h < nseg; ++h)
+        rank += (int)(sl[h].active != 0) & (int)(sl[h].incl == 2) & (int)(sl[h].prefix < own);
       const bool chosen = rank < k;
       s.grp_x[g] -= chosen ? 0 : 1;
       fh[g] = chosen ? 1 : 0;  // applied after every thread has read the flags
@@ -1963,10 +2051,11 @@ __global__ void __launch_bounds__(1024) k_list_finish(DevState s, int single) {
   }
   // the list's victims: keys below (or at, if incl) the threshold
   for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
-    const uint64_t key = key_at(e);
-    const FinSeg& f = sl[seg_at(e)];
+    const bool mine = e == (int64_t)threadIdx.x;
+    const uint64_t key = mine ? my_key : ldcg_u64(s.lst_key + e);
+    const FinSeg& f = sl[mine ? my_seg : (int)s.lst_seg[e]];
     if (f.active && (key < f.prefix || (f.incl && key == f.prefix))) {
-      const uint32_t b = s.lst_blk[e];
+      const uint32_t b = mine ? my_blk : s.lst_blk[e];
       atomicOr(s.bm_victim + (b >> 5), 1u << (b & 31));
     }
   }
@@ -2010,21 +2099,6 @@ __global__ void __launch_bounds__(kBmChunk) k_bm_count(DevState s) {
 // at most 8192 ids of each kind), so one block scan carries all three.
 __device__ __forceinline__ uint64_t pack3(uint64_t a, uint64_t b, uint64_t c) { return a | b << 21 | c << 42; }
 __device__ __forceinline__ int64_t field3(uint64_t v, int k) { return (int64_t)((v >> (21 * k)) & 0x1FFFFF); }
-// The lowest 'want' set bits of f, 0 <= want <= popc(f) (a search for the
-// want-th set bit by halves; __fns is a loop of up to 32 rounds).
-__device__ __forceinline__ uint32_t lowest_bits(uint32_t f, int want) {
-  if (want == 0) return 0;
-  int left = want, p = 0;
-#pragma unroll
-  for (int st = 16; st > 0; st >>= 1) {
-    const int n = __popc((f >> p) & ((1u << st) - 1u));
-    if (left > n) {
-      left -= n;
-      p += st;
-    }
-  }
-  return f & ((2u << p) - 1u);
-}
 // The ids of nw bitmap words from w0 on to the three lists: a warp takes a
 // word, a lane an id, so a list's stores coalesce (a thread a word wrote up to
 // 32 ids one after the other, in as many rounds as the fullest word).
