@@ -245,6 +245,7 @@ size_t carve(const Dims& d, char* base, DevState* s, ps_handle* h) {
   t.rq_h = cv.take<int32_t>(R);
   t.rq_s = cv.take<int32_t>(R);
   t.rq_cbase = cv.take<int32_t>(R);
+  t.rq_qbase = cv.take<int32_t>(R);
   t.rq_a = cv.take<int32_t>(R);
   t.rq_e = cv.take<int32_t>(R);
   t.rq_fu = cv.take<uint32_t>(R);
@@ -261,6 +262,7 @@ size_t carve(const Dims& d, char* base, DevState* s, ps_handle* h) {
   t.seg_word = cv.take<uint64_t>((size_t)d.max_segments);
   t.pos_blk = cv.take<uint32_t>(B);
   t.pos_claim = cv.take<uint32_t>(B);
+  t.claim_pos = cv.take<uint64_t>(B);
   t.pos_elig = cv.take<uint8_t>(B);
   t.claims = cv.take<ClaimEntry>((size_t)kClaimWays << d.cl_log2);
   t.bm_victim = cv.take<uint32_t>((size_t)d.nwords);

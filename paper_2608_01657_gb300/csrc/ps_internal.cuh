@@ -292,6 +292,7 @@ struct DevState {
   int32_t* rq_h;           // cached prefix length
   int32_t* rq_s;           // first own claim
   int32_t* rq_cbase;       // exclusive scan of claims
+  int32_t* rq_qbase;       // the step's own claims of earlier requests
   int32_t* rq_a;           // granted (admitted) blocks
   int32_t* rq_e;           // in-step hits
   uint32_t* rq_fu;         // first ungranted in-step position
@@ -308,6 +309,7 @@ struct DevState {
   uint64_t* seg_word;      // the chunk's published chain total and miss bit (k_hash_lookup)
   uint32_t* pos_blk;       // resident block hit by lookup (or kNone)
   uint32_t* pos_claim;     // claim-map slot (or kNone)
+  uint64_t* claim_pos;     // own claims in (request, position) order: request (high half), position
   uint8_t* pos_elig;       // touch was promotion-eligible
   ClaimEntry* claims;
   uint32_t* bm_victim;     // per-step bitmaps over block ids

@@ -856,6 +856,7 @@ __global__ void __launch_bounds__(1024) k_grant(DevState s0) {
         // granted keys are paired with the allocated ids in (request,
         // position) order: request i's first granted key is the lo-th
         s.rq_cbase[i] = (int32_t)lo;
+        s.rq_qbase[i] = (int32_t)base_c;
         s.rq_a[i] = a;
         s.out.admitted_blocks[i] = a;
         s.out.admitted_offsets[i] = (int32_t)lo;
@@ -952,7 +953,8 @@ __global__ void __launch_bounds__(1024) k_grant_quota(DevState s) {
 
 // In-step hits: positions of [h_i, s_i) belong to earlier requests' claims;
 // the leading granted ones are hits.  A position whose owner's key was not
-// granted lowers the request's first-ungranted mark.
+// granted lowers the request's first-ungranted mark.  The positions from s_i
+// on are the request's own claims: they are listed for the insertion.
 __global__ void __launch_bounds__(kThreads) k_instep(DevState s) {
   s = with_args(s);
   const Ctl* c = s.ctl;
@@ -967,6 +969,8 @@ __global__ void __launch_bounds__(kThreads) k_instep(DevState s) {
     h = s.rq_h[r.i];
     sown = s.rq_s[r.i];
     slot = s.pos_claim[pos];
+    const int32_t qb = s.rq_qbase[r.i];
+    if (r.m >= sown) s.claim_pos[qb + (r.m - sown)] = (uint64_t)r.i << 32 | (uint64_t)(uint32_t)pos;
   }
   if (valid && r.m >= h && r.m < sown) {
     // the owner's claims are ranked consecutively: its key here is granted
@@ -2180,43 +2184,43 @@ __global__ void __launch_bounds__(kBmThreads, 3) k_bm_write(DevState s) {
   write_ids(s, sm, w0, kBmChunk);
 }
 
-// Stage 6: place granted claims (thread per position).  The allocated ids
-// (ascending) go to the granted keys in (request, position) order; each new
-// block carries the metadata OnCacheFullBlocks attached plus any in-step
-// touches.  An allocated id that is still resident is a victim (every victim
-// is allocated again in its step): its old content leaves the pool first, in
-// the same thread (Alg. 2 Evict: table entry and record), so no other thread
-// ever sees the block between its two contents.  Each claim's owning position
-// then clears its claim-map slot (no other thread reads it here), and each
-// request's first position commits its OnRequest / RecordSuccessfulAdmission
-// history update.
+// Stage 6: place granted claims, a thread per claim of the step (k_instep
+// listed them; a thread per position left most lanes idle: at 2^20 blocks half
+// of the positions are hits).  The allocated ids (ascending) go to the granted
+// keys in (request, position) order; each new block carries the metadata
+// OnCacheFullBlocks attached plus any in-step touches.  An allocated id that
+// is still resident is a victim (every victim is allocated again in its step):
+// its old content leaves the pool first, in the same thread (Alg. 2 Evict:
+// table entry and record), so no other thread ever sees the block between its
+// two contents.  Each claim's thread then clears its claim-map slot (no other
+// thread reads it here).  The first R threads also commit a request's
+// OnRequest / RecordSuccessfulAdmission history update each.
 __global__ void __launch_bounds__(kThreads, 5) k_insert(DevState s) {
   s = with_args(s);
   Ctl* c = s.ctl;
   if (c->status != PS_OK) return;
-  const int64_t pos = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (pos == 0) c->hist_live += c->hist_new;
-  PosRef r;
+  const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   bool placed = false, evicted = false;
   uint32_t g = 0, gold = 0;
-  if (pos_ref(s, pos, &r)) {
-    // Three rounds of loads, each issued as a whole before anything is stored
-    // (a store or an atomic in between would hold back the loads after it):
-    // the position's and its request's records; the id and the claim; the
-    // id's old record.
-    const uint32_t i = r.i;
+  if (q < c->total_claims) {
+    // Rounds of loads, each issued as a whole before anything is stored (a
+    // store or an atomic in between would hold back the loads after it): the
+    // claim's position; its and its request's records; the id and the claim;
+    // the id's old record.
+    const uint64_t cp = s.claim_pos[q];
+    const uint32_t i = (uint32_t)(cp >> 32);
+    const int64_t pos = (int64_t)(uint32_t)cp;
     const int si = s.rq_s[i], a = s.rq_a[i], cbase = s.rq_cbase[i], n = s.rq_n[i], pbase = s.rq_pbase[i];
     const int cid = s.rq_cid[i];
-    const uint32_t hs = s.rq_hs[i];
     const uint64_t p = s.rq_p[i], key = s.pos_key[pos];
     const uint8_t knew = s.rq_knew[i];
-    const uint32_t pc = s.pos_claim[pos];
+    const uint32_t slot = s.pos_claim[pos];
     const int64_t n_alloc = c->n_alloc;
     const uint64_t base = c->stamp_base;
     g = (uint32_t)s.in_group[i];
-    const uint32_t slot = r.m >= si ? pc : kNone;  // an own claim
-    const bool grant = r.m >= si && r.m < si + a;
-    const int64_t rank = (int64_t)cbase + (r.m - si);
+    const int m = (int)(pos - pbase);
+    const bool grant = m < si + a;
+    const int64_t rank = (int64_t)cbase + (m - si);
     ClaimEntry e{};
     uint32_t b = kNone;
     if (grant) {
@@ -2235,10 +2239,6 @@ __global__ void __launch_bounds__(kThreads, 5) k_insert(DevState s) {
       okey = s.blk_key[b];
       ogrp = s.blk_group[b];
     }
-    if (r.m == 0 && hs != kNone) {  // history commit of request i (it has a full block)
-      atomicAdd(&s.hist[hs].refadm, 1u);
-      if (a > 0) atomicOr(&s.hist[hs].refadm, 0x80000000u);
-    }
     if (grant) {
       if (b >= (uint64_t)s.N) {
         c->internal_error = 1;  // the allocated set is short: never expected
@@ -2251,7 +2251,7 @@ __global__ void __launch_bounds__(kThreads, 5) k_insert(DevState s) {
         const uint32_t nslot = table_insert(s, key, g, b);
         // the latest request that touched it: an in-step toucher's stamp, or
         // the owner's own
-        const uint64_t st = tmax<uint64_t>(e.stamp, make_stamp(base, pbase, n, r.m));
+        const uint64_t st = tmax<uint64_t>(e.stamp, make_stamp(base, pbase, n, m));
         s.blk_key[b] = key;
         s.blk_group[b] = (uint16_t)g;
         s.blk_contract[b] = (uint8_t)cid;
@@ -2266,8 +2266,17 @@ __global__ void __launch_bounds__(kThreads, 5) k_insert(DevState s) {
         placed = true;  // its resident bit was set with the allocated set
       }
     }
-    if (slot != kNone) s.claims[slot] = empty_claim();
+    s.claims[slot] = empty_claim();
   }
+  if (q < s.R) {  // history commit of request q (no entry: no full block)
+    const uint32_t hs = s.rq_hs[q];
+    const int a = s.rq_a[q];
+    if (hs != kNone) {
+      atomicAdd(&s.hist[hs].refadm, 1u);
+      if (a > 0) atomicOr(&s.hist[hs].refadm, 0x80000000u);
+    }
+  }
+  if (q == 0) c->hist_live += c->hist_new;
   agg_stat(s, gold, PS_STAT_EVICTED_BLOCKS, 1, evicted);
   agg_stat(s, gold, PS_STAT_RESIDENT_BLOCKS, -1, evicted);
   agg_stat(s, g, PS_STAT_RESIDENT_BLOCKS, 1, placed);
@@ -2362,6 +2371,7 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
   const int R = s.max_requests;
   const int pgrid = grid_for(s.max_blocks, kThreads, 1 << 30);
   const int prgrid = grid_for(s.max_blocks + R, kThreads, 1 << 30);
+  const int igrid = grid_for(s.max_blocks > R ? s.max_blocks : R, kThreads, 1 << 30);
   const int cgrid = grid_for(s.N, 256, 152 * 8);
   int launches = 0;
   auto mark = [&](int stage) {
@@ -2498,9 +2508,9 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
   mark(9);
   if (fork2) {  // the touch branch joins the insertion
     if (cudaStreamWaitEvent(st, cap->join2, 0) != cudaSuccess) return PS_ERR_CUDA;
-    PS_LAUNCH((k_insert<<<pgrid, kThreads, 0, st>>>(s)));  // after the join: plain
+    PS_LAUNCH((k_insert<<<igrid, kThreads, 0, st>>>(s)));  // after the join: plain
   } else {
-    PS_LAUNCH(launch_k(k_insert, pgrid, kThreads, 0, st, s));
+    PS_LAUNCH(launch_k(k_insert, igrid, kThreads, 0, st, s));
   }
   if (s.policy == PS_S3FIFO && launch_s3_insert(s, st, &launches) != PS_OK) return PS_ERR_CUDA;
   if (s.lg_on && launch_queue_append(s, st, cap, &launches) != PS_OK) return PS_ERR_CUDA;
