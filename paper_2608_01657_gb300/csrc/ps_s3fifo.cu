@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(kPT) k_s3_plan(DevState s) {
   Ctl* c = s.ctl;
   if (c->status != PS_OK) return;
   S3Plan* pl = s.s3_plan;
-  __shared__ int64_t sv[8];
+  __shared__ int64_t sv[16];
   __shared__ uint32_t hmain[kS3Bins], hmov[kS3Bins];
   const int buf = c->s3_buf;
   const int64_t lenS = c->s3_len[0], lenM = c->s3_len[1];
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(kPT) k_s3_plan(DevState s) {
   const int64_t m = c->mvict;
   const uint32_t cap = (uint32_t)s.s3_freq_cap, mm = (uint32_t)s.s3_move_min;
   if (threadIdx.x < kS3Bins) { hmain[threadIdx.x] = 0; hmov[threadIdx.x] = 0; }
-  if (threadIdx.x < 8) sv[threadIdx.x] = -1;
+  if (threadIdx.x < 16) sv[threadIdx.x] = -1;
   if (threadIdx.x == 0) {
     pl->lenS = lenS; pl->lenM = lenM;
     pl->ctr0 = c->s3_ctr;
@@ -311,16 +311,59 @@ __global__ void __launch_bounds__(kPT) k_s3_plan(DevState s) {
     pl->fb = 0;
   }
   __syncthreads();
+  // The chunks in list order, main queue first: thread t holds a run of them
+  // (one up to kPT chunks) and its exclusive prefixes in registers, so each
+  // question below ("which chunk holds the n-th ...") is a look at registers
+  // and a barrier, and several counts share a scan.
+  const int64_t nch = chM + chS;
+  const int64_t run = (nch + kPT - 1) / kPT;
+  const int64_t r0 = tmin<int64_t>((int64_t)threadIdx.x * run, nch), r1 = tmin<int64_t>(r0 + run, nch);
+  auto rec = [&](int64_t i) -> const S3Chunk& { return i < chM ? ckM[i] : ckS[i - chM]; };
+  // per bin, the warp's sum added once (a lane each would queue up on 16 addresses)
+  auto add_bins = [&](uint32_t* bins, const uint32_t (&h)[kS3Bins]) {
+#pragma unroll
+    for (int r = 0; r < kS3Bins; ++r) {
+      const uint32_t w = __reduce_add_sync(kFull, h[r]);
+      if (lane_id() == 0 && w) atomicAdd(bins + r, w);
+    }
+  };
   // ---- sizes: unpinned and victim-grade members of the small queue, main's unpinned
-  const uint64_t tS = plan_scan(chS, [&](int64_t i) { return (uint64_t)ckS[i].nu << 32 | ckS[i].nev; },
-                                [&](int64_t i, uint64_t ex, uint64_t) { bS[i].u = (uint32_t)(ex >> 32); bS[i].ev = (uint32_t)ex; });
-  const int64_t K = (int64_t)(tS >> 32), T = (int64_t)(uint32_t)tS;
-  const int64_t nS0 = (int64_t)plan_scan(chS, [&](int64_t i) { return (uint64_t)ckS[i].nlive; }, [&](int64_t, uint64_t, uint64_t) {});
-  const int64_t UMo = (int64_t)plan_scan(chM, [&](int64_t i) { return (uint64_t)ckM[i].nu; },
-                                         [&](int64_t i, uint64_t ex, uint64_t) { bM[i].u = (uint32_t)ex; });
-  for (int64_t i = threadIdx.x; i < chM; i += kPT)
-    for (int r = 0; r < kS3Bins; ++r)
-      if (ckM[i].hist[r]) atomicAdd(&hmain[r], ckM[i].hist[r]);
+  uint32_t h[kS3Bins];
+#pragma unroll
+  for (int r = 0; r < kS3Bins; ++r) h[r] = 0;
+  uint64_t a0 = 0, a1 = 0;  // unpinned of main (high) and small (low); small's victim-grade (high) and live (low)
+  for (int64_t i = r0; i < r1; ++i) {
+    const S3Chunk& k = rec(i);
+    if (i < chM) {
+      a0 += (uint64_t)k.nu << 32;
+#pragma unroll
+      for (int r = 0; r < kS3Bins; ++r) h[r] += k.hist[r];
+    } else {
+      a0 += k.nu;
+      a1 += (uint64_t)k.nev << 32 | k.nlive;
+    }
+  }
+  add_bins(hmain, h);
+  uint64_t t0, t1;
+  const uint64_t e0 = block_excl_scan<uint64_t>(a0, &t0);
+  const uint64_t e1 = block_excl_scan<uint64_t>(a1, &t1);
+  {
+    uint32_t um = (uint32_t)(e0 >> 32), us = (uint32_t)e0, ev = (uint32_t)(e1 >> 32);
+    for (int64_t i = r0; i < r1; ++i) {
+      const S3Chunk& k = rec(i);
+      if (i < chM) {
+        bM[i].u = um;
+        um += k.nu;
+      } else {
+        bS[i - chM].u = us;
+        bS[i - chM].ev = ev;
+        us += k.nu;
+        ev += k.nev;
+      }
+    }
+  }
+  const int64_t UMo = (int64_t)(t0 >> 32), K = (int64_t)(uint32_t)t0, T = (int64_t)(t1 >> 32);
+  const int64_t nS0 = (int64_t)(uint32_t)t1;
   // ---- small phase: how many evictions take the small queue, and where they stop
   const int64_t D = nS0 - s.s3_small_cap;
   int64_t nA = 0;
@@ -329,13 +372,17 @@ __global__ void __launch_bounds__(kPT) k_s3_plan(DevState s) {
     int64_t TD = 0;
     if (Dp >= 1) {
       // the chunk holding unpinned member number Dp, then the victims among the first Dp
-      if (threadIdx.x == 0) { sv[0] = -1; sv[1] = -1; }
-      plan_scan(chS, [&](int64_t i) { return (uint64_t)ckS[i].nu; }, [&](int64_t i, uint64_t ex, uint64_t v) {
-        if ((int64_t)ex < Dp && Dp <= (int64_t)(ex + v)) sv[0] = i;
-      });
+      uint32_t us = (uint32_t)e0, ev = (uint32_t)(e1 >> 32);
+      for (int64_t i = tmax(r0, chM); i < r1; ++i) {
+        const S3Chunk& k = rec(i);
+        if ((int64_t)us < Dp && Dp <= (int64_t)(us + k.nu)) { sv[0] = i - chM; sv[1] = -1; sv[2] = us; sv[3] = ev; }
+        us += k.nu;
+        ev += k.nev;
+      }
+      __syncthreads();
       const int64_t cd = sv[0];
       if (cd < 0) { lost_locate(s); return; }
-      const int64_t want = Dp - bS[cd].u;
+      const int64_t want = Dp - sv[2];
       const int n = (int)tmin<int64_t>(kS3Chunk, lenS - cd * kS3Chunk);
       const uint8_t* at = atS + cd * kS3Chunk;
       chunk_scan(n, [&](int j) {
@@ -345,27 +392,30 @@ __global__ void __launch_bounds__(kPT) k_s3_plan(DevState s) {
         if ((own >> 32) && (int64_t)(incl >> 32) == want) sv[1] = (int64_t)(uint32_t)incl;
       });
       if (sv[1] < 0) { lost_locate(s); return; }
-      TD = bS[cd].ev + sv[1];
+      TD = sv[3] + sv[1];
     }
     nA = tmin<int64_t>(m, 1 + TD);
   }
   int64_t pcut = 0, kS = 0;
   if (nA > 0 && nA <= T) {
-    if (threadIdx.x == 0) { sv[2] = -1; sv[3] = -1; }
-    plan_scan(chS, [&](int64_t i) { return (uint64_t)ckS[i].nev; }, [&](int64_t i, uint64_t ex, uint64_t v) {
-      if ((int64_t)ex < nA && nA <= (int64_t)(ex + v)) sv[2] = i;
-    });
-    const int64_t ce = sv[2];
+    uint32_t ev = (uint32_t)(e1 >> 32);
+    for (int64_t i = tmax(r0, chM); i < r1; ++i) {
+      const S3Chunk& k = rec(i);
+      if ((int64_t)ev < nA && nA <= (int64_t)(ev + k.nev)) { sv[4] = i - chM; sv[5] = ev; sv[6] = -1; }
+      ev += k.nev;
+    }
+    __syncthreads();
+    const int64_t ce = sv[4];
     if (ce < 0) { lost_locate(s); return; }
-    const int64_t want = nA - bS[ce].ev;
+    const int64_t want = nA - sv[5];
     const int n = (int)tmin<int64_t>(kS3Chunk, lenS - ce * kS3Chunk);
     const uint8_t* at = atS + ce * kS3Chunk;
     chunk_scan(n, [&](int j) { const uint32_t a = at[j]; return (uint64_t)(a_un(a) && a_f(a) < mm); },
                [&](int j, uint64_t incl, uint64_t own) {
-                 if (own && (int64_t)incl == want) sv[3] = j;
+                 if (own && (int64_t)incl == want) sv[6] = j;
                });
-    if (sv[3] < 0) { lost_locate(s); return; }
-    pcut = ce * kS3Chunk + sv[3] + 1;
+    if (sv[6] < 0) { lost_locate(s); return; }
+    pcut = ce * kS3Chunk + sv[6] + 1;
     kS = nA;
   } else if (nA > T) {
     pcut = lenS;
@@ -380,12 +430,14 @@ __global__ void __launch_bounds__(kPT) k_s3_plan(DevState s) {
   __syncthreads();
   if (cpart >= 0) {
     const uint8_t* at = atS + cpart * kS3Chunk;
-    for (int j = threadIdx.x; j < (int)(pcut - cpart * kS3Chunk); j += kPT) {
-      const uint32_t a = at[j];
-      if (a_un(a)) {
-        atomicAdd(&part_u, 1u);
-        atomicAdd(&part_h[a_f(a)], 1u);
-      }
+    const int n = (int)(pcut - cpart * kS3Chunk);
+    for (int j0 = 0; j0 < n; j0 += kPT) {
+      const int j = j0 + (int)threadIdx.x;
+      const uint32_t a = j < n ? at[j] : 0u;
+      const bool un = a_un(a);
+      const unsigned bal = __ballot_sync(kFull, un);
+      if (lane_id() == 0 && bal) atomicAdd(&part_u, (uint32_t)__popc(bal));
+      agg_inc(part_h, a_f(a), un);
     }
   }
   __syncthreads();
@@ -398,33 +450,48 @@ __global__ void __launch_bounds__(kPT) k_s3_plan(DevState s) {
     }
     return n;
   };
-  const int64_t MA = (int64_t)plan_scan(chS, [&](int64_t i) { return (uint64_t)mv_of(i, 0); },
-                                        [&](int64_t i, uint64_t ex, uint64_t) { bS[i].mv = (uint32_t)ex; });
-  for (int64_t i = threadIdx.x; i < chS; i += kPT) {
-    if (i < cfull) {
-      for (int r = (int)mm; r < kS3Bins; ++r)
-        if (ckS[i].hist[r]) atomicAdd(&hmov[r], ckS[i].hist[r]);
-    } else if (i == cpart) {
-      for (int r = (int)mm; r < kS3Bins; ++r)
-        if (part_h[r]) atomicAdd(&hmov[r], part_h[r]);
+#pragma unroll
+  for (int r = 0; r < kS3Bins; ++r) h[r] = 0;
+  uint64_t mvs = 0;
+  for (int64_t i = tmax(r0, chM); i < r1; ++i) {
+    mvs += mv_of(i - chM, 0);
+    if (i - chM < cfull) {
+#pragma unroll
+      for (int r = 0; r < kS3Bins; ++r)
+        if (r >= (int)mm) h[r] += ckS[i - chM].hist[r];
+    } else if (i - chM == cpart) {
+#pragma unroll
+      for (int r = 0; r < kS3Bins; ++r)
+        if (r >= (int)mm) h[r] += part_h[r];
     }
   }
-  __syncthreads();
+  add_bins(hmov, h);
+  uint64_t tmv;
+  uint64_t emv = block_excl_scan<uint64_t>(mvs, &tmv);
+  const int64_t MA = (int64_t)tmv;
+  {
+    uint64_t mv = emv;
+    for (int64_t i = tmax(r0, chM); i < r1; ++i) {
+      bS[i - chM].mv = (uint32_t)mv;
+      mv += mv_of(i - chM, 0);
+    }
+  }
   const int64_t nL = UMo + MA;
   const int64_t mB = m - kS;
   if (cap >= (uint32_t)kS3Bins || mB > nL || (s.flags & PS_FLAG_S3_SEQUENTIAL)) {  // sequential kernel
     if (threadIdx.x == 0) pl->fb = 1;
     return;
   }
-  // ---- main phase: the final round Rs and the position P of its last visit
+  // ---- main phase: the final round Rs, and list-order prefixes of f >= Rs and
+  // f == Rs; the small queue's kept members (live and not consumed) beside them
   int Rs = 0;
-  int64_t P = -1, rge_P1 = 0, rgt_P1 = 0, base_R = 0, base_Rm1 = 0, cpP = -1;
+  int64_t P = -1, rge_P1 = 0, rgt_P1 = 0, base_R = 0, base_Rm1 = 0, kth = 0;
   if (mB > 0) {
-    int64_t cum = 0, k = 0;
+    int64_t cum = 0;
     for (int r = 0; r < kS3Bins; ++r) {
-      const int64_t h = (int64_t)hmain[r] + hmov[r];
-      if (cum + h >= mB) { Rs = r; k = mB - cum; break; }
-      cum += h;
+      const int64_t hr = (int64_t)hmain[r] + hmov[r];
+      if (cum + hr >= mB) { Rs = r; kth = mB - cum; break; }
+      cum += hr;
     }
     // reinsertions of the complete rounds: round r reinserts every member with f > r
     for (int r = 0; r < Rs; ++r) {
@@ -433,15 +500,53 @@ __global__ void __launch_bounds__(kPT) k_s3_plan(DevState s) {
       if (r < Rs - 1) base_Rm1 += gt;
       base_R += gt;
     }
-    // the k-th member with f == Rs, in list order (main chunks, then small chunks)
-    if (threadIdx.x == 0) { sv[4] = -1; sv[6] = -1; }
-    plan_scan(chM + chS, [&](int64_t i) -> uint64_t {
-      return i < chM ? ckM[i].hist[Rs] : (Rs >= (int)mm ? mv_of(i - chM, Rs) - mv_of(i - chM, Rs + 1) : 0u);
-    }, [&](int64_t i, uint64_t ex, uint64_t v) {
-      if ((int64_t)ex < k && k <= (int64_t)(ex + v)) { sv[4] = i; sv[5] = (int64_t)ex; }
-    });
-    if (sv[4] < 0) { lost_locate(s); return; }
-    const int64_t cp = sv[4], want = k - sv[5];
+  }
+  auto ge_eq = [&](int64_t i) -> uint64_t {  // members with f >= Rs (high) and f == Rs (low) of list chunk i
+    uint32_t ge = 0, gt = 0;
+    if (i < chM) {
+      for (int r = Rs; r < kS3Bins; ++r) ge += ckM[i].hist[r];
+      gt = ge - ckM[i].hist[Rs];
+    } else {
+      ge = mv_of(i - chM, Rs);
+      gt = mv_of(i - chM, Rs + 1);
+    }
+    return (uint64_t)ge << 32 | (ge - gt);
+  };
+  auto keep_s = [&](int64_t i) -> uint32_t {
+    return ckS[i].nlive - (i < cfull ? ckS[i].nu : (i == cpart ? part_u : 0u));
+  };
+  uint64_t ags = 0, aks = 0;
+  for (int64_t i = r0; i < r1; ++i) {
+    ags += ge_eq(i);
+    if (i >= chM) aks += keep_s(i - chM);
+  }
+  uint64_t tg, tks;
+  uint64_t eg = block_excl_scan<uint64_t>(ags, &tg);
+  uint64_t eks = block_excl_scan<uint64_t>(aks, &tks);
+  for (int64_t i = r0; i < r1; ++i) {
+    const uint64_t v = ge_eq(i);
+    S3Base& bb = i < chM ? bM[i] : bS[i - chM];
+    const uint32_t ge = (uint32_t)(eg >> 32), eq = (uint32_t)eg;
+    bb.ge = ge;
+    bb.gt = ge - eq;
+    if (mB > 0 && (int64_t)eq < kth && kth <= (int64_t)(eq + (uint32_t)v)) {  // the last visit's chunk
+      sv[7] = i;
+      sv[8] = eq;
+      sv[9] = ge;
+      sv[10] = -1;
+      sv[11] = i < chM ? bM[i].u : bS[i - chM].mv;  // list members before the chunk (of its queue)
+    }
+    eg += v;
+    if (i >= chM) {
+      bS[i - chM].keep = (uint32_t)eks;
+      eks += keep_s(i - chM);
+    }
+  }
+  if (mB > 0) {
+    // the kth member with f == Rs, in list order: the position P of the last visit
+    __syncthreads();
+    if (sv[7] < 0) { lost_locate(s); return; }
+    const int64_t cp = sv[7], want = kth - sv[8];
     const bool inM = cp < chM;
     const int64_t ci = inM ? cp : cp - chM;
     const int n = (int)tmin<int64_t>(kS3Chunk, (inM ? lenM : lenS) - ci * kS3Chunk);
@@ -457,53 +562,45 @@ __global__ void __launch_bounds__(kPT) k_s3_plan(DevState s) {
              (uint64_t)(f > (uint32_t)Rs) << 48;
     }, [&](int, uint64_t incl, uint64_t own) {
       if ((own & 0xFFFF) && (int64_t)(incl & 0xFFFF) == want) {
-        sv[6] = (int64_t)((incl >> 16) & 0xFFFF) - 1;  // members before it in the chunk
-        sv[7] = (int64_t)(incl >> 32);                  // ge (16 bits) | gt (16 bits) up to it
+        sv[10] = (int64_t)((incl >> 16) & 0xFFFF) - 1;  // members before it in the chunk
+        sv[12] = (int64_t)(incl >> 32);                  // ge (16 bits) | gt (16 bits) up to it
       }
     });
-    if (sv[6] < 0) { lost_locate(s); return; }
-    const int64_t before = sv[6];
-    P = inM ? (int64_t)bM[ci].u + before : UMo + (int64_t)bS[ci].mv + before;
-    // within the chunk; the chunk's list-order bases are added below
-    rge_P1 = sv[7] & 0xFFFF;
-    rgt_P1 = (sv[7] >> 16) & 0xFFFF;
-    cpP = cp;
-  }
-  // ---- list-order bases of f >= Rs and f > Rs (main chunks, then small chunks)
-  const uint64_t tg = plan_scan(chM + chS, [&](int64_t i) -> uint64_t {
-    uint32_t ge = 0, gt = 0;
-    if (i < chM) {
-      for (int r = Rs; r < kS3Bins; ++r) ge += ckM[i].hist[r];
-      gt = ge - ckM[i].hist[Rs];
-    } else {
-      ge = mv_of(i - chM, Rs);
-      gt = mv_of(i - chM, Rs + 1);
-    }
-    return (uint64_t)ge << 32 | gt;
-  }, [&](int64_t i, uint64_t ex, uint64_t) {
-    S3Base& b = i < chM ? bM[i] : bS[i - chM];
-    b.ge = (uint32_t)(ex >> 32);
-    b.gt = (uint32_t)ex;
-  });
-  if (mB > 0) {
-    const S3Base& b = cpP < chM ? bM[cpP] : bS[cpP - chM];
-    rge_P1 += b.ge;
-    rgt_P1 += b.gt;
+    if (sv[10] < 0) { lost_locate(s); return; }
+    P = (inM ? 0 : UMo) + sv[11] + sv[10];
+    rge_P1 = sv[9] + (sv[12] & 0xFFFF);
+    rgt_P1 = (sv[9] - sv[8]) + ((sv[12] >> 16) & 0xFFFF);
   }
   const int64_t GE = (int64_t)(tg >> 32);
   const int64_t nG1 = Rs >= 1 ? GE - rge_P1 : 0;
   const int64_t nUnvMov = Rs == 0 ? nL - tmax<int64_t>(P + 1, UMo) : 0;
   const int64_t nMid = nG1 + nUnvMov + rgt_P1;
-  // ---- kept entries: small = live and not consumed; main = pinned, or unvisited
-  const int64_t nKeepS = (int64_t)plan_scan(chS, [&](int64_t i) -> uint64_t {
-    const uint32_t cons = i < cfull ? ckS[i].nu : (i == cpart ? part_u : 0u);
-    return ckS[i].nlive - cons;
-  }, [&](int64_t i, uint64_t ex, uint64_t) { bS[i].keep = (uint32_t)ex; });
-  const int64_t nKeepM = (int64_t)plan_scan(chM, [&](int64_t i) -> uint64_t {
+  // ---- main's kept entries: pinned, or unvisited
+  const int64_t nKeepS = (int64_t)tks;
+  auto keep_m = [&](int64_t i, int64_t u) -> uint32_t {
     int64_t unv = 0;
-    if (Rs == 0) unv = tmin<int64_t>(tmax<int64_t>((int64_t)bM[i].u + ckM[i].nu - (P + 1), 0), ckM[i].nu);
-    return (uint64_t)(ckM[i].nlive - ckM[i].nu + unv);
-  }, [&](int64_t i, uint64_t ex, uint64_t) { bM[i].keep = (uint32_t)ex; });
+    if (Rs == 0) unv = tmin<int64_t>(tmax<int64_t>(u + ckM[i].nu - (P + 1), 0), ckM[i].nu);
+    return (uint32_t)(ckM[i].nlive - ckM[i].nu + unv);
+  };
+  uint64_t akm = 0;
+  {
+    int64_t u = (int64_t)(e0 >> 32);
+    for (int64_t i = r0; i < tmin(r1, chM); ++i) {
+      akm += keep_m(i, u);
+      u += ckM[i].nu;
+    }
+  }
+  uint64_t tkm;
+  uint64_t ekm = block_excl_scan<uint64_t>(akm, &tkm);
+  const int64_t nKeepM = (int64_t)tkm;
+  {
+    int64_t u = (int64_t)(e0 >> 32);
+    for (int64_t i = r0; i < tmin(r1, chM); ++i) {
+      bM[i].keep = (uint32_t)ekm;
+      ekm += keep_m(i, u);
+      u += ckM[i].nu;
+    }
+  }
   // ---- the ghost FIFO: pushes, trimming, room
   __shared__ uint64_t gq;
   const uint64_t tail = c->ghost_tail, head = c->ghost_head;
@@ -513,8 +610,8 @@ __global__ void __launch_bounds__(kPT) k_s3_plan(DevState s) {
   const int64_t born = tmax<int64_t>(X - live_old, 0);
   const int gc = ((int64_t)(head - tail) + kS > (int64_t)s.ghost_ring_cap ||
                   ((s.flags & PS_FLAG_S3_COMPACT_GHOST) && head > tail)) ? 1 : 0;
-  const uint64_t a0 = tail & ~(uint64_t)(kS3Chunk - 1);
-  const int64_t nrch = head > tail ? cdiv64((int64_t)(head - a0), kS3Chunk) : 0;
+  const uint64_t ra0 = tail & ~(uint64_t)(kS3Chunk - 1);
+  const int64_t nrch = head > tail ? cdiv64((int64_t)(head - ra0), kS3Chunk) : 0;
   if (threadIdx.x == 0) gq = tail;
   __syncthreads();
   if (gc) {
@@ -528,18 +625,18 @@ __global__ void __launch_bounds__(kPT) k_s3_plan(DevState s) {
     });
     if (sv[2] < 0) { lost_locate(s); return; }
     const int64_t rc = sv[2];
-    const uint64_t p0 = a0 + (uint64_t)rc * kS3Chunk;
+    const uint64_t p0 = ra0 + (uint64_t)rc * kS3Chunk;
     const uint32_t* rbits = bits_of(s, c->ghost_rbuf);
     const uint64_t rmask = s.ghost_ring_cap - 1;
     if (threadIdx.x < 32) {
       // a warp: two words a lane, in order
       uint32_t w[2];
-      for (int h = 0; h < 2; ++h) {
-        const uint64_t pw = p0 + 32u * (2 * threadIdx.x + h);
+      for (int q = 0; q < 2; ++q) {
+        const uint64_t pw = p0 + 32u * (2 * threadIdx.x + q);
         uint32_t x = rbits[(pw & rmask) >> 5];
         if (pw < tail) x = tail - pw >= 32 ? 0u : x & (~0u << (uint32_t)(tail - pw));
         if (pw + 32 > head) x = head <= pw ? 0u : x & (~0u >> (uint32_t)(pw + 32 - head));
-        w[h] = x;
+        w[q] = x;
       }
       const uint32_t n = __popc(w[0]) + __popc(w[1]);
       const uint32_t incl = warp_incl_scan(n);
@@ -547,10 +644,10 @@ __global__ void __launch_bounds__(kPT) k_s3_plan(DevState s) {
       const int64_t exl = (int64_t)(incl - n);
       if (exl < want && want <= (int64_t)incl) {
         int64_t left = want - exl;
-        const int h = left <= __popc(w[0]) ? 0 : 1;
-        if (h == 1) left -= __popc(w[0]);
-        const int bit = (int)__fns(w[h], 0, (int)left);
-        gq = p0 + 32u * (2 * threadIdx.x + h) + (uint64_t)bit + 1;
+        const int q = left <= __popc(w[0]) ? 0 : 1;
+        if (q == 1) left -= __popc(w[0]);
+        const int bit = (int)__fns(w[q], 0, (int)left);
+        gq = p0 + 32u * (2 * threadIdx.x + q) + (uint64_t)bit + 1;
       }
     }
     __syncthreads();
@@ -563,7 +660,7 @@ __global__ void __launch_bounds__(kPT) k_s3_plan(DevState s) {
     pl->nKeepS = nKeepS; pl->nKeepM = nKeepM;
     pl->ctr_end = c->s3_ctr + MA + base_R + rgt_P1;
     pl->gc = gc; pl->rbuf = c->ghost_rbuf;
-    pl->g_head = head; pl->g_tail = tail; pl->ra0 = a0; pl->nrch = nrch;
+    pl->g_head = head; pl->g_tail = tail; pl->ra0 = ra0; pl->nrch = nrch;
     pl->live_old = live_old; pl->X = X; pl->born = born;
     pl->gctr0 = c->ghost_ctr;
     uint64_t q;
