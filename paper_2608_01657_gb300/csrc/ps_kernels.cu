@@ -2499,13 +2499,25 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
   } else if (launch_s3_select(s, st, fork2, &launches) != PS_OK) {
     return PS_ERR_CUDA;
   }
+  // The ghost pushes run beside the id lists (the candidate scan's branch,
+  // which S3-FIFO has no use for), joined before the insertion.
+  const bool fork3 = cap != nullptr && s.policy == PS_S3FIFO;
+  if (fork3) {
+    if (cudaEventRecord(cap->fork, st) != cudaSuccess || cudaStreamWaitEvent(cap->side, cap->fork, 0) != cudaSuccess ||
+        launch_s3_push(s, cap->side, true, &launches) != PS_OK || cudaEventRecord(cap->join, cap->side) != cudaSuccess)
+      return PS_ERR_CUDA;
+  } else if (s.policy == PS_S3FIFO && launch_s3_push(s, st, false, &launches) != PS_OK) {
+    return PS_ERR_CUDA;
+  }
   mark(7);
   const int nchunks = (int)((s.nwords + kBmChunk - 1) / kBmChunk);
-  PS_LAUNCH(launch_k(k_bm_count, nchunks, kBmChunk, 0, st, s));
+  if (fork3) PS_LAUNCH((k_bm_count<<<nchunks, kBmChunk, 0, st>>>(s)));  // after the fork: plain
+  else PS_LAUNCH(launch_k(k_bm_count, nchunks, kBmChunk, 0, st, s));
   PS_LAUNCH(launch_k(k_bm_write, nchunks, kBmThreads, 0, st, s));
   mark(8);
   // (evictions happen in k_insert: every victim is allocated again in its step)
   mark(9);
+  if (fork3 && cudaStreamWaitEvent(st, cap->join, 0) != cudaSuccess) return PS_ERR_CUDA;
   if (fork2) {  // the touch branch joins the insertion
     if (cudaStreamWaitEvent(st, cap->join2, 0) != cudaSuccess) return PS_ERR_CUDA;
     PS_LAUNCH((k_insert<<<igrid, kThreads, 0, st>>>(s)));  // after the join: plain

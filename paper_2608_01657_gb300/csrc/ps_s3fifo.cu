@@ -282,16 +282,178 @@ __global__ void __launch_bounds__(kCT) k_s3_count(DevState s) {
 }
 
 // ===========================================================================
-// 2. The plan: one CTA turns the chunk counts into the step's closed form
+// 2. The published loop, one eviction at a time, on the same arrays: used
+//    when the closed form does not apply (the main queue runs empty within the
+//    step, or frequencies reach kS3Bins).  Writes what the plan's kernels
+//    write: victims, moved and reinserted blocks, the new arrays' kept and
+//    re-sequenced parts, the ghost pushes, and the plan's totals.
+__device__ void s3_sequential(const DevState& s, Ctl* c) {  // one thread
+  S3Plan* pl = s.s3_plan;
+  const int buf = c->s3_buf;
+  const uint32_t* S = q_region(s, buf, 0);
+  const uint32_t* M = q_region(s, buf, 1);
+  uint32_t* oS = q_region(s, buf ^ 1, 0);
+  uint32_t* oM = q_region(s, buf ^ 1, 1);
+  const int64_t lenS = pl->lenS, lenM = pl->lenM, N = s.N;
+  const uint32_t step32 = (uint32_t)c->step;
+  const uint32_t mm = (uint32_t)s.s3_move_min;
+  uint32_t* um = reinterpret_cast<uint32_t*>(s.csk);  // the main queue's unpinned members: a ring of N
+  uint32_t* pushes = push_list(s);                    // the step's small-queue victims, in order
+  auto live = [&](uint32_t b) { return (s.blk_flags[b] & 1) != 0; };
+  auto unpinned = [&](uint32_t b) { return live(b) && s.blk_pin[b] != step32; };
+  int64_t uh = 0, ut = 0, ucount = 0;
+  for (int64_t j = 0; j < lenM; ++j) {
+    const uint32_t b = M[j];
+    if (unpinned(b)) { um[ut] = b; ut = ut + 1 == N ? 0 : ut + 1; ++ucount; }
+  }
+  int64_t nS = 0, Krem = 0;
+  for (int64_t j = 0; j < lenS; ++j) {
+    const uint32_t b = S[j];
+    nS += live(b);
+    Krem += unpinned(b);
+  }
+  const uint64_t ctr0 = c->s3_ctr;
+  uint64_t ctr = ctr0;
+  int64_t ps = 0, kS = 0, moved = 0;
+  const int64_t m = c->mvict;
+  int64_t budget = 4 * (N + 1) * ((int64_t)s.s3_freq_cap + 2) + lenS + 16;
+  bool bad = false;
+  auto evict_main = [&]() {
+    for (;;) {
+      if (ucount == 0 || --budget < 0) { bad = true; return; }
+      const uint32_t b = um[uh];
+      uh = uh + 1 == N ? 0 : uh + 1;
+      --ucount;
+      const uint32_t f = eff_freq(s, b);
+      if (f > 0) {
+        s.blk_freq[b] = f - 1;
+        s.blk_s3seq[b] = ++ctr;
+        um[ut] = b;
+        ut = ut + 1 == N ? 0 : ut + 1;
+        ++ucount;
+      } else {
+        mark_victim(s, b);
+        return;
+      }
+    }
+  };
+  for (int64_t v = 0; v < m && !bad; ++v) {
+    const bool use_small = (nS >= s.s3_small_cap && Krem > 0) || ucount == 0;
+    bool done = false;
+    if (use_small) {
+      while (Krem > 0 && !bad) {
+        uint32_t b = kNone;
+        while (ps < lenS) {
+          const uint32_t x = S[ps++];
+          if (unpinned(x)) { b = x; break; }
+        }
+        if (b == kNone || --budget < 0) { bad = true; break; }
+        --Krem;
+        --nS;
+        if (eff_freq(s, b) >= mm) {  // to the main queue's head
+          s.blk_flags[b] |= 2;
+          s.blk_s3seq[b] = ++ctr;
+          um[ut] = b;
+          ut = ut + 1 == N ? 0 : ut + 1;
+          ++ucount;
+          ++moved;
+        } else {                     // out, its key into the ghost
+          mark_victim(s, b);
+          pushes[kS++] = b;
+          done = true;
+          break;
+        }
+      }
+    }
+    if (!done && !bad) evict_main();
+  }
+  // the new arrays' kept and re-sequenced parts
+  int64_t nKeepS = 0, nKeepM = 0, nMid = 0;
+  for (int64_t j = 0; j < lenS; ++j) {
+    const uint32_t b = S[j];
+    if (live(b) && !(j < ps && unpinned(b))) oS[nKeepS++] = b;
+  }
+  for (int64_t j = 0; j < lenM; ++j) {
+    const uint32_t b = M[j];
+    const bool vic = (s.bm_victim[b >> 5] >> (b & 31)) & 1;
+    if (live(b) && !vic && s.blk_s3seq[b] <= ctr0) oM[nKeepM++] = b;
+  }
+  for (int64_t i = 0; i < ucount; ++i) {
+    const uint32_t b = um[(uh + i) % N];
+    if (s.blk_s3seq[b] > ctr0) oM[nKeepM + nMid++] = b;
+  }
+  // the ghost: trim the oldest live entries, compact when the ring lacks room, push
+  const uint64_t rcap = s.ghost_ring_cap, rmask = rcap - 1;
+  int rb = c->ghost_rbuf;
+  uint64_t tail = c->ghost_tail, head = c->ghost_head;
+  const int64_t live_old = c->ghost_live;
+  const int64_t X = live_old + kS - s.s3_ghost_cap;
+  const int64_t Xo = tmin<int64_t>(tmax<int64_t>(X, 0), live_old);
+  const int64_t born = tmax<int64_t>(X - live_old, 0);
+  uint32_t* ring = ring_of(s, rb);
+  uint32_t* bits = bits_of(s, rb);
+  auto bit_at = [&](uint32_t* bw, uint64_t p) { return (bw[(p & rmask) >> 5] >> (p & 31)) & 1; };
+  int64_t erased = 0;
+  while (erased < Xo && tail < head) {
+    if (bit_at(bits, tail)) {
+      gh_erase(s, ring[tail & rmask]);
+      bits[(tail & rmask) >> 5] &= ~(1u << (tail & 31));
+      ++erased;
+    }
+    ++tail;
+  }
+  uint64_t pbase = head;
+  if ((int64_t)(head - tail) + kS > (int64_t)rcap || ((s.flags & PS_FLAG_S3_COMPACT_GHOST) && head > tail)) {
+    uint32_t* nring = ring_of(s, rb ^ 1);
+    uint32_t* nbits = bits_of(s, rb ^ 1);
+    uint64_t w = 0;
+    for (uint64_t p = tail; p < head; ++p) {
+      if (!bit_at(bits, p)) continue;
+      const uint32_t slot = ring[p & rmask];
+      nring[w] = slot;
+      s.ghost_map[slot].blk = (uint32_t)w;
+      nbits[w >> 5] |= 1u << (w & 31);
+      ++w;
+    }
+    for (uint64_t p = tail & ~31ull; p < head; p += 32) bits[(p & rmask) >> 5] = 0;
+    rb ^= 1;
+    ring = nring;
+    bits = nbits;
+    tail = 0;
+    head = w;
+    pbase = head - (uint64_t)born;
+  } else if (born > 0) {
+    tail = head + (uint64_t)born;
+  }
+  for (int64_t t = born; t < kS; ++t) {
+    const uint32_t b = pushes[t];
+    const uint64_t p = pbase + (uint64_t)t;
+    const uint32_t slot = gh_insert(s, s.blk_key[b], s.blk_group[b], (uint32_t)(p & rmask), c->ghost_ctr + (uint64_t)t + 1);
+    if (slot == kNone) { bad = true; break; }
+    ring[p & rmask] = slot;
+    bits[(p & rmask) >> 5] |= 1u << (p & 31);
+  }
+  c->ghost_ctr += (uint64_t)kS;
+  c->ghost_live = live_old - Xo + (kS - born);
+  c->ghost_tail = tail;
+  c->ghost_head = pbase + (uint64_t)kS;
+  c->ghost_rbuf = rb;
+  pl->kS = kS;
+  pl->MA = moved;
+  pl->nKeepS = nKeepS;
+  pl->nKeepM = nKeepM;
+  pl->nMid = nMid;
+  pl->ctr_end = ctr;
+  if (bad) c->internal_error = 1;
+}
+
+// ===========================================================================
+// 3. The plan: one CTA turns the chunk counts into the step's closed form
 //    (or hands the step to the sequential kernel), and every chunk's bases.
-__global__ void __launch_bounds__(kPT) k_s3_plan(DevState s) {
-  s = with_args(s);
-  Ctl* c = s.ctl;
-  if (c->status != PS_OK) return;
+__device__ __forceinline__ void s3_plan(const DevState& s, Ctl* c) {
   S3Plan* pl = s.s3_plan;
   __shared__ int64_t sv[16];
   __shared__ uint32_t hmain[kS3Bins], hmov[kS3Bins];
-  const int buf = c->s3_buf;
   const int64_t lenS = c->s3_len[0], lenM = c->s3_len[1];
   const int64_t chS = cdiv64(lenS, kS3Chunk), chM = cdiv64(lenM, kS3Chunk);
   const S3Chunk* ckS = s.s3_ck;
@@ -680,175 +842,15 @@ __global__ void __launch_bounds__(kPT) k_s3_plan(DevState s) {
     if (gc) c->ghost_rbuf ^= 1;
   }
 }
-
-// ===========================================================================
-// 3. The published loop, one eviction at a time, on the same arrays: used
-//    when the closed form does not apply (the main queue runs empty within the
-//    step, or frequencies reach kS3Bins).  Writes what the plan's kernels
-//    write: victims, moved and reinserted blocks, the new arrays' kept and
-//    re-sequenced parts, the ghost pushes, and the plan's totals.
-__global__ void k_s3_fallback(DevState s) {
+// The plan, then (where it does not apply) the loop on one of its threads: a
+// kernel of its own for the loop cost every step a launch.
+__global__ void __launch_bounds__(kPT) k_s3_plan(DevState s) {
   s = with_args(s);
   Ctl* c = s.ctl;
-  S3Plan* pl = s.s3_plan;
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  if (c->status != PS_OK || !pl->fb) return;
-  const int buf = c->s3_buf;
-  const uint32_t* S = q_region(s, buf, 0);
-  const uint32_t* M = q_region(s, buf, 1);
-  uint32_t* oS = q_region(s, buf ^ 1, 0);
-  uint32_t* oM = q_region(s, buf ^ 1, 1);
-  const int64_t lenS = pl->lenS, lenM = pl->lenM, N = s.N;
-  const uint32_t step32 = (uint32_t)c->step;
-  const uint32_t mm = (uint32_t)s.s3_move_min;
-  uint32_t* um = reinterpret_cast<uint32_t*>(s.csk);  // the main queue's unpinned members: a ring of N
-  uint32_t* pushes = push_list(s);                    // the step's small-queue victims, in order
-  auto live = [&](uint32_t b) { return (s.blk_flags[b] & 1) != 0; };
-  auto unpinned = [&](uint32_t b) { return live(b) && s.blk_pin[b] != step32; };
-  int64_t uh = 0, ut = 0, ucount = 0;
-  for (int64_t j = 0; j < lenM; ++j) {
-    const uint32_t b = M[j];
-    if (unpinned(b)) { um[ut] = b; ut = ut + 1 == N ? 0 : ut + 1; ++ucount; }
-  }
-  int64_t nS = 0, Krem = 0;
-  for (int64_t j = 0; j < lenS; ++j) {
-    const uint32_t b = S[j];
-    nS += live(b);
-    Krem += unpinned(b);
-  }
-  const uint64_t ctr0 = c->s3_ctr;
-  uint64_t ctr = ctr0;
-  int64_t ps = 0, kS = 0, moved = 0;
-  const int64_t m = c->mvict;
-  int64_t budget = 4 * (N + 1) * ((int64_t)s.s3_freq_cap + 2) + lenS + 16;
-  bool bad = false;
-  auto evict_main = [&]() {
-    for (;;) {
-      if (ucount == 0 || --budget < 0) { bad = true; return; }
-      const uint32_t b = um[uh];
-      uh = uh + 1 == N ? 0 : uh + 1;
-      --ucount;
-      const uint32_t f = eff_freq(s, b);
-      if (f > 0) {
-        s.blk_freq[b] = f - 1;
-        s.blk_s3seq[b] = ++ctr;
-        um[ut] = b;
-        ut = ut + 1 == N ? 0 : ut + 1;
-        ++ucount;
-      } else {
-        mark_victim(s, b);
-        return;
-      }
-    }
-  };
-  for (int64_t v = 0; v < m && !bad; ++v) {
-    const bool use_small = (nS >= s.s3_small_cap && Krem > 0) || ucount == 0;
-    bool done = false;
-    if (use_small) {
-      while (Krem > 0 && !bad) {
-        uint32_t b = kNone;
-        while (ps < lenS) {
-          const uint32_t x = S[ps++];
-          if (unpinned(x)) { b = x; break; }
-        }
-        if (b == kNone || --budget < 0) { bad = true; break; }
-        --Krem;
-        --nS;
-        if (eff_freq(s, b) >= mm) {  // to the main queue's head
-          s.blk_flags[b] |= 2;
-          s.blk_s3seq[b] = ++ctr;
-          um[ut] = b;
-          ut = ut + 1 == N ? 0 : ut + 1;
-          ++ucount;
-          ++moved;
-        } else {                     // out, its key into the ghost
-          mark_victim(s, b);
-          pushes[kS++] = b;
-          done = true;
-          break;
-        }
-      }
-    }
-    if (!done && !bad) evict_main();
-  }
-  // the new arrays' kept and re-sequenced parts
-  int64_t nKeepS = 0, nKeepM = 0, nMid = 0;
-  for (int64_t j = 0; j < lenS; ++j) {
-    const uint32_t b = S[j];
-    if (live(b) && !(j < ps && unpinned(b))) oS[nKeepS++] = b;
-  }
-  for (int64_t j = 0; j < lenM; ++j) {
-    const uint32_t b = M[j];
-    const bool vic = (s.bm_victim[b >> 5] >> (b & 31)) & 1;
-    if (live(b) && !vic && s.blk_s3seq[b] <= ctr0) oM[nKeepM++] = b;
-  }
-  for (int64_t i = 0; i < ucount; ++i) {
-    const uint32_t b = um[(uh + i) % N];
-    if (s.blk_s3seq[b] > ctr0) oM[nKeepM + nMid++] = b;
-  }
-  // the ghost: trim the oldest live entries, compact when the ring lacks room, push
-  const uint64_t rcap = s.ghost_ring_cap, rmask = rcap - 1;
-  int rb = c->ghost_rbuf;
-  uint64_t tail = c->ghost_tail, head = c->ghost_head;
-  const int64_t live_old = c->ghost_live;
-  const int64_t X = live_old + kS - s.s3_ghost_cap;
-  const int64_t Xo = tmin<int64_t>(tmax<int64_t>(X, 0), live_old);
-  const int64_t born = tmax<int64_t>(X - live_old, 0);
-  uint32_t* ring = ring_of(s, rb);
-  uint32_t* bits = bits_of(s, rb);
-  auto bit_at = [&](uint32_t* bw, uint64_t p) { return (bw[(p & rmask) >> 5] >> (p & 31)) & 1; };
-  int64_t erased = 0;
-  while (erased < Xo && tail < head) {
-    if (bit_at(bits, tail)) {
-      gh_erase(s, ring[tail & rmask]);
-      bits[(tail & rmask) >> 5] &= ~(1u << (tail & 31));
-      ++erased;
-    }
-    ++tail;
-  }
-  uint64_t pbase = head;
-  if ((int64_t)(head - tail) + kS > (int64_t)rcap || ((s.flags & PS_FLAG_S3_COMPACT_GHOST) && head > tail)) {
-    uint32_t* nring = ring_of(s, rb ^ 1);
-    uint32_t* nbits = bits_of(s, rb ^ 1);
-    uint64_t w = 0;
-    for (uint64_t p = tail; p < head; ++p) {
-      if (!bit_at(bits, p)) continue;
-      const uint32_t slot = ring[p & rmask];
-      nring[w] = slot;
-      s.ghost_map[slot].blk = (uint32_t)w;
-      nbits[w >> 5] |= 1u << (w & 31);
-      ++w;
-    }
-    for (uint64_t p = tail & ~31ull; p < head; p += 32) bits[(p & rmask) >> 5] = 0;
-    rb ^= 1;
-    ring = nring;
-    bits = nbits;
-    tail = 0;
-    head = w;
-    pbase = head - (uint64_t)born;
-  } else if (born > 0) {
-    tail = head + (uint64_t)born;
-  }
-  for (int64_t t = born; t < kS; ++t) {
-    const uint32_t b = pushes[t];
-    const uint64_t p = pbase + (uint64_t)t;
-    const uint32_t slot = gh_insert(s, s.blk_key[b], s.blk_group[b], (uint32_t)(p & rmask), c->ghost_ctr + (uint64_t)t + 1);
-    if (slot == kNone) { bad = true; break; }
-    ring[p & rmask] = slot;
-    bits[(p & rmask) >> 5] |= 1u << (p & 31);
-  }
-  c->ghost_ctr += (uint64_t)kS;
-  c->ghost_live = live_old - Xo + (kS - born);
-  c->ghost_tail = tail;
-  c->ghost_head = pbase + (uint64_t)kS;
-  c->ghost_rbuf = rb;
-  pl->kS = kS;
-  pl->MA = moved;
-  pl->nKeepS = nKeepS;
-  pl->nKeepM = nKeepM;
-  pl->nMid = nMid;
-  pl->ctr_end = ctr;
-  if (bad) c->internal_error = 1;
+  if (c->status != PS_OK) return;
+  s3_plan(s, c);
+  __syncthreads();
+  if (threadIdx.x == 0 && s.s3_plan->fb) s3_sequential(s, c);
 }
 
 // ===========================================================================
@@ -1142,10 +1144,15 @@ int32_t launch_s3_select(const DevState& s, cudaStream_t st, bool plain_first, i
   if (plain_first) k_s3_count<<<152 * 4, kCT, 0, st>>>(s);
   else launch_k(k_s3_count, 152 * 4, kCT, 0, st, s);
   launch_k(k_s3_plan, 1, kPT, 0, st, s);
-  launch_k(k_s3_fallback, 1, 32, 0, st, s);
   launch_k(k_s3_apply, 152 * 4, kCT, 0, st, s);
-  launch_k(k_s3_push, 152 * 4, kCT, 0, st, s);
-  *launches += 5;
+  *launches += 3;
+  return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
+}
+
+int32_t launch_s3_push(const DevState& s, cudaStream_t st, bool plain, int* launches) {
+  if (plain) k_s3_push<<<152 * 4, kCT, 0, st>>>(s);
+  else launch_k(k_s3_push, 152 * 4, kCT, 0, st, s);
+  ++*launches;
   return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
 }
 
