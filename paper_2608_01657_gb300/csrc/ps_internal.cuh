@@ -457,8 +457,7 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
 // phase, 1 its global fallback, 2 lru, 3 StaticQuota.
 void launch_queue_init(const DevState& s, cudaStream_t st);
 int32_t launch_queue_cand(const DevState& s, cudaStream_t st, int* launches);
-int32_t launch_queue_select(const DevState& s, cudaStream_t st, const CaptureCtx* cap, int phase, int depth,
-                            bool plain_first, int* launches);
+int32_t launch_queue_select(const DevState& s, cudaStream_t st, int phase, bool plain_first, int* launches);
 int32_t launch_queue_append(const DevState& s, cudaStream_t st, const CaptureCtx* cap, int* launches);
 // S3-FIFO (ps_s3fifo.cu)
 // The select: per-chunk counts, the closed-form plan, the sequential kernel

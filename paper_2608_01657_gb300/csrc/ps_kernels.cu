@@ -1435,7 +1435,7 @@ __global__ void __launch_bounds__(1024) k_quota_sel(DevState s) {
 // each) the ones with the smallest candidate keys are taken (resolved after
 // the radix select finds those keys).  What the debt phase cannot cover goes
 // to the global fallback in (class, stamp) order.
-__global__ void __launch_bounds__(1024) k_waterfill(DevState s0, cudaGraphConditionalHandle fb_cond, int has_cond) {
+__global__ void __launch_bounds__(1024) k_waterfill(DevState s0) {
   // contract arrays are read from the parameter block (see k_grant)
   const DevState s = with_args(s0);
   Ctl* c = s.ctl;
@@ -1499,7 +1499,6 @@ __global__ void __launch_bounds__(1024) k_waterfill(DevState s0, cudaGraphCondit
     }
     if (threadIdx.x == 0) {
       c->m_fb = m - E; c->sel_ntie = 0; c->sel_k = 0; c->lst_n = 0;
-      if (has_cond && m > E) cudaGraphSetConditional(fb_cond, 1);  // the queues' fallback phase runs
     }
     return;
   }
@@ -2455,21 +2454,14 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
   if (fork && cudaStreamWaitEvent(st, cap->join, 0) != cudaSuccess) return PS_ERR_CUDA;
   if (s.lg_on) {
     // indexed queues: the same victims, taken from the queues' heads
-    cudaGraphConditionalHandle hq_fb = 0;
     if (s.policy == PS_PREFIXSHIELD) {
-      if (cap && !cond_handle(st, &hq_fb)) return PS_ERR_CUDA;
       // the first kernel after the side branch's join depends on two nodes:
       // a plain launch (a programmatic edge takes a single kernel predecessor)
-      PS_LAUNCH(k_waterfill<<<1, 1024, 0, st>>>(s, hq_fb, cap ? 1 : 0));
-      if (launch_queue_select(s, st, cap, 0, 0, false, &launches) != PS_OK) return PS_ERR_CUDA;
-      cudaStream_t f = st;
-      if (cap) {
-        if (!cond_open(st, cap->aux, hq_fb)) return PS_ERR_CUDA;
-        f = cap->aux;
-      }
-      if (launch_queue_select(s, f, cap, 1, 1, false, &launches) != PS_OK) return PS_ERR_CUDA;
-      if (cap && !cond_close(cap->aux)) return PS_ERR_CUDA;
-    } else if (launch_queue_select(s, st, cap, s.policy == PS_LRU ? 2 : 3, 0, fork, &launches) != PS_OK) {
+      PS_LAUNCH(k_waterfill<<<1, 1024, 0, st>>>(s));
+      if (launch_queue_select(s, st, 0, false, &launches) != PS_OK) return PS_ERR_CUDA;
+      // the fallback: its plan finds nothing owed when the debts covered all
+      if (launch_queue_select(s, st, 1, false, &launches) != PS_OK) return PS_ERR_CUDA;
+    } else if (launch_queue_select(s, st, s.policy == PS_LRU ? 2 : 3, fork, &launches) != PS_OK) {
       return PS_ERR_CUDA;
     }
   }
@@ -2487,7 +2479,7 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
   if (s.lg_on) {
     // selected above
   } else if (s.policy == PS_PREFIXSHIELD) {
-    PS_LAUNCH(k_waterfill<<<1, 1024, 0, st>>>(s, 0, 0));  // after the join: plain
+    PS_LAUNCH(k_waterfill<<<1, 1024, 0, st>>>(s));  // after the join: plain
     select(0, 0);
     select(1, 1);  // the global fallback, started by the debt phase's finish
   } else if (s.policy == PS_STATICQUOTA) {

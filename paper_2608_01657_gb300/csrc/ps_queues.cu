@@ -231,8 +231,7 @@ __global__ void __launch_bounds__(1024) k_lg_plan(DevState s, int phase, int rou
 constexpr uint64_t kAgg = 1ull << 62, kIncl = 2ull << 62, kValMask = (1ull << 62) - 1;
 constexpr int kLookbackSpins = 1 << 22;
 
-__global__ void __launch_bounds__(kScanThreads) k_lg_take(DevState s, int phase, cudaGraphConditionalHandle next,
-                                                          int has_next) {
+__global__ void __launch_bounds__(kScanThreads) k_lg_take(DevState s, int phase) {
   s = with_args(s);
   __shared__ int32_t sc0[kMaxLogs + 1];
   __shared__ int s_q;
@@ -348,7 +347,6 @@ __global__ void __launch_bounds__(kScanThreads) k_lg_take(DevState s, int phase,
           c->internal_error = 1;  // the log holds fewer live entries than counted
         } else {
           c->lg_more = 1;
-          if (has_next) cudaGraphSetConditional(next, 1);
         }
       }
     }
@@ -698,26 +696,15 @@ int32_t launch_queue_cand(const DevState& s, cudaStream_t st, int* launches) {
   return PS_OK;
 }
 
-int32_t launch_queue_select(const DevState& s, cudaStream_t st, const CaptureCtx* cap, int phase, int depth,
-                            bool plain_first, int* launches) {
-  cudaGraphConditionalHandle h1 = 0;
-  if (cap && !cond_handle(st, &h1)) return PS_ERR_CUDA;
-  auto round = [&](cudaStream_t q, int r) {
-    if (plain_first && r == 0) k_lg_plan<<<1, 1024, 0, q>>>(s, phase, r);  // its predecessor is a join
-    else launch_k(k_lg_plan, 1, 1024, 0, q, s, phase, r);
-    launch_k(k_lg_take, kScanGrid, kScanThreads, 0, q, s, phase, h1, (cap && r == 0) ? 1 : 0);
+int32_t launch_queue_select(const DevState& s, cudaStream_t st, int phase, bool plain_first, int* launches) {
+  // Both rounds are launched on every step (a round with nothing to do
+  // returns at once): a conditional graph node costs about 10 us even when
+  // its body is skipped, these two launches about 3.
+  for (int r = 0; r < 2; ++r) {
+    if (plain_first && r == 0) k_lg_plan<<<1, 1024, 0, st>>>(s, phase, r);  // its predecessor is a join
+    else launch_k(k_lg_plan, 1, 1024, 0, st, s, phase, r);
+    launch_k(k_lg_take, kScanGrid, kScanThreads, 0, st, s, phase);
     *launches += 2;
-  };
-  round(st, 0);
-  if (cap) {
-    // the second round is a conditional body (depth 0 phases nest on aux,
-    // the fallback's on aux2)
-    cudaStream_t body = depth == 0 ? cap->aux : cap->aux2;
-    if (!cond_open(st, body, h1)) return PS_ERR_CUDA;
-    round(body, 1);
-    if (!cond_close(body)) return PS_ERR_CUDA;
-  } else {
-    round(st, 1);
   }
   if (phase == 0) {
     launch_k(k_lg_tie, 1, PS_MAX_GROUPS, 0, st, s);
