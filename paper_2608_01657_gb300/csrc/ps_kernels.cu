@@ -2136,12 +2136,11 @@ __global__ void __launch_bounds__(kBmThreads, 3) k_bm_write(DevState s) {
   const uint32_t vic = in ? s.bm_victim[w] : 0u, inv = in ? s.bm_inval[w] : 0u;
   // earlier chunks' free, evicted and invalidated ids
   int64_t fb = 0, vb = 0, ib = 0;
-  for (int j = t; j < (int)blockIdx.x; j += kBmThreads) {
+  for (int j = t; j < (int)blockIdx.x; j += kBmThreads) {  // (none in a single chunk)
     fb += s.bm_chunk_cnt[0 * nchunks + j];
     vb += s.bm_chunk_cnt[1 * nchunks + j];
     ib += s.bm_chunk_cnt[2 * nchunks + j];
   }
-  const int64_t here = s.bm_chunk_cnt[blockIdx.x];
   {
     __shared__ int64_t s_before[3][kBmThreads / 32];
     fb = warp_sum(fb); vb = warp_sum(vb); ib = warp_sum(ib);
@@ -2152,11 +2151,11 @@ __global__ void __launch_bounds__(kBmThreads, 3) k_bm_write(DevState s) {
     vb = warp_sum(hold ? s_before[1][lane_id()] : (int64_t)0);
     ib = warp_sum(hold ? s_before[2][lane_id()] : (int64_t)0);
   }
-  const int64_t take_here = tmin(ftake, fb + here) - tmin(ftake, fb);
-  // this word's taken free ids: the chunk's lowest take_here free ids
-  const uint32_t f = (in && take_here > 0) ? free_word(s, w) : 0u;
+  const uint32_t f = (in && ftake > 0) ? free_word(s, w) : 0u;
   uint64_t tot1;
   const uint64_t ex1 = block_excl_scan<uint64_t>(pack3(__popc(f), __popc(vic), __popc(inv)), &tot1);
+  // this word's taken free ids: the chunk's lowest take_here free ids
+  const int64_t take_here = tmin(ftake, fb + field3(tot1, 0)) - tmin(ftake, fb);
   const int64_t fl = field3(ex1, 0);
   const int64_t want = tmin<int64_t>(tmax<int64_t>(take_here - fl, 0), __popc(f));
   const uint32_t alloc = lowest_bits(f, (int)want) | vic;
@@ -2503,9 +2502,13 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
   }
   mark(7);
   const int nchunks = (int)((s.nwords + kBmChunk - 1) / kBmChunk);
-  if (fork3) PS_LAUNCH((k_bm_count<<<nchunks, kBmChunk, 0, st>>>(s)));  // after the fork: plain
-  else PS_LAUNCH(launch_k(k_bm_count, nchunks, kBmChunk, 0, st, s));
-  PS_LAUNCH(launch_k(k_bm_write, nchunks, kBmThreads, 0, st, s));
+  // a pool of one chunk (8192 blocks) has no earlier chunks to count
+  if (nchunks > 1) {
+    if (fork3) PS_LAUNCH((k_bm_count<<<nchunks, kBmChunk, 0, st>>>(s)));  // after the fork: plain
+    else PS_LAUNCH(launch_k(k_bm_count, nchunks, kBmChunk, 0, st, s));
+  }
+  if (fork3 && nchunks == 1) PS_LAUNCH((k_bm_write<<<nchunks, kBmThreads, 0, st>>>(s)));
+  else PS_LAUNCH(launch_k(k_bm_write, nchunks, kBmThreads, 0, st, s));
   mark(8);
   // (evictions happen in k_insert: every victim is allocated again in its step)
   mark(9);
