@@ -232,7 +232,7 @@ size_t carve(const Dims& d, char* base, DevState* s, ps_handle* h) {
   t.ghost_ring = cv.take<uint32_t>(2 * (size_t)d.ghost_ring_cap);
   t.ghost_bits = cv.take<uint32_t>(2 * (size_t)(d.ghost_ring_cap / 32));
   t.table = cv.take<TableEntry>((size_t)kTableWays << d.tb_log2);
-  t.table_ovf = cv.take<uint32_t>((size_t)1 << d.tb_log2);
+  t.tags = cv.take<TagBucket>((size_t)1 << d.tb_log2);
   t.ledger = cv.take<int64_t>(G * d.C);
   t.ledger_b0 = cv.take<int64_t>(G * d.C);
   t.contract_of_group = cv.take<int32_t>(G);

@@ -44,6 +44,12 @@ struct __align__(16) TableEntry {   // native prefix table (group, key) -> block
   uint32_t grp;
 };
 
+struct __align__(32) TagBucket {    // native prefix table: what a lookup reads first
+  uint16_t tag[kTableWays];  // of the last key inserted into each way (0: none yet)
+  uint32_t ovf;              // live keys probing past the bucket
+  uint32_t pad[3];
+};
+
 struct __align__(32) ClaimEntry {   // per-step: first request that needs a new key
   uint64_t key;     // 0 when empty
   uint32_t minreq;  // lowest request index containing the key (atomicMin)
@@ -278,7 +284,7 @@ struct DevState {
   uint32_t* ghost_ring;    // [2][ghost_ring_cap] map slot of each FIFO position
   uint32_t* ghost_bits;    // [2][ghost_ring_cap / 32] live FIFO positions
   TableEntry* table;
-  uint32_t* table_ovf;     // per bucket: live keys probing past it
+  TagBucket* tags;         // per bucket: a tag of each way's key, and the live keys probing past it
   int64_t* ledger;         // B_{g,c}, fixed point
   int64_t* ledger_b0;      // per step: B_{g,c} refilled to now, before the step's charges
   int32_t* contract_of_group;

@@ -83,29 +83,88 @@ __device__ __forceinline__ uint64_t mul61(uint64_t a, uint64_t b) {  // a, b < p
 }
 
 // ---- native prefix table ---------------------------------------------------
-// Lookup by one thread: the 128-byte home bucket (8 entries), then following
-// buckets while the overflow count says some key probed past.
-// All eight ways and the overflow count are loaded before any is compared,
-// so a bucket costs one round trip (a return inside the loads would keep the
-// compiler from issuing a later way's load before an earlier way's compare).
+// Lookup by one thread: the home bucket's 32-byte tag sector (a 16-bit tag per
+// way, and the overflow count), then the entry of each way whose tag matches,
+// then following buckets while the overflow count says some key probed past.
+// A miss reads one sector instead of the whole 128-byte bucket, a hit one more:
+// at 2^20 blocks the tags are 16 MB, which stay in L2, beside a 64 MB table.
+// Tags are never cleared (a delete that cleared one could land after a later
+// insert's): a stale tag costs a look at an empty or another key's entry.
+__device__ __forceinline__ uint32_t table_tag(uint64_t key, uint32_t g) {
+  const uint64_t x = (key ^ ((uint64_t)(g + 1) * 0x9E3779B97F4A7C15ull)) * 0xD6E8FEB86659FD93ull;
+  const uint32_t t = (uint32_t)(x >> 16) & 0xFFFFu;  // away from the bits that choose the bucket
+  return t ? t : 1u;
+}
+// The ways of a bucket whose tag matches: way 2k at bit k, way 2k + 1 at bit
+// 16 + k; and the way of the lowest such bit.
+__device__ __forceinline__ uint32_t tag_matches(const uint4& t, uint32_t tag) {
+  const uint32_t t2 = tag * 0x10001u;
+  return (__vcmpeq2(t.x, t2) & 0x10001u) | (__vcmpeq2(t.y, t2) & 0x20002u) | (__vcmpeq2(t.z, t2) & 0x40004u) |
+         (__vcmpeq2(t.w, t2) & 0x80008u);
+}
+__device__ __forceinline__ uint32_t tag_bit(uint32_t w) { return 1u << ((w >> 1) + 16 * (w & 1)); }
+__device__ __forceinline__ int tag_way(uint32_t m) {
+  const int k = __ffs((int)m) - 1;
+  return k < 16 ? 2 * k : 2 * (k - 16) + 1;
+}
 __device__ uint32_t table_find(const DevState& s, uint64_t key, uint32_t g) {
   const uint32_t mask = (1u << s.tb_nbuckets_log2) - 1;
+  const uint32_t tag = table_tag(key, g);
   uint32_t b = table_home(key, g, s.tb_nbuckets_log2);
   for (uint32_t it = 0; it <= mask; ++it) {
-    const uint4* e = reinterpret_cast<const uint4*>(s.table + (size_t)b * kTableWays);
-    uint4 raw[kTableWays];
-#pragma unroll
-    for (int w = 0; w < kTableWays; ++w) raw[w] = __ldg(e + w);
-    const uint32_t ovf = __ldg(s.table_ovf + b);  // issued with the bucket: a miss needs no second trip
-    uint32_t hit = kNone;
-#pragma unroll
-    for (int w = 0; w < kTableWays; ++w)
-      if (raw[w].z != kNone && raw[w].x == (uint32_t)key && raw[w].y == (uint32_t)(key >> 32) && raw[w].w == g)
-        hit = raw[w].z;
-    if (hit != kNone || ovf == 0) return hit;
+    const uint4 tg = __ldg(reinterpret_cast<const uint4*>(s.tags + b));
+    const uint32_t ovf = __ldg(&s.tags[b].ovf);  // issued with the tags: a miss needs no second trip
+    for (uint32_t m = tag_matches(tg, tag); m; m &= m - 1) {
+      const uint4 raw = __ldg(reinterpret_cast<const uint4*>(s.table + (size_t)b * kTableWays + tag_way(m)));
+      if (raw.z != kNone && raw.x == (uint32_t)key && raw.y == (uint32_t)(key >> 32) && raw.w == g) return raw.z;
+    }
+    if (ovf == 0) return kNone;
     b = (b + 1) & mask;
   }
   return kNone;
+}
+
+// The way of its home bucket where a key's insertion tries first.
+__device__ __forceinline__ uint32_t table_way0(uint64_t key) { return (uint32_t)(key >> 7) & (kTableWays - 1); }
+
+// The same for two keys of a thread, in one round of loads where possible:
+// both tag sectors and, beside them, the entry each key's insertion tries
+// first (at a quarter load it is usually there).  The first entry of another
+// matching way costs a second trip; a key not settled by these (several ways'
+// tags match, or keys probed past the bucket) takes the general walk.
+__device__ __forceinline__ void table_find2(const DevState& s, uint64_t keyA, uint64_t keyB, uint32_t g, bool doA,
+                                            bool doB, uint32_t* blkA, uint32_t* blkB) {
+  const uint32_t bA = table_home(keyA, g, s.tb_nbuckets_log2), bB = table_home(keyB, g, s.tb_nbuckets_log2);
+  const uint32_t wA = table_way0(keyA), wB = table_way0(keyB);
+  uint4 tA = make_uint4(0, 0, 0, 0), tB = tA, eA = make_uint4(0, 0, kNone, 0), eB = eA;
+  uint32_t oA = 0, oB = 0;
+  if (doA) {
+    tA = __ldg(reinterpret_cast<const uint4*>(s.tags + bA));
+    oA = __ldg(&s.tags[bA].ovf);
+    eA = __ldg(reinterpret_cast<const uint4*>(s.table + (size_t)bA * kTableWays + wA));
+  }
+  if (doB) {
+    tB = __ldg(reinterpret_cast<const uint4*>(s.tags + bB));
+    oB = __ldg(&s.tags[bB].ovf);
+    eB = __ldg(reinterpret_cast<const uint4*>(s.table + (size_t)bB * kTableWays + wB));
+  }
+  auto is_key = [&](const uint4& e, uint64_t key) {
+    return e.z != kNone && e.x == (uint32_t)key && e.y == (uint32_t)(key >> 32) && e.w == g;
+  };
+  bool hitA = is_key(eA, keyA), hitB = is_key(eB, keyB);
+  // other ways with the key's tag
+  const uint32_t mA = hitA ? 0u : tag_matches(tA, table_tag(keyA, g)) & ~tag_bit(wA);
+  const uint32_t mB = hitB ? 0u : tag_matches(tB, table_tag(keyB, g)) & ~tag_bit(wB);
+  if (mA) {
+    eA = __ldg(reinterpret_cast<const uint4*>(s.table + (size_t)bA * kTableWays + tag_way(mA)));
+    hitA = is_key(eA, keyA);
+  }
+  if (mB) {
+    eB = __ldg(reinterpret_cast<const uint4*>(s.table + (size_t)bB * kTableWays + tag_way(mB)));
+    hitB = is_key(eB, keyB);
+  }
+  *blkA = hitA ? eA.z : ((mA & (mA - 1)) != 0 || oA != 0 ? table_find(s, keyA, g) : kNone);
+  *blkB = hitB ? eB.z : ((mB & (mB - 1)) != 0 || oB != 0 ? table_find(s, keyB, g) : kNone);
 }
 
 // Returns the slot, with kDisplaced set when it lies past the home bucket
@@ -117,7 +176,8 @@ constexpr uint32_t kDisplaced = 0x80000000u;
 __device__ uint32_t table_insert(const DevState& s, uint64_t key, uint32_t g, uint32_t blk) {
   const uint32_t mask = (1u << s.tb_nbuckets_log2) - 1;
   uint32_t b = table_home(key, g, s.tb_nbuckets_log2);
-  const uint32_t w0 = (uint32_t)(key >> 7) & (kTableWays - 1);
+  const uint32_t w0 = table_way0(key);
+  const uint16_t tag = (uint16_t)table_tag(key, g);
   for (uint32_t it = 0; it <= mask; ++it) {
     TableEntry* e = s.table + (size_t)b * kTableWays;
     for (int q = 0; q < kTableWays; ++q) {
@@ -125,10 +185,11 @@ __device__ uint32_t table_insert(const DevState& s, uint64_t key, uint32_t g, ui
       if (atomicCAS(&e[w].blk, kNone, blk) == kNone) {
         e[w].key = key;
         e[w].grp = g;
+        s.tags[b].tag[w] = tag;
         return (b * kTableWays + w) | (it ? kDisplaced : 0u);
       }
     }
-    atomicAdd(s.table_ovf + b, 1u);
+    atomicAdd(&s.tags[b].ovf, 1u);
     b = (b + 1) & mask;
   }
   return kNone;  // unreachable: the table is at most a quarter full
@@ -147,7 +208,7 @@ __device__ __forceinline__ void table_delete_known(const DevState& s, uint32_t t
   if (!(tagged & kDisplaced)) return;  // in its home bucket: no counter passed
   const uint32_t bucket = slot / kTableWays;
   uint32_t x = table_home(key, g, s.tb_nbuckets_log2);
-  for (uint32_t it = 0; x != bucket && it <= mask; ++it, x = (x + 1) & mask) atomicSub(s.table_ovf + x, 1u);
+  for (uint32_t it = 0; x != bucket && it <= mask; ++it, x = (x + 1) & mask) atomicSub(&s.tags[x].ovf, 1u);
 }
 __device__ void table_delete(const DevState& s, uint32_t blk) {
   const uint32_t mask = (1u << s.tb_nbuckets_log2) - 1;
@@ -157,7 +218,7 @@ __device__ void table_delete(const DevState& s, uint32_t blk) {
   if (!(tagged & kDisplaced)) return;  // in its home bucket: no counter passed
   const uint32_t bucket = slot / kTableWays;
   uint32_t x = table_home(s.blk_key[blk], s.blk_group[blk], s.tb_nbuckets_log2);
-  for (uint32_t it = 0; x != bucket && it <= mask; ++it, x = (x + 1) & mask) atomicSub(s.table_ovf + x, 1u);
+  for (uint32_t it = 0; x != bucket && it <= mask; ++it, x = (x + 1) & mask) atomicSub(&s.tags[x].ovf, 1u);
 }
 
 // ---- per-step claim map ------------------------------------------------------
@@ -583,8 +644,7 @@ __device__ __forceinline__ bool hash_lookup_chunk(const DevState& s, Ctl* c, con
     const uint64_t C = add61(mul61(kc[lane + 1], cinB), bB);
     keyB = fix_reserved(mix64(C ^ ((uint64_t)(mB + 1) * 0xD1B54A32D192ED03ull)));
   }
-  if (lane < nbA) blkA = table_find(s, keyA, g);
-  if (lane < nbB) blkB = table_find(s, keyB, g);
+  table_find2(s, keyA, keyB, g, lane < nbA, lane < nbB, &blkA, &blkB);
   const unsigned missA = __ballot_sync(kFull, lane < nbA && blkA == kNone);
   const unsigned missB = __ballot_sync(kFull, lane < nbB && blkB == kNone);
   const bool anymiss = (missA | missB) != 0;
