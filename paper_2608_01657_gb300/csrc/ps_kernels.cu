@@ -274,6 +274,19 @@ __device__ __forceinline__ bool pos_ref(const DevState& s, int64_t pos, PosRef* 
   r->m = (int)s.pos_m[pos];
   return true;
 }
+// The position of a position-parallel kernel, false past the step's blocks or
+// in a failed step.  The step's status and size and the position's record are
+// loaded in one round trip: the records reach to max_blocks whatever the
+// step's size, so they may be loaded before it is known.  (A status looked at
+// first cost every such kernel two trips before its work began.)
+__device__ __forceinline__ bool pos_open(const DevState& s, const Ctl* c, int64_t pos, PosRef* r) {
+  const int32_t st = c->status;
+  const int64_t nb = c->nblocks;
+  const bool in = pos < s.max_blocks;
+  r->i = in ? s.pos_req[pos] : 0u;
+  r->m = in ? (int)s.pos_m[pos] : 0;
+  return st == PS_OK && pos < nb;
+}
 
 // ===========================================================================
 // Init: an empty pool, every balance at beta (Sec. III-B, B = beta at t = 0).
@@ -743,12 +756,11 @@ __global__ void __launch_bounds__(256, kHashCtasPerSm) k_hash_lookup(DevState s,
   __shared__ uint32_t sk[BS + 2];                // the NH key words (read by every lane alike)
   __shared__ uint64_t kc[2 * (kSegBlocks + 1)];  // Kc^j, then Kc^(32 t)
   Ctl* c = s.ctl;
-  if (c->status != PS_OK) return;
+  const int64_t nsegs = c->nsegs;  // none in a failed call
   if (threadIdx.x < BS + 2) sk[threadIdx.x] = s.key_words[threadIdx.x];
   if (threadIdx.x < 2 * (kSegBlocks + 1)) kc[threadIdx.x] = s.kc_pow[threadIdx.x];
   __syncthreads();
   const int lane = lane_id();
-  const int64_t nsegs = c->nsegs;
   for (;;) {
     uint32_t t = 0;
     if (lane == 0) t = atomicAdd(&c->hash_ticket, 1u);
@@ -819,18 +831,18 @@ __device__ __forceinline__ HistEntry ldcg_hist(const HistEntry* p) {
 __global__ void __launch_bounds__(kThreads) k_claims(DevState s) {
   s = with_args(s);
   Ctl* c = s.ctl;
-  if (c->status != PS_OK) return;
-  if (history_overflows(s, c)) {
-    undo_pin_claim(s, c, blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
+  const int64_t pos = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  PosRef r;
+  const bool overflow = history_overflows(s, c);
+  const uint32_t step32 = (uint32_t)c->step;
+  const bool valid = pos_open(s, c, pos, &r);
+  if (overflow) {
+    if (c->status == PS_OK) undo_pin_claim(s, c, pos);
     return;
   }
-  const int64_t pos = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const uint32_t step32 = (uint32_t)c->step;
   bool inv = false;
   uint32_t ginv = 0, kinv = 0;
-  PosRef r;
   bool own = false;
-  const bool valid = pos_ref(s, pos, &r);
   if (valid) {
     // the position's records in one round of loads, then what they point to
     const int h = s.rq_h[r.i];
@@ -1018,11 +1030,10 @@ __global__ void __launch_bounds__(1024) k_grant_quota(DevState s) {
 __global__ void __launch_bounds__(kThreads) k_instep(DevState s) {
   s = with_args(s);
   const Ctl* c = s.ctl;
-  if (c->status != PS_OK) return;
   const int64_t pos = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   PosRef r;
   bool past = false;
-  const bool valid = pos_ref(s, pos, &r);
+  const bool valid = pos_open(s, c, pos, &r);
   int h = 0, sown = 0;
   uint32_t slot = kNone;
   if (valid) {  // one round of loads
@@ -1193,10 +1204,10 @@ __global__ void __launch_bounds__(kMeterThreads) k_meter(DevState s0) {
 __global__ void __launch_bounds__(kThreads) k_touch(DevState s) {
   s = with_args(s);
   const Ctl* c = s.ctl;
-  if (c->status != PS_OK) return;
   const int64_t pos = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const uint64_t step = c->step, base = c->stamp_base;
   PosRef r;
-  if (!pos_ref(s, pos, &r)) return;
+  if (!pos_open(s, c, pos, &r)) return;
   // every record of the position and its request in one round of loads (an
   // atomic in between would hold back the loads after it), then the block's
   const uint32_t i = r.i;
@@ -1205,7 +1216,6 @@ __global__ void __launch_bounds__(kThreads) k_touch(DevState s) {
   const uint8_t fl = s.rq_flags[i];
   const uint64_t p = s.rq_p[i];
   const uint32_t b = s.pos_blk[pos], slot = s.pos_claim[pos];
-  const uint64_t step = c->step, base = c->stamp_base;
   if (m >= h + re) return;
   const bool proven = fl & 1, gate = fl & 2;
   const uint64_t stamp = make_stamp(base, pbase, n, m);
@@ -1237,7 +1247,6 @@ __global__ void __launch_bounds__(kThreads) k_touch(DevState s) {
 __global__ void __launch_bounds__(kThreads) k_touch2(DevState s) {
   s = with_args(s);
   const Ctl* c = s.ctl;
-  if (c->status != PS_OK) return;
   const int64_t pos = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   PosRef r;
   bool gated = false, promoted = false;
@@ -1247,7 +1256,7 @@ __global__ void __launch_bounds__(kThreads) k_touch2(DevState s) {
   uint32_t b = kNone, slot = kNone;
   uint8_t fl = 0;
   const uint64_t step = c->step;
-  if (pos_ref(s, pos, &r)) {  // one round of loads (an untouched position's eligibility is stale, and not used)
+  if (pos_open(s, c, pos, &r)) {  // one round of loads (an untouched position's eligibility is stale, and not used)
     const uint8_t el = s.pos_elig[pos];
     const int re = s.rq_e[r.i];
     h = s.rq_h[r.i];
@@ -1287,8 +1296,9 @@ __global__ void __launch_bounds__(kThreads) k_touch2(DevState s) {
 __global__ void __launch_bounds__(1024) k_cand(DevState s) {
   s = with_args(s);
   extern __shared__ uint32_t cand_smem[];  // 5 arrays of nseg * kClasses
-  Ctl* c = s.ctl;
-  if (c->status != PS_OK) return;  // runs beside S3-S4: the victim count is not known yet
+  // runs beside S3-S4: the victim count is not known yet, and a failed step
+  // ignores what is written here
+  const Ctl* c = s.ctl;
   const uint32_t step32 = (uint32_t)c->step;
   // segments: groups for prefixshield and staticquota, one for lru; retention
   // classes only for prefixshield
@@ -1505,16 +1515,20 @@ __global__ void __launch_bounds__(1024) k_waterfill(DevState s0) {
   const int G = s.G;
   const int64_t eps = s.eps;
   const bool seg = !(s.flags & PS_FLAG_NO_SEGMENTATION);
-  const int64_t m = (c->status == PS_OK) ? c->mvict : 0;
+  const int32_t st = c->status;
+  const int64_t mv = c->mvict;
+  for (int g = threadIdx.x; g < G; g += blockDim.x) {  // loaded beside the victim count
+    sP[g] = s.grp_P[g];
+    sD[g] = s.grp_delta[g];
+    sQ[g] = s.grp_qsize[g];
+  }
+  const int64_t m = st == PS_OK ? mv : 0;
   if (m == 0) {
     for (int g = threadIdx.x; g < G; g += blockDim.x) { s.sel[g].active = 0; s.grp_x[g] = 0; s.grp_full[g] = 0; }
     if (threadIdx.x == 0) c->m_fb = 0;
     return;
   }
   for (int g = threadIdx.x; g < G; g += blockDim.x) {
-    sP[g] = s.grp_P[g];
-    sD[g] = s.grp_delta[g];
-    sQ[g] = s.grp_qsize[g];
     uint64_t rcp = 0;
     for (int cc = 0; cc < s.C; ++cc)
       if (s0.delta[cc] == sD[g]) rcp = s0.delta_rcp[cc];
@@ -2144,13 +2158,16 @@ __device__ __forceinline__ uint32_t free_word(const DevState& s, int64_t w) {
 __global__ void __launch_bounds__(kBmChunk) k_bm_count(DevState s) {
   s = with_args(s);
   const Ctl* c = s.ctl;
-  if (c->status != PS_OK) return;
   const int64_t w = (int64_t)blockIdx.x * kBmChunk + threadIdx.x;
   const int nchunks = gridDim.x;
   const bool in = w < s.nwords;
+  const int32_t st = c->status;
+  const int64_t ftake = c->ftake;
   const int nv = in ? __popc(s.bm_victim[w]) : 0;
   const int ni = in ? __popc(s.bm_inval[w]) : 0;
-  const int nf = (in && c->ftake > 0) ? __popc(free_word(s, w)) : 0;
+  const int fr = in ? __popc(free_word(s, w)) : 0;
+  if (st != PS_OK) return;
+  const int nf = ftake > 0 ? fr : 0;
   const int tv = block_sum(nv), ti = block_sum(ni), tf = block_sum(nf);
   if (threadIdx.x == 0) {
     s.bm_chunk_cnt[0 * nchunks + blockIdx.x] = tf;
@@ -2187,13 +2204,15 @@ __global__ void __launch_bounds__(kBmThreads, 3) k_bm_write(DevState s) {
   s = with_args(s);
   __shared__ ListSmem sm;
   Ctl* c = s.ctl;
-  if (c->status != PS_OK) return;
+  const int32_t st = c->status;
   const int t = (int)threadIdx.x;
   const int64_t w0 = (int64_t)blockIdx.x * kBmChunk, w = w0 + t;
   const int nchunks = gridDim.x;
   const bool in = t < kBmChunk && w < s.nwords;  // the first kBmChunk threads hold a word each
   const int64_t ftake = c->ftake;
   const uint32_t vic = in ? s.bm_victim[w] : 0u, inv = in ? s.bm_inval[w] : 0u;
+  const uint32_t fw = in ? free_word(s, w) : 0u;
+  if (st != PS_OK) return;
   // earlier chunks' free, evicted and invalidated ids
   int64_t fb = 0, vb = 0, ib = 0;
   for (int j = t; j < (int)blockIdx.x; j += kBmThreads) {  // (none in a single chunk)
@@ -2211,7 +2230,7 @@ __global__ void __launch_bounds__(kBmThreads, 3) k_bm_write(DevState s) {
     vb = warp_sum(hold ? s_before[1][lane_id()] : (int64_t)0);
     ib = warp_sum(hold ? s_before[2][lane_id()] : (int64_t)0);
   }
-  const uint32_t f = (in && ftake > 0) ? free_word(s, w) : 0u;
+  const uint32_t f = ftake > 0 ? fw : 0u;
   uint64_t tot1;
   const uint64_t ex1 = block_excl_scan<uint64_t>(pack3(__popc(f), __popc(vic), __popc(inv)), &tot1);
   // this word's taken free ids: the chunk's lowest take_here free ids
@@ -2256,16 +2275,20 @@ __global__ void __launch_bounds__(kBmThreads, 3) k_bm_write(DevState s) {
 __global__ void __launch_bounds__(kThreads, 5) k_insert(DevState s) {
   s = with_args(s);
   Ctl* c = s.ctl;
-  if (c->status != PS_OK) return;
   const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  // in one round trip (the claims' list reaches to max_blocks)
+  const int32_t st = c->status;
+  const int64_t nclaims = c->total_claims, n_alloc = c->n_alloc;
+  const uint64_t base = c->stamp_base;
+  const uint64_t cp = q < s.max_blocks ? s.claim_pos[q] : 0ull;
+  if (st != PS_OK) return;
   bool placed = false, evicted = false;
   uint32_t g = 0, gold = 0;
-  if (q < c->total_claims) {
+  if (q < nclaims) {
     // Rounds of loads, each issued as a whole before anything is stored (a
     // store or an atomic in between would hold back the loads after it): the
     // claim's position; its and its request's records; the id and the claim;
     // the id's old record.
-    const uint64_t cp = s.claim_pos[q];
     const uint32_t i = (uint32_t)(cp >> 32);
     const int64_t pos = (int64_t)(uint32_t)cp;
     const int si = s.rq_s[i], a = s.rq_a[i], cbase = s.rq_cbase[i], n = s.rq_n[i], pbase = s.rq_pbase[i];
@@ -2273,8 +2296,6 @@ __global__ void __launch_bounds__(kThreads, 5) k_insert(DevState s) {
     const uint64_t p = s.rq_p[i], key = s.pos_key[pos];
     const uint8_t knew = s.rq_knew[i];
     const uint32_t slot = s.pos_claim[pos];
-    const int64_t n_alloc = c->n_alloc;
-    const uint64_t base = c->stamp_base;
     g = (uint32_t)s.in_group[i];
     const int m = (int)(pos - pbase);
     const bool grant = m < si + a;
