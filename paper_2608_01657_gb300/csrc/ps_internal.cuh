@@ -98,6 +98,7 @@ struct Ctl {
   int64_t n_evicted, n_alloc;
   int64_t m_fb;            // prefixshield: victims left to the global fallback
   int32_t sel_ntie, sel_k; // prefixshield tie bookkeeping
+  int32_t sel_mode;        // what the select's first pass does (kSel*)
   int64_t lst_n;              // members of the select's split list
   uint32_t ticket;         // last-block-done counter for the radix passes and the split
   int32_t nlaunch;         // kernels launched by the step (conditional bodies run or not)
@@ -173,6 +174,10 @@ struct TieItem {
   int32_t log;
 };
 constexpr int kClasses = 3;
+// The select's first pass: a segment per group; one global segment; one global
+// segment beside groups that are taken whole.  (Its second pass, the fallback
+// after a pass of group segments, is global over what that left.)
+constexpr int32_t kSelGroups = 0, kSelGlobal = 1, kSelWhole = 2;
 // Buckets a select cuts a segment's key range into.
 constexpr int kDigBits = 12;
 constexpr int kDigBins = 1 << kDigBits;

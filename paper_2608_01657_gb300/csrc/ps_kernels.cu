@@ -886,8 +886,18 @@ __global__ void __launch_bounds__(1024) k_grant(DevState s0) {
   const DevState s = with_args(s0);
   extern __shared__ unsigned long long g_sum[];  // [G * C] the step's charges per (group, contract)
   Ctl* c = s.ctl;
+  // the first tile's claims (see below) in the status's round trip
+  int32_t n4[4], s4[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int i = u * (int)blockDim.x + (int)threadIdx.x;
+    n4[u] = i < s.R ? s.rq_n[i] : 0;
+    s4[u] = i < s.R ? s.rq_s[i] : 0;
+  }
+  const int64_t pinned = c->pinned, n_resident = c->n_resident, t_prev = c->t_prev;
+  const bool overflow = history_overflows(s, c);
   if (c->status != PS_OK) return;
-  if (history_overflows(s, c)) {  // undone by k_claims; the error is sticky
+  if (overflow) {  // undone by k_claims; the error is sticky
     if (threadIdx.x == 0) { c->status = PS_ERR_CAPACITY; c->sticky = PS_ERR_CAPACITY; }
     return;
   }
@@ -896,7 +906,7 @@ __global__ void __launch_bounds__(1024) k_grant(DevState s0) {
   const bool quota = s.policy == PS_STATICQUOTA;  // a_i already granted per group
   for (int k = threadIdx.x; k < s.G * C; k += blockDim.x) g_sum[k] = 0;
   __syncthreads();
-  const int64_t avail = s.N - c->pinned;
+  const int64_t avail = s.N - pinned;
   // Granted ranks are the first avail in (request, position) order, so the
   // grants before request i number min(avail, base_i), base_i the claims
   // before it, and a_i = min(avail, base_i + c_i) - min(avail, base_i).  One
@@ -911,7 +921,11 @@ __global__ void __launch_bounds__(1024) k_grant(DevState s0) {
     for (int u = 0; u < 4; ++u) {
       const int i = t0 + u * (int)blockDim.x + (int)threadIdx.x;
       const bool in = i < R;
-      cl[u] = in ? s.rq_n[i] - s.rq_s[i] : 0;
+      if (t0 > 0) {
+        n4[u] = in ? s.rq_n[i] : 0;
+        s4[u] = in ? s.rq_s[i] : 0;
+      }
+      cl[u] = n4[u] - s4[u];
       aq[u] = in && quota ? s.rq_a[i] : 0;
       v[u] = (uint64_t)cl[u] << 32 | (uint64_t)aq[u];
     }
@@ -947,7 +961,7 @@ __global__ void __launch_bounds__(1024) k_grant(DevState s0) {
   if (threadIdx.x == 0) {
     const int64_t need = carry_a;
     s.out.admitted_offsets[R] = (int32_t)need;
-    const int64_t nfree = s.N - c->n_resident;
+    const int64_t nfree = s.N - n_resident;
     c->avail = avail;
     c->total_claims = carry_c;
     c->need = need;
@@ -965,7 +979,7 @@ __global__ void __launch_bounds__(1024) k_grant(DevState s0) {
     // the Eq. 8 decrement of the largest indebted rate is the smallest one
     int64_t raw = 0, norm = 0, delta = 0;
     for (int cc = 0; cc < C; ++cc) {
-      const int64_t b0 = refill(s.ledger[g * C + cc], s0.beta[cc], s0.rho[cc], s.now - c->t_prev);
+      const int64_t b0 = refill(s.ledger[g * C + cc], s0.beta[cc], s0.rho[cc], s.now - t_prev);
       s.ledger_b0[g * C + cc] = b0;
       const int64_t b = b0 - (int64_t)g_sum[g * C + cc] * unit;  // Eq. 2 over the step's charges
       s.ledger[g * C + cc] = b;
@@ -1473,10 +1487,11 @@ __device__ void start_global_select(const DevState& s, Ctl* c, int fallback) {
   sel_start_cls(z, cnt, lo, hi, segmented);
   s.sel[0] = z;
   c->lst_n = 0;
+  if (!fallback) c->sel_mode = kSelGlobal;
 }
-__global__ void __launch_bounds__(32) k_sel_single(DevState s, int fallback) {
+__global__ void __launch_bounds__(32) k_sel_single(DevState s) {
   s = with_args(s);
-  start_global_select(s, s.ctl, fallback);
+  start_global_select(s, s.ctl, 0);
 }
 
 // StaticQuota: each group reclaims its overflow m_g from its own blocks, in
@@ -1493,7 +1508,7 @@ __global__ void __launch_bounds__(1024) k_quota_sel(DevState s) {
     sel_start_group(s, g, z, false);
     s.sel[g] = z;
   }
-  if (threadIdx.x == 0) { c->m_fb = 0; c->sel_ntie = 0; c->sel_k = 0; c->lst_n = 0; }
+  if (threadIdx.x == 0) { c->m_fb = 0; c->sel_ntie = 0; c->sel_k = 0; c->lst_n = 0; c->sel_mode = kSelGroups; }
 }
 
 // Alg. 2 in closed form (one CTA).  Group g's j-th victim would be taken at
@@ -1558,21 +1573,34 @@ __global__ void __launch_bounds__(1024) k_waterfill(DevState s0) {
   if (E <= m) {
     // a group that gives all its candidates needs no select: the split takes
     // them whole
+    int part = 0, whole = 0;
     for (int g = threadIdx.x; g < G; g += blockDim.x) {
       const int64_t x = items_gt(g, eps);
       const bool full = x > 0 && x == sQ[g];
       s.grp_x[g] = x;
       s.grp_full[g] = full ? 1 : 0;
-      if (x == 0) continue;  // k_grant left the segment inactive
+      whole |= full;
+      if (x == 0 || full) continue;  // k_grant left the segment inactive
+      part = 1;
       SelSeg z = s.sel[g];
-      z.rank = full ? 0 : x;
-      z.active = x > 0 && !full;
+      z.rank = x;
+      z.active = 1;
       z.incl = 1;
       sel_start_group(s, g, z, seg);
       s.sel[g] = z;
     }
+    part = __syncthreads_or(part);
+    whole = __syncthreads_or(whole);
     if (threadIdx.x == 0) {
       c->m_fb = m - E; c->sel_ntie = 0; c->sel_k = 0; c->lst_n = 0;
+      c->sel_mode = part ? kSelGroups : (whole ? kSelWhole : kSelGlobal);
+    }
+    // No group gives only some of its candidates (nothing is owed, or the
+    // indebted groups go whole): what is left is one global select, which the
+    // select's first pass does, and the fallback's pass has nothing to do.
+    if (!part && !s.lg_on) {
+      __syncthreads();
+      if (threadIdx.x < 32) start_global_select(s, c, 1);
     }
     return;
   }
@@ -1651,6 +1679,7 @@ __global__ void __launch_bounds__(1024) k_waterfill(DevState s0) {
   if (threadIdx.x == 0) {
     c->m_fb = 0;
     c->lst_n = 0;
+    c->sel_mode = kSelGroups;
     c->sel_ntie = (int32_t)ntie;
     c->sel_k = (int32_t)(m - above);  // tied items to take, 1..ntie
   }
@@ -1691,24 +1720,25 @@ struct CountSmem {
 // as the warp-aggregated increment needs).  Neighbouring blocks were mostly
 // admitted together and share buckets, so a warp's increments combine.
 // Bound by the scan of N keys (8 B) and groups (2 B).
-__device__ __forceinline__ void select_count(const DevState& s, CountSmem& sm, int single, int fallback, int bid,
+__device__ __forceinline__ void select_count(const DevState& s, CountSmem& sm, int mode, int fallback, int bid,
                                              int nb) {
-  const int nseg = single ? 1 : s.G;
+  // indexed by group, or one entry for all
+  const int nseg = mode == kSelGlobal ? 1 : s.G;
   int any = 0;
   for (int g = threadIdx.x; g < nseg; g += blockDim.x) {
-    const SelSeg z = s.sel[g];
+    const SelSeg z = s.sel[mode == kSelGroups ? g : 0];
+    const bool on = z.active && !(mode == kSelWhole && s.grp_full[g]);
     sm.kmin[g] = z.kmin;
     sm.span[g] = z.kmax - z.kmin;
-    sm.shift[g] = z.active ? (uint8_t)bucket_shift(z.kmin, z.kmax) : (uint8_t)64;
-    any |= z.active;
+    sm.shift[g] = on ? (uint8_t)bucket_shift(z.kmin, z.kmax) : (uint8_t)64;
+    any |= on;
   }
-  if (!__syncthreads_or(any)) return;
   constexpr int kU = 4;
   const int64_t span = (int64_t)nb * blockDim.x;
-  for (int64_t b0 = bid * (int64_t)blockDim.x; b0 < s.N; b0 += span * kU) {
-    uint64_t key[kU];
-    int seg[kU];
-    uint32_t vw[kU];
+  uint64_t key[kU];
+  int seg[kU];
+  uint32_t vw[kU];
+  auto load = [&](int64_t b0) {
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
       const int64_t e = b0 + u * span + threadIdx.x;
@@ -1717,10 +1747,15 @@ __device__ __forceinline__ void select_count(const DevState& s, CountSmem& sm, i
       vw[u] = 0;
       if (e < s.N) {
         key[u] = s.csk[e];
-        if (!single) seg[u] = s.blk_group[e];
+        if (mode != kSelGlobal) seg[u] = s.blk_group[e];
         if (fallback) vw[u] = s.bm_victim[e >> 5];
       }
     }
+  };
+  load(bid * (int64_t)blockDim.x);  // the first batch beside the segments' state
+  if (!__syncthreads_or(any)) return;
+  for (int64_t b0 = bid * (int64_t)blockDim.x; b0 < s.N; b0 += span * kU) {
+    if (b0 != bid * (int64_t)blockDim.x) load(b0);
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
       const int64_t e = b0 + u * span + threadIdx.x;
@@ -1730,7 +1765,7 @@ __device__ __forceinline__ void select_count(const DevState& s, CountSmem& sm, i
         const int sh = sm.shift[seg[u]];
         const uint64_t d = key[u] - sm.kmin[seg[u]];  // keys below the range wrap past any span
         act = sh < 64 && d <= sm.span[seg[u]];
-        idx = (uint32_t)seg[u] * kDigBins + (act ? (uint32_t)(d >> sh) : 0u);
+        idx = (mode == kSelGroups ? (uint32_t)seg[u] * kDigBins : 0u) + (act ? (uint32_t)(d >> sh) : 0u);
       }
       agg_inc(s.dig_bins, idx, act);
     }
@@ -1740,8 +1775,7 @@ __device__ __forceinline__ void select_count(const DevState& s, CountSmem& sm, i
 // One CTA per segment: the bucket holding the segment's rank-th key, as a key
 // range [blo, bhi], and the rank left inside it.  The counts are cleared for
 // the next select.
-__device__ __forceinline__ void select_resolve(const DevState& s, int g) {
-  const SelSeg z = s.sel[g];
+__device__ __forceinline__ void select_resolve(const DevState& s, int g, const SelSeg& z) {
   if (!z.active) return;
   constexpr int kV = 4;  // bins a thread reads at once
   uint4* bins = reinterpret_cast<uint4*>(s.dig_bins + (size_t)g * kDigBins);
@@ -1778,26 +1812,25 @@ struct SplitSmem {
   uint64_t lo[PS_MAX_GROUPS], hi[PS_MAX_GROUPS];  // the bucket; a segment taken whole: [~0, ~0]
   uint8_t act[PS_MAX_GROUPS];
 };
-__device__ __forceinline__ void select_split(const DevState& s, Ctl* c, SplitSmem& sm, int single, int fallback,
+__device__ __forceinline__ void select_split(const DevState& s, Ctl* c, SplitSmem& sm, int mode, int fallback,
                                              int bid, int nb) {
-  const int nseg = single ? 1 : s.G;
-  const bool whole = !single && s.policy == PS_PREFIXSHIELD;
+  const int nseg = mode == kSelGlobal ? 1 : s.G;
+  const bool whole = mode != kSelGlobal && s.policy == PS_PREFIXSHIELD;
   int any = 0;
   for (int g = threadIdx.x; g < nseg; g += blockDim.x) {
-    const SelSeg z = s.sel[g];
+    const SelSeg z = s.sel[mode == kSelGroups ? g : 0];
     const bool w = whole && s.grp_full[g];
     sm.lo[g] = w ? ~0ull : z.blo;
     sm.hi[g] = w ? ~0ull : z.bhi;
     sm.act[g] = w || z.active;
     any |= sm.act[g];
   }
-  if (!__syncthreads_or(any)) return;
   constexpr int kU = 4;
   const int64_t span = (int64_t)nb * blockDim.x;
-  for (int64_t b0 = bid * (int64_t)blockDim.x; b0 < s.N; b0 += span * kU) {
-    uint64_t key[kU];
-    int seg[kU];
-    uint32_t vw[kU];
+  uint64_t key[kU];
+  int seg[kU];
+  uint32_t vw[kU];
+  auto load = [&](int64_t b0) {
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
       const int64_t b = b0 + u * span + threadIdx.x;
@@ -1806,10 +1839,15 @@ __device__ __forceinline__ void select_split(const DevState& s, Ctl* c, SplitSme
       vw[u] = 0;
       if (b < s.N) {
         key[u] = s.csk[b];
-        if (!single) seg[u] = s.blk_group[b];
+        if (mode != kSelGlobal) seg[u] = s.blk_group[b];
         if (fallback) vw[u] = s.bm_victim[b >> 5];
       }
     }
+  };
+  load(bid * (int64_t)blockDim.x);  // the first batch beside the segments' state
+  if (!__syncthreads_or(any)) return;
+  for (int64_t b0 = bid * (int64_t)blockDim.x; b0 < s.N; b0 += span * kU) {
+    if (b0 != bid * (int64_t)blockDim.x) load(b0);
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
       const int64_t b = b0 + u * span + threadIdx.x;
@@ -1822,6 +1860,7 @@ __device__ __forceinline__ void select_split(const DevState& s, Ctl* c, SplitSme
       if (bits && lane_id() == 0) atomicOr(s.bm_victim + ((b - lane_id()) >> 5), bits);
       const unsigned lm = __ballot_sync(kFull, to_list);
       if (!lm) continue;
+      const uint32_t row = mode == kSelGroups ? (uint32_t)seg[u] : 0u;
       unsigned long long base = 0;
       if (lane_id() == 0) base = atomicAdd(reinterpret_cast<unsigned long long*>(&c->lst_n), (unsigned long long)__popc(lm));
       base = __shfl_sync(kFull, base, 0);
@@ -1829,43 +1868,49 @@ __device__ __forceinline__ void select_split(const DevState& s, Ctl* c, SplitSme
         const int64_t slot = (int64_t)base + __popc(lm & ((1u << lane_id()) - 1));
         s.lst_key[slot] = key[u];
         s.lst_blk[slot] = (uint32_t)b;
-        s.lst_seg[slot] = (uint16_t)seg[u];
+        s.lst_seg[slot] = (uint16_t)row;
       }
       // the list's key range per segment (lanes of one segment combined)
-      const unsigned peers = __match_any_sync(kFull, to_list ? (uint32_t)seg[u] : ~0u);
+      const unsigned peers = __match_any_sync(kFull, to_list ? row : ~0u);
       if (to_list) {
         const uint32_t hi = (uint32_t)(key[u] >> 32), lo = (uint32_t)key[u];
         const uint32_t hmin = __reduce_min_sync(peers, hi), hmax = __reduce_max_sync(peers, hi);
         const uint32_t lmin = __reduce_min_sync(peers, hi == hmin ? lo : ~0u);
         const uint32_t lmax = __reduce_max_sync(peers, hi == hmax ? lo : 0u);
         if (lane_id() == __ffs(peers) - 1) {
-          atomicMin(reinterpret_cast<unsigned long long*>(&s.sel[seg[u]].qmin), ((unsigned long long)hmin << 32) | lmin);
-          atomicMax(reinterpret_cast<unsigned long long*>(&s.sel[seg[u]].qmax), ((unsigned long long)hmax << 32) | lmax);
+          atomicMin(reinterpret_cast<unsigned long long*>(&s.sel[row].qmin), ((unsigned long long)hmin << 32) | lmin);
+          atomicMax(reinterpret_cast<unsigned long long*>(&s.sel[row].qmax), ((unsigned long long)hmax << 32) | lmax);
         }
       }
     }
   }
 }
 
-__global__ void __launch_bounds__(256) k_sel_count(DevState s, int single, int fallback) {
+// What a pass of the select has to do: its mode, or -1 for nothing.
+__device__ __forceinline__ int select_mode(const Ctl* c, int fallback) {
+  const int32_t st = c->status, mode = c->sel_mode;  // one round trip
+  const int64_t m = c->mvict, mf = c->m_fb;
+  if (st != PS_OK || m == 0) return -1;
+  if (!fallback) return mode;
+  return mode == kSelGroups && mf > 0 ? kSelGlobal : -1;
+}
+__global__ void __launch_bounds__(256) k_sel_count(DevState s, int fallback) {
   s = with_args(s);
   __shared__ CountSmem sm;
-  Ctl* c = s.ctl;
-  if (c->status != PS_OK || c->mvict == 0) return;
-  select_count(s, sm, single, fallback, blockIdx.x, gridDim.x);
+  const int mode = select_mode(s.ctl, fallback);
+  if (mode >= 0) select_count(s, sm, mode, fallback, blockIdx.x, gridDim.x);
 }
-__global__ void __launch_bounds__(1024) k_sel_resolve(DevState s) {
+__global__ void __launch_bounds__(1024) k_sel_resolve(DevState s, int fallback) {
   s = with_args(s);
-  const Ctl* c = s.ctl;
-  if (c->status != PS_OK || c->mvict == 0) return;
-  select_resolve(s, blockIdx.x);
+  const SelSeg z = s.sel[blockIdx.x];  // in the mode's round trip
+  const int mode = select_mode(s.ctl, fallback);
+  if (mode == kSelGroups || (mode > 0 && blockIdx.x == 0)) select_resolve(s, blockIdx.x, z);
 }
-__global__ void __launch_bounds__(256) k_sel_split(DevState s, int single, int fallback) {
+__global__ void __launch_bounds__(256) k_sel_split(DevState s, int fallback) {
   s = with_args(s);
   __shared__ SplitSmem sm;
-  Ctl* c = s.ctl;
-  if (c->status != PS_OK || c->mvict == 0) return;
-  select_split(s, c, sm, single, fallback, blockIdx.x, gridDim.x);
+  const int mode = select_mode(s.ctl, fallback);
+  if (mode >= 0) select_split(s, s.ctl, sm, mode, fallback, blockIdx.x, gridDim.x);
 }
 
 // The digits of the list's finish: bytes, from the highest one where the
@@ -1917,7 +1962,7 @@ constexpr int kFinWords = (int)(kFinList / 4);  // bitmap words in the list's pl
 constexpr int kFinSegWords = 1024;              // of one segment (one warp searches them)
 constexpr size_t kFinSmem = kFinList + (size_t)PS_MAX_GROUPS * (sizeof(FinSeg) + 8 + 4 + 2);
 
-__global__ void __launch_bounds__(1024) k_list_finish(DevState s, int single) {
+__global__ void __launch_bounds__(1024) k_list_finish(DevState s, int fallback) {
   s = with_args(s);
   extern __shared__ __align__(16) unsigned char fin_smem[];
   FinSeg* sl = reinterpret_cast<FinSeg*>(fin_smem);
@@ -1931,13 +1976,18 @@ __global__ void __launch_bounds__(1024) k_list_finish(DevState s, int single) {
   __shared__ int16_t seg_of_row[PS_MAX_GROUPS];
   __shared__ int s_nrows;
   Ctl* c = s.ctl;
-  if (c->status != PS_OK || c->mvict == 0) return;
-  // the debt phase's launch also starts the fallback's select (the groups'
+  const int64_t n = c->lst_n;  // in the mode's round trip
+  const int mode = select_mode(c, fallback);
+  if (mode < 0) return;
+  const bool single = mode != kSelGroups;
+  // a pass over the groups also starts the fallback's select (the groups'
   // final take counts are known here)
   const bool start_fb = !single && s.policy == PS_PREFIXSHIELD;
-  if (single && !s.sel[0].active) return;
   const int nseg = single ? 1 : s.G;
-  const int64_t n = c->lst_n;
+  if (n == 0) {  // no segment selects
+    if (start_fb && threadIdx.x < 32) start_global_select(s, c, 1);
+    return;
+  }
   const bool small = n <= kFinCap;
   const int warp = threadIdx.x >> 5, lane = lane_id();
   // each thread's first member, loaded beside the segments' state
@@ -2550,24 +2600,24 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
   // step (a kernel of a phase with nothing to select returns at once): a
   // conditional graph node measured about 10 us a step even when its body
   // was skipped, more than the phase's early-returning launches.
-  auto select = [&](int single, int fallback) {
-    PS_LAUNCH(launch_k(k_sel_count, cgrid, 256, 0, st, s, single, fallback));
-    PS_LAUNCH(launch_k(k_sel_resolve, single ? 1 : s.G, 1024, 0, st, s));
-    PS_LAUNCH(launch_k(k_sel_split, cgrid, 256, 0, st, s, single, fallback));
-    PS_LAUNCH(launch_k(k_list_finish, 1, 1024, kFinSmem, st, s, single));
+  auto select = [&](int fallback) {
+    PS_LAUNCH(launch_k(k_sel_count, cgrid, 256, 0, st, s, fallback));
+    PS_LAUNCH(launch_k(k_sel_resolve, fallback || s.policy == PS_LRU ? 1 : s.G, 1024, 0, st, s, fallback));
+    PS_LAUNCH(launch_k(k_sel_split, cgrid, 256, 0, st, s, fallback));
+    PS_LAUNCH(launch_k(k_list_finish, 1, 1024, kFinSmem, st, s, fallback));
   };
   if (s.lg_on) {
     // selected above
   } else if (s.policy == PS_PREFIXSHIELD) {
     PS_LAUNCH(k_waterfill<<<1, 1024, 0, st>>>(s));  // after the join: plain
-    select(0, 0);
-    select(1, 1);  // the global fallback, started by the debt phase's finish
+    select(0);
+    select(1);  // the global fallback, started by the debt phase's finish
   } else if (s.policy == PS_STATICQUOTA) {
     PS_LAUNCH(k_quota_sel<<<1, 1024, 0, st>>>(s));  // after the join: plain
-    select(0, 0);
+    select(0);
   } else if (s.policy == PS_LRU) {
-    PS_LAUNCH(k_sel_single<<<1, 32, 0, st>>>(s, 0));  // after the join: plain
-    select(1, 0);
+    PS_LAUNCH(k_sel_single<<<1, 32, 0, st>>>(s));  // after the join: plain
+    select(0);
   } else if (launch_s3_select(s, st, fork2, &launches) != PS_OK) {
     return PS_ERR_CUDA;
   }
