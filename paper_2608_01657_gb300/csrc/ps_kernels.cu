@@ -1520,168 +1520,217 @@ __global__ void __launch_bounds__(1024) k_quota_sel(DevState s) {
 // each) the ones with the smallest candidate keys are taken (resolved after
 // the radix select finds those keys).  What the debt phase cannot cover goes
 // to the global fallback in (class, stamp) order.
-__global__ void __launch_bounds__(1024) k_waterfill(DevState s0) {
+//
+// A thread holds a group (PS_MAX_GROUPS threads) with everything loaded in one
+// round trip; sums over the groups take one barrier each (per-warp partials,
+// every warp adding them up for itself).  tau is bracketed first: a group with
+// m items of its own puts tau at or above its m-th, and some group gives at
+// least ceil(m / groups) of the m items, so tau is at most the largest such
+// item.  The search then narrows the bracket to one decrement, within which
+// each group has at most one item: tau is one of those.  (One indebted group
+// needs no search at all; the search over all values took four to six rounds.)
+__global__ void __launch_bounds__(PS_MAX_GROUPS) k_waterfill(DevState s0) {
   // contract arrays are read from the parameter block (see k_grant)
   const DevState s = with_args(s0);
   Ctl* c = s.ctl;
-  __shared__ int64_t sP[PS_MAX_GROUPS], sD[PS_MAX_GROUPS], sQ[PS_MAX_GROUPS];
-  __shared__ uint64_t sRcp[PS_MAX_GROUPS];  // floor((2^64 - 1) / d) for the division below (d: some contract's)
-  __shared__ int64_t s_pmax;
-  const int G = s.G;
+  __shared__ int64_t hP[PS_MAX_GROUPS], hD[PS_MAX_GROUPS], hQ[PS_MAX_GROUPS];  // the groups that can give victims
+  __shared__ uint64_t hRcp[PS_MAX_GROUPS];
+  __shared__ int64_t w_a[32], w_b[32], w_c[32], w_d[32];  // per-warp partials
+  __shared__ int32_t w_n[32], w_f[32];
+  __shared__ int64_t s_tau;
+  const int g = (int)threadIdx.x, warp = g >> 5, lane = lane_id();
+  const bool mine = g < s.G;
   const int64_t eps = s.eps;
   const bool seg = !(s.flags & PS_FLAG_NO_SEGMENTATION);
   const int32_t st = c->status;
   const int64_t mv = c->mvict;
-  for (int g = threadIdx.x; g < G; g += blockDim.x) {  // loaded beside the victim count
-    sP[g] = s.grp_P[g];
-    sD[g] = s.grp_delta[g];
-    sQ[g] = s.grp_qsize[g];
-  }
+  const int64_t P = mine ? s.grp_P[g] : 0, d = mine ? s.grp_delta[g] : 0, q = mine ? s.grp_qsize[g] : 0;
+  ClsRange r[kClasses];
+#pragma unroll
+  for (int k = 0; k < kClasses; ++k) r[k] = mine ? s.cls[g * kClasses + k] : ClsRange{0, ~0u, 0, ~0u, 0};
   const int64_t m = st == PS_OK ? mv : 0;
   if (m == 0) {
-    for (int g = threadIdx.x; g < G; g += blockDim.x) { s.sel[g].active = 0; s.grp_x[g] = 0; s.grp_full[g] = 0; }
-    if (threadIdx.x == 0) c->m_fb = 0;
+    if (mine) { s.sel[g].active = 0; s.grp_x[g] = 0; s.grp_full[g] = 0; }
+    if (g == 0) c->m_fb = 0;
     return;
   }
-  for (int g = threadIdx.x; g < G; g += blockDim.x) {
-    uint64_t rcp = 0;
-    for (int cc = 0; cc < s.C; ++cc)
-      if (s0.delta[cc] == sD[g]) rcp = s0.delta_rcp[cc];
-    sRcp[g] = rcp;
-  }
-  if (threadIdx.x == 0) s_pmax = 0;
-  __syncthreads();
+  uint64_t rcp = 0;  // floor((2^64 - 1) / d): d is some contract's decrement
+  for (int cc = 0; cc < s.C; ++cc)
+    if (s0.delta[cc] == d) rcp = s0.delta_rcp[cc];
   // floor(x / d) for x >= 0 from the reciprocal: the estimate is at most two
   // below the quotient, and the correction makes it exact
-  auto div_d = [&](int g, uint64_t x) -> uint64_t {
-    const uint64_t d = (uint64_t)sD[g];
-    if (d == 1) return x;
-    uint64_t q = __umul64hi(x, sRcp[g]);
-    while (x - q * d >= d) ++q;
-    return q;
+  auto div_d = [](uint64_t x, uint64_t dd, uint64_t rr) -> uint64_t {
+    if (dd == 1) return x;
+    uint64_t z = __umul64hi(x, rr);
+    while (x - z * dd >= dd) ++z;
+    return z;
   };
-  // items of group g with value > t: min(q, floor((P - t - 1) / d) + 1) if P > t
-  auto items_gt = [&](int g, int64_t t) -> int64_t {
-    const int64_t P = sP[g], d = sD[g];
-    return (P > t && d > 0) ? tmin<int64_t>(sQ[g], (int64_t)div_d(g, (uint64_t)(P - t - 1)) + 1) : 0;
+  // items of a group with value > t: min(q, floor((P - t - 1) / d) + 1) if P > t
+  auto items_gt = [&](int64_t pp, int64_t dd, int64_t qq, uint64_t rr, int64_t t) -> int64_t {
+    return (pp > t && dd > 0) ? tmin<int64_t>(qq, (int64_t)div_d((uint64_t)(pp - t - 1), (uint64_t)dd, rr) + 1) : 0;
   };
-  int64_t e = 0, pm = 0;
-  for (int g = threadIdx.x; g < G; g += blockDim.x) { e += items_gt(g, eps); pm = tmax(pm, sP[g]); }
-  const int64_t E = block_sum(e);
-  if (pm) atomicMax(reinterpret_cast<unsigned long long*>(&s_pmax), (unsigned long long)pm);
+  // a segment started over the group's rank smallest candidates
+  auto start = [&](int64_t rank, int incl) {
+    SelSeg z{};
+    z.rank = rank;
+    z.active = 1;
+    z.incl = incl;
+    z.qmin = ~0ull;
+    int64_t cnt[kClasses];
+    uint64_t lo[kClasses], hi[kClasses];
+#pragma unroll
+    for (int k = 0; k < kClasses; ++k) {
+      cnt[k] = r[k].cnt;
+      cls_stamp_range(r[k], &lo[k], &hi[k]);
+    }
+    sel_start_cls(z, cnt, lo, hi, seg);
+    s.sel[g] = z;
+  };
+  const int64_t x = items_gt(P, d, q, rcp, eps);  // the group's items above epsilon
+  const bool holds = x > 0, full = holds && x == q;
+  const unsigned hb = __ballot_sync(kFull, holds);
+  const unsigned fl = (__ballot_sync(kFull, full) ? 1u : 0u) | (__ballot_sync(kFull, holds && !full) ? 2u : 0u);
+  {
+    const int64_t e = warp_sum(x);
+    int64_t dm = holds ? d : INT64_MAX;
+    for (int o = 16; o > 0; o >>= 1) dm = tmin(dm, (int64_t)__shfl_xor_sync(kFull, dm, o));
+    if (lane == 0) {
+      w_a[warp] = e;
+      w_d[warp] = dm;
+      w_n[warp] = __popc(hb);
+      w_f[warp] = (int32_t)fl;
+    }
+  }
   __syncthreads();
+  const int64_t E = warp_sum(w_a[lane]);
+  const int32_t nw = w_n[lane], nin = warp_incl_scan(nw);
+  const int ng = __shfl_sync(kFull, nin, 31);
+  const int hbase = __shfl_sync(kFull, nin - nw, warp);
+  int64_t dmin = w_d[lane];
+  for (int o = 16; o > 0; o >>= 1) dmin = tmin(dmin, (int64_t)__shfl_xor_sync(kFull, dmin, o));
+  const uint32_t flags = __reduce_or_sync(kFull, (uint32_t)w_f[lane]);
   if (E <= m) {
     // a group that gives all its candidates needs no select: the split takes
     // them whole
-    int part = 0, whole = 0;
-    for (int g = threadIdx.x; g < G; g += blockDim.x) {
-      const int64_t x = items_gt(g, eps);
-      const bool full = x > 0 && x == sQ[g];
+    if (mine) {
       s.grp_x[g] = x;
       s.grp_full[g] = full ? 1 : 0;
-      whole |= full;
-      if (x == 0 || full) continue;  // k_grant left the segment inactive
-      part = 1;
-      SelSeg z = s.sel[g];
-      z.rank = x;
-      z.active = 1;
-      z.incl = 1;
-      sel_start_group(s, g, z, seg);
-      s.sel[g] = z;
     }
-    part = __syncthreads_or(part);
-    whole = __syncthreads_or(whole);
-    if (threadIdx.x == 0) {
+    if (holds && !full) start(x, 1);
+    const bool part = flags & 2u;
+    if (g == 0) {
       c->m_fb = m - E; c->sel_ntie = 0; c->sel_k = 0; c->lst_n = 0;
-      c->sel_mode = part ? kSelGroups : (whole ? kSelWhole : kSelGlobal);
+      c->sel_mode = part ? kSelGroups : ((flags & 1u) ? kSelWhole : kSelGlobal);
     }
     // No group gives only some of its candidates (nothing is owed, or the
     // indebted groups go whole): what is left is one global select, which the
     // select's first pass does, and the fallback's pass has nothing to do.
     if (!part && !s.lg_on) {
       __syncthreads();
-      if (threadIdx.x < 32) start_global_select(s, c, 1);
+      if (warp == 0) start_global_select(s, c, 1);
     }
     return;
   }
-  // tau = max{t in [eps+1, pmax] : items_gt(t - 1) summed >= m}.  Only the
-  // groups that can hold an item above eps count (d > 0, q > 0, P > eps);
-  // each round tests T thresholds spread over the interval, L lanes (a power
-  // of two covering them, at most 32) splitting the groups of one: each
+  // tau = max{t > eps : the items at or above t number at least m}
+  if (holds) {
+    const int k = hbase + __popc(hb & ((1u << lane) - 1u));
+    hP[k] = P;
+    hD[k] = d;
+    hQ[k] = q;
+    hRcp[k] = rcp;
+  }
+  {
+    const int64_t share = (m + ng - 1) / ng;
+    int64_t lo = holds && x >= m ? P - (m - 1) * d : eps + 1;
+    int64_t hi = holds && x >= share ? P - (share - 1) * d : eps + 1;
+    for (int o = 16; o > 0; o >>= 1) {
+      lo = tmax(lo, (int64_t)__shfl_xor_sync(kFull, lo, o));
+      hi = tmax(hi, (int64_t)__shfl_xor_sync(kFull, hi, o));
+    }
+    if (lane == 0) {
+      w_b[warp] = lo;
+      w_c[warp] = hi;
+    }
+    if (g == 0) s_tau = eps;
+  }
+  __syncthreads();
+  int64_t lo = w_b[lane], hi = w_c[lane];
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = tmax(lo, (int64_t)__shfl_xor_sync(kFull, lo, o));
+    hi = tmax(hi, (int64_t)__shfl_xor_sync(kFull, hi, o));
+  }
+  // Each round tests T thresholds spread over the bracket, L lanes (a power of
+  // two covering the groups, at most 32) splitting the groups of one: each
   // evaluation is a chain of dependent 64-bit steps, so one per thread and
   // more rounds beat several per thread and fewer rounds.
-  __shared__ int16_t s_gid[PS_MAX_GROUPS];
-  __shared__ int s_ng;
-  {
-    int k = 0;
-    for (int base = 0; base < G; base += blockDim.x) {
-      const int g = base + threadIdx.x;
-      const bool holds = g < G && sD[g] > 0 && sQ[g] > 0 && sP[g] > eps;
-      int tot;
-      const int ex = block_excl_scan((int)holds, &tot);
-      if (holds) s_gid[k + ex] = (int16_t)g;
-      k += tot;
-    }
-    if (threadIdx.x == 0) s_ng = k;
-    __syncthreads();
-  }
-  const int ng = s_ng;
-  int64_t lo = eps + 1, hi = s_pmax;
-  {
-    int L = 1, logT = 10;  // blockDim.x == 1024 == T * L
-    while (L < ng && L < 32) { L <<= 1; --logT; }
-    const int T = 1 << logT;
-    const int jt = threadIdx.x / L, gl = threadIdx.x % L;
-    while (lo < hi) {
-      const int64_t span = hi - lo;  // >= 1
-      const int64_t stride = tmax<int64_t>(1, (span + T - 1) >> logT);
-      auto thr = [&](int jj) -> int64_t { return jj == T - 1 ? hi : tmin<int64_t>(hi, lo + 1 + stride * jj); };
-      const int64_t t = thr(jt);
-      int64_t cnt = 0;
-      for (int k = gl; k < ng; k += L) cnt += items_gt(s_gid[k], t - 1);
-      for (int o = L / 2; o > 0; o >>= 1) cnt += __shfl_xor_sync(kFull, cnt, o);
-      // J = the largest threshold still holding m items: counts fall as the
-      // threshold rises, so it is the number of such thresholds less one, and
-      // the round's one barrier counts them (a shared maximum taken by up to
-      // 1024 threads made a round 1.1 us, six of them a search)
-      const int J = __syncthreads_count(gl == 0 && cnt >= m) - 1;
-      if (J < 0) {
-        hi = lo;
-      } else {
-        // both ends from this round's lo (thr reads lo and hi by reference)
-        const int64_t nlo = thr(J), nhi = J + 1 < T ? thr(J + 1) - 1 : hi;
-        lo = nlo;
-        hi = nhi < nlo ? nlo : nhi;
-      }
+  int logL = 0;
+  while ((1 << logL) < ng && logL < 5) ++logL;
+  const int L = 1 << logL, logT = 10 - logL, T = 1 << logT;  // blockDim.x == 1024 == T * L
+  const int jt = g >> logL, gl = g & (L - 1);
+  auto at_least = [&](int64_t t) -> int64_t {  // items at or above t, by the L lanes of a threshold
+    int64_t cnt = 0;
+    for (int k = gl; k < ng; k += L) cnt += items_gt(hP[k], hD[k], hQ[k], hRcp[k], t - 1);
+    for (int o = L / 2; o > 0; o >>= 1) cnt += __shfl_xor_sync(kFull, cnt, o);
+    return cnt;
+  };
+  while (hi - lo >= dmin) {
+    const int64_t span = hi - lo;
+    const int64_t stride = tmax<int64_t>(1, (span + T - 1) >> logT);
+    const int64_t l0 = lo, h0 = hi;
+    auto thr = [&](int jj) -> int64_t { return jj == T - 1 ? h0 : tmin<int64_t>(h0, l0 + 1 + stride * jj); };
+    const int64_t cnt = at_least(thr(jt));
+    // J = the largest threshold still holding m items: counts fall as the
+    // threshold rises, so it is the number of such thresholds less one, and
+    // the round's one barrier counts them
+    const int J = __syncthreads_count(gl == 0 && cnt >= m) - 1;
+    if (J < 0) {
+      hi = lo;
+    } else {
+      lo = thr(J);
+      hi = tmax(lo, J + 1 < T ? thr(J + 1) - 1 : h0);
     }
   }
-  const int64_t tau = lo;
-  int64_t above = 0, ntie = 0;
-  for (int g = threadIdx.x; g < G; g += blockDim.x) {
-    const int64_t P = sP[g], d = sD[g], q = sQ[g];
-    const int64_t xa = items_gt(g, tau);
-    const uint64_t qt = (d > 0 && P >= tau) ? div_d(g, (uint64_t)(P - tau)) : 0;
-    const bool tied = d > 0 && P >= tau && qt * (uint64_t)d == (uint64_t)(P - tau) && (int64_t)qt < q;
-    above += xa;
-    ntie += tied;
+  // each group's one item inside the bracket, if any; tau is the largest of
+  // these with m items at or above it
+  for (int k0 = 0; k0 < ng; k0 += T) {
+    const int k = k0 + jt;
+    int64_t v = eps;
+    if (k < ng) {
+      const int64_t dk = hD[k], pk = hP[k];
+      const int64_t j = pk > hi ? (int64_t)div_d((uint64_t)(pk - hi + dk - 1), (uint64_t)dk, hRcp[k]) : 0;
+      if (j < hQ[k] && pk - j * dk >= lo) v = pk - j * dk;
+    }
+    const int64_t cnt = at_least(tmax(v, eps + 1));
+    if (gl == 0 && v > eps && cnt >= m)
+      atomicMax(reinterpret_cast<long long*>(&s_tau), (long long)v);
+  }
+  __syncthreads();
+  const int64_t tau = s_tau;
+  const int64_t xa = mine ? items_gt(P, d, q, rcp, tau) : 0;
+  const uint64_t qt = (mine && d > 0 && P >= tau) ? div_d((uint64_t)(P - tau), (uint64_t)d, rcp) : 0;
+  const bool tied = mine && d > 0 && P >= tau && qt * (uint64_t)d == (uint64_t)(P - tau) && (int64_t)qt < q;
+  if (mine) {
     s.grp_x[g] = xa + (tied ? 1 : 0);
     s.grp_full[g] = 0;
-    if (xa == 0 && !tied) continue;  // k_grant left the segment inactive
-    SelSeg z = s.sel[g];
-    z.rank = xa + (tied ? 1 : 0);
-    z.active = 1;
-    z.incl = tied ? 2 : 1;  // 2: the tie item is taken only if the tie rule chooses it
-    sel_start_group(s, g, z, seg);
-    s.sel[g] = z;
   }
-  above = block_sum(above);
-  ntie = block_sum(ntie);
-  if (threadIdx.x == 0) {
-    c->m_fb = 0;
-    c->lst_n = 0;
-    c->sel_mode = kSelGroups;
-    c->sel_ntie = (int32_t)ntie;
-    c->sel_k = (int32_t)(m - above);  // tied items to take, 1..ntie
+  if (xa > 0 || tied) start(xa + (tied ? 1 : 0), tied ? 2 : 1);  // 2: taken only if the tie rule chooses it
+  const int64_t above = warp_sum(xa);
+  const int nt = __popc(__ballot_sync(kFull, tied));
+  if (lane == 0) {
+    w_a[warp] = above;
+    w_n[warp] = nt;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const int64_t a = warp_sum(w_a[lane]);
+    const int32_t n = warp_sum(w_n[lane]);
+    if (lane == 0) {
+      c->m_fb = 0;
+      c->lst_n = 0;
+      c->sel_mode = kSelGroups;
+      c->sel_ntie = n;
+      c->sel_k = (int32_t)(m - a);  // tied items to take, 1..ntie
+    }
   }
 }
 
