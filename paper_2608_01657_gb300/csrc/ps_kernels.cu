@@ -757,8 +757,8 @@ __global__ void __launch_bounds__(256, kHashCtasPerSm) k_hash_lookup(DevState s,
   __shared__ uint64_t kc[2 * (kSegBlocks + 1)];  // Kc^j, then Kc^(32 t)
   Ctl* c = s.ctl;
   const int64_t nsegs = c->nsegs;  // none in a failed call
-  if (threadIdx.x < BS + 2) sk[threadIdx.x] = s.key_words[threadIdx.x];
-  if (threadIdx.x < 2 * (kSegBlocks + 1)) kc[threadIdx.x] = s.kc_pow[threadIdx.x];
+  for (int k = threadIdx.x; k < BS + 2; k += blockDim.x) sk[k] = s.key_words[k];
+  for (int k = threadIdx.x; k < 2 * (kSegBlocks + 1); k += blockDim.x) kc[k] = s.kc_pow[k];
   __syncthreads();
   const int lane = lane_id();
   for (;;) {
@@ -2290,6 +2290,7 @@ __device__ __forceinline__ void write_ids(const DevState& s, const ListSmem& sm,
   const int lane = lane_id();
   const unsigned lt = (1u << lane) - 1u;
   for (int w = (int)(threadIdx.x >> 5); w < nw; w += (int)(blockDim.x >> 5)) {
+    if (!(sm.word[0][w] | sm.word[2][w])) continue;  // victims are allocated again
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const uint32_t bits = sm.word[k][w];
@@ -2357,7 +2358,7 @@ __global__ void __launch_bounds__(kBmThreads, 3) k_bm_write(DevState s) {
     c->n_evicted = vb + field3(tot1, 1);
   }
   __syncthreads();
-  write_ids(s, sm, w0, kBmChunk);
+  write_ids(s, sm, w0, (int)tmin<int64_t>(kBmChunk, s.nwords - w0));
 }
 
 // Stage 6: place granted claims, a thread per claim of the step (k_instep
@@ -2520,9 +2521,15 @@ static void launch_hash_lookup_t(const DevState& s, cudaStream_t st, int probe) 
   // persistent: the CTAs that fit at once (more only queue behind them)
   int dev = 0, nsm = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t want = (s.max_segments + 7) / 8;
-  const int grid = (int)(want < (int64_t)nsm * kHashCtasPerSm ? want : (int64_t)nsm * kHashCtasPerSm);
-  k_hash_lookup<BS><<<grid > 0 ? grid : 1, 256, 0, st>>>(s, probe);
+  // 8 warps a CTA, or fewer where all chunks have a warp then and more SMs
+  // share them (a chunk's probes keep an SM's L1 busy: 8 warps on each of 37
+  // SMs took longer than 2 on each of 148)
+  int warps = 8;
+  while (warps > 1 && s.max_segments <= (int64_t)nsm * (warps / 2)) warps >>= 1;
+  const int64_t want = (s.max_segments + warps - 1) / warps;
+  const int64_t most = (int64_t)nsm * kHashCtasPerSm * 8 / warps;
+  const int grid = (int)(want < most ? want : most);
+  k_hash_lookup<BS><<<grid > 0 ? grid : 1, 32 * warps, 0, st>>>(s, probe);
 }
 static int32_t launch_hash_lookup(const DevState& s, cudaStream_t st, int probe) {
   switch (s.bs) {
