@@ -288,6 +288,7 @@ size_t carve(const Dims& d, char* base, DevState* s, ps_handle* h) {
   t.s3_rbase = cv.take<uint32_t>((size_t)d.s3_nrch);
   t.s3_plan = cv.take<S3Plan>(1);
   t.s3_hit = cv.take<uint8_t>(B);
+  t.s3_slot = cv.take<uint32_t>(B);
   t.s3_ick = cv.take<uint32_t>(B / kS3Chunk + 1);
   if (d.lg) {
     const size_t L = (size_t)d.lg_L;

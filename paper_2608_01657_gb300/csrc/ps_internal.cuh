@@ -347,6 +347,7 @@ struct DevState {
   uint32_t* s3_rbase;      // [s3_nrch] their exclusive prefix
   S3Plan* s3_plan;
   uint8_t* s3_hit;         // [max_blocks] inserted block found in the ghost
+  uint32_t* s3_slot;       // [max_blocks] ghost map slot of each claim's key (or kNone)
   uint32_t* s3_ick;        // [max_blocks / kS3Chunk + 1] ghost hits per chunk of inserts
   // indexed queues (allocated only with PS_FLAG_INDEXED_QUEUES)
   int32_t lg_on;           // victims come from the queues instead of a candidate scan
@@ -471,15 +472,20 @@ int32_t launch_queue_cand(const DevState& s, cudaStream_t st, int* launches);
 int32_t launch_queue_select(const DevState& s, cudaStream_t st, int phase, bool plain_first, int* launches);
 int32_t launch_queue_append(const DevState& s, cudaStream_t st, const CaptureCtx* cap, int* launches);
 // S3-FIFO (ps_s3fifo.cu)
-// The select: per-chunk counts, the closed-form plan, the sequential kernel
-// (used when the plan does not apply), the plan's application.
-// plain_first: the first kernel follows a fork of the step graph (a plain
-// launch: a programmatic edge is kept for a kernel's only dependent).
-int32_t launch_s3_select(const DevState& s, cudaStream_t st, bool plain_first, int* launches);
+// The ghost's entries for the step's claims (before anything leaves the ghost).
+int32_t launch_s3_probe(const DevState& s, cudaStream_t st, int* launches);
+// The select: per-chunk counts; then the closed-form plan (the one-at-a-time
+// loop where it does not apply) and its application, which trim the ghost and
+// so follow the lookups.
+// plain: the (first) kernel follows a fork or a join of the step graph (a plain
+// launch: a programmatic edge is kept for a kernel's only dependent and takes
+// one predecessor).
+int32_t launch_s3_count(const DevState& s, cudaStream_t st, bool plain, int* launches);
+int32_t launch_s3_select(const DevState& s, cudaStream_t st, bool plain, int* launches);
 // The step's ghost pushes: they read the victims' records, so before the
 // insertion, but nothing of the id lists.
 int32_t launch_s3_push(const DevState& s, cudaStream_t st, bool plain, int* launches);
-// After the insertions: ghost lookups of the new blocks, their array places.
+// After the insertions: the new blocks' ghost entries, their array places.
 int32_t launch_s3_insert(const DevState& s, cudaStream_t st, int* launches);
 // A step's outputs (device) written into page-locked host buffers, the id
 // lists by their device-side counts (ps_step_host_async).

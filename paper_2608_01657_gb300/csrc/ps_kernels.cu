@@ -2630,6 +2630,11 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
   }
   if (fork2 && early) PS_LAUNCH((k_instep<<<pgrid, kThreads, 0, ms>>>(s)));  // after the join: plain
   else PS_LAUNCH(launch_k(k_instep, pgrid, kThreads, 0, ms, s));
+  if (s.policy == PS_S3FIFO) {
+    if (launch_s3_probe(s, ms, &launches) != PS_OK) return PS_ERR_CUDA;
+    // the plan trims the ghost: it waits for the lookups
+    if (fork2 && cudaEventRecord(cap->fork, ms) != cudaSuccess) return PS_ERR_CUDA;
+  }
   mark(4);
   PS_LAUNCH(launch_k(k_meter, s.G, 512, 0, ms, s));
   mark(5);
@@ -2674,8 +2679,10 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
   } else if (s.policy == PS_LRU) {
     PS_LAUNCH(k_sel_single<<<1, 32, 0, st>>>(s));  // after the join: plain
     select(0);
-  } else if (launch_s3_select(s, st, fork2, &launches) != PS_OK) {
-    return PS_ERR_CUDA;
+  } else {
+    if (launch_s3_count(s, st, fork2, &launches) != PS_OK) return PS_ERR_CUDA;
+    if (fork2 && cudaStreamWaitEvent(st, cap->fork, 0) != cudaSuccess) return PS_ERR_CUDA;
+    if (launch_s3_select(s, st, fork2, &launches) != PS_OK) return PS_ERR_CUDA;
   }
   // The ghost pushes run beside the id lists (the candidate scan's branch,
   // which S3-FIFO has no use for), joined before the insertion.

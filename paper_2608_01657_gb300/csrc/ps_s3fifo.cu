@@ -480,7 +480,34 @@ __device__ __forceinline__ void s3_plan(const DevState& s, Ctl* c) {
   const int64_t nch = chM + chS;
   const int64_t run = (nch + kPT - 1) / kPT;
   const int64_t r0 = tmin<int64_t>((int64_t)threadIdx.x * run, nch), r1 = tmin<int64_t>(r0 + run, nch);
-  auto rec = [&](int64_t i) -> const S3Chunk& { return i < chM ? ckM[i] : ckS[i - chM]; };
+  // a chunk record in five 16-byte loads; its bins are used with static
+  // indexes only (a loop from a run-time bin reads them one by one)
+  struct Rec {
+    uint32_t nlive, nu, nev, h[kS3Bins];
+  };
+  auto rec = [&](int64_t i) -> Rec {
+    const uint4* p = reinterpret_cast<const uint4*>(i < chM ? ckM + i : ckS + (i - chM));
+    const uint4 v = p[0];
+    Rec k;
+    k.nlive = v.x;
+    k.nu = v.y;
+    k.nev = v.z;
+#pragma unroll
+    for (int q = 0; q < kS3Bins / 4; ++q) {
+      const uint4 w = p[1 + q];
+      k.h[4 * q] = w.x;
+      k.h[4 * q + 1] = w.y;
+      k.h[4 * q + 2] = w.z;
+      k.h[4 * q + 3] = w.w;
+    }
+    return k;
+  };
+  auto bins_from = [&](const uint32_t (&b)[kS3Bins], int lo) -> uint32_t {  // entries with f >= lo
+    uint32_t n = 0;
+#pragma unroll
+    for (int q = 0; q < kS3Bins; ++q) n += q >= lo ? b[q] : 0u;
+    return n;
+  };
   // per bin, the warp's sum added once (a lane each would queue up on 16 addresses)
   auto add_bins = [&](uint32_t* bins, const uint32_t (&h)[kS3Bins]) {
 #pragma unroll
@@ -495,11 +522,11 @@ __device__ __forceinline__ void s3_plan(const DevState& s, Ctl* c) {
   for (int r = 0; r < kS3Bins; ++r) h[r] = 0;
   uint64_t a0 = 0, a1 = 0;  // unpinned of main (high) and small (low); small's victim-grade (high) and live (low)
   for (int64_t i = r0; i < r1; ++i) {
-    const S3Chunk& k = rec(i);
+    const Rec k = rec(i);
     if (i < chM) {
       a0 += (uint64_t)k.nu << 32;
 #pragma unroll
-      for (int r = 0; r < kS3Bins; ++r) h[r] += k.hist[r];
+      for (int r = 0; r < kS3Bins; ++r) h[r] += k.h[r];
     } else {
       a0 += k.nu;
       a1 += (uint64_t)k.nev << 32 | k.nlive;
@@ -512,7 +539,7 @@ __device__ __forceinline__ void s3_plan(const DevState& s, Ctl* c) {
   {
     uint32_t um = (uint32_t)(e0 >> 32), us = (uint32_t)e0, ev = (uint32_t)(e1 >> 32);
     for (int64_t i = r0; i < r1; ++i) {
-      const S3Chunk& k = rec(i);
+      const Rec k = rec(i);
       if (i < chM) {
         bM[i].u = um;
         um += k.nu;
@@ -536,7 +563,7 @@ __device__ __forceinline__ void s3_plan(const DevState& s, Ctl* c) {
       // the chunk holding unpinned member number Dp, then the victims among the first Dp
       uint32_t us = (uint32_t)e0, ev = (uint32_t)(e1 >> 32);
       for (int64_t i = tmax(r0, chM); i < r1; ++i) {
-        const S3Chunk& k = rec(i);
+        const Rec k = rec(i);
         if ((int64_t)us < Dp && Dp <= (int64_t)(us + k.nu)) { sv[0] = i - chM; sv[1] = -1; sv[2] = us; sv[3] = ev; }
         us += k.nu;
         ev += k.nev;
@@ -562,7 +589,7 @@ __device__ __forceinline__ void s3_plan(const DevState& s, Ctl* c) {
   if (nA > 0 && nA <= T) {
     uint32_t ev = (uint32_t)(e1 >> 32);
     for (int64_t i = tmax(r0, chM); i < r1; ++i) {
-      const S3Chunk& k = rec(i);
+      const Rec k = rec(i);
       if ((int64_t)ev < nA && nA <= (int64_t)(ev + k.nev)) { sv[4] = i - chM; sv[5] = ev; sv[6] = -1; }
       ev += k.nev;
     }
@@ -603,29 +630,22 @@ __device__ __forceinline__ void s3_plan(const DevState& s, Ctl* c) {
     }
   }
   __syncthreads();
-  auto mv_of = [&](int64_t i, int lo) -> uint32_t {  // movers of small chunk i with f >= lo
-    uint32_t n = 0;
-    if (i < cfull) {
-      for (int r = tmax<int>(lo, (int)mm); r < kS3Bins; ++r) n += ckS[i].hist[r];
-    } else if (i == cpart) {
-      for (int r = tmax<int>(lo, (int)mm); r < kS3Bins; ++r) n += part_h[r];
-    }
-    return n;
+  // a small chunk's bins, cut to its movers' part: all of a chunk before the
+  // cut, the cut chunk's counted part, none after it
+  auto mover_bins = [&](int64_t i, Rec& k) {
+#pragma unroll
+    for (int q = 0; q < kS3Bins; ++q)
+      k.h[q] = q < (int)mm ? 0u : (i < cfull ? k.h[q] : (i == cpart ? part_h[q] : 0u));
   };
 #pragma unroll
   for (int r = 0; r < kS3Bins; ++r) h[r] = 0;
   uint64_t mvs = 0;
   for (int64_t i = tmax(r0, chM); i < r1; ++i) {
-    mvs += mv_of(i - chM, 0);
-    if (i - chM < cfull) {
+    Rec k = rec(i);
+    mover_bins(i - chM, k);
+    mvs += bins_from(k.h, 0);
 #pragma unroll
-      for (int r = 0; r < kS3Bins; ++r)
-        if (r >= (int)mm) h[r] += ckS[i - chM].hist[r];
-    } else if (i - chM == cpart) {
-#pragma unroll
-      for (int r = 0; r < kS3Bins; ++r)
-        if (r >= (int)mm) h[r] += part_h[r];
-    }
+    for (int q = 0; q < kS3Bins; ++q) h[q] += k.h[q];
   }
   add_bins(hmov, h);
   uint64_t tmv;
@@ -635,7 +655,11 @@ __device__ __forceinline__ void s3_plan(const DevState& s, Ctl* c) {
     uint64_t mv = emv;
     for (int64_t i = tmax(r0, chM); i < r1; ++i) {
       bS[i - chM].mv = (uint32_t)mv;
-      mv += mv_of(i - chM, 0);
+      if (i + 1 < r1) {
+        Rec k = rec(i);
+        mover_bins(i - chM, k);
+        mv += bins_from(k.h, 0);
+      }
     }
   }
   const int64_t nL = UMo + MA;
@@ -663,30 +687,31 @@ __device__ __forceinline__ void s3_plan(const DevState& s, Ctl* c) {
       base_R += gt;
     }
   }
-  auto ge_eq = [&](int64_t i) -> uint64_t {  // members with f >= Rs (high) and f == Rs (low) of list chunk i
-    uint32_t ge = 0, gt = 0;
-    if (i < chM) {
-      for (int r = Rs; r < kS3Bins; ++r) ge += ckM[i].hist[r];
-      gt = ge - ckM[i].hist[Rs];
-    } else {
-      ge = mv_of(i - chM, Rs);
-      gt = mv_of(i - chM, Rs + 1);
+  // members with f >= Rs (high) and f == Rs (low) of list chunk i, and the
+  // kept ones of a small chunk
+  auto ge_eq = [&](int64_t i, uint32_t* keep) -> uint64_t {
+    Rec k = rec(i);
+    *keep = 0;
+    if (i >= chM) {
+      const int64_t j = i - chM;
+      *keep = k.nlive - (j < cfull ? k.nu : (j == cpart ? part_u : 0u));
+      mover_bins(j, k);
     }
+    const uint32_t ge = bins_from(k.h, Rs), gt = bins_from(k.h, Rs + 1);
     return (uint64_t)ge << 32 | (ge - gt);
-  };
-  auto keep_s = [&](int64_t i) -> uint32_t {
-    return ckS[i].nlive - (i < cfull ? ckS[i].nu : (i == cpart ? part_u : 0u));
   };
   uint64_t ags = 0, aks = 0;
   for (int64_t i = r0; i < r1; ++i) {
-    ags += ge_eq(i);
-    if (i >= chM) aks += keep_s(i - chM);
+    uint32_t keep;
+    ags += ge_eq(i, &keep);
+    aks += keep;
   }
   uint64_t tg, tks;
   uint64_t eg = block_excl_scan<uint64_t>(ags, &tg);
   uint64_t eks = block_excl_scan<uint64_t>(aks, &tks);
   for (int64_t i = r0; i < r1; ++i) {
-    const uint64_t v = ge_eq(i);
+    uint32_t keep;
+    const uint64_t v = ge_eq(i, &keep);
     S3Base& bb = i < chM ? bM[i] : bS[i - chM];
     const uint32_t ge = (uint32_t)(eg >> 32), eq = (uint32_t)eg;
     bb.ge = ge;
@@ -701,7 +726,7 @@ __device__ __forceinline__ void s3_plan(const DevState& s, Ctl* c) {
     eg += v;
     if (i >= chM) {
       bS[i - chM].keep = (uint32_t)eks;
-      eks += keep_s(i - chM);
+      eks += keep;
     }
   }
   if (mB > 0) {
@@ -1061,28 +1086,49 @@ __global__ void __launch_bounds__(kCT) k_s3_push(DevState s) {
 }
 
 // ===========================================================================
-// 6. After the insertions: each new block (in rank order, the order of its
-//    sequence number) looks its key up in the ghost; a hit leaves the ghost
-//    and enters the main queue, any other block the small queue.
+// 6. The new blocks and the ghost.  Every claimed key is looked up beside the
+//    plan (k_s3_probe): the step's own pushes are keys that were resident, so
+//    no claim can meet them, and an entry found may only be trimmed before its
+//    block is inserted.  After the insertions each new block (in rank order,
+//    the order of its sequence number; a granted claim's rank is its place
+//    among the claims) looks at its one slot again: a key still there leaves
+//    the ghost and enters the main queue, any other block the small queue.
+//    (The lookup of 128-byte buckets after the insertions took 20 us of a step
+//    at 2^20 blocks.)
+__global__ void __launch_bounds__(kCT) k_s3_probe(DevState s) {
+  s = with_args(s);
+  const Ctl* c = s.ctl;
+  const int64_t q = blockIdx.x * (int64_t)kCT + threadIdx.x;
+  const int32_t st = c->status;
+  const int64_t nclaims = c->total_claims;
+  const uint64_t cp = q < s.max_blocks ? s.claim_pos[q] : 0ull;
+  if (st != PS_OK || q >= nclaims) return;
+  s.s3_slot[q] = gh_find(s, s.pos_key[(uint32_t)cp], (uint32_t)s.in_group[cp >> 32]);
+}
+
 __global__ void __launch_bounds__(kCT) k_s3_ins(DevState s) {
   s = with_args(s);
   Ctl* c = s.ctl;
   S3Plan* pl = s.s3_plan;
-  if (c->status != PS_OK) return;
-  const int64_t n_ins = c->need < c->n_alloc ? c->need : c->n_alloc;
   const int64_t r = blockIdx.x * (int64_t)kCT + threadIdx.x;
+  const int32_t st = c->status;
+  const int64_t need = c->need, n_alloc = c->n_alloc;
+  const bool room = r < s.max_blocks;
+  const uint32_t b = room ? (uint32_t)s.out.admitted_ids[r] : 0u;
+  const uint32_t slot = room ? s.s3_slot[r] : kNone;
+  if (st != PS_OK) return;
   bool hit = false;
-  if (r < n_ins) {
-    const uint32_t b = (uint32_t)s.out.admitted_ids[r];
-    const uint64_t key = s.blk_key[b];
-    const uint32_t g = s.blk_group[b];
-    const uint32_t slot = gh_find(s, key, g);
+  if (r < tmin(need, n_alloc)) {
     if (slot != kNone) {
-      const uint32_t ridx = s.ghost_map[slot].blk;
-      gh_erase_known(s, slot, key, g);
-      atomicAnd(bits_of(s, c->ghost_rbuf) + (ridx >> 5), ~(1u << (ridx & 31)));
-      s.blk_flags[b] = 3;
-      hit = true;
+      const TableEntry e = s.ghost_map[slot];
+      const uint64_t key = s.blk_key[b];
+      const uint32_t g = s.blk_group[b];
+      if (e.blk != kNone && e.key == key && e.grp == g) {
+        gh_erase_known(s, slot, key, g);
+        atomicAnd(bits_of(s, c->ghost_rbuf) + (e.blk >> 5), ~(1u << (e.blk & 31)));
+        s.blk_flags[b] = 3;
+        hit = true;
+      }
     }
     s.blk_s3seq[b] = pl->ctr_end + (uint64_t)r + 1;
     s.s3_hit[r] = hit ? 1 : 0;
@@ -1140,12 +1186,23 @@ __global__ void __launch_bounds__(kCT) k_s3_place(DevState s) {
   }
 }
 
-int32_t launch_s3_select(const DevState& s, cudaStream_t st, bool plain_first, int* launches) {
-  if (plain_first) k_s3_count<<<152 * 4, kCT, 0, st>>>(s);
+int32_t launch_s3_probe(const DevState& s, cudaStream_t st, int* launches) {
+  const int64_t B = s.max_blocks > 0 ? s.max_blocks : 1;
+  launch_k(k_s3_probe, (int)((B + kCT - 1) / kCT), kCT, 0, st, s);
+  ++*launches;
+  return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
+}
+int32_t launch_s3_count(const DevState& s, cudaStream_t st, bool plain, int* launches) {
+  if (plain) k_s3_count<<<152 * 4, kCT, 0, st>>>(s);
   else launch_k(k_s3_count, 152 * 4, kCT, 0, st, s);
-  launch_k(k_s3_plan, 1, kPT, 0, st, s);
+  ++*launches;
+  return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
+}
+int32_t launch_s3_select(const DevState& s, cudaStream_t st, bool plain, int* launches) {
+  if (plain) k_s3_plan<<<1, kPT, 0, st>>>(s);
+  else launch_k(k_s3_plan, 1, kPT, 0, st, s);
   launch_k(k_s3_apply, 152 * 4, kCT, 0, st, s);
-  *launches += 3;
+  *launches += 2;
   return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
 }
 
