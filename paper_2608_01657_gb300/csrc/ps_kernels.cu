@@ -314,7 +314,8 @@ __global__ void k_init_ctl(DevState s) {
 // without inclusive prefixes: a tile sums every earlier tile's total, and no
 // total waits on anything).  The last CTA to finish sets the call's status
 // and per-step scalars, and clears the tile words for the next call.
-// 'probe' skips the clock and step checks.  Every write is bounds-checked, so
+// A probe (probe_status set: where its outcome goes) skips the clock and step
+// checks.  Every write is bounds-checked, so
 // inputs that turn out invalid write nothing outside the scratch arrays.
 // A warp's requests' chunk descriptors, a lane per chunk: its request is found
 // among the warp's by the chunks before it, and the request's values come by
@@ -347,10 +348,11 @@ __device__ __forceinline__ void write_chunks(const DevState& s, int32_t ns, int3
 
 constexpr uint64_t kTileFlag = 1ull << 63;
 
-__global__ void __launch_bounds__(kValTile) k_validate(DevState s, int probe) {
+__global__ void __launch_bounds__(kValTile) k_validate(DevState s, int32_t* probe_status) {
   s = with_args(s);
   __shared__ uint64_t s_base;
   __shared__ bool s_last;
+  const bool probe = probe_status != nullptr;
   Ctl* c = s.ctl;
   const int R = s.R;
   const int tile = blockIdx.x;
@@ -451,6 +453,7 @@ __global__ void __launch_bounds__(kValTile) k_validate(DevState s, int probe) {
   else if (!probe && step > kMaxStep) st = PS_ERR_CAPACITY;
   else if (vb || first_off != 0 || T > s.max_tokens) st = PS_ERR_INVALID_ARG;
   c->status = st;
+  if (probe) *probe_status = st;
   c->T = T;
   c->hash_ticket = 0;
   if (st != PS_OK) {
@@ -588,7 +591,7 @@ __device__ __forceinline__ void block_nh(const DevState& s, const uint32_t* sk, 
 // a predecessor ran out (never expected).
 template <int BS>
 __device__ __forceinline__ bool hash_lookup_chunk(const DevState& s, Ctl* c, const uint32_t* sk, const uint64_t* kc,
-                                                  int64_t j, int probe) {
+                                                  int64_t j, int32_t* probe_out) {
   const int lane = lane_id();
   const ChunkDesc d = load_chunk(s.chunks + j);
   const uint32_t i = d.req;
@@ -677,8 +680,11 @@ __device__ __forceinline__ bool hash_lookup_chunk(const DevState& s, Ctl* c, con
   if (!__all_sync(kFull, ok)) return false;  // a predecessor never published
   // first miss in this chunk
   const int first = missA ? __ffs(missA) - 1 : (missB ? kSegBlocks + __ffs(missB) - 1 : kChunkBlocks);
+  if (probe_out) {  // the chunk of the first miss, or the last chunk, knows the count
+    if (lane == 0 && !missbefore && (anymiss || m0 + nb == n)) probe_out[i] = anymiss ? m0 + first : n;
+    return true;
+  }
   if (!missbefore && anymiss && lane == 0) s.rq_h[i] = m0 + first;  // h_i: its only writer
-  if (probe) return true;
   const uint32_t step32 = (uint32_t)c->step;
   // the cached prefix is pinned, every later block claimed
   auto place = [&](bool act, int half, uint64_t key, uint32_t blk, uint32_t* klass) -> bool {
@@ -747,11 +753,11 @@ __device__ __forceinline__ bool hash_lookup_chunk(const DevState& s, Ctl* c, con
 // (lower tickets) have always started hashing before it, and their totals
 // arrive about when its own does.  A chunk waits only on chunks of lower
 // tickets, each held by a running warp: the waits always make progress.
-// probe = 1: the read-only probe (ps_cached_prefix): h_i only, no pins,
+// probe_out: the read-only probe (ps_cached_prefix) stores h_i there; no pins,
 // claims, history or per-position records.
 constexpr int kHashCtasPerSm = 5;
 template <int BS>
-__global__ void __launch_bounds__(256, kHashCtasPerSm) k_hash_lookup(DevState s, int probe) {
+__global__ void __launch_bounds__(256, kHashCtasPerSm) k_hash_lookup(DevState s, int32_t* probe_out) {
   s = with_args(s);
   __shared__ uint32_t sk[BS + 2];                // the NH key words (read by every lane alike)
   __shared__ uint64_t kc[2 * (kSegBlocks + 1)];  // Kc^j, then Kc^(32 t)
@@ -761,12 +767,15 @@ __global__ void __launch_bounds__(256, kHashCtasPerSm) k_hash_lookup(DevState s,
   for (int k = threadIdx.x; k < 2 * (kSegBlocks + 1); k += blockDim.x) kc[k] = s.kc_pow[k];
   __syncthreads();
   const int lane = lane_id();
+  if (probe_out && c->status == PS_OK)  // a prompt without a full block has no chunk
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < s.R; i += gridDim.x * blockDim.x)
+      if (s.rq_n[i] == 0) probe_out[i] = 0;
   for (;;) {
     uint32_t t = 0;
     if (lane == 0) t = atomicAdd(&c->hash_ticket, 1u);
     t = __shfl_sync(kFull, t, 0);
     if ((int64_t)t >= nsegs) return;
-    if (!hash_lookup_chunk<BS>(s, c, sk, kc, (int64_t)t, probe)) {
+    if (!hash_lookup_chunk<BS>(s, c, sk, kc, (int64_t)t, probe_out)) {
       if (lane == 0) c->internal_error = 1;
       return;
     }
@@ -2491,16 +2500,6 @@ __global__ void k_finalize(DevState s) {
   }
 }
 
-// Read-only probe output: h_i per request, and the probe's status.
-__global__ void k_probe_out(DevState s, int32_t* out, int32_t* status) {
-  s = with_args(s);
-  const Ctl* c = s.ctl;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) *status = c->status;
-  if (c->status != PS_OK || i >= s.R) return;
-  out[i] = s.rq_h[i];
-}
-
 // ===========================================================================
 // host launchers
 static int grid_for(int64_t items, int threads, int max_ctas) {
@@ -2517,7 +2516,7 @@ void launch_init(const DevState& s, cudaStream_t st) {
 }
 
 template <int BS>
-static void launch_hash_lookup_t(const DevState& s, cudaStream_t st, int probe) {
+static void launch_hash_lookup_t(const DevState& s, cudaStream_t st, int32_t* probe_out) {
   // persistent: the CTAs that fit at once (more only queue behind them)
   int dev = 0, nsm = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -2529,16 +2528,16 @@ static void launch_hash_lookup_t(const DevState& s, cudaStream_t st, int probe) 
   const int64_t want = (s.max_segments + warps - 1) / warps;
   const int64_t most = (int64_t)nsm * kHashCtasPerSm * 8 / warps;
   const int grid = (int)(want < most ? want : most);
-  k_hash_lookup<BS><<<grid > 0 ? grid : 1, 32 * warps, 0, st>>>(s, probe);
+  k_hash_lookup<BS><<<grid > 0 ? grid : 1, 32 * warps, 0, st>>>(s, probe_out);
 }
-static int32_t launch_hash_lookup(const DevState& s, cudaStream_t st, int probe) {
+static int32_t launch_hash_lookup(const DevState& s, cudaStream_t st, int32_t* probe_out) {
   switch (s.bs) {
-    case 2: launch_hash_lookup_t<2>(s, st, probe); break;
-    case 4: launch_hash_lookup_t<4>(s, st, probe); break;
-    case 8: launch_hash_lookup_t<8>(s, st, probe); break;
-    case 16: launch_hash_lookup_t<16>(s, st, probe); break;
-    case 32: launch_hash_lookup_t<32>(s, st, probe); break;
-    case 64: launch_hash_lookup_t<64>(s, st, probe); break;
+    case 2: launch_hash_lookup_t<2>(s, st, probe_out); break;
+    case 4: launch_hash_lookup_t<4>(s, st, probe_out); break;
+    case 8: launch_hash_lookup_t<8>(s, st, probe_out); break;
+    case 16: launch_hash_lookup_t<16>(s, st, probe_out); break;
+    case 32: launch_hash_lookup_t<32>(s, st, probe_out); break;
+    case 64: launch_hash_lookup_t<64>(s, st, probe_out); break;
     default: return PS_ERR_INVALID_ARG;
   }
   return PS_OK;
@@ -2569,9 +2568,9 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
   };
 #define PS_LAUNCH(...) do { __VA_ARGS__; ++launches; } while (0)
   mark(0);
-  PS_LAUNCH(launch_k(k_validate, grid_for(R, kValTile, 1 << 20), kValTile, 0, st, s, 0));
+  PS_LAUNCH(launch_k(k_validate, grid_for(R, kValTile, 1 << 20), kValTile, 0, st, s, nullptr));
   mark(1);
-  if (launch_hash_lookup(s, st, 0) != PS_OK) return PS_ERR_INVALID_ARG;
+  if (launch_hash_lookup(s, st, nullptr) != PS_OK) return PS_ERR_INVALID_ARG;
   ++launches;
   mark(2);
   PS_LAUNCH(launch_k(k_claims, prgrid, kThreads, 0, st, s));
@@ -2753,13 +2752,10 @@ void launch_host_out(const ps_step_out_t& dev, const ps_step_out_t& host, int32_
 }
 
 int32_t launch_probe(const DevState& s, cudaStream_t st, int32_t* out, int32_t* status) {
-  const int rgrid = grid_for(s.R, 256, 1 << 20);
-  const int pgrid = grid_for(s.max_blocks, kThreads, 1 << 30);
   DevState p = s;
   p.args = nullptr;  // the probe's kernels take every argument by value
-  k_validate<<<grid_for(p.max_requests, kValTile, 1 << 20), kValTile, 0, st>>>(p, 1);
-  if (s.R > 0 && launch_hash_lookup(p, st, 1) != PS_OK) return PS_ERR_INVALID_ARG;
-  k_probe_out<<<rgrid, 256, 0, st>>>(p, out, status);
+  k_validate<<<grid_for(p.max_requests, kValTile, 1 << 20), kValTile, 0, st>>>(p, status);
+  if (s.R > 0 && launch_hash_lookup(p, st, out) != PS_OK) return PS_ERR_INVALID_ARG;
   return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
 }
 
