@@ -536,6 +536,21 @@ int32_t ps_step(ps_handle_t* h, void* stream, int64_t now_ticks, int32_t num_req
   return launch_step(s, st, &h->trace);
 }
 
+namespace {
+constexpr size_t kHostKernelBytes = (size_t)8 << 20;
+inline bool aligned_to(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
+// A host array a kernel may read or write: page-locked (or otherwise device-mapped).
+bool device_writable(const void* p) {
+  if (!p) return true;
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeHost || a.type == cudaMemoryTypeManaged;
+}
+}  // namespace
+
 int32_t ps_step_host(ps_handle_t* h, void* stream, int64_t now_ticks, int32_t num_requests, const int32_t* h_group_ids,
                      const int64_t* h_token_offsets, const int32_t* h_tokens, const int32_t* h_contract_ids,
                      const uint64_t* h_prefix_ids, const ps_host_out_t* h_out) {
@@ -551,10 +566,23 @@ int32_t ps_step_host(ps_handle_t* h, void* stream, int64_t now_ticks, int32_t nu
     return bytes == 0 || cudaMemcpyAsync(d, src, bytes, cudaMemcpyHostToDevice, st) == cudaSuccess;
   };
   const ps_handle::Staging& sg = h->stg[0];
-  if (!h2d(sg.offsets, h_token_offsets, (R + 1) * 8) || !h2d(sg.group, h_group_ids, R * 4) ||
-      !h2d(sg.tokens, h_tokens, (size_t)T * 4) || (h_contract_ids && !h2d(sg.contract, h_contract_ids, R * 4)) ||
-      (h_prefix_ids && !h2d(sg.prefix, h_prefix_ids, R * 8)))
+  // Page-locked inputs of up to kHostKernelBytes are read by a kernel (larger
+  // ones are the copy engine's), page-locked outputs written by one, id lists
+  // by their device-side counts: one wait instead of two and no copy calls.
+  const void* in[5] = {h_token_offsets, h_group_ids, h_tokens, h_contract_ids, h_prefix_ids};
+  bool in_locked = (size_t)T * 4 <= kHostKernelBytes;
+  for (const void* p : in) in_locked = in_locked && aligned_to(p, 4) && device_writable(p);
+  if (in_locked) {
+    void* dst[5] = {sg.offsets, sg.group, sg.tokens, sg.contract, sg.prefix};
+    const int64_t words[5] = {2 * ((int64_t)R + 1), (int64_t)R, T, (int64_t)R, 2 * (int64_t)R};
+    launch_host_in(in, dst, words, st);
+    if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
+  } else if (!h2d(sg.offsets, h_token_offsets, (R + 1) * 8) || !h2d(sg.group, h_group_ids, R * 4) ||
+             !h2d(sg.tokens, h_tokens, (size_t)T * 4) ||
+             (h_contract_ids && !h2d(sg.contract, h_contract_ids, R * 4)) ||
+             (h_prefix_ids && !h2d(sg.prefix, h_prefix_ids, R * 8))) {
     return PS_ERR_CUDA;
+  }
   int32_t rc = ps_step(h, stream, now_ticks, num_requests, sg.group, sg.offsets, sg.tokens,
                        h_contract_ids ? sg.contract : nullptr, h_prefix_ids ? sg.prefix : nullptr, &h->st_out);
   if (rc != PS_OK) return rc;
@@ -562,6 +590,18 @@ int32_t ps_step_host(ps_handle_t* h, void* stream, int64_t now_ticks, int32_t nu
   auto d2h = [&](void* dst, const void* d, size_t bytes) {
     return bytes == 0 || !dst || cudaMemcpyAsync(dst, d, bytes, cudaMemcpyDeviceToHost, st) == cudaSuccess;
   };
+  bool out_locked = h_out->counts != nullptr;
+  for (const void* p : {(const void*)h_out->hit_blocks, (const void*)h_out->admitted_blocks,
+                        (const void*)h_out->admitted_offsets, (const void*)h_out->admitted_ids,
+                        (const void*)h_out->evicted_ids, (const void*)h_out->invalidated_ids,
+                        (const void*)h_out->counts, (const void*)h_out->debt_raw, (const void*)h_out->debt_norm})
+    out_locked = out_locked && aligned_to(p, 4) && device_writable(p);
+  out_locked = out_locked && aligned_to(h_out->debt_raw, 8) && aligned_to(h_out->debt_norm, 8);
+  if (out_locked) {
+    launch_host_out(o, *h_out, num_requests, h->base.G, st);
+    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return PS_ERR_CUDA;
+    return h_out->counts[3];
+  }
   const size_t G = (size_t)h->base.G;
   if (!d2h(h_out->counts, o.counts, 16) || !d2h(h_out->hit_blocks, o.hit_blocks, R * 4) ||
       !d2h(h_out->admitted_blocks, o.admitted_blocks, R * 4) ||
@@ -576,19 +616,6 @@ int32_t ps_step_host(ps_handle_t* h, void* stream, int64_t now_ticks, int32_t nu
     return PS_ERR_CUDA;
   return PS_OK;
 }
-
-namespace {
-// A host array a kernel may write: page-locked (or otherwise device-mapped).
-bool device_writable(const void* p) {
-  if (!p) return true;
-  cudaPointerAttributes a{};
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return a.type == cudaMemoryTypeHost || a.type == cudaMemoryTypeManaged;
-}
-}  // namespace
 
 int32_t ps_step_host_async(ps_handle_t* h, void* stream, int32_t slot, int64_t now_ticks, int32_t num_requests,
                            const int32_t* h_group_ids, const int64_t* h_token_offsets, const int32_t* h_tokens,

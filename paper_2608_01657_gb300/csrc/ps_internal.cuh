@@ -490,6 +490,8 @@ int32_t launch_s3_insert(const DevState& s, cudaStream_t st, int* launches);
 // A step's outputs (device) written into page-locked host buffers, the id
 // lists by their device-side counts (ps_step_host_async).
 void launch_host_out(const ps_step_out_t& dev, const ps_step_out_t& host, int32_t R, int32_t G, cudaStream_t st);
+// Five input arrays copied from page-locked host memory (null ones skipped).
+void launch_host_in(const void* const* src, void* const* dst, const int64_t* words, cudaStream_t st);
 // Read-only cached-prefix probe; 'out' receives h_i per request, 'status' the outcome.
 int32_t launch_probe(const DevState& s, cudaStream_t st, int32_t* out, int32_t* status);
 

@@ -2751,6 +2751,36 @@ void launch_host_out(const ps_step_out_t& dev, const ps_step_out_t& host, int32_
   k_host_out<<<152 * 2, 256, 0, st>>>(dev, host, R, G);
 }
 
+// A step's inputs from the caller's page-locked host buffers into the staging
+// area, one pass of all SMs over the host link: a small call's five copies
+// took longer to issue, one after the other, than to run.
+struct HostIn {
+  const void* src[5];
+  void* dst[5];
+  int64_t words[5];  // 32-bit words
+};
+__global__ void __launch_bounds__(256) k_host_in(HostIn a) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const int64_t n = a.words[k];
+    const uint32_t* src = static_cast<const uint32_t*>(a.src[k]);
+    uint32_t* dst = static_cast<uint32_t*>(a.dst[k]);
+    const int64_t nv = (reinterpret_cast<uintptr_t>(src) & 15) ? 0 : n / 4;  // the staging areas are aligned
+    for (int64_t i = t; i < nv; i += nt) reinterpret_cast<uint4*>(dst)[i] = reinterpret_cast<const uint4*>(src)[i];
+    for (int64_t i = 4 * nv + t; i < n; i += nt) dst[i] = src[i];
+  }
+}
+void launch_host_in(const void* const* src, void* const* dst, const int64_t* words, cudaStream_t st) {
+  HostIn a{};
+  for (int k = 0; k < 5; ++k) {
+    a.src[k] = src[k];
+    a.dst[k] = dst[k];
+    a.words[k] = src[k] ? words[k] : 0;
+  }
+  k_host_in<<<152 * 4, 256, 0, st>>>(a);
+}
+
 int32_t launch_probe(const DevState& s, cudaStream_t st, int32_t* out, int32_t* status) {
   DevState p = s;
   p.args = nullptr;  // the probe's kernels take every argument by value
