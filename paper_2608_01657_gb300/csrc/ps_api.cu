@@ -34,8 +34,6 @@ struct ps_handle {
   // the step as one CUDA graph, captured on a private stream at first use
   StepArgs* step_args;
   cudaStream_t cap_stream = nullptr;
-  cudaStream_t cap_aux = nullptr;   // conditional bodies are captured here
-  cudaStream_t cap_aux2 = nullptr;  // and bodies nested in them here
   cudaStream_t cap_side = nullptr;  // a parallel branch of the step graph
   cudaStream_t cap_side2 = nullptr; // a second one
   cudaEvent_t cap_fork = nullptr, cap_join = nullptr, cap_fork2 = nullptr, cap_join2 = nullptr;
@@ -386,18 +384,8 @@ void capture_step(ps_handle* h) {
   tmpl.R = 0;
   bool ok = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
   if (ok) {
-    const CaptureCtx ctx{h->cap_aux, h->cap_aux2, h->cap_side, h->cap_fork, h->cap_join,
-                         h->cap_side2, h->cap_fork2, h->cap_join2};
+    const CaptureCtx ctx{h->cap_side, h->cap_fork, h->cap_join, h->cap_side2, h->cap_fork2, h->cap_join2};
     const int32_t rc = launch_step(tmpl, h->cap_stream, &h->trace, &ctx);
-    // a body whose capture did not close leaves an auxiliary stream capturing
-    // (the side stream joined the main capture: it ends with it)
-    for (cudaStream_t a : {h->cap_aux2, h->cap_aux}) {
-      cudaStreamCaptureStatus aux_cs = cudaStreamCaptureStatusNone;
-      if (cudaStreamIsCapturing(a, &aux_cs) == cudaSuccess && aux_cs != cudaStreamCaptureStatusNone) {
-        cudaGraph_t body = nullptr;
-        cudaStreamEndCapture(a, &body);
-      }
-    }
     cudaGraph_t g = nullptr;
     const bool ended = cudaStreamEndCapture(h->cap_stream, &g) == cudaSuccess;
     ok = rc == PS_OK && ended && g;
@@ -484,8 +472,6 @@ int32_t ps_create(ps_handle_t** out, int64_t capacity_blocks, int32_t block_size
   int32_t rc = init_state(h, st);
   if (rc == PS_OK) rc = upload_constants(h, st);
   if (rc == PS_OK && (cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
-                      cudaStreamCreateWithFlags(&h->cap_aux, cudaStreamNonBlocking) != cudaSuccess ||
-                      cudaStreamCreateWithFlags(&h->cap_aux2, cudaStreamNonBlocking) != cudaSuccess ||
                       cudaStreamCreateWithFlags(&h->cap_side, cudaStreamNonBlocking) != cudaSuccess ||
                       cudaStreamCreateWithFlags(&h->cap_side2, cudaStreamNonBlocking) != cudaSuccess ||
                       cudaEventCreateWithFlags(&h->cap_fork, cudaEventDisableTiming) != cudaSuccess ||
@@ -708,8 +694,6 @@ void ps_destroy(ps_handle_t* h) {
   if (!h) return;
   drop_graph(h);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
-  if (h->cap_aux) cudaStreamDestroy(h->cap_aux);
-  if (h->cap_aux2) cudaStreamDestroy(h->cap_aux2);
   if (h->cap_side) cudaStreamDestroy(h->cap_side);
   if (h->cap_side2) cudaStreamDestroy(h->cap_side2);
   if (h->cap_fork) cudaEventDestroy(h->cap_fork);
@@ -744,7 +728,7 @@ int32_t ps_get_stage_times(ps_handle_t* h, float* h_ms, int32_t max_stages, int3
   if (h_launches) *h_launches = h->trace.launches;
   if (!h->trace.timing) return 0;
   if (cudaEventSynchronize(h->trace.ev[PS_NUM_STAGES]) != cudaSuccess) return PS_ERR_CUDA;
-  // kernels the step actually launched (conditional bodies included or not)
+  // kernels the step actually launched
   if (h_launches && cudaMemcpy(h_launches, &h->base.ctl->nlaunch, 4, cudaMemcpyDeviceToHost) != cudaSuccess)
     return PS_ERR_CUDA;
   const int n = max_stages < PS_NUM_STAGES ? max_stages : PS_NUM_STAGES;

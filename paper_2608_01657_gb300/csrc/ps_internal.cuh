@@ -101,7 +101,7 @@ struct Ctl {
   int32_t sel_mode;        // what the select's first pass does (kSel*)
   int64_t lst_n;              // members of the select's split list
   uint32_t ticket;         // last-block-done counter for the radix passes and the split
-  int32_t nlaunch;         // kernels launched by the step (conditional bodies run or not)
+  int32_t nlaunch;         // kernels launched by the step
   int32_t pad2;
   int32_t internal_error;  // an invariant of the step failed (reported, never expected)
   // indexed queues (PS_FLAG_INDEXED_QUEUES)
@@ -115,6 +115,7 @@ struct Ctl {
   uint32_t v_ticket;       // k_validate: CTAs done (the last one finishes the call)
   uint32_t v_bad;          // k_validate: bit 0 an invalid request, bit 1 a look-back ran out
   uint64_t v_sum;          // k_validate: blocks (high half) and chunks (low half) of the call
+  uint64_t bar;            // k_lg_compact's grid barrier: arrivals so far (a multiple of its grid between steps)
 };
 
 // One hashing chunk: up to kChunkBlocks consecutive blocks of one request.
@@ -416,11 +417,8 @@ struct StepTrace {
   int launches = 0;
 };
 
-// Stream capture of a step: a second private stream on which the bodies of
-// conditional graph nodes are captured (phases that many steps skip).
+// Stream capture of a step: the streams and events of its parallel branches.
 struct CaptureCtx {
-  cudaStream_t aux;   // bodies of top-level conditional nodes
-  cudaStream_t aux2;  // bodies of conditional nodes inside those
   cudaStream_t side;  // a parallel branch of the step graph (the candidate scan)
   cudaEvent_t fork, join;
   cudaStream_t side2;  // a second branch (in-step hits, metering, touch passes)
@@ -470,7 +468,7 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
 void launch_queue_init(const DevState& s, cudaStream_t st);
 int32_t launch_queue_cand(const DevState& s, cudaStream_t st, int* launches);
 int32_t launch_queue_select(const DevState& s, cudaStream_t st, int phase, bool plain_first, int* launches);
-int32_t launch_queue_append(const DevState& s, cudaStream_t st, const CaptureCtx* cap, int* launches);
+int32_t launch_queue_append(const DevState& s, cudaStream_t st, int* launches);
 // S3-FIFO (ps_s3fifo.cu)
 // The ghost's entries for the step's claims (before anything leaves the ghost).
 int32_t launch_s3_probe(const DevState& s, cudaStream_t st, int* launches);

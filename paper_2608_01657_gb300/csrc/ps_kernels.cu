@@ -2713,7 +2713,7 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
     PS_LAUNCH(launch_k(k_insert, igrid, kThreads, 0, st, s));
   }
   if (s.policy == PS_S3FIFO && launch_s3_insert(s, st, &launches) != PS_OK) return PS_ERR_CUDA;
-  if (s.lg_on && launch_queue_append(s, st, cap, &launches) != PS_OK) return PS_ERR_CUDA;
+  if (s.lg_on && launch_queue_append(s, st, &launches) != PS_OK) return PS_ERR_CUDA;
   mark(10);
   PS_LAUNCH(launch_k(k_finalize, 1, 32, 0, st, s));
   mark(11);

@@ -38,6 +38,7 @@ namespace {
 
 constexpr int kScanThreads = 256;          // 4 consecutive entries a thread per chunk
 constexpr int kScanGrid = 152 * 8;         // grid-stride over the chunks of a scan
+constexpr int kCompactGrid = 152 * 2;      // all resident (a cooperative launch)
 static_assert(kScanThreads * 4 == kLogChunk, "a scan CTA covers one chunk");
 
 __device__ __forceinline__ const uint32_t* ent_blk(const DevState& s, int buf) { return s.lg_blk + (int64_t)buf * s.lg_P; }
@@ -416,10 +417,10 @@ __global__ void __launch_bounds__(kAppChunk) k_lg_app_count(DevState s) {
 }
 
 // Per log (a CTA each): chunk offsets of the appends, their total, and
-// whether the log has room for them.  Each thread scans a run of
+// whether the log has room for them (if not, every log is compacted first).  Each thread scans a run of
 // consecutive chunks, so the loads of a log's row are all in flight at once.
 constexpr int kScanRun = 16;  // chunk counts a thread holds (up to 4096 x 16 chunks per pass)
-__global__ void __launch_bounds__(256) k_lg_app_scan(DevState s, cudaGraphConditionalHandle hc, int has_cond) {
+__global__ void __launch_bounds__(256) k_lg_app_scan(DevState s) {
   s = with_args(s);
   Ctl* c = s.ctl;
   if (c->status != PS_OK) return;
@@ -449,22 +450,12 @@ __global__ void __launch_bounds__(256) k_lg_app_scan(DevState s, cudaGraphCondit
   if (threadIdx.x == 0) {
     s.lg_add[l] = before;
     const LogDesc d = s.lg_desc[l];
-    if (d.tail + (int64_t)before > d.end) {
-      c->lg_cmp = 1;
-      if (has_cond) cudaGraphSetConditional(hc, 1);
-    }
+    if (d.tail + (int64_t)before > d.end) c->lg_cmp = 1;
   }
 }
 
 // Compaction: chunks over every log's [head, tail).
-__global__ void __launch_bounds__(1024) k_lg_cmp_plan(DevState s) {
-  s = with_args(s);
-  Ctl* c = s.ctl;
-  if (c->status != PS_OK || !c->lg_cmp) {
-    __syncthreads();
-    if (threadIdx.x == 0) c->lg_nchunks = 0;
-    return;
-  }
+__device__ __forceinline__ void lg_cmp_plan(const DevState& s, Ctl* c) {
   int base = 0;
   for (int l0 = 0; l0 < s.lg_L; l0 += blockDim.x) {
     const int l = l0 + threadIdx.x;
@@ -484,16 +475,9 @@ __global__ void __launch_bounds__(1024) k_lg_cmp_plan(DevState s) {
   }
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_lg_cmp_count(DevState s) {
-  s = with_args(s);
-  __shared__ int32_t sc0[kMaxLogs + 1];
-  const Ctl* c = s.ctl;
-  if (c->status != PS_OK || !c->lg_cmp) return;
+__device__ __forceinline__ void lg_cmp_count(const DevState& s, const Ctl* c, const int32_t* sc0) {
   const int nch = c->lg_nchunks;
-  if (nch == 0) return;
   const int L = s.lg_L;
-  for (int t = threadIdx.x; t <= L; t += blockDim.x) sc0[t] = s.lg_c0[t];
-  __syncthreads();
   const uint32_t* eb = ent_blk(s, c->lg_buf);
   const uint64_t* es = ent_st(s, c->lg_buf);
   for (int q = blockIdx.x; q < nch; q += gridDim.x) {
@@ -512,11 +496,7 @@ __global__ void __launch_bounds__(kScanThreads) k_lg_cmp_count(DevState s) {
 }
 
 // Per log (a CTA each): its live entries, and each chunk's offset inside it.
-__global__ void __launch_bounds__(256) k_lg_cmp_live(DevState s) {
-  s = with_args(s);
-  Ctl* c = s.ctl;
-  if (c->status != PS_OK || !c->lg_cmp) return;
-  const int l = blockIdx.x;
+__device__ __forceinline__ void lg_cmp_live(const DevState& s, Ctl* c, int l) {
   const int q0 = s.lg_c0[l], q1 = s.lg_c0[l + 1];
   int64_t before = 0;
   for (int base = q0; base < q1; base += (int)blockDim.x * kScanRun) {
@@ -546,10 +526,7 @@ __global__ void __launch_bounds__(256) k_lg_cmp_live(DevState s) {
 
 // The new layout: each log gets its live entries, this step's appends, and a
 // share of the free room in proportion to its appends (plus one).
-__global__ void __launch_bounds__(1024) k_lg_cmp_layout(DevState s) {
-  s = with_args(s);
-  Ctl* c = s.ctl;
-  if (c->status != PS_OK || !c->lg_cmp) return;
+__device__ __forceinline__ void lg_cmp_layout(const DevState& s, Ctl* c) {
   const int L = s.lg_L;
   const int per = (L + (int)blockDim.x - 1) / (int)blockDim.x;
   const int l0 = threadIdx.x * per, l1 = l0 + per < L ? l0 + per : L;
@@ -574,15 +551,9 @@ __global__ void __launch_bounds__(1024) k_lg_cmp_layout(DevState s) {
   }
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_lg_cmp_write(DevState s) {
-  s = with_args(s);
-  __shared__ int32_t sc0[kMaxLogs + 1];
-  Ctl* c = s.ctl;
-  if (c->status != PS_OK || !c->lg_cmp) return;
+__device__ __forceinline__ void lg_cmp_write(const DevState& s, Ctl* c, const int32_t* sc0) {
   const int nch = c->lg_nchunks;
   const int L = s.lg_L;
-  for (int t = threadIdx.x; t <= L; t += blockDim.x) sc0[t] = s.lg_c0[t];
-  __syncthreads();
   const int src = c->lg_buf;
   const uint32_t* eb = ent_blk(s, src);
   const uint64_t* es = ent_st(s, src);
@@ -617,12 +588,62 @@ __global__ void __launch_bounds__(kScanThreads) k_lg_cmp_write(DevState s) {
         ++o;
       }
   }
-  if (last_cta(c)) {
-    for (int l = threadIdx.x; l < L; l += blockDim.x) s.lg_desc[l] = s.lg_new[l];
-    if (threadIdx.x == 0) {
-      c->lg_buf = src ^ 1;
-      c->lg_ticket = 0;
+}
+
+// Every CTA adds one to a counter that only grows and waits (bounded) for the
+// next multiple of the grid: a grid barrier of a cooperative launch, whose
+// CTAs are all resident.  False if the wait ran out (never expected).
+__device__ __forceinline__ bool grid_sync(Ctl* c, uint64_t* target) {
+  __shared__ int s_ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    *target += gridDim.x;
+    __threadfence();
+    atomicAdd(reinterpret_cast<unsigned long long*>(&c->bar), 1ull);
+    int ok = 0;
+    for (int it = 0; it < kLookbackSpins && !ok; ++it) {
+      uint64_t v;
+      asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&c->bar) : "memory");
+      ok = v >= *target;
     }
+    __threadfence();
+    if (!ok) c->internal_error = 1;
+    s_ok = ok;
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
+// The compaction as one cooperative kernel, launched on every step and gone at
+// once on the many that need none: its five phases as kernels behind a
+// conditional graph node cost every step about 10 us.
+__global__ void __launch_bounds__(kScanThreads) k_lg_compact(DevState s) {
+  s = with_args(s);
+  __shared__ int32_t sc0[kMaxLogs + 1];
+  Ctl* c = s.ctl;
+  const int32_t st = c->status, need = c->lg_cmp;
+  if (st != PS_OK || !need) return;
+  // a CTA has not arrived yet, so fewer than a grid of this launch's arrivals
+  // are in the counter
+  uint64_t target = threadIdx.x == 0 ? ldcg_u64(&c->bar) / gridDim.x * gridDim.x : 0;
+  if (blockIdx.x == 0) lg_cmp_plan(s, c);
+  if (!grid_sync(c, &target)) return;
+  const int L = s.lg_L;
+  for (int t = threadIdx.x; t <= L; t += blockDim.x) sc0[t] = s.lg_c0[t];
+  __syncthreads();
+  lg_cmp_count(s, c, sc0);
+  if (!grid_sync(c, &target)) return;
+  for (int l = blockIdx.x; l < L; l += gridDim.x) lg_cmp_live(s, c, l);
+  if (!grid_sync(c, &target)) return;
+  if (blockIdx.x == 0) lg_cmp_layout(s, c);
+  if (!grid_sync(c, &target)) return;
+  lg_cmp_write(s, c, sc0);
+  if (!grid_sync(c, &target)) return;
+  if (blockIdx.x != 0) return;
+  for (int l = threadIdx.x; l < L; l += blockDim.x) s.lg_desc[l] = s.lg_new[l];
+  if (threadIdx.x == 0) {
+    c->lg_buf ^= 1;
+    c->lg_nchunks = 0;
   }
 }
 
@@ -713,27 +734,22 @@ int32_t launch_queue_select(const DevState& s, cudaStream_t st, int phase, bool 
   return PS_OK;
 }
 
-int32_t launch_queue_append(const DevState& s, cudaStream_t st, const CaptureCtx* cap, int* launches) {
+int32_t launch_queue_append(const DevState& s, cudaStream_t st, int* launches) {
   const int ach = (int)s.lg_app_chunks;
-  cudaGraphConditionalHandle hc = 0;
-  if (cap && !cond_handle(st, &hc)) return PS_ERR_CUDA;
   launch_k(k_lg_app_count, ach, kAppChunk, 0, st, s);
-  launch_k(k_lg_app_scan, s.lg_L, 256, 0, st, s, hc, cap ? 1 : 0);
-  *launches += 2;
-  cudaStream_t b = st;
-  if (cap) {
-    if (!cond_open(st, cap->aux, hc)) return PS_ERR_CUDA;
-    b = cap->aux;
-  }
-  launch_k(k_lg_cmp_plan, 1, 1024, 0, b, s);
-  launch_k(k_lg_cmp_count, kScanGrid, kScanThreads, 0, b, s);
-  launch_k(k_lg_cmp_live, s.lg_L, 256, 0, b, s);
-  launch_k(k_lg_cmp_layout, 1, 1024, 0, b, s);
-  launch_k(k_lg_cmp_write, kScanGrid, kScanThreads, 0, b, s);
-  *launches += 5;
-  if (cap && !cond_close(cap->aux)) return PS_ERR_CUDA;
+  launch_k(k_lg_app_scan, s.lg_L, 256, 0, st, s);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.gridDim = dim3(kCompactGrid);
+  cfg.blockDim = dim3(kScanThreads);
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, k_lg_compact, s) != cudaSuccess) return PS_ERR_CUDA;
   launch_k(k_lg_app_write, ach, kAppChunk, 0, st, s);
-  ++*launches;
+  *launches += 4;
   return PS_OK;
 }
 
