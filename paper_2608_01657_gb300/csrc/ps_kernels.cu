@@ -71,15 +71,18 @@ __device__ __forceinline__ uint64_t red61(uint64_t x) {  // any 64-bit x -> [0, 
   const uint64_t r = (x & kP61) + (x >> 61);
   return r >= kP61 ? r - kP61 : r;
 }
-__device__ __forceinline__ uint64_t add61(uint64_t a, uint64_t b) {  // a, b < p
-  const uint64_t r = a + b;
-  return r >= kP61 ? r - kP61 : r;
-}
-__device__ __forceinline__ uint64_t mul61(uint64_t a, uint64_t b) {  // a, b < p
-  const uint64_t lo = a * b, hi = __umul64hi(a, b);
-  uint64_t r = (lo & kP61) + ((lo >> 61) | (hi << 3));
-  r = (r & kP61) + (r >> 61);
-  return r >= kP61 ? r - kP61 : r;
+// A chain of products keeps its values below p + 8 instead of below p, and
+// reduces fully only where a value leaves it: k x + c from four 32-bit
+// products and one reduction is half the instructions of a full product, a
+// full sum and their two compares and subtractions.
+__device__ __forceinline__ uint64_t weak61(uint64_t x) { return (x & kP61) + (x >> 61); }  // any 64-bit x -> <= p + 7
+__device__ __forceinline__ uint64_t mad61(uint64_t k, uint64_t x, uint64_t c) {  // k < p, x <= p + 7, c <= 2 (p + 7)
+  const uint32_t k0 = (uint32_t)k, k1 = (uint32_t)(k >> 32), x0 = (uint32_t)x, x1 = (uint32_t)(x >> 32);  // x1 <= 2^29
+  const uint64_t mid = (uint64_t)k0 * x1 + (uint64_t)k1 * x0, low = (uint64_t)k0 * x0;                    // mid <= 2^62
+  uint64_t r = (uint64_t)(k1 << 3) * x1 + c;  // 2^64 = 8 (mod p); at most 3 2^61 so far, 5 2^61 in all
+  r += (low & kP61) + (low >> 61);
+  r += ((uint64_t)((uint32_t)mid & 0x1FFFFFFFu) << 32) + (mid >> 29);  // 2^32 mid
+  return weak61(r);
 }
 
 // ---- native prefix table ---------------------------------------------------
@@ -612,26 +615,26 @@ __device__ __forceinline__ bool hash_lookup_chunk(const DevState& s, Ctl* c, con
   if (lane < nbA) {
     uint64_t d1, d2;
     block_nh<BS>(s, sk, o0 + (int64_t)mA * BS, (int)(o0 & 3), s.tokens_aligned16 != 0, T, &d1, &d2);
-    bA = add61(red61(d1), mul61(s.digest_mul, red61(d2)));
+    bA = mad61(s.digest_mul, weak61(d2), weak61(d1));
   }
   if (lane < nbB) {
     uint64_t d1, d2;
     block_nh<BS>(s, sk, o0 + (int64_t)mB * BS, (int)(o0 & 3), s.tokens_aligned16 != 0, T, &d1, &d2);
-    bB = add61(red61(d1), mul61(s.digest_mul, red61(d2)));
+    bB = mad61(s.digest_mul, weak61(d2), weak61(d1));
   }
 #pragma unroll
   for (int q = 0; q < 5; ++q) {
     const uint64_t tA = __shfl_up_sync(kFull, bA, 1 << q);
     const uint64_t tB = __shfl_up_sync(kFull, bB, 1 << q);
     if (lane >= (1 << q)) {
-      bA = add61(bA, mul61(kc[1 << q], tA));
-      bB = add61(bB, mul61(kc[1 << q], tB));
+      bA = mad61(kc[1 << q], tA, bA);
+      bB = mad61(kc[1 << q], tB, bB);
     }
   }
   const uint64_t totA = __shfl_sync(kFull, bA, nbA - 1);
   const uint64_t totB = __shfl_sync(kFull, bB, nbB > 0 ? nbB - 1 : 0);
   // a second half follows a full first half (Kc^32 times it)
-  const uint64_t total = nbB > 0 ? add61(mul61(kc[nbB], totA), totB) : totA;
+  const uint64_t total = red61(nbB > 0 ? mad61(kc[nbB], totA, totB) : totA);
   if (lane == 0) st_relaxed_u64(s.seg_word + j, total | kWordTotal);
   // the chain value entering the chunk
   bool ok = true;
@@ -642,22 +645,25 @@ __device__ __forceinline__ bool hash_lookup_chunk(const DevState& s, Ctl* c, con
     if (lane < w) {
       const uint64_t v = wait_word(s.seg_word + sb + l0 + lane, kWordTotal);
       ok = ok && v != 0;
-      term = mul61(kc[(kSegBlocks + 1) + (w - 1 - lane)], v & kP61);
+      term = mad61(kc[(kSegBlocks + 1) + (w - 1 - lane)], v & kP61, 0);
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) term = add61(term, __shfl_xor_sync(kFull, term, o));
-    cin = add61(mul61(kc[(kSegBlocks + 1) + w], cin), term);
+    for (int o = 16; o > 0; o >>= 1) {
+      term += __shfl_xor_sync(kFull, term, o);
+      if (o == 8 || o == 2) term = weak61(term);  // four terms at most are below 2^64
+    }
+    cin = mad61(kc[(kSegBlocks + 1) + w], cin, term);
   }
   // the lane's keys and their table probes
   uint64_t keyA = 0, keyB = 0;
   uint32_t blkA = kNone, blkB = kNone;
   if (lane < nbA) {
-    const uint64_t C = add61(mul61(kc[lane + 1], cin), bA);
+    const uint64_t C = red61(mad61(kc[lane + 1], cin, bA));
     keyA = fix_reserved(mix64(C ^ ((uint64_t)(mA + 1) * 0xD1B54A32D192ED03ull)));
   }
   if (lane < nbB) {
-    const uint64_t cinB = add61(mul61(kc[kSegBlocks], cin), totA);
-    const uint64_t C = add61(mul61(kc[lane + 1], cinB), bB);
+    const uint64_t cinB = mad61(kc[kSegBlocks], cin, totA);
+    const uint64_t C = red61(mad61(kc[lane + 1], cinB, bB));
     keyB = fix_reserved(mix64(C ^ ((uint64_t)(mB + 1) * 0xD1B54A32D192ED03ull)));
   }
   table_find2(s, keyA, keyB, g, lane < nbA, lane < nbB, &blkA, &blkB);
