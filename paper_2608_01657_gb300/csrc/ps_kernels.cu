@@ -1544,10 +1544,8 @@ __global__ void __launch_bounds__(1024) k_quota_sel(DevState s) {
 // item.  The search then narrows the bracket to one decrement, within which
 // each group has at most one item: tau is one of those.  (One indebted group
 // needs no search at all; the search over all values took four to six rounds.)
-__global__ void __launch_bounds__(PS_MAX_GROUPS) k_waterfill(DevState s0) {
-  // contract arrays are read from the parameter block (see k_grant)
-  const DevState s = with_args(s0);
-  Ctl* c = s.ctl;
+// (PS_MAX_GROUPS threads; contract arrays are read from the parameter block s0, see k_grant)
+__device__ __forceinline__ void waterfill(const DevState& s, const DevState& s0, Ctl* c) {
   __shared__ int64_t hP[PS_MAX_GROUPS], hD[PS_MAX_GROUPS], hQ[PS_MAX_GROUPS];  // the groups that can give victims
   __shared__ uint64_t hRcp[PS_MAX_GROUPS];
   __shared__ int64_t w_a[32], w_b[32], w_c[32], w_d[32];  // per-warp partials
@@ -1747,6 +1745,10 @@ __global__ void __launch_bounds__(PS_MAX_GROUPS) k_waterfill(DevState s0) {
       c->sel_k = (int32_t)(m - a);  // tied items to take, 1..ntie
     }
   }
+}
+__global__ void __launch_bounds__(PS_MAX_GROUPS) k_waterfill(DevState s0) {
+  const DevState s = with_args(s0);
+  waterfill(s, s0, s.ctl);
 }
 
 // ---- exact segmented select -------------------------------------------------
@@ -2026,9 +2028,7 @@ constexpr int kFinWords = (int)(kFinList / 4);  // bitmap words in the list's pl
 constexpr int kFinSegWords = 1024;              // of one segment (one warp searches them)
 constexpr size_t kFinSmem = kFinList + (size_t)PS_MAX_GROUPS * (sizeof(FinSeg) + 8 + 4 + 2);
 
-__global__ void __launch_bounds__(1024) k_list_finish(DevState s, int fallback) {
-  s = with_args(s);
-  extern __shared__ __align__(16) unsigned char fin_smem[];
+__device__ __forceinline__ void list_finish(const DevState& s, Ctl* c, unsigned char* fin_smem, int mode, int64_t n) {
   FinSeg* sl = reinterpret_cast<FinSeg*>(fin_smem);
   uint64_t* blo = reinterpret_cast<uint64_t*>(sl + PS_MAX_GROUPS);  // the segments' buckets
   int32_t* woff = reinterpret_cast<int32_t*>(blo + PS_MAX_GROUPS);  // and bitmaps
@@ -2039,10 +2039,6 @@ __global__ void __launch_bounds__(1024) k_list_finish(DevState s, int fallback) 
   __shared__ int16_t row_of[PS_MAX_GROUPS];
   __shared__ int16_t seg_of_row[PS_MAX_GROUPS];
   __shared__ int s_nrows;
-  Ctl* c = s.ctl;
-  const int64_t n = c->lst_n;  // in the mode's round trip
-  const int mode = select_mode(c, fallback);
-  if (mode < 0) return;
   const bool single = mode != kSelGroups;
   // a pass over the groups also starts the fallback's select (the groups'
   // final take counts are known here)
@@ -2255,6 +2251,13 @@ __global__ void __launch_bounds__(1024) k_list_finish(DevState s, int fallback) 
     if ((threadIdx.x >> 5) == 0) start_global_select(s, c, 1);
   }
 }
+__global__ void __launch_bounds__(1024) k_list_finish(DevState s, int fallback) {
+  s = with_args(s);
+  extern __shared__ __align__(16) unsigned char fin_smem[];
+  const int64_t n = s.ctl->lst_n;  // in the mode's round trip
+  const int mode = select_mode(s.ctl, fallback);
+  if (mode >= 0) list_finish(s, s.ctl, fin_smem, mode, n);
+}
 
 // TakeTrueFree (Alg. 2) and the step's id lists (allocated, evicted,
 // invalidated), all ascending, from the bitmaps.  Each CTA owns kBmChunk
@@ -2315,14 +2318,11 @@ __device__ __forceinline__ void write_ids(const DevState& s, const ListSmem& sm,
   }
 }
 constexpr int kBmThreads = 512;
-__global__ void __launch_bounds__(kBmThreads, 3) k_bm_write(DevState s) {
-  s = with_args(s);
-  __shared__ ListSmem sm;
-  Ctl* c = s.ctl;
+template <int NT>  // threads of the CTA
+__device__ __forceinline__ void list_chunk(const DevState& s, Ctl* c, ListSmem& sm, int chunk, int nchunks) {
   const int32_t st = c->status;
   const int t = (int)threadIdx.x;
-  const int64_t w0 = (int64_t)blockIdx.x * kBmChunk, w = w0 + t;
-  const int nchunks = gridDim.x;
+  const int64_t w0 = (int64_t)chunk * kBmChunk, w = w0 + t;
   const bool in = t < kBmChunk && w < s.nwords;  // the first kBmChunk threads hold a word each
   const int64_t ftake = c->ftake;
   const uint32_t vic = in ? s.bm_victim[w] : 0u, inv = in ? s.bm_inval[w] : 0u;
@@ -2330,17 +2330,17 @@ __global__ void __launch_bounds__(kBmThreads, 3) k_bm_write(DevState s) {
   if (st != PS_OK) return;
   // earlier chunks' free, evicted and invalidated ids
   int64_t fb = 0, vb = 0, ib = 0;
-  for (int j = t; j < (int)blockIdx.x; j += kBmThreads) {  // (none in a single chunk)
+  for (int j = t; j < chunk; j += NT) {  // (none in a single chunk)
     fb += s.bm_chunk_cnt[0 * nchunks + j];
     vb += s.bm_chunk_cnt[1 * nchunks + j];
     ib += s.bm_chunk_cnt[2 * nchunks + j];
   }
   {
-    __shared__ int64_t s_before[3][kBmThreads / 32];
+    __shared__ int64_t s_before[3][NT / 32];
     fb = warp_sum(fb); vb = warp_sum(vb); ib = warp_sum(ib);
     if (lane_id() == 0) { s_before[0][t >> 5] = fb; s_before[1][t >> 5] = vb; s_before[2][t >> 5] = ib; }
     __syncthreads();
-    const bool hold = lane_id() < kBmThreads / 32;
+    const bool hold = lane_id() < NT / 32;
     fb = warp_sum(hold ? s_before[0][lane_id()] : (int64_t)0);
     vb = warp_sum(hold ? s_before[1][lane_id()] : (int64_t)0);
     ib = warp_sum(hold ? s_before[2][lane_id()] : (int64_t)0);
@@ -2368,12 +2368,108 @@ __global__ void __launch_bounds__(kBmThreads, 3) k_bm_write(DevState s) {
     sm.base[1][t] = (int32_t)(vb + field3(ex1, 1));
     sm.base[2][t] = (int32_t)(ib + field3(ex1, 2));
   }
-  if (blockIdx.x == nchunks - 1 && t == 0) {
+  if (chunk == nchunks - 1 && t == 0) {
     c->n_alloc = vb + tmin(ftake, fb) + take_here + field3(tot1, 1);
     c->n_evicted = vb + field3(tot1, 1);
   }
   __syncthreads();
   write_ids(s, sm, w0, (int)tmin<int64_t>(kBmChunk, s.nwords - w0));
+}
+__global__ void __launch_bounds__(kBmThreads, 3) k_bm_write(DevState s) {
+  s = with_args(s);
+  __shared__ ListSmem sm;
+  list_chunk<kBmThreads>(s, s.ctl, sm, blockIdx.x, gridDim.x);
+}
+
+// The whole select of a small pool, and its id lists, by one CTA: the stage
+// kernels above as phases between CTA barriers.  With a few thousand blocks
+// each of those kernels is a launch and a chain of dependent loads around a
+// few hundred instructions, ten launches under PrefixShield (four of them the
+// fallback's, which mostly finds nothing to do) and six under LRU.
+// Measured a step, stage kernels against this: prefixshield over 512 blocks
+// 55.9 -> 50.7 us, over 2048 59.5 -> 53.4, over 4096 66.2 -> 65.5 (2 groups)
+// and 62.6 -> 57.0 (32); over 8192 it lost from 16 groups on (65.7 -> 72.7 us
+// with 32).  LRU has no fallback to skip: 50.7 -> 48.3 us over 512 blocks,
+// 53.7 -> 53.1 over 2048, 56.4 -> 57.1 over 4096.  StaticQuota selects in
+// every group on every step, which one CTA does more slowly (2048 blocks,
+// 8 groups: 57.5 -> 58.5 us; 32 groups: 58.7 -> 65.2), so it is left alone.
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallPool = 4 * kSmallThreads;     // one batch of loads a thread in the counts and in the split
+constexpr int kSmallPoolLru = 2 * kSmallThreads;
+constexpr int kSmallGroups = kSmallThreads / 32;  // a warp for each segment
+inline bool small_select(const DevState& s) {
+  if (s.lg_on) return false;
+  return s.policy == PS_PREFIXSHIELD ? s.N <= kSmallPool && s.G <= kSmallGroups
+                                     : s.policy == PS_LRU && s.N <= kSmallPoolLru;
+}
+// select_resolve by one warp, 128 buckets at a time.
+__device__ __forceinline__ void select_resolve_warp(const DevState& s, int g) {
+  const SelSeg z = s.sel[g];
+  if (!z.active) return;
+  const int lane = lane_id();
+  uint4* bins = reinterpret_cast<uint4*>(s.dig_bins + (size_t)g * kDigBins) + lane;
+  const uint64_t rank = (uint64_t)z.rank;
+  uint64_t before = 0;
+  constexpr int kV = 8;  // loads in flight
+  for (int k0 = 0; k0 < kDigBins / 128; k0 += kV) {
+    uint4 v[kV];
+#pragma unroll
+    for (int u = 0; u < kV; ++u) v[u] = __ldcg(bins + 32 * (k0 + u));
+#pragma unroll
+    for (int u = 0; u < kV; ++u) {
+      bins[32 * (k0 + u)] = make_uint4(0, 0, 0, 0);
+      const uint32_t sum = v[u].x + v[u].y + v[u].z + v[u].w;
+      if (!__any_sync(kFull, sum != 0)) continue;
+      const uint32_t incl = warp_incl_scan(sum);
+      uint64_t run = before + incl - sum;
+      if (run < rank && rank <= run + sum) {  // one lane
+        uint32_t d = 128u * (uint32_t)(k0 + u) + 4u * (uint32_t)lane;
+        if (rank > run + v[u].x) { run += v[u].x; ++d;
+          if (rank > run + v[u].y) { run += v[u].y; ++d;
+            if (rank > run + v[u].z) { run += v[u].z; ++d; } } }
+        const int sh = bucket_shift(z.kmin, z.kmax);
+        SelSeg* o = s.sel + g;
+        o->blo = z.kmin + ((uint64_t)d << sh);
+        o->bhi = tmin<uint64_t>(o->blo + ((1ull << sh) - 1), z.kmax);
+        o->rank = (int64_t)(rank - run);
+      }
+      before += __shfl_sync(kFull, incl, 31);
+    }
+  }
+}
+__device__ __forceinline__ void small_pass(const DevState& s, Ctl* c, unsigned char* smem, int mode, int fallback) {
+  select_count(s, *reinterpret_cast<CountSmem*>(smem), mode, fallback, 0, 1);
+  __syncthreads();
+  if (mode == kSelGroups) {
+    const int g = (int)(threadIdx.x >> 5);
+    if (g < s.G) select_resolve_warp(s, g);
+  } else {
+    const SelSeg z = s.sel[0];
+    select_resolve(s, 0, z);
+  }
+  __syncthreads();
+  select_split(s, c, *reinterpret_cast<SplitSmem*>(smem), mode, fallback, 0, 1);
+  __syncthreads();
+  list_finish(s, c, smem, mode, c->lst_n);
+  __syncthreads();
+}
+__global__ void __launch_bounds__(kSmallThreads) k_small_select(DevState s0) {
+  const DevState s = with_args(s0);
+  extern __shared__ __align__(16) unsigned char fin_smem[];
+  Ctl* c = s.ctl;
+  if (s.policy == PS_LRU) {
+    if (threadIdx.x < 32) start_global_select(s, c, 0);
+  } else {
+    waterfill(s, s0, c);
+  }
+  __syncthreads();
+  const int mode = select_mode(c, 0);
+  if (mode >= 0) {
+    small_pass(s, c, fin_smem, mode, 0);
+    const int again = s.policy == PS_PREFIXSHIELD ? select_mode(c, 1) : -1;
+    if (again >= 0) small_pass(s, c, fin_smem, again, 1);
+  }
+  list_chunk<kSmallThreads>(s, c, *reinterpret_cast<ListSmem*>(fin_smem), 0, 1);
 }
 
 // Stage 6: place granted claims, a thread per claim of the step (k_instep
@@ -2552,6 +2648,7 @@ static int32_t launch_hash_lookup(const DevState& s, cudaStream_t st, int32_t* p
 void configure_kernels(const DevState& s) {
   (void)s;
   cudaFuncSetAttribute(k_list_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFinSmem);
+  cudaFuncSetAttribute(k_small_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFinSmem);
   cudaFuncSetAttribute(k_cand, cudaFuncAttributeMaxDynamicSharedMemorySize, PS_MAX_GROUPS * kClasses * 5 * 4);
   cudaFuncSetAttribute(k_grant, cudaFuncAttributeMaxDynamicSharedMemorySize, PS_MAX_GROUPS * PS_MAX_CONTRACTS * 8);
 }
@@ -2672,8 +2769,12 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
     PS_LAUNCH(launch_k(k_sel_split, cgrid, 256, 0, st, s, fallback));
     PS_LAUNCH(launch_k(k_list_finish, 1, 1024, kFinSmem, st, s, fallback));
   };
+  // stage timing tells the select from the lists, so it runs them apart
+  const bool one_cta = small_select(s) && !(tr && tr->timing);
   if (s.lg_on) {
     // selected above
+  } else if (one_cta) {
+    PS_LAUNCH(k_small_select<<<1, kSmallThreads, kFinSmem, st>>>(s));  // after the join: plain
   } else if (s.policy == PS_PREFIXSHIELD) {
     PS_LAUNCH(k_waterfill<<<1, 1024, 0, st>>>(s));  // after the join: plain
     select(0);
@@ -2706,7 +2807,9 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
     if (fork3) PS_LAUNCH((k_bm_count<<<nchunks, kBmChunk, 0, st>>>(s)));  // after the fork: plain
     else PS_LAUNCH(launch_k(k_bm_count, nchunks, kBmChunk, 0, st, s));
   }
-  if (fork3 && nchunks == 1) PS_LAUNCH((k_bm_write<<<nchunks, kBmThreads, 0, st>>>(s)));
+  if (one_cta) {
+    // listed already
+  } else if (fork3 && nchunks == 1) PS_LAUNCH((k_bm_write<<<nchunks, kBmThreads, 0, st>>>(s)));
   else PS_LAUNCH(launch_k(k_bm_write, nchunks, kBmThreads, 0, st, s));
   mark(8);
   // (evictions happen in k_insert: every victim is allocated again in its step)
