@@ -318,7 +318,7 @@ int32_t ps_get_stage_times(ps_handle_t* h, float* h_ms, int32_t max_stages, int3
 
 /* 1 if the handle replays its step as one captured CUDA graph (the step's
  * per-call arguments live in a device block that every kernel reads, so one
- * graph serves every step; phases many steps skip are conditional nodes), 0
+ * graph serves every step; a phase that a step skips returns at once), 0
  * if it launches kernel by kernel (the graph could not be captured or
  * instantiated: results are the same).  Known after the first ps_step().
  * Measurement hook; the paper has no counterpart. */
@@ -326,8 +326,8 @@ int32_t ps_uses_graph(const ps_handle_t* h);
 
 /* Launch mode of ps_step(): enable = 1 (the default) replays the step as one
  * captured CUDA graph, enable = 0 launches its kernels one by one on the
- * caller's stream (for profilers that cannot see inside graphs with
- * conditional nodes).  The same kernels do the same work either way.
+ * caller's stream (for profilers that cannot see inside graphs).  The same
+ * kernels do the same work either way.
  * Measurement hook; the paper has no counterpart. */
 int32_t ps_set_graph(ps_handle_t* h, int32_t enable);
 

@@ -1,0 +1,214 @@
+"""The step's size-dependent branches against the oracle, at the sizes where
+each begins, ends or leaves a remainder.  Every output, the exported state and
+the statistics are whole numbers: the tolerance is zero.
+"""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2608_01657_gb300 import workloads as W
+from _util import compare_outputs, compare_state
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _pair(N, bs, G, policy, params_kw, max_requests, max_tokens):
+    from paper_2608_01657_gb300 import binding as B
+    gpu = B.Cache(N, bs, G, policy, B.Params(**params_kw), max_requests=max_requests, max_tokens=max_tokens)
+    return gpu, O.OracleCache(N, bs, G, policy, O.Params(**params_kw))
+
+
+def _run(gpu, orc, steps, state_every=8, label=""):
+    dev = torch.device("cuda")
+    for k, st in enumerate(steps):
+        g = torch.from_numpy(st.groups).to(dev)
+        o = torch.from_numpy(st.offsets).to(dev)
+        t = torch.from_numpy(st.tokens if st.num_tokens else np.zeros(4, np.int32)).to(dev)
+        c = None if st.contracts is None else torch.from_numpy(st.contracts).to(dev)
+        p = None if st.prefixes is None else torch.from_numpy(st.prefixes.view(np.int64)).to(dev)
+        assert gpu.step(st.now, g, o, t, c, p) == 0, f"{label} step {k}"
+        want = orc.step(st.now, st.groups, st.offsets, st.tokens, st.contracts, st.prefixes)
+        compare_outputs(gpu.fetch(st.num_requests), want, f"{label} step {k}")
+        if k % state_every == state_every - 1 or k == len(steps) - 1:
+            compare_state(gpu.export(), orc.export(), f"{label} step {k}", s3=gpu.policy == "s3fifo")
+    assert np.array_equal(gpu.stats(), orc.stats()), f"{label}: stats differ"
+    return orc.stats()
+
+
+def _evicted(stats):
+    return int(stats[:, O.STAT_NAMES.index("evicted_blocks")].sum())
+
+
+def _prompts(lengths, groups, seed, docs=None):
+    """One step's prompts: `lengths` tokens each, the first from documents."""
+    rng = np.random.default_rng(seed)
+    pieces = []
+    for k, n in enumerate(lengths):
+        if docs is not None and k % 2 == 0:
+            d = docs[k % len(docs)]
+            pieces.append(np.concatenate([d[:n], rng.integers(0, W.VOCAB, size=max(0, n - len(d)), dtype=np.int32)]))
+        else:
+            pieces.append(rng.integers(0, W.VOCAB, size=n, dtype=np.int32))
+    off = np.concatenate([[0], np.cumsum([len(p) for p in pieces])]).astype(np.int64)
+    toks = np.concatenate(pieces).astype(np.int32) if pieces else np.zeros(0, np.int32)
+    return np.asarray(groups, np.int32), off, toks
+
+
+@pytest.mark.parametrize("policy,N,G,beta", [
+    ("prefixshield", 511, 1, 4.0), ("prefixshield", 4096, 2, 40.0), ("prefixshield", 4097, 2, 40.0),
+    ("prefixshield", 2000, 32, 8.0), ("prefixshield", 2000, 33, 8.0), ("prefixshield", 31, 3, 1e6),
+    ("lru", 2048, 2, 8.0), ("lru", 2049, 2, 8.0), ("lru", 1, 1, 8.0)])
+def test_small_pool_select(policy, N, G, beta):
+    """The one-CTA select and lists, at and past the largest pool and number
+    of groups; large balances (no debt) leave every victim to the fallback."""
+    steps = W.fuzz_steps(N + G, G, 12, 40, docs_per_group=2, doc_blocks=max(2, N // 24), now_stride=2,
+                         fresh_max_blocks=max(2, N // 16), empty_every=11)
+    gpu, orc = _pair(N, 16, G, policy, dict(rho=(1.0,), beta=(beta,)), 12, 12 * 16 * (N // 24 + N // 16 + 8))
+    assert _evicted(_run(gpu, orc, steps, label=f"{policy}/{N}/{G}")) > 0
+
+
+@pytest.mark.parametrize("N", [8191, 8192, 8193, 16400])
+@pytest.mark.parametrize("policy", ["lru", "staticquota"])
+def test_id_lists_at_chunk_edges(policy, N):
+    """Free, evicted and invalidated ids over one chunk of 8192 ids, a last
+    partial word, and a second chunk."""
+    steps = W.fuzz_steps(N, 2, 8, 24, docs_per_group=2, doc_blocks=N // 16, fresh_max_blocks=N // 12, now_stride=2)
+    gpu, orc = _pair(N, 16, 2, policy, dict(rho=(2.0,), beta=(64.0,)), 8, 8 * 16 * (N // 16 + N // 12 + 2))
+    assert _evicted(_run(gpu, orc, steps, label=f"lists/{policy}/{N}")) > 0
+
+
+@pytest.mark.parametrize("max_blocks", [64 * 152, 64 * 153, 64 * 608 + 64, 64 * 1300])
+@pytest.mark.parametrize("bs", [8, 16, 32])
+def test_hashing_widths_and_chunk_edges(bs, max_blocks):
+    """CTAs of one to eight hashing warps (chosen by the handle's bound), with
+    prompts of 0 to 130 blocks around the half (32) and the chunk (64), at
+    every offset of a prompt's first token in its 16-byte word."""
+    blocks = [0, 1, 2, 31, 32, 33, 63, 64, 65, 96, 127, 128, 129, 130]
+    rng = np.random.default_rng(bs)
+    docs = [rng.integers(0, W.VOCAB, size=130 * bs, dtype=np.int32) for _ in range(2)]
+    steps = []
+    for k in range(4):
+        lengths = [b * bs + int(rng.integers(0, bs)) for b in blocks]
+        g, o, t = _prompts(lengths, [i % 2 for i in range(len(blocks))], 10 * bs + k, docs)
+        steps.append(W.Step(k, k, g, o, t, None, None))
+    gpu, orc = _pair(2500, bs, 2, "prefixshield", dict(rho=(1.0,), beta=(50.0,)), len(blocks), max_blocks * bs)
+    _run(gpu, orc, steps, 1, f"hash/{bs}/{max_blocks}")
+
+
+@pytest.mark.parametrize("R,max_blocks", [(300, 4), (64, 8), (5, 512)])
+def test_more_requests_than_blocks(R, max_blocks):
+    """Claims and history entries share the insertion's threads: more requests
+    than blocks in a step, and the other way round, most of them empty or hits."""
+    rng = np.random.default_rng(R)
+    doc = rng.integers(0, W.VOCAB, size=max_blocks * 16, dtype=np.int32)
+    steps = []
+    for k in range(12):
+        n = int(rng.integers(1, max_blocks + 1))
+        lengths = [0] * R
+        lengths[int(rng.integers(0, R)) & ~1] = n * 16
+        g, o, t = _prompts(lengths, rng.integers(0, 3, size=R), k, [doc])
+        steps.append(W.Step(k, k, g, o, t, None, None))
+    gpu, orc = _pair(max_blocks + 2, 16, 3, "prefixshield", dict(rho=(1.0,), beta=(2.0,)), R, max_blocks * 16)
+    _run(gpu, orc, steps, 1, f"R/{R}")
+
+
+@pytest.mark.parametrize("G,contracts", [(2, 1), (40, 3), (1000, 3)])
+def test_many_indebted_groups(G, contracts):
+    """The water-filling's search with one, some and a thousand groups in debt
+    (a thread a group), whole groups taken and partial ones."""
+    steps = W.fuzz_steps(G, G, 64, 24, docs_per_group=1, doc_blocks=6, fresh_max_blocks=12,
+                         with_contracts=contracts if contracts > 1 else 0, now_stride=2)
+    rho, beta = (0.5, 1.0, 2.0)[:contracts], (1.0, 3.0, 2.0)[:contracts]
+    kw = dict(rho=rho, beta=beta, contract_of_group=[g % contracts for g in range(G)])
+    gpu, orc = _pair(4500, 16, G, "prefixshield", kw, 64, 64 * 16 * 19)
+    assert _evicted(_run(gpu, orc, steps, label=f"debt/{G}")) > 0
+
+
+@pytest.mark.parametrize("gap", [0, 3000])
+@pytest.mark.parametrize("need", [40, 1500])
+def test_list_finish_widths(gap, need):
+    """A select's list: dense stamps leave a few members a segment; stamps
+    spread by many hits (gap steps' worth) leave hundreds in one bucket, which
+    a bitmap of the bucket ranks."""
+    rng = np.random.default_rng(gap + need)
+    doc = rng.integers(0, W.VOCAB, size=3000 * 16, dtype=np.int32)
+    other = rng.integers(0, W.VOCAB, size=2000 * 16, dtype=np.int32)
+    fresh = rng.integers(0, W.VOCAB, size=need * 16, dtype=np.int32)
+    seq = [doc, other] + [other] * (gap // 60) + [rng.integers(0, W.VOCAB, size=10 * 16, dtype=np.int32), fresh]
+    steps = [W.Step(k, k, np.zeros(1, np.int32), np.array([0, len(t)], np.int64), t, None, None)
+             for k, t in enumerate(seq)]
+    gpu, orc = _pair(5020, 16, 2, "prefixshield", dict(rho=(1.0,), beta=(100.0,)), 1, 3000 * 16)
+    assert _evicted(_run(gpu, orc, steps, 16, f"finish/{gap}/{need}")) >= need - 10
+
+
+@pytest.mark.parametrize("N,blocks", [(64, 12), (2000, 400)])
+def test_s3fifo_ghost_readmission(N, blocks):
+    """Keys evicted and asked for again: ghost hits, among them keys that two
+    requests of a step share and keys that the same step trims."""
+    steps = W.fuzz_steps(N, 2, 5, 40, docs_per_group=3, doc_blocks=blocks, fresh_max_blocks=blocks // 4, now_stride=2)
+    gpu, orc = _pair(N, 16, 2, "s3fifo", dict(rho=(2.0,), beta=(6.0,)), 5, 5 * 16 * (2 * blocks + 2))
+    assert _evicted(_run(gpu, orc, steps, label=f"ghost/{N}")) > 0
+
+
+@pytest.mark.parametrize("policy", ["lru", "prefixshield"])
+def test_queue_logs_fill_and_compact(policy):
+    """Indexed queues whose logs run full again and again."""
+    steps = W.fuzz_steps(3, 3, 8, 300, docs_per_group=3, doc_blocks=6, fresh_max_blocks=1, now_stride=2)
+    gpu, orc = _pair(40, 16, 3, policy, dict(rho=(2.0,), beta=(6.0,), flags=O.FLAG_INDEXED_QUEUES), 8, 4096)
+    assert _evicted(_run(gpu, orc, steps, 25, f"queues/{policy}")) > 0
+
+
+@pytest.mark.parametrize("R", [1, 7, 600])
+def test_probe_edges(R):
+    """Prompts without a full block count 0 whatever the output held; a call
+    with an invalid request reports it and leaves the outputs untouched."""
+    rng = np.random.default_rng(R)
+    lengths = [int(n) for n in rng.choice([0, 5, 16, 40, 100 * 16 + 3], size=R)]
+    g, o, t = _prompts(lengths, rng.integers(0, 2, size=R), R, [rng.integers(0, W.VOCAB, size=1700, dtype=np.int32)])
+    gpu, orc = _pair(9000, 16, 2, "lru", dict(rho=(1.0,), beta=(1.0,)), R, max(64, len(t)))
+    dev = torch.device("cuda")
+    half = slice(0, max(1, R // 2))
+    n = len(g[half])
+    first = (g[half], o[:n + 1], t[:o[n]])
+    gg, oo, tt = (torch.from_numpy(np.ascontiguousarray(x)).to(dev) for x in (g, o, t if len(t) else np.zeros(4, np.int32)))
+    assert gpu.step(0, gg[:n], oo[:n + 1], tt) == 0
+    compare_outputs(gpu.fetch(n), orc.step(0, *first), "first")
+    out = torch.full((R,), -7, dtype=torch.int32, device=dev)
+    _, status = gpu.cached_prefix(gg, oo, tt, out=out)
+    assert int(status.item()) == 0
+    assert np.array_equal(out.cpu().numpy(), orc.cached_prefix(g, o, t))
+    bad = gg.clone()
+    bad[R - 1] = 2
+    out.fill_(-7)
+    _, status = gpu.cached_prefix(bad, oo, tt, out=out)
+    assert int(status.item()) == O.ERR_INVALID_ARG and bool((out == -7).all())
+
+
+@pytest.mark.parametrize("tokens_pinned,outputs_pinned,shift", [
+    (True, True, 0), (True, True, 1), (True, False, 0), (False, True, 0), (False, False, 3)])
+def test_step_host_buffers(tokens_pinned, outputs_pinned, shift):
+    """Page-locked buffers (read and written by kernels), pageable ones
+    (copied), mixtures, and token buffers off a 16-byte boundary."""
+    from paper_2608_01657_gb300 import binding as B
+    steps = W.fuzz_steps(61, 3, 5, 16, docs_per_group=3, doc_blocks=6, with_contracts=2, with_prefixes=True, empty_every=7)
+    kw = dict(rho=(2.0, 1.0), beta=(6.0, 3.0), contract_of_group=[0, 1, 0])
+    gpu, orc = _pair(40, 16, 3, "prefixshield", kw, 5, 2048)
+
+    def host(x, by=0):
+        buf = torch.empty(len(x) + by + 4, dtype=torch.from_numpy(x[:0]).dtype, pin_memory=tokens_pinned).numpy()
+        buf[by:by + len(x)] = x
+        return buf[by:by + len(x)]
+
+    for st in steps:
+        out = B.host_outputs(5, gpu.max_blocks, 3, pinned=outputs_pinned)
+        R = st.num_requests
+        res = gpu.step_host(st.now, host(st.groups), host(st.offsets), host(st.tokens, shift), host(st.contracts),
+                            host(st.prefixes.view(np.int64)), out=out)
+        assert res["rc"] == 0
+        cnt = out["counts"]
+        got = {"status": int(cnt[3]), "hit_blocks": out["hit_blocks"][:R], "admitted_blocks": out["admitted_blocks"][:R],
+               "admitted_offsets": out["admitted_offsets"][:R + 1], "admitted_ids": out["admitted_ids"][:cnt[0]],
+               "evicted_ids": out["evicted_ids"][:cnt[1]], "invalidated_ids": out["invalidated_ids"][:cnt[2]],
+               "debt_raw": out["debt_raw"], "debt_norm": out["debt_norm"]}
+        compare_outputs(got, orc.step(st.now, st.groups, st.offsets, st.tokens, st.contracts, st.prefixes), f"step {st.index}")
