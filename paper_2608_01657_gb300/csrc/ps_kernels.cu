@@ -227,7 +227,9 @@ __device__ void table_delete(const DevState& s, uint32_t blk) {
 // ---- per-step claim map ------------------------------------------------------
 // The bucket's keys are loaded first, so the many requests that claim one
 // popular key in a step mostly find it with a plain load and swap nothing
-// (a swap first would serialize them on one address).
+// (a swap first would serialize them on one address).  Keys kept apart from
+// the entries, a bucket's in one sector, took 171 us a step at 2^20 blocks
+// against 155: a second scattered line a claim costs more than the sectors.
 __device__ uint32_t claim_insert(const DevState& s, uint64_t key, uint32_t req) {
   const uint32_t mask = (1u << s.cl_nbuckets_log2) - 1;
   uint32_t b = claim_home(key, s.cl_nbuckets_log2);
@@ -759,6 +761,14 @@ __device__ __forceinline__ bool hash_lookup_chunk(const DevState& s, Ctl* c, con
 // (lower tickets) have always started hashing before it, and their totals
 // arrive about when its own does.  A chunk waits only on chunks of lower
 // tickets, each held by a running warp: the waits always make progress.
+// What bounds it: the memory system under scattered accesses, not instructions
+// (28% of issue slots) or DRAM bandwidth (20%).  Clocks read inside it at 2^20
+// blocks, in thousands of cycles a chunk: ticket 12, descriptor 3, tokens and
+// digests 13, scan 4, predecessors' totals 9, table 20, predecessors' misses 8,
+// pins and claims 14.  Measured there and not kept (155 us a step): tokens read
+// coalesced, four lanes a block (159 to 171), a CTA's first tickets drawn at
+// once (156), a warp's next ticket drawn early (158), two claims at a time
+// (155), no way loaded before its tag matched (155).
 // probe_out: the read-only probe (ps_cached_prefix) stores h_i there; no pins,
 // claims, history or per-position records.
 constexpr int kHashCtasPerSm = 5;

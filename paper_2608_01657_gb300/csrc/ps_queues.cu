@@ -520,7 +520,7 @@ __device__ __forceinline__ void lg_cmp_live(const DevState& s, Ctl* c, int l) {
   }
   if (threadIdx.x == 0) {
     if (before != s.lg_live[l]) c->internal_error = 1;  // the live count drifted
-    s.lg_new[l].tail = before;  // live count, for k_lg_cmp_layout
+    s.lg_new[l].tail = before;  // live count, for lg_cmp_layout
   }
 }
 
