@@ -614,15 +614,24 @@ __device__ __forceinline__ bool hash_lookup_chunk(const DevState& s, Ctl* c, con
   // D_m of the lane's two blocks, then the inclusive scans of the affine maps
   // x -> Kc x + D, one per half
   uint64_t bA = 0, bB = 0;
-  if (lane < nbA) {
-    uint64_t d1, d2;
-    block_nh<BS>(s, sk, o0 + (int64_t)mA * BS, (int)(o0 & 3), s.tokens_aligned16 != 0, T, &d1, &d2);
-    bA = mad61(s.digest_mul, weak61(d2), weak61(d1));
-  }
+  // The halves' digests in a rolled loop: half the code, and no spills (155.2 ->
+  // 152.8 us a step at 2^20 blocks; it cost 0.4 us with a few chunks in all).
+  // The second half's tokens are on their way from DRAM meanwhile (-> 152.2).
   if (lane < nbB) {
-    uint64_t d1, d2;
-    block_nh<BS>(s, sk, o0 + (int64_t)mB * BS, (int)(o0 & 3), s.tokens_aligned16 != 0, T, &d1, &d2);
-    bB = mad61(s.digest_mul, weak61(d2), weak61(d1));
+    const int32_t* src = s.in_tokens + o0 + (int64_t)mB * BS;
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(src));
+    if (BS >= 16) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + BS / 2));
+  }
+#pragma unroll 1
+  for (int half = 0; half < 2; ++half) {
+    uint64_t D = 0;
+    if (lane < (half ? nbB : nbA)) {
+      uint64_t d1, d2;
+      block_nh<BS>(s, sk, o0 + (int64_t)(half ? mB : mA) * BS, (int)(o0 & 3), s.tokens_aligned16 != 0, T, &d1, &d2);
+      D = mad61(s.digest_mul, weak61(d2), weak61(d1));
+    }
+    if (half) bB = D;
+    else bA = D;
   }
 #pragma unroll
   for (int q = 0; q < 5; ++q) {
