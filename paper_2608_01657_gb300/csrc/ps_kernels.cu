@@ -678,6 +678,19 @@ __device__ __forceinline__ bool hash_lookup_chunk(const DevState& s, Ctl* c, con
     keyB = fix_reserved(mix64(C ^ ((uint64_t)(mB + 1) * 0xD1B54A32D192ED03ull)));
   }
   table_find2(s, keyA, keyB, g, lane < nbA, lane < nbB, &blkA, &blkB);
+  // What place() below swaps is fetched into L2 while the warp waits for its
+  // predecessors' misses: a hit's pin, a miss's claim bucket (152.6 -> 149.8 us
+  // a step at 2^20 blocks).  A hit past the first miss is claimed after all and
+  // only goes without.
+  auto ahead = [&](uint64_t key, uint32_t blk) {
+    const void* p = blk == kNone ? (const void*)(s.claims + (size_t)claim_home(key, s.cl_nbuckets_log2) * kClaimWays)
+                                 : (const void*)(s.blk_pin + blk);
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+  };
+  if (!probe_out) {
+    if (lane < nbA) ahead(keyA, blkA);
+    if (lane < nbB) ahead(keyB, blkB);
+  }
   const unsigned missA = __ballot_sync(kFull, lane < nbA && blkA == kNone);
   const unsigned missB = __ballot_sync(kFull, lane < nbB && blkB == kNone);
   const bool anymiss = (missA | missB) != 0;
