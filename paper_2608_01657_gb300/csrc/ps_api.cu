@@ -274,7 +274,7 @@ size_t carve(const Dims& d, char* base, DevState* s, ps_handle* h) {
   t.grp_full = cv.take<uint8_t>(G);
   t.sel = cv.take<SelSeg>(G);
   t.cls = cv.take<ClsRange>(G * kClasses);
-  t.dig_bins = cv.take<uint32_t>(G * kDigBins);
+  t.dig_bins = cv.take<uint32_t>(G << dig_row_bits(d.N, d.G));
   t.lst_key = cv.take<uint64_t>(N);
   t.lst_blk = cv.take<uint32_t>(N);
   t.lst_seg = cv.take<uint16_t>(N);

@@ -179,9 +179,17 @@ constexpr int kClasses = 3;
 // segment beside groups that are taken whole.  (Its second pass, the fallback
 // after a pass of group segments, is global over what that left.)
 constexpr int32_t kSelGroups = 0, kSelGlobal = 1, kSelWhole = 2;
-// Buckets a select cuts a segment's key range into.
-constexpr int kDigBits = 12;
+// Buckets a select cuts a segment's key range into: 2^kDigBits, or 2^kWideBits
+// where the range has more than kWideRange bits and the handle has counters for
+// that (more blocks than kWidePool, at most kWideGroups groups).
+constexpr int kDigBits = 12, kWideBits = 16, kWideRange = 25;
 constexpr int kDigBins = 1 << kDigBits;
+constexpr int64_t kWidePool = 4096;
+constexpr int kWideGroups = 64;
+// Counters of one segment, as a power of two.
+__host__ __device__ __forceinline__ int dig_row_bits(int64_t N, int32_t G) {
+  return N > kWidePool && G <= kWideGroups ? kWideBits : kDigBits;
+}
 
 // ---- S3-FIFO as sequence-ordered arrays ------------------------------------
 // Both queues are arrays of block ids in sequence order (oldest first),
@@ -335,7 +343,7 @@ struct DevState {
   uint8_t* grp_full;       // the debt phase takes all of the group's candidates
   SelSeg* sel;             // [G] segments
   ClsRange* cls;           // [G * kClasses] candidates per (segment, class)
-  uint32_t* dig_bins;      // [G][kDigBins] candidates per bucket (zero between selects)
+  uint32_t* dig_bins;      // [G][2^dig_row_bits] candidates per bucket (zero between selects)
   uint64_t* lst_key;       // split list of the select: key, block, segment
   uint32_t* lst_blk;
   uint16_t* lst_seg;

@@ -1787,8 +1787,8 @@ __global__ void __launch_bounds__(PS_MAX_GROUPS) k_waterfill(DevState s0) {
 // Each active segment (a group in the debt phase, one global segment for lru
 // and for the fallback) looks for the rank-th smallest key among its
 // candidates of one class.  The class's key range [kmin, kmax] is cut into
-// kDigBins equal buckets (a power of two wide), the candidates are counted by
-// bucket, and the bucket holding the rank is found; candidates below it are
+// 4096 or 65536 equal buckets (a power of two wide), the candidates are counted
+// by bucket, and the bucket holding the rank is found; candidates below it are
 // victims, its members go to a short list that one CTA finishes exactly.
 //
 // Stamps are dense (a step's blocks take consecutive ones), so a range cut
@@ -1799,11 +1799,42 @@ __global__ void __launch_bounds__(PS_MAX_GROUPS) k_waterfill(DevState s0) {
 // histogram beside it.  Measured a step, byte digits against this: staticquota
 // over 100,003 blocks 90.2 -> 82.0 us, prefixshield over 256 blocks 76.2 ->
 // 71.9 us and over 2^20 blocks 186.3 -> 184.5 us (the launches dominate).
+//
+// A class that holds blocks much older than the rest has a range far wider than
+// its dense parts (a group that stood idle, a pool of hot prompts that starts to
+// turn over), and a 4096th of it can hold most of a step's blocks: a list of
+// thousands of members for the one CTA of list_finish.  Past 2^kWideRange stamps
+// a segment is therefore cut into 65536 buckets.  Measured a step of the
+// 2^20-block workloads whose stamps jump by a gap before every step, the pool
+// holding a few such gaps, 4096 buckets against 65536: lru 155 -> 151 us at a
+// gap of 2^22, 198 -> 154 at 2^25, 413 -> 173 at 2^28, 597 -> 230 at 2^30;
+// prefixshield of 2 groups 118 -> 112, 251 -> 118, 304 -> 179, 306 -> 290.  At a
+// range of 2^22 and below the longer resolve shows instead (149 -> 155, 108 ->
+// 116).  2^25 is where a bucket (2^13 stamps) still leaves room for 64 groups'
+// bitmaps in list_finish.  Counters for 65536 buckets are 16 MB at 64 groups; a
+// handle of more groups, whose segments are shorter, keeps 4096, and so does a
+// pool whose whole list fits one CTA's shared memory (4096 blocks: no
+// difference at any gap).
 
+// SMALL: of a pool of at most kWidePool blocks.
+template <bool SMALL>
+__device__ __forceinline__ int dig_row_log2(const DevState& s) {
+  return SMALL ? kDigBits : dig_row_bits(s.N, s.G);
+}
+// A segment whose range takes 2^kWideBits buckets.
+template <bool SMALL>
+__device__ __forceinline__ bool wide_range(const DevState& s, uint64_t kmin, uint64_t kmax) {
+  return ((kmax - kmin) >> kWideRange) != 0 && dig_row_log2<SMALL>(s) == kWideBits;
+}
 // The bucket width of a range, as a shift.
-__device__ __forceinline__ int bucket_shift(uint64_t kmin, uint64_t kmax) {
-  const int bits = 64 - __clzll((long long)(kmax - kmin));
-  return bits > kDigBits ? bits - kDigBits : 0;
+template <bool SMALL>
+__device__ __forceinline__ int bucket_shift(const DevState& s, uint64_t kmin, uint64_t kmax) {
+  const int bits = 64 - __clzll((long long)(kmax - kmin)), dig = wide_range<SMALL>(s, kmin, kmax) ? kWideBits : kDigBits;
+  return bits > dig ? bits - dig : 0;
+}
+template <bool SMALL>
+__device__ __forceinline__ uint4* dig_row(const DevState& s, int g) {
+  return reinterpret_cast<uint4*>(s.dig_bins + ((size_t)g << dig_row_log2<SMALL>(s)));
 }
 
 // A segment as the counting pass sees it (shared memory).
@@ -1818,6 +1849,7 @@ struct CountSmem {
 // as the warp-aggregated increment needs).  Neighbouring blocks were mostly
 // admitted together and share buckets, so a warp's increments combine.
 // Bound by the scan of N keys (8 B) and groups (2 B).
+template <bool SMALL>
 __device__ __forceinline__ void select_count(const DevState& s, CountSmem& sm, int mode, int fallback, int bid,
                                              int nb) {
   // indexed by group, or one entry for all
@@ -1828,11 +1860,12 @@ __device__ __forceinline__ void select_count(const DevState& s, CountSmem& sm, i
     const bool on = z.active && !(mode == kSelWhole && s.grp_full[g]);
     sm.kmin[g] = z.kmin;
     sm.span[g] = z.kmax - z.kmin;
-    sm.shift[g] = on ? (uint8_t)bucket_shift(z.kmin, z.kmax) : (uint8_t)64;
+    sm.shift[g] = on ? (uint8_t)bucket_shift<SMALL>(s, z.kmin, z.kmax) : (uint8_t)64;
     any |= on;
   }
   constexpr int kU = 4;
   const int64_t span = (int64_t)nb * blockDim.x;
+  const int row = dig_row_log2<SMALL>(s);
   uint64_t key[kU];
   int seg[kU];
   uint32_t vw[kU];
@@ -1863,20 +1896,89 @@ __device__ __forceinline__ void select_count(const DevState& s, CountSmem& sm, i
         const int sh = sm.shift[seg[u]];
         const uint64_t d = key[u] - sm.kmin[seg[u]];  // keys below the range wrap past any span
         act = sh < 64 && d <= sm.span[seg[u]];
-        idx = (mode == kSelGroups ? (uint32_t)seg[u] * kDigBins : 0u) + (act ? (uint32_t)(d >> sh) : 0u);
+        idx = (mode == kSelGroups ? (uint32_t)seg[u] << row : 0u) + (act ? (uint32_t)(d >> sh) : 0u);
       }
       agg_inc(s.dig_bins, idx, act);
     }
   }
 }
 
+// One warp: of the 128 'rows' buckets from bucket d0 on ('bins' is the lane's
+// place in the first 128; 'before' of the segment's keys lie below them), the
+// one holding the segment's rank-th key, if any, as a key range [blo, bhi], and
+// the rank left inside it.  The counts are cleared.
+template <bool SMALL>
+__device__ __forceinline__ void resolve_rows(const DevState& s, int g, const SelSeg& z, uint4* bins, int rows,
+                                             uint32_t d0, uint64_t before) {
+  const int lane = lane_id();
+  const uint64_t rank = (uint64_t)z.rank;
+  constexpr int kV = 8;  // loads in flight
+  for (int k0 = 0; k0 < rows; k0 += kV) {
+    uint4 v[kV];
+#pragma unroll
+    for (int u = 0; u < kV; ++u) v[u] = __ldcg(bins + 32 * (k0 + u));
+#pragma unroll
+    for (int u = 0; u < kV; ++u) {
+      bins[32 * (k0 + u)] = make_uint4(0, 0, 0, 0);
+      const uint32_t sum = v[u].x + v[u].y + v[u].z + v[u].w;
+      if (!__any_sync(kFull, sum != 0)) continue;
+      const uint32_t incl = warp_incl_scan(sum);
+      uint64_t run = before + incl - sum;
+      if (run < rank && rank <= run + sum) {  // one lane
+        uint32_t d = d0 + 128u * (uint32_t)(k0 + u) + 4u * (uint32_t)lane;
+        if (rank > run + v[u].x) { run += v[u].x; ++d;
+          if (rank > run + v[u].y) { run += v[u].y; ++d;
+            if (rank > run + v[u].z) { run += v[u].z; ++d; } } }
+        const int sh = bucket_shift<SMALL>(s, z.kmin, z.kmax);
+        SelSeg* o = s.sel + g;
+        o->blo = z.kmin + ((uint64_t)d << sh);
+        o->bhi = tmin<uint64_t>(o->blo + ((1ull << sh) - 1), z.kmax);
+        o->rank = (int64_t)(rank - run);
+      }
+      before += __shfl_sync(kFull, incl, 31);
+    }
+  }
+}
+// A wide range's buckets, by a CTA of 32 warps: each sums a 32nd of them, and
+// the one whose share holds the rank looks through it.
+__device__ __forceinline__ void select_resolve_wide(const DevState& s, int g, const SelSeg& z) {
+  __shared__ uint32_t w_sum[32];
+  constexpr int kRows = (1 << kWideBits) / 128 / 32, kV = 8;
+  const int warp = (int)(threadIdx.x >> 5), lane = lane_id();
+  uint4* bins = dig_row<false>(s, g) + warp * kRows * 32 + lane;
+  uint32_t sum = 0;
+  for (int k0 = 0; k0 < kRows; k0 += kV) {
+    uint4 v[kV];
+#pragma unroll
+    for (int u = 0; u < kV; ++u) v[u] = __ldcg(bins + 32 * (k0 + u));
+#pragma unroll
+    for (int u = 0; u < kV; ++u) sum += v[u].x + v[u].y + v[u].z + v[u].w;
+  }
+  sum = __reduce_add_sync(kFull, sum);
+  if (lane == 0) w_sum[warp] = sum;
+  __syncthreads();
+  const uint32_t ws = w_sum[lane], ex = warp_incl_scan(ws) - ws;
+  const uint64_t before = __shfl_sync(kFull, ex, warp), rank = (uint64_t)z.rank;
+  if (before < rank && rank <= before + sum) {
+    resolve_rows<false>(s, g, z, bins, kRows, (uint32_t)(warp * kRows) * 128u, before);
+  } else if (sum) {
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) bins[32 * k] = make_uint4(0, 0, 0, 0);
+  }
+}
+
 // One CTA per segment: the bucket holding the segment's rank-th key, as a key
 // range [blo, bhi], and the rank left inside it.  The counts are cleared for
 // the next select.
+template <bool SMALL>
 __device__ __forceinline__ void select_resolve(const DevState& s, int g, const SelSeg& z) {
   if (!z.active) return;
+  if (!SMALL && wide_range<SMALL>(s, z.kmin, z.kmax)) {
+    select_resolve_wide(s, g, z);
+    return;
+  }
   constexpr int kV = 4;  // bins a thread reads at once
-  uint4* bins = reinterpret_cast<uint4*>(s.dig_bins + (size_t)g * kDigBins);
+  uint4* bins = dig_row<SMALL>(s, g);
   uint64_t before = 0;
   for (int base = 0; base < kDigBins / kV; base += blockDim.x) {
     const int k = base + (int)threadIdx.x;
@@ -1894,7 +1996,7 @@ __device__ __forceinline__ void select_resolve(const DevState& s, int g, const S
       if (rank > run + v.x) { run += v.x; ++d;
         if (rank > run + v.y) { run += v.y; ++d;
           if (rank > run + v.z) { run += v.z; ++d; } } }
-      const int sh = bucket_shift(z.kmin, z.kmax);
+      const int sh = bucket_shift<SMALL>(s, z.kmin, z.kmax);
       SelSeg* o = s.sel + g;
       o->blo = z.kmin + ((uint64_t)d << sh);
       o->bhi = tmin<uint64_t>(o->blo + ((1ull << sh) - 1), z.kmax);
@@ -1996,13 +2098,13 @@ __global__ void __launch_bounds__(256) k_sel_count(DevState s, int fallback) {
   s = with_args(s);
   __shared__ CountSmem sm;
   const int mode = select_mode(s.ctl, fallback);
-  if (mode >= 0) select_count(s, sm, mode, fallback, blockIdx.x, gridDim.x);
+  if (mode >= 0) select_count<false>(s, sm, mode, fallback, blockIdx.x, gridDim.x);
 }
 __global__ void __launch_bounds__(1024) k_sel_resolve(DevState s, int fallback) {
   s = with_args(s);
   const SelSeg z = s.sel[blockIdx.x];  // in the mode's round trip
   const int mode = select_mode(s.ctl, fallback);
-  if (mode == kSelGroups || (mode > 0 && blockIdx.x == 0)) select_resolve(s, blockIdx.x, z);
+  if (mode == kSelGroups || (mode > 0 && blockIdx.x == 0)) select_resolve<false>(s, blockIdx.x, z);
 }
 __global__ void __launch_bounds__(256) k_sel_split(DevState s, int fallback) {
   s = with_args(s);
@@ -2427,6 +2529,7 @@ __global__ void __launch_bounds__(kBmThreads, 3) k_bm_write(DevState s) {
 // 8 groups: 57.5 -> 58.5 us; 32 groups: 58.7 -> 65.2), so it is left alone.
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallPool = 4 * kSmallThreads;     // one batch of loads a thread in the counts and in the split
+static_assert(kSmallPool <= kWidePool, "a warp resolves a small pool's segment: no 2^kWideBits buckets there");
 constexpr int kSmallPoolLru = 2 * kSmallThreads;
 constexpr int kSmallGroups = kSmallThreads / 32;  // a warp for each segment
 inline bool small_select(const DevState& s) {
@@ -2434,50 +2537,20 @@ inline bool small_select(const DevState& s) {
   return s.policy == PS_PREFIXSHIELD ? s.N <= kSmallPool && s.G <= kSmallGroups
                                      : s.policy == PS_LRU && s.N <= kSmallPoolLru;
 }
-// select_resolve by one warp, 128 buckets at a time.
+// select_resolve by one warp (4096 buckets).
 __device__ __forceinline__ void select_resolve_warp(const DevState& s, int g) {
   const SelSeg z = s.sel[g];
-  if (!z.active) return;
-  const int lane = lane_id();
-  uint4* bins = reinterpret_cast<uint4*>(s.dig_bins + (size_t)g * kDigBins) + lane;
-  const uint64_t rank = (uint64_t)z.rank;
-  uint64_t before = 0;
-  constexpr int kV = 8;  // loads in flight
-  for (int k0 = 0; k0 < kDigBins / 128; k0 += kV) {
-    uint4 v[kV];
-#pragma unroll
-    for (int u = 0; u < kV; ++u) v[u] = __ldcg(bins + 32 * (k0 + u));
-#pragma unroll
-    for (int u = 0; u < kV; ++u) {
-      bins[32 * (k0 + u)] = make_uint4(0, 0, 0, 0);
-      const uint32_t sum = v[u].x + v[u].y + v[u].z + v[u].w;
-      if (!__any_sync(kFull, sum != 0)) continue;
-      const uint32_t incl = warp_incl_scan(sum);
-      uint64_t run = before + incl - sum;
-      if (run < rank && rank <= run + sum) {  // one lane
-        uint32_t d = 128u * (uint32_t)(k0 + u) + 4u * (uint32_t)lane;
-        if (rank > run + v[u].x) { run += v[u].x; ++d;
-          if (rank > run + v[u].y) { run += v[u].y; ++d;
-            if (rank > run + v[u].z) { run += v[u].z; ++d; } } }
-        const int sh = bucket_shift(z.kmin, z.kmax);
-        SelSeg* o = s.sel + g;
-        o->blo = z.kmin + ((uint64_t)d << sh);
-        o->bhi = tmin<uint64_t>(o->blo + ((1ull << sh) - 1), z.kmax);
-        o->rank = (int64_t)(rank - run);
-      }
-      before += __shfl_sync(kFull, incl, 31);
-    }
-  }
+  if (z.active) resolve_rows<true>(s, g, z, dig_row<true>(s, g) + lane_id(), kDigBins / 128, 0, 0);
 }
 __device__ __forceinline__ void small_pass(const DevState& s, Ctl* c, unsigned char* smem, int mode, int fallback) {
-  select_count(s, *reinterpret_cast<CountSmem*>(smem), mode, fallback, 0, 1);
+  select_count<true>(s, *reinterpret_cast<CountSmem*>(smem), mode, fallback, 0, 1);
   __syncthreads();
   if (mode == kSelGroups) {
     const int g = (int)(threadIdx.x >> 5);
     if (g < s.G) select_resolve_warp(s, g);
   } else {
     const SelSeg z = s.sel[0];
-    select_resolve(s, 0, z);
+    select_resolve<true>(s, 0, z);
   }
   __syncthreads();
   select_split(s, c, *reinterpret_cast<SplitSmem*>(smem), mode, fallback, 0, 1);

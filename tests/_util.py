@@ -210,3 +210,36 @@ def compare_state(got, want, where="", s3=False):
         assert got["s3_ctr"] == want["s3_ctr"] and got["ghost_ctr"] == want["ghost_ctr"]
         for a, b in zip(got["ghost"], want["ghost"]):
             assert np.array_equal(a, b), f"{where}: ghost differs"
+
+
+# ---------------------------------------------------------------------------
+# A handle's device state, read (or set) where a test has to see which branch a
+# step took or to age a handle: the offsets come from the library's own header.
+LAYOUT = {"Ctl": ("step", "stamp_base", "lst_n", "bar", "lg_buf", "internal_error"),
+          "DevState": ("ctl", "lg_live")}
+_layout = {}
+
+
+def device_layout():
+    """{(struct, field): byte offset} of the fields in LAYOUT."""
+    if not _layout:
+        import subprocess
+        import tempfile
+        from paper_2608_01657_gb300 import build as B
+        names = [(s, f) for s, fs in LAYOUT.items() for f in fs]
+        body = "".join(f'printf("%zu\\n", offsetof(ps::{s}, {f}));' for s, f in names)
+        with tempfile.TemporaryDirectory() as d:
+            src, exe = os.path.join(d, "layout.cu"), os.path.join(d, "layout")
+            with open(src, "w") as f:
+                f.write('#include <cstddef>\n#include <cstdio>\n#include "ps_internal.cuh"\nint main() {' + body + "}\n")
+            subprocess.run([B._nvcc(), *B.ARCH, "-std=c++17", "-I" + B.INCLUDE, "-I" + B.CSRC, "-o", exe, src], check=True)
+            out = subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split()
+        _layout.update(zip(names, map(int, out)))
+    return _layout
+
+
+def ctl_word(cache, field, dtype):
+    """One element tensor over a field of the handle's control block (which starts its workspace)."""
+    import torch
+    at = device_layout()["Ctl", field]
+    return cache.workspace[at:at + torch.empty(0, dtype=dtype).element_size()].view(dtype)

@@ -7,7 +7,7 @@ import pytest
 
 import oracle as O
 from paper_2608_01657_gb300 import workloads as W
-from _util import compare_outputs, compare_state
+from _util import compare_outputs, compare_state, ctl_word
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -140,6 +140,62 @@ def test_list_finish_widths(gap, need):
              for k, t in enumerate(seq)]
     gpu, orc = _pair(5020, 16, 2, "prefixshield", dict(rho=(1.0,), beta=(100.0,)), 1, 3000 * 16)
     assert _evicted(_run(gpu, orc, steps, 16, f"finish/{gap}/{need}")) >= need - 10
+
+
+def _aged(policy, old, new, need, gap, N=None):
+    """A pool of `old` blocks, `gap` stamps, then `new` blocks, and a prompt
+    that takes `need` victims among the old ones: a handle that served other
+    prompts in between, as the recency counter tells it.  Returns the length
+    of the select's split list."""
+    N = N or old + new
+    rng = np.random.default_rng(old + need)
+    seq = [rng.integers(0, W.VOCAB, size=n * 2, dtype=np.int32) for n in (old, new, need + N - old - new)]
+    gpu, orc = _pair(N, 2, 2, policy, dict(rho=(1.0,), beta=(0.0,)), 1, 2 * max(len(t) for t in seq))
+    dev = torch.device("cuda")
+    for k, t in enumerate(seq):
+        if k == 1:
+            ctl_word(gpu, "stamp_base", torch.int64).add_(gap)
+        g, o = np.zeros(1, np.int32), np.array([0, len(t)], np.int64)
+        assert gpu.step(k, torch.from_numpy(g).to(dev), torch.from_numpy(o).to(dev), torch.from_numpy(t).to(dev)) == 0
+        want = orc.step(k, g, o, t)
+        compare_outputs(gpu.fetch(1), want, f"aged/{policy}/{old}/{need}/{gap} step {k}")
+        if k == 2:
+            assert len(want["evicted_ids"]) == need
+    listed = int(ctl_word(gpu, "lst_n", torch.int64).item())
+    got, want = gpu.export(), orc.export()
+    assert int(got["stamp"].max()) > gap  # the counter did jump
+    for e in (got, want):  # the stamps' order is what has to agree
+        e["stamp"] = np.unique(e["stamp"], return_inverse=True)[1]
+    compare_state(got, want, f"aged/{policy}/{old}/{need}/{gap}")
+    return listed
+
+
+@pytest.mark.parametrize("policy", ["lru", "prefixshield"])
+@pytest.mark.parametrize("gap,most", [(1 << 22, 1 << 11), (1 << 24, 1 << 13), (1 << 26, 1 << 11), (1 << 27, 1 << 12)])
+def test_aged_range_is_cut_finely(policy, gap, most):
+    """Old blocks beside new ones much later: past 2^25 stamps the range is cut
+    into 65536 buckets, so the list stays a few thousand long (4096 buckets
+    would put all 20,000 old blocks on it from 2^27 on)."""
+    for need in (1, 9000, 20000):
+        listed = _aged(policy, 20000, 3000, need, gap)
+        assert policy != "lru" or 1 <= listed <= most  # (a debt phase's list is reset for its fallback)
+
+
+@pytest.mark.parametrize("N,G", [(4096, 64), (4097, 64), (9000, 65), (9000, 64)])
+def test_wide_buckets_at_the_rule_s_edges(N, G):
+    """Quota groups that select over ranges of mixed widths, at the largest
+    pool without and the smallest with 65536 buckets, and at 64 and 65 groups."""
+    steps = W.fuzz_steps(N + G, G, 64, 30, docs_per_group=2, doc_blocks=max(2, N // G // 2), now_stride=2,
+                         fresh_max_blocks=max(2, N // G // 2), block_size=2)
+    gpu, orc = _pair(N, 2, G, "staticquota", dict(rho=(2.0,), beta=(64.0,)), 64, 64 * 2 * (2 * (N // G) + 4))
+    dev = torch.device("cuda")
+    base = ctl_word(gpu, "stamp_base", torch.int64)
+    for k, st in enumerate(steps):
+        base.add_((0, 1 << 13, 1 << 24, 1 << 25, 1 << 33)[k % 5])
+        assert gpu.step(st.now, *(torch.from_numpy(x).to(dev) for x in (st.groups, st.offsets, st.tokens))) == 0
+        want = orc.step(st.now, st.groups, st.offsets, st.tokens)
+        compare_outputs(gpu.fetch(st.num_requests), want, f"wide/{N}/{G} step {k}")
+    assert _evicted(orc.stats()) > 0
 
 
 @pytest.mark.parametrize("N,blocks", [(64, 12), (2000, 400)])
