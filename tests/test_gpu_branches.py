@@ -113,6 +113,18 @@ def test_more_requests_than_blocks(R, max_blocks):
     _run(gpu, orc, steps, 1, f"R/{R}")
 
 
+@pytest.mark.parametrize("max_blocks", [1, 5, 8, 9, 10, 11, 12, 17, 19, 4099])
+def test_claim_map_holds_a_full_step_of_new_blocks(max_blocks):
+    """Every block of the largest step is new, at sizes just past a power of
+    two times the claim map's four ways a bucket."""
+    steps = []
+    for k in range(3):
+        g, o, t = _prompts([(max_blocks - 1) * 2, 2], [0, 1], 100 * max_blocks + k)
+        steps.append(W.Step(k, k, g, o, t, None, None))
+    gpu, orc = _pair(max_blocks + 1, 2, 2, "prefixshield", dict(rho=(1.0,), beta=(3.0,)), 2, max_blocks * 2)
+    _run(gpu, orc, steps, 1, f"claims/{max_blocks}")
+
+
 @pytest.mark.parametrize("G,contracts", [(2, 1), (40, 3), (1000, 3)])
 def test_many_indebted_groups(G, contracts):
     """The water-filling's search with one, some and a thousand groups in debt
