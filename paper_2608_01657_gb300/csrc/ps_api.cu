@@ -471,6 +471,7 @@ int32_t ps_create(ps_handle_t** out, int64_t capacity_blocks, int32_t block_size
   configure_kernels(s);  // per device: attributes are set on the current one
   int32_t rc = init_state(h, st);
   if (rc == PS_OK) rc = upload_constants(h, st);
+  if (rc == PS_OK && s.lg_on) h->base.lg_grid = queue_compact_grid(s, st);
   if (rc == PS_OK && (cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
                       cudaStreamCreateWithFlags(&h->cap_side, cudaStreamNonBlocking) != cudaSuccess ||
                       cudaStreamCreateWithFlags(&h->cap_side2, cudaStreamNonBlocking) != cudaSuccess ||

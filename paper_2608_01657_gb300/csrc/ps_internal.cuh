@@ -361,6 +361,7 @@ struct DevState {
   // indexed queues (allocated only with PS_FLAG_INDEXED_QUEUES)
   int32_t lg_on;           // victims come from the queues instead of a candidate scan
   int32_t lg_L;            // logs: 3G + 3
+  int32_t lg_grid;         // CTAs of a compaction
   int64_t lg_P;            // entries per buffer
   int64_t lg_max_chunks;   // chunks a scan can span
   int64_t lg_app_chunks;   // append chunks of the largest step
@@ -477,6 +478,8 @@ void launch_queue_init(const DevState& s, cudaStream_t st);
 int32_t launch_queue_cand(const DevState& s, cudaStream_t st, int* launches);
 int32_t launch_queue_select(const DevState& s, cudaStream_t st, int phase, bool plain_first, int* launches);
 int32_t launch_queue_append(const DevState& s, cudaStream_t st, int* launches);
+// The CTAs a compaction may take on this device (an initialized handle without one due).
+int32_t queue_compact_grid(const DevState& s, cudaStream_t st);
 // S3-FIFO (ps_s3fifo.cu)
 // The ghost's entries for the step's claims (before anything leaves the ghost).
 int32_t launch_s3_probe(const DevState& s, cudaStream_t st, int* launches);

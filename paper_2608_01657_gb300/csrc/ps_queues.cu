@@ -38,7 +38,7 @@ namespace {
 
 constexpr int kScanThreads = 256;          // 4 consecutive entries a thread per chunk
 constexpr int kScanGrid = 152 * 8;         // grid-stride over the chunks of a scan
-constexpr int kCompactGrid = 152 * 2;      // all resident (a cooperative launch)
+constexpr int kCompactGrid = 152 * 2;      // at most; all resident (a cooperative launch)
 static_assert(kScanThreads * 4 == kLogChunk, "a scan CTA covers one chunk");
 
 __device__ __forceinline__ const uint32_t* ent_blk(const DevState& s, int buf) { return s.lg_blk + (int64_t)buf * s.lg_P; }
@@ -734,20 +734,40 @@ int32_t launch_queue_select(const DevState& s, cudaStream_t st, int phase, bool 
   return PS_OK;
 }
 
-int32_t launch_queue_append(const DevState& s, cudaStream_t st, int* launches) {
-  const int ach = (int)s.lg_app_chunks;
-  launch_k(k_lg_app_count, ach, kAppChunk, 0, st, s);
-  launch_k(k_lg_app_scan, s.lg_L, 256, 0, st, s);
+static cudaError_t launch_compact(const DevState& s, int grid, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;
-  cfg.gridDim = dim3(kCompactGrid);
+  cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(kScanThreads);
   cfg.stream = st;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, k_lg_compact, s) != cudaSuccess) return PS_ERR_CUDA;
+  cfg.numAttrs = grid > 1 ? 1 : 0;  // one CTA waits for no other
+  return cudaLaunchKernelEx(&cfg, k_lg_compact, s);
+}
+// The CTAs of a handle's compactions: kCompactGrid, or fewer where the SMs the
+// handle may use do not hold as many at once (a cooperative launch of more is
+// refused; a captured one is not even that, and could never start).  What the device counts can be more than what a partition of it
+// (a green context) is given, so the launch itself is asked: with no
+// compaction due, the kernel returns at once.
+int32_t queue_compact_grid(const DevState& s, cudaStream_t st) {
+  int dev = 0, nsm = 0, per = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_lg_compact, kScanThreads, 0) != cudaSuccess)
+    nsm = 0;
+  int grid = nsm * per < kCompactGrid ? nsm * per : kCompactGrid;
+  while (grid > 1 && launch_compact(s, grid, st) != cudaSuccess) grid /= 2;
+  cudaGetLastError();  // a refused size
+  return grid > 1 ? grid : 1;
+}
+
+int32_t launch_queue_append(const DevState& s, cudaStream_t st, int* launches) {
+  const int ach = (int)s.lg_app_chunks;
+  launch_k(k_lg_app_count, ach, kAppChunk, 0, st, s);
+  launch_k(k_lg_app_scan, s.lg_L, 256, 0, st, s);
+  if (launch_compact(s, s.lg_grid, st) != cudaSuccess) return PS_ERR_CUDA;
   launch_k(k_lg_app_write, ach, kAppChunk, 0, st, s);
   *launches += 4;
   return PS_OK;
