@@ -31,6 +31,8 @@
  *    than history_capacity distinct (group, prefix id) entries) also leaves
  *    all state unchanged, and is sticky: every later step is a no-op
  *    reporting PS_ERR_CAPACITY until ps_clear_status() or ps_reset().
+ *    PS_ERR_DEVICE_STATUS reports a broken invariant of the library (never
+ *    expected); with indexed queues it is sticky until ps_reset().
  *  - A handle is not thread-safe; steps on one handle must be issued in
  *    order on one stream (or with equivalent ordering).
  */

@@ -76,7 +76,7 @@ struct __align__(32) HistEntry {    // (group, prefix id) -> reference history
 struct Ctl {
   // persistent
   int32_t sticky;          // PS_OK or PS_ERR_CAPACITY
-  int32_t pad0;
+  int32_t lg_lost;         // a step with indexed queues hit an internal error: PS_ERR_DEVICE_STATUS until ps_reset
   uint64_t step;           // index of the step being / next to be processed (from 1)
   uint64_t stamp_base;     // first recency stamp of this step (from 1)
   int64_t t_prev;          // last refill time
@@ -115,7 +115,7 @@ struct Ctl {
   uint32_t v_ticket;       // k_validate: CTAs done (the last one finishes the call)
   uint32_t v_bad;          // k_validate: bit 0 an invalid request, bit 1 a look-back ran out
   uint64_t v_sum;          // k_validate: blocks (high half) and chunks (low half) of the call
-  uint64_t bar;            // k_lg_compact's grid barrier: arrivals so far (a multiple of its grid between steps)
+  uint64_t bar;            // k_lg_compact's grid barrier: arrivals so far (zeroed in each step)
 };
 
 // One hashing chunk: up to kChunkBlocks consecutive blocks of one request.

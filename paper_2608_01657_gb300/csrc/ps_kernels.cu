@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(kValTile) k_validate(DevState s, int32_t* prob
   const uint64_t all = ldcg_u64(&c->v_sum);  // blocks (high half) and chunks (low half) of the step
   const int64_t T = R > 0 ? s.in_offsets[R] : 0;
   const int64_t first_off = R > 0 ? s.in_offsets[0] : 0;
-  const int32_t sticky = c->sticky;
+  const int32_t sticky = c->sticky, lost = c->lg_lost;
   const int64_t t_prev = c->t_prev;
   const uint64_t step = c->step;
   c->v_bad = 0;
@@ -454,6 +454,7 @@ __global__ void __launch_bounds__(kValTile) k_validate(DevState s, int32_t* prob
   c->v_sum = 0;
   int32_t st = PS_OK;
   if (!probe && sticky != PS_OK) st = sticky;
+  else if (!probe && lost) st = PS_ERR_DEVICE_STATUS;
   else if (!probe && s.now < t_prev) st = PS_ERR_CLOCK;
   else if (!probe && step > kMaxStep) st = PS_ERR_CAPACITY;
   else if (vb || first_off != 0 || T > s.max_tokens) st = PS_ERR_INVALID_ARG;
@@ -2687,6 +2688,8 @@ __global__ void k_finalize(DevState s) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const int32_t st = c->internal_error ? PS_ERR_DEVICE_STATUS : c->status;
   s.out.counts[3] = st;
+  // the queues' logs no longer agree with the pool: no later step uses them
+  if (c->internal_error && s.lg_on) c->lg_lost = 1;
   if (c->status != PS_OK) return;
   s.out.counts[0] = (int32_t)c->need;
   s.out.counts[1] = (int32_t)c->n_evicted;

@@ -400,6 +400,7 @@ __global__ void __launch_bounds__(kAppChunk) k_lg_app_count(DevState s) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     c->lg_cmp = 0;
     c->lg_ticket = 0;  // k_lg_take left its chunk count there
+    c->bar = 0;
   }
   if (c->status != PS_OK) return;
   const int64_t nb = c->nblocks;
@@ -590,9 +591,11 @@ __device__ __forceinline__ void lg_cmp_write(const DevState& s, Ctl* c, const in
   }
 }
 
-// Every CTA adds one to a counter that only grows and waits (bounded) for the
-// next multiple of the grid: a grid barrier of a cooperative launch, whose
-// CTAs are all resident.  False if the wait ran out (never expected).
+// Every CTA adds one to a counter, zero at the launch, and waits (bounded) for
+// the next multiple of the grid: a grid barrier of a cooperative launch, whose
+// CTAs are all resident.  False if the wait ran out (never expected): the CTA
+// then leaves the compaction, the step appends nothing, and the handle's
+// queues are not used again (k_finalize).
 __device__ __forceinline__ bool grid_sync(Ctl* c, uint64_t* target) {
   __shared__ int s_ok;
   __syncthreads();
@@ -623,9 +626,7 @@ __global__ void __launch_bounds__(kScanThreads) k_lg_compact(DevState s) {
   Ctl* c = s.ctl;
   const int32_t st = c->status, need = c->lg_cmp;
   if (st != PS_OK || !need) return;
-  // a CTA has not arrived yet, so fewer than a grid of this launch's arrivals
-  // are in the counter
-  uint64_t target = threadIdx.x == 0 ? ldcg_u64(&c->bar) / gridDim.x * gridDim.x : 0;
+  uint64_t target = 0;
   if (blockIdx.x == 0) lg_cmp_plan(s, c);
   if (!grid_sync(c, &target)) return;
   const int L = s.lg_L;
@@ -653,7 +654,8 @@ __global__ void __launch_bounds__(kAppChunk) k_lg_app_write(DevState s) {
   s = with_args(s);
   __shared__ uint32_t cnt[kMaxLogs];
   Ctl* c = s.ctl;
-  if (c->status != PS_OK) return;
+  // after an error the logs may lack the room (a compaction that gave up)
+  if (c->status != PS_OK || c->internal_error) return;
   const int64_t nb = c->nblocks;
   const int q = blockIdx.x;
   const int L = s.lg_L;
@@ -690,9 +692,14 @@ __global__ void __launch_bounds__(kAppChunk) k_lg_app_write(DevState s) {
 #pragma unroll
     for (int i = 0; i < 2; ++i)
       if (key[i] >= 0) {
-        const int64_t o = s.lg_desc[key[i]].tail + s.lg_app[(int64_t)key[i] * s.lg_app_chunks + q] + rank[i];
-        ob[o] = b;
-        os[o] = c->stamp_base + (uint64_t)j;
+        const LogDesc d = s.lg_desc[key[i]];
+        const int64_t o = d.tail + s.lg_app[(int64_t)key[i] * s.lg_app_chunks + q] + rank[i];
+        if (o < d.end) {
+          ob[o] = b;
+          os[o] = c->stamp_base + (uint64_t)j;
+        } else {
+          c->internal_error = 1;  // a full log was compacted first: cannot happen
+        }
       }
   }
   if (last_cta(c)) {
@@ -748,9 +755,10 @@ static cudaError_t launch_compact(const DevState& s, int grid, cudaStream_t st) 
 }
 // The CTAs of a handle's compactions: kCompactGrid, or fewer where the SMs the
 // handle may use do not hold as many at once (a cooperative launch of more is
-// refused; a captured one is not even that, and could never start).  What the device counts can be more than what a partition of it
-// (a green context) is given, so the launch itself is asked: with no
-// compaction due, the kernel returns at once.
+// refused; a captured one is not even that, and could never start).  What the
+// device counts can be more than what a partition of it (a green context) is
+// given, so the launch itself is asked: with no compaction due, the kernel
+// returns at once.
 int32_t queue_compact_grid(const DevState& s, cudaStream_t st) {
   int dev = 0, nsm = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||

@@ -2,12 +2,14 @@
 each begins, ends or leaves a remainder.  Every output, the exported state and
 the statistics are whole numbers: the tolerance is zero.
 """
+import ctypes
+
 import numpy as np
 import pytest
 
 import oracle as O
 from paper_2608_01657_gb300 import workloads as W
-from _util import compare_outputs, compare_state, ctl_word
+from _util import compare_outputs, compare_state, ctl_word, device_layout
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -225,6 +227,58 @@ def test_queue_logs_fill_and_compact(policy):
     steps = W.fuzz_steps(3, 3, 8, 300, docs_per_group=3, doc_blocks=6, fresh_max_blocks=1, now_stride=2)
     gpu, orc = _pair(40, 16, 3, policy, dict(rho=(2.0,), beta=(6.0,), flags=O.FLAG_INDEXED_QUEUES), 8, 4096)
     assert _evicted(_run(gpu, orc, steps, 25, f"queues/{policy}")) > 0
+
+
+def _queue_steps(gpu, orc, steps, before=None):
+    """Steps against the oracle; returns the entry buffers seen after them
+    (two: a compaction ran)."""
+    dev, buffers = torch.device("cuda"), set()
+    for k, st in enumerate(steps):
+        if before:
+            before()
+        assert gpu.step(st.now, *(torch.from_numpy(x).to(dev) for x in (st.groups, st.offsets, st.tokens))) == 0
+        compare_outputs(gpu.fetch(st.num_requests), orc.step(st.now, st.groups, st.offsets, st.tokens), f"step {k}")
+        buffers.add(int(ctl_word(gpu, "lg_buf", torch.int32).item()))
+    return buffers
+
+
+def test_queue_barrier_starts_from_any_count():
+    """The compaction's barrier does not depend on what an earlier launch left
+    in its counter."""
+    steps = W.fuzz_steps(3, 3, 8, 120, docs_per_group=3, doc_blocks=6, fresh_max_blocks=1, now_stride=2)
+    gpu, orc = _pair(40, 16, 3, "lru", dict(rho=(2.0,), beta=(6.0,), flags=O.FLAG_INDEXED_QUEUES), 8, 4096)
+    bar = ctl_word(gpu, "bar", torch.int64)
+    assert _queue_steps(gpu, orc, steps, lambda: bar.fill_(17)) == {0, 1}
+
+
+def test_queue_error_is_kept_until_reset():
+    """A live count that disagrees with its log is found by the next
+    compaction: that step and every later one report it (ps_clear_status does
+    not help), and no later one changes the pool, until ps_reset."""
+    steps = W.fuzz_steps(3, 3, 8, 300, docs_per_group=3, doc_blocks=6, fresh_max_blocks=1, now_stride=2)
+    kw = dict(rho=(2.0,), beta=(6.0,), flags=O.FLAG_INDEXED_QUEUES)
+    gpu, orc = _pair(40, 16, 3, "lru", kw, 8, 4096)
+    dev = torch.device("cuda")
+    _queue_steps(gpu, orc, steps[:5])
+    at = device_layout()["DevState", "lg_live"]  # the handle starts with its DevState
+    live = int.from_bytes(ctypes.string_at(gpu._h.value + at, 8), "little") - gpu.workspace.data_ptr()
+    live += 8 * 3 * 3  # the global log
+    gpu.workspace[live:live + 8].view(torch.int64).add_(1)
+    status = []
+    for st in steps[5:]:
+        if len(status) == 3:
+            break
+        if status:
+            gpu.clear_status()
+            before = gpu.export()
+        assert gpu.step(st.now, *(torch.from_numpy(x).to(dev) for x in (st.groups, st.offsets, st.tokens))) == 0
+        if status:
+            compare_state(gpu.export(), before, "a refused step")
+        if status or gpu.fetch(st.num_requests)["status"]:
+            status.append(gpu.fetch(st.num_requests)["status"])
+    assert status == [-6] * 3  # PS_ERR_DEVICE_STATUS
+    assert gpu.reset() == 0
+    assert _queue_steps(gpu, O.OracleCache(40, 16, 3, "lru", O.Params(**kw)), steps[:120]) == {0, 1}
 
 
 @pytest.mark.parametrize("R", [1, 7, 600])
