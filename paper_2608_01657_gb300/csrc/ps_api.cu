@@ -525,6 +525,11 @@ int32_t ps_step(ps_handle_t* h, void* stream, int64_t now_ticks, int32_t num_req
 
 namespace {
 constexpr size_t kHostKernelBytes = (size_t)8 << 20;
+// A refused copy leaves no error behind for the next call's launch check.
+inline bool copied(cudaError_t e) {
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess;
+}
 inline bool aligned_to(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 // A host array a kernel may read or write: page-locked (or otherwise device-mapped).
 bool device_writable(const void* p) {
@@ -535,6 +540,15 @@ bool device_writable(const void* p) {
     return false;
   }
   return a.type == cudaMemoryTypeHost || a.type == cudaMemoryTypeManaged;
+}
+// The same of a whole array, by its first and its last byte: one that starts in
+// registered memory and runs out of it is left to the copy calls, which refuse it.
+// (Memory is registered by pages: an array inside one needs one question.)
+bool whole_writable(const void* p, size_t bytes) {
+  if (!p || bytes == 0) return true;
+  const char* last = static_cast<const char*>(p) + bytes - 1;
+  const bool one_page = ((reinterpret_cast<uintptr_t>(p) ^ reinterpret_cast<uintptr_t>(last)) >> 12) == 0;
+  return device_writable(p) && (one_page || device_writable(last));
 }
 }  // namespace
 
@@ -550,7 +564,7 @@ int32_t ps_step_host(ps_handle_t* h, void* stream, int64_t now_ticks, int32_t nu
   cudaStream_t st = as_stream(stream);
   const size_t R = (size_t)num_requests;
   auto h2d = [&](void* d, const void* src, size_t bytes) {
-    return bytes == 0 || cudaMemcpyAsync(d, src, bytes, cudaMemcpyHostToDevice, st) == cudaSuccess;
+    return bytes == 0 || copied(cudaMemcpyAsync(d, src, bytes, cudaMemcpyHostToDevice, st));
   };
   const ps_handle::Staging& sg = h->stg[0];
   // Page-locked inputs of up to kHostKernelBytes are read by a kernel (larger
@@ -558,10 +572,11 @@ int32_t ps_step_host(ps_handle_t* h, void* stream, int64_t now_ticks, int32_t nu
   // by their device-side counts: one wait instead of two and no copy calls.
   const void* in[5] = {h_token_offsets, h_group_ids, h_tokens, h_contract_ids, h_prefix_ids};
   bool in_locked = (size_t)T * 4 <= kHostKernelBytes;
-  for (const void* p : in) in_locked = in_locked && aligned_to(p, 4) && device_writable(p);
+  const int64_t words[5] = {2 * ((int64_t)R + 1), (int64_t)R, T, (int64_t)R, 2 * (int64_t)R};
+  for (int k = 0; k < 5; ++k)
+    in_locked = in_locked && aligned_to(in[k], 4) && whole_writable(in[k], 4 * (size_t)words[k]);
   if (in_locked) {
     void* dst[5] = {sg.offsets, sg.group, sg.tokens, sg.contract, sg.prefix};
-    const int64_t words[5] = {2 * ((int64_t)R + 1), (int64_t)R, T, (int64_t)R, 2 * (int64_t)R};
     launch_host_in(in, dst, words, st);
     if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
   } else if (!h2d(sg.offsets, h_token_offsets, (R + 1) * 8) || !h2d(sg.group, h_group_ids, R * 4) ||
@@ -575,21 +590,22 @@ int32_t ps_step_host(ps_handle_t* h, void* stream, int64_t now_ticks, int32_t nu
   if (rc != PS_OK) return rc;
   const ps_step_out_t& o = h->st_out;
   auto d2h = [&](void* dst, const void* d, size_t bytes) {
-    return bytes == 0 || !dst || cudaMemcpyAsync(dst, d, bytes, cudaMemcpyDeviceToHost, st) == cudaSuccess;
+    return bytes == 0 || !dst || copied(cudaMemcpyAsync(dst, d, bytes, cudaMemcpyDeviceToHost, st));
   };
+  const size_t G = (size_t)h->base.G, ids = 4 * (size_t)h->base.max_blocks;
+  const struct {
+    const void* p;
+    size_t bytes, align;
+  } outs[9] = {{h_out->hit_blocks, R * 4, 4}, {h_out->admitted_blocks, R * 4, 4}, {h_out->admitted_offsets, (R + 1) * 4, 4},
+               {h_out->admitted_ids, ids, 4}, {h_out->evicted_ids, ids, 4}, {h_out->invalidated_ids, ids, 4},
+               {h_out->counts, 16, 4}, {h_out->debt_raw, G * 8, 8}, {h_out->debt_norm, G * 8, 8}};
   bool out_locked = h_out->counts != nullptr;
-  for (const void* p : {(const void*)h_out->hit_blocks, (const void*)h_out->admitted_blocks,
-                        (const void*)h_out->admitted_offsets, (const void*)h_out->admitted_ids,
-                        (const void*)h_out->evicted_ids, (const void*)h_out->invalidated_ids,
-                        (const void*)h_out->counts, (const void*)h_out->debt_raw, (const void*)h_out->debt_norm})
-    out_locked = out_locked && aligned_to(p, 4) && device_writable(p);
-  out_locked = out_locked && aligned_to(h_out->debt_raw, 8) && aligned_to(h_out->debt_norm, 8);
+  for (const auto& x : outs) out_locked = out_locked && aligned_to(x.p, x.align) && whole_writable(x.p, x.bytes);
   if (out_locked) {
     launch_host_out(o, *h_out, num_requests, h->base.G, st);
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return PS_ERR_CUDA;
     return h_out->counts[3];
   }
-  const size_t G = (size_t)h->base.G;
   if (!d2h(h_out->counts, o.counts, 16) || !d2h(h_out->hit_blocks, o.hit_blocks, R * 4) ||
       !d2h(h_out->admitted_blocks, o.admitted_blocks, R * 4) ||
       !d2h(h_out->admitted_offsets, o.admitted_offsets, (R + 1) * 4) || !d2h(h_out->debt_raw, o.debt_raw, G * 8) ||
@@ -623,7 +639,7 @@ int32_t ps_step_host_async(ps_handle_t* h, void* stream, int32_t slot, int64_t n
   const size_t R = (size_t)num_requests;
   const ps_handle::Staging& sg = h->stg[slot];
   auto h2d = [&](void* d, const void* src, size_t bytes) {
-    return bytes == 0 || cudaMemcpyAsync(d, src, bytes, cudaMemcpyHostToDevice, cs) == cudaSuccess;
+    return bytes == 0 || copied(cudaMemcpyAsync(d, src, bytes, cudaMemcpyHostToDevice, cs));
   };
   // the slot's staging is free once the step that last read it has run
   if (cudaStreamWaitEvent(cs, h->slot_free[slot], 0) != cudaSuccess) return PS_ERR_CUDA;

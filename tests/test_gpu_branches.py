@@ -334,3 +334,45 @@ def test_step_host_buffers(tokens_pinned, outputs_pinned, shift):
                "evicted_ids": out["evicted_ids"][:cnt[1]], "invalidated_ids": out["invalidated_ids"][:cnt[2]],
                "debt_raw": out["debt_raw"], "debt_norm": out["debt_norm"]}
         compare_outputs(got, orc.step(st.now, st.groups, st.offsets, st.tokens, st.contracts, st.prefixes), f"step {st.index}")
+
+
+@pytest.mark.parametrize("which", ["tokens", "admitted_ids"])
+def test_step_host_array_that_leaves_page_locked_memory(which):
+    """An array of which only the first pages are page-locked goes to the copy
+    calls, which refuse it; the next call is as if that one had not been made
+    (a refused input) or had only lost its outputs."""
+    from paper_2608_01657_gb300 import binding as B
+    bs, n = 2, 1 << 18
+    rng = np.random.default_rng(5)
+    docs = [rng.integers(0, W.VOCAB, size=n, dtype=np.int32) for _ in range(2)]
+    gpu, orc = _pair(n // bs, bs, 2, "lru", dict(rho=(1.0,), beta=(1.0,)), 1, n)
+    cudart = torch.cuda.cudart()
+    raw = np.zeros(4 * n + (1 << 17), np.uint8)
+    at = -raw.ctypes.data % (1 << 16)
+    part = raw[at:at + 4 * n].view(np.int32)[:n if which == "tokens" else n // bs]
+
+    def pinned(x):
+        return torch.from_numpy(x).pin_memory().numpy()
+
+    g, o = np.zeros(1, np.int32), np.array([0, n], np.int64)
+    out = B.host_outputs(1, gpu.max_blocks, 2, pinned=True)
+    assert int(cudart.cudaHostRegister(part.ctypes.data, 1 << 16, 0)) == 0
+    try:
+        if which == "tokens":
+            part[:] = docs[0]
+            res = gpu.step_host(0, pinned(g), pinned(o), part, out=out)
+        else:
+            orc.step(0, g, o, docs[0])
+            res = gpu.step_host(0, pinned(g), pinned(o), pinned(docs[0]), out=dict(out, admitted_ids=part))
+        assert res["rc"] == -4  # PS_ERR_CUDA
+    finally:
+        torch.cuda.synchronize()
+        cudart.cudaHostUnregister(part.ctypes.data)
+    res = gpu.step_host(1, pinned(g), pinned(o), pinned(docs[1]), out=out)
+    assert res["rc"] == 0
+    cnt = out["counts"]
+    got = {"status": int(cnt[3]), **{k: out[k][:m] for k, m in (
+        ("hit_blocks", 1), ("admitted_blocks", 1), ("admitted_offsets", 2), ("admitted_ids", cnt[0]),
+        ("evicted_ids", cnt[1]), ("invalidated_ids", cnt[2]), ("debt_raw", 2), ("debt_norm", 2))}}
+    compare_outputs(got, orc.step(1, g, o, docs[1]), which)
+    compare_state(gpu.export(), orc.export(), which)
