@@ -2767,7 +2767,10 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
   const int pgrid = grid_for(s.max_blocks, kThreads, 1 << 30);
   const int prgrid = grid_for(s.max_blocks + R, kThreads, 1 << 30);
   const int igrid = grid_for(s.max_blocks > R ? s.max_blocks : R, kThreads, 1 << 30);
-  const int cgrid = grid_for(s.N, 256, 152 * 8);
+  // The select's scans, four CTAs an SM: with eight, a step that has nothing to
+  // select waits for as many CTAs to come and go four times (prefixshield over
+  // 2^20 blocks: a step of one request 69.4 -> 66.0 us, of 4096 147.6 -> 142.6).
+  const int cgrid = grid_for(s.N, 256, 152 * 4);
   int launches = 0;
   auto mark = [&](int stage) {
     // under capture an external record becomes an event-record node of the
@@ -2832,14 +2835,11 @@ int32_t launch_step(const DevState& s, cudaStream_t st, StepTrace* tr, const Cap
     if (cudaEventRecord(cap->fork2, st) != cudaSuccess || cudaStreamWaitEvent(cap->side2, cap->fork2, 0) != cudaSuccess)
       return PS_ERR_CUDA;
     ms = cap->side2;
-    // The candidate scan has the GPU to itself first: the select waits for it,
-    // and beside these kernels it took three times as long (28 us of a 177 us
-    // step at 2^20 blocks); they fill the time of the select's one-CTA kernels
-    // instead.
-    if (early && cudaStreamWaitEvent(ms, cap->join, 0) != cudaSuccess) return PS_ERR_CUDA;
+    // (Held back until the candidate scan was done they cost more than they
+    // slow it down: prefixshield over 2^20 blocks 149.3 us a step of 4096
+    // requests against 148.1, and 71.6 against 68.2 for one of a single one.)
   }
-  if (fork2 && early) PS_LAUNCH((k_instep<<<pgrid, kThreads, 0, ms>>>(s)));  // after the join: plain
-  else PS_LAUNCH(launch_k(k_instep, pgrid, kThreads, 0, ms, s));
+  PS_LAUNCH(launch_k(k_instep, pgrid, kThreads, 0, ms, s));
   if (s.policy == PS_S3FIFO) {
     if (launch_s3_probe(s, ms, &launches) != PS_OK) return PS_ERR_CUDA;
     // the plan trims the ghost: it waits for the lookups
