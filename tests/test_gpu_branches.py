@@ -80,13 +80,17 @@ def test_id_lists_at_chunk_edges(policy, N):
     assert _evicted(_run(gpu, orc, steps, label=f"lists/{policy}/{N}")) > 0
 
 
-@pytest.mark.parametrize("max_blocks", [64 * 152, 64 * 153, 64 * 608 + 64, 64 * 1300])
+@pytest.mark.parametrize("per_sm,more", [(1, 0), (1, 1), (2, 0), (2, 1), (4, 0), (4, 1)])
 @pytest.mark.parametrize("bs", [8, 16, 32])
-def test_hashing_widths_and_chunk_edges(bs, max_blocks):
-    """CTAs of one to eight hashing warps (chosen by the handle's bound), with
+def test_hashing_widths_and_chunk_edges(bs, per_sm, more):
+    """CTAs of one, two, four and eight hashing warps, at both sides of each
+    switch (the handle's largest number of chunks against the SMs), with
     prompts of 0 to 130 blocks around the half (32) and the chunk (64), at
     every offset of a prompt's first token in its 16-byte word."""
     blocks = [0, 1, 2, 31, 32, 33, 63, 64, 65, 96, 127, 128, 129, 130]
+    chunks = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + more
+    max_blocks = 64 * (chunks - len(blocks) - 1)  # chunks = max_blocks / 64 + requests + 1
+    assert max_blocks >= sum(blocks)
     rng = np.random.default_rng(bs)
     docs = [rng.integers(0, W.VOCAB, size=130 * bs, dtype=np.int32) for _ in range(2)]
     steps = []
@@ -95,7 +99,7 @@ def test_hashing_widths_and_chunk_edges(bs, max_blocks):
         g, o, t = _prompts(lengths, [i % 2 for i in range(len(blocks))], 10 * bs + k, docs)
         steps.append(W.Step(k, k, g, o, t, None, None))
     gpu, orc = _pair(2500, bs, 2, "prefixshield", dict(rho=(1.0,), beta=(50.0,)), len(blocks), max_blocks * bs)
-    _run(gpu, orc, steps, 1, f"hash/{bs}/{max_blocks}")
+    _run(gpu, orc, steps, 1, f"hash/{bs}/{chunks}")
 
 
 @pytest.mark.parametrize("R,max_blocks", [(300, 4), (64, 8), (5, 512)])
@@ -139,23 +143,6 @@ def test_many_indebted_groups(G, contracts):
     assert _evicted(_run(gpu, orc, steps, label=f"debt/{G}")) > 0
 
 
-@pytest.mark.parametrize("gap", [0, 3000])
-@pytest.mark.parametrize("need", [40, 1500])
-def test_list_finish_widths(gap, need):
-    """A select's list: dense stamps leave a few members a segment; stamps
-    spread by many hits (gap steps' worth) leave hundreds in one bucket, which
-    a bitmap of the bucket ranks."""
-    rng = np.random.default_rng(gap + need)
-    doc = rng.integers(0, W.VOCAB, size=3000 * 16, dtype=np.int32)
-    other = rng.integers(0, W.VOCAB, size=2000 * 16, dtype=np.int32)
-    fresh = rng.integers(0, W.VOCAB, size=need * 16, dtype=np.int32)
-    seq = [doc, other] + [other] * (gap // 60) + [rng.integers(0, W.VOCAB, size=10 * 16, dtype=np.int32), fresh]
-    steps = [W.Step(k, k, np.zeros(1, np.int32), np.array([0, len(t)], np.int64), t, None, None)
-             for k, t in enumerate(seq)]
-    gpu, orc = _pair(5020, 16, 2, "prefixshield", dict(rho=(1.0,), beta=(100.0,)), 1, 3000 * 16)
-    assert _evicted(_run(gpu, orc, steps, 16, f"finish/{gap}/{need}")) >= need - 10
-
-
 def _aged(policy, old, new, need, gap, N=None):
     """A pool of `old` blocks, `gap` stamps, then `new` blocks, and a prompt
     that takes `need` victims among the old ones: a handle that served other
@@ -184,6 +171,24 @@ def _aged(policy, old, new, need, gap, N=None):
     return listed
 
 
+# Old blocks that fill the first bucket of the range, so the list holds all of
+# them: bitmaps of the bucket rank more than 128 of them where it is at most
+# 32768 stamps wide, counting ranks up to 512, byte digits the rest (up to 8192
+# in shared memory).
+@pytest.mark.parametrize("n,log2gap", [
+    (128, 24),                                                                # counting
+    (129, 24), (1024, 24), (1025, 24), (8192, 24), (16384, 29), (20000, 30),  # bitmaps: 5 to 1024 words
+    (129, 40), (512, 40),                                                     # no room for a bitmap: counting
+    (513, 40), (8192, 40),                                                    # digits, shared memory
+    (8193, 40), (20000, 31)])                                                 # digits, global memory
+@pytest.mark.parametrize("policy", ["lru", "prefixshield"])
+def test_list_finish(policy, n, log2gap):
+    """The split list at the edges of each way to finish it."""
+    for need in (1, n // 2, n):
+        listed = _aged(policy, n, max(3000, 5000 - n), need, 1 << log2gap)
+        assert policy != "lru" or listed == n  # (a debt phase's list is reset for its fallback)
+
+
 @pytest.mark.parametrize("policy", ["lru", "prefixshield"])
 @pytest.mark.parametrize("gap,most", [(1 << 22, 1 << 11), (1 << 24, 1 << 13), (1 << 26, 1 << 11), (1 << 27, 1 << 12)])
 def test_aged_range_is_cut_finely(policy, gap, most):
@@ -195,38 +200,45 @@ def test_aged_range_is_cut_finely(policy, gap, most):
         assert policy != "lru" or 1 <= listed <= most  # (a debt phase's list is reset for its fallback)
 
 
+@pytest.mark.parametrize("policy", ["staticquota", "prefixshield"])
 @pytest.mark.parametrize("N,G", [(4096, 64), (4097, 64), (9000, 65), (9000, 64)])
-def test_wide_buckets_at_the_rule_s_edges(N, G):
-    """Quota groups that select over ranges of mixed widths, at the largest
-    pool without and the smallest with 65536 buckets, and at 64 and 65 groups."""
+def test_wide_buckets_at_the_rule_s_edges(policy, N, G):
+    """Groups that select over ranges of mixed widths, at the largest pool
+    without and the smallest with 65536 buckets, and at 64 and 65 groups."""
     steps = W.fuzz_steps(N + G, G, 64, 30, docs_per_group=2, doc_blocks=max(2, N // G // 2), now_stride=2,
                          fresh_max_blocks=max(2, N // G // 2), block_size=2)
-    gpu, orc = _pair(N, 2, G, "staticquota", dict(rho=(2.0,), beta=(64.0,)), 64, 64 * 2 * (2 * (N // G) + 4))
+    gpu, orc = _pair(N, 2, G, policy, dict(rho=(2.0,), beta=(4.0,)), 64, 64 * 2 * (2 * (N // G) + 4))
     dev = torch.device("cuda")
     base = ctl_word(gpu, "stamp_base", torch.int64)
     for k, st in enumerate(steps):
         base.add_((0, 1 << 13, 1 << 24, 1 << 25, 1 << 33)[k % 5])
         assert gpu.step(st.now, *(torch.from_numpy(x).to(dev) for x in (st.groups, st.offsets, st.tokens))) == 0
         want = orc.step(st.now, st.groups, st.offsets, st.tokens)
-        compare_outputs(gpu.fetch(st.num_requests), want, f"wide/{N}/{G} step {k}")
+        compare_outputs(gpu.fetch(st.num_requests), want, f"wide/{policy}/{N}/{G} step {k}")
     assert _evicted(orc.stats()) > 0
 
 
 @pytest.mark.parametrize("N,blocks", [(64, 12), (2000, 400)])
 def test_s3fifo_ghost_readmission(N, blocks):
-    """Keys evicted and asked for again: ghost hits, among them keys that two
-    requests of a step share and keys that the same step trims."""
+    """Keys evicted and asked for again: ghost hits, and keys found in the ghost
+    that the same step's pushes trim before their block is inserted; some of
+    the step's new blocks are shared by its requests."""
     steps = W.fuzz_steps(N, 2, 5, 40, docs_per_group=3, doc_blocks=blocks, fresh_max_blocks=blocks // 4, now_stride=2)
-    gpu, orc = _pair(N, 16, 2, "s3fifo", dict(rho=(2.0,), beta=(6.0,)), 5, 5 * 16 * (2 * blocks + 2))
-    assert _evicted(_run(gpu, orc, steps, label=f"ghost/{N}")) > 0
-
-
-@pytest.mark.parametrize("policy", ["lru", "prefixshield"])
-def test_queue_logs_fill_and_compact(policy):
-    """Indexed queues whose logs run full again and again."""
-    steps = W.fuzz_steps(3, 3, 8, 300, docs_per_group=3, doc_blocks=6, fresh_max_blocks=1, now_stride=2)
-    gpu, orc = _pair(40, 16, 3, policy, dict(rho=(2.0,), beta=(6.0,), flags=O.FLAG_INDEXED_QUEUES), 8, 4096)
-    assert _evicted(_run(gpu, orc, steps, 25, f"queues/{policy}")) > 0
+    params, limits = dict(rho=(2.0,), beta=(6.0,)), (5, 5 * 16 * (2 * blocks + 2))
+    gpu, orc = _pair(N, 16, 2, "s3fifo", params, *limits)
+    _run(gpu, orc, steps, label=f"ghost/{N}")
+    again = O.OracleCache(N, 16, 2, "s3fifo", O.Params(**params))
+    hits = trimmed = 0
+    for st in steps:
+        ghost = set(zip(*(x.tolist() for x in again.export()["ghost"][:2])))
+        new = again.step(st.now, st.groups, st.offsets, st.tokens)["admitted_ids"]
+        e = again.export()
+        for b in new:
+            if (int(e["group"][b]), int(e["key"][b])) in ghost:
+                hits += int(e["s3q"][b] == 1)
+                trimmed += int(e["s3q"][b] == 0)
+    assert hits > 0 and trimmed > 0
+    assert int(orc.stats()[:, O.STAT_NAMES.index("instep_hit_blocks")].sum()) > 0
 
 
 def _queue_steps(gpu, orc, steps, before=None):
@@ -240,6 +252,16 @@ def _queue_steps(gpu, orc, steps, before=None):
         compare_outputs(gpu.fetch(st.num_requests), orc.step(st.now, st.groups, st.offsets, st.tokens), f"step {k}")
         buffers.add(int(ctl_word(gpu, "lg_buf", torch.int32).item()))
     return buffers
+
+
+@pytest.mark.parametrize("policy", ["lru", "prefixshield", "staticquota"])
+def test_queue_logs_fill_and_compact(policy):
+    """Indexed queues whose logs run full again and again."""
+    steps = W.fuzz_steps(3, 3, 8, 300, docs_per_group=3, doc_blocks=6, fresh_max_blocks=1, now_stride=2)
+    gpu, orc = _pair(40, 16, 3, policy, dict(rho=(2.0,), beta=(6.0,), flags=O.FLAG_INDEXED_QUEUES), 8, 4096)
+    assert _queue_steps(gpu, orc, steps) == {0, 1}
+    compare_state(gpu.export(), orc.export(), f"queues/{policy}")
+    assert np.array_equal(gpu.stats(), orc.stats()) and _evicted(orc.stats()) > 0
 
 
 def test_queue_barrier_starts_from_any_count():
@@ -334,6 +356,26 @@ def test_step_host_buffers(tokens_pinned, outputs_pinned, shift):
                "evicted_ids": out["evicted_ids"][:cnt[1]], "invalidated_ids": out["invalidated_ids"][:cnt[2]],
                "debt_raw": out["debt_raw"], "debt_norm": out["debt_norm"]}
         compare_outputs(got, orc.step(st.now, st.groups, st.offsets, st.tokens, st.contracts, st.prefixes), f"step {st.index}")
+
+
+@pytest.mark.parametrize("tokens", [1 << 21, (1 << 21) + 1])
+def test_step_host_tokens_at_the_kernel_s_limit(tokens):
+    """Page-locked tokens of 8 MB are read by a kernel, more are copied."""
+    from paper_2608_01657_gb300 import binding as B
+    rng = np.random.default_rng(tokens)
+    t = torch.from_numpy(rng.integers(0, W.VOCAB, size=tokens, dtype=np.int32)).pin_memory().numpy()
+    cut = tokens // 3
+    g = torch.zeros(2, dtype=torch.int32, pin_memory=True).numpy()
+    o = torch.tensor([0, cut, tokens], dtype=torch.int64).pin_memory().numpy()
+    gpu, orc = _pair(20000, 64, 2, "lru", dict(rho=(1.0,), beta=(1.0,)), 2, tokens)
+    for now in range(2):  # the second step hits what the first left
+        out = B.host_outputs(2, gpu.max_blocks, 2, pinned=True)
+        assert gpu.step_host(now, g, o, t, out=out)["rc"] == 0
+        cnt = out["counts"]
+        got = {"status": int(cnt[3]), **{k: out[k][:m] for k, m in (
+            ("hit_blocks", 2), ("admitted_blocks", 2), ("admitted_offsets", 3), ("admitted_ids", cnt[0]),
+            ("evicted_ids", cnt[1]), ("invalidated_ids", cnt[2]), ("debt_raw", 2), ("debt_norm", 2))}}
+        compare_outputs(got, orc.step(now, g, o, t), f"step {now}")
 
 
 @pytest.mark.parametrize("which", ["tokens", "admitted_ids"])

@@ -532,10 +532,10 @@ def test_parity_graph_replay_streams_and_timing(policy):
 
 
 def test_parity_long_split_list():
-    """A select whose split list is longer than one CTA finishes in shared
-    memory: one indebted group holds 12,001 Probationary and 12,000 Normal
-    candidates, and 5,425 victims fall inside the Probationary class, so the
-    first digit (the class byte) leaves the whole class on the list."""
+    """A select inside one class of many: one indebted group holds 12,001
+    Probationary and 12,000 Normal candidates, and 5,425 victims fall inside
+    the Probationary class, whose stamps alone are searched (the split list's
+    lengths are test_gpu_branches.py's)."""
     rng = np.random.default_rng(77)
     steps = []
     for k, (pid, nb) in enumerate([(7, 1), (7, 12000), (9, 12000), (11, 6000)]):
