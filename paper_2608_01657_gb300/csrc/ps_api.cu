@@ -524,6 +524,12 @@ int32_t ps_step(ps_handle_t* h, void* stream, int64_t now_ticks, int32_t num_req
 }
 
 namespace {
+// Page-locked tokens up to this size are read by a kernel, more are copied.  The
+// kernel saves a call of any size 2 to 9 us (measured a call, copies against
+// the kernel: 0.9 MB 114.8 -> 112.6 us, 3.6 MB 144.6 -> 138.9, 7.2 MB 169.7 ->
+// 163.7, 14.5 MB 220.3 -> 210.8, 41.5 MB 434.0 -> 425.1), and its 608 CTAs
+// hold their SMs for as long as the link takes: 40 us at 8 MB.  Past that the
+// gain is a few percent, and the SMs are left to the caller's other streams.
 constexpr size_t kHostKernelBytes = (size_t)8 << 20;
 // A refused copy leaves no error behind for the next call's launch check.
 inline bool copied(cudaError_t e) {

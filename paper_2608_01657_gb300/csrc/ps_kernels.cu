@@ -615,8 +615,9 @@ __device__ __forceinline__ bool hash_lookup_chunk(const DevState& s, Ctl* c, con
   // D_m of the lane's two blocks, then the inclusive scans of the affine maps
   // x -> Kc x + D, one per half
   uint64_t bA = 0, bB = 0;
-  // The halves' digests in a rolled loop: half the code, and no spills (155.2 ->
-  // 152.8 us a step at 2^20 blocks; it cost 0.4 us with a few chunks in all).
+  // The halves' digests in a rolled loop: half the code, and no spills with
+  // blocks of up to 16 tokens (32 and 64 spill 20 bytes a thread): 155.2 -> 152.8
+  // us a step at 2^20 blocks; it cost 0.4 us with a few chunks in all.
   // The second half's tokens are on their way from DRAM meanwhile (-> 152.2).
   if (lane < nbB) {
     const int32_t* src = s.in_tokens + o0 + (int64_t)mB * BS;
@@ -785,10 +786,11 @@ __device__ __forceinline__ bool hash_lookup_chunk(const DevState& s, Ctl* c, con
 // arrive about when its own does.  A chunk waits only on chunks of lower
 // tickets, each held by a running warp: the waits always make progress.
 // What bounds it: the memory system under scattered accesses, not instructions
-// (28% of issue slots) or DRAM bandwidth (20%).  Clocks read inside it at 2^20
-// blocks, in thousands of cycles a chunk: ticket 12, descriptor 3, tokens and
-// digests 13, scan 4, predecessors' totals 9, table 20, predecessors' misses 8,
-// pins and claims 14.  Measured there and not kept (155 us a step): tokens read
+// (34% of issue slots) or DRAM bandwidth (20%).  Clocks read inside it at 2^20
+// blocks, before the digests were rolled and the pins and claims fetched ahead,
+// in thousands of cycles a chunk: ticket 12, descriptor 3, tokens and digests 13,
+// scan 4, predecessors' totals 9, table 20, predecessors' misses 8, pins and
+// claims 14.  Measured there and not kept (155 us a step): tokens read
 // coalesced, four lanes a block (159 to 171), a CTA's first tickets drawn at
 // once (156), a warp's next ticket drawn early (158), two claims at a time
 // (155), no way loaded before its tag matched (155).
@@ -799,7 +801,7 @@ template <int BS>
 __global__ void __launch_bounds__(256, kHashCtasPerSm) k_hash_lookup(DevState s, int32_t* probe_out) {
   s = with_args(s);
   __shared__ uint32_t sk[BS + 2];                // the NH key words (read by every lane alike)
-  __shared__ uint64_t kc[2 * (kSegBlocks + 1)];  // Kc^j, then Kc^(32 t)
+  __shared__ uint64_t kc[2 * (kSegBlocks + 1)];  // Kc^j, then Kc^(64 t)
   Ctl* c = s.ctl;
   const int64_t nsegs = c->nsegs;  // none in a failed call
   for (int k = threadIdx.x; k < BS + 2; k += blockDim.x) sk[k] = s.key_words[k];

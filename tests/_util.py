@@ -215,8 +215,8 @@ def compare_state(got, want, where="", s3=False):
 # ---------------------------------------------------------------------------
 # A handle's device state, read (or set) where a test has to see which branch a
 # step took or to age a handle: the offsets come from the library's own header.
-LAYOUT = {"Ctl": ("step", "stamp_base", "lst_n", "bar", "lg_buf", "internal_error"),
-          "DevState": ("ctl", "lg_live")}
+LAYOUT = {"Ctl": ("stamp_base", "lst_n", "bar", "lg_buf"),
+          "DevState": ("lg_live",)}
 _layout = {}
 
 
