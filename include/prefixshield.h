@@ -79,7 +79,9 @@ enum {
  * every candidate.  Same victims, same results; lru, prefixshield and
  * staticquota (ignored for s3fifo, which keeps its own queues).  The
  * workspace grows by two buffers of 16 x (N + max_tokens / block_size)
- * entries of 12 bytes each, plus per-step scratch. */
+ * entries of 12 bytes each, plus per-step scratch.  The queues' compaction
+ * takes as many CTAs as fit at once on the SMs that ps_create() runs on: steps
+ * must not run on fewer (a smaller green context, a lower SM limit). */
 #define PS_FLAG_INDEXED_QUEUES 4u
 /* With PS_FLAG_INDEXED_QUEUES: the first scan round of a take covers a single
  * 1024-entry chunk, so a take that needs more finishes in the second round.
